@@ -91,6 +91,10 @@ __device__ __forceinline__ float val(float x) { return x; }
 __device__ __forceinline__ float val(Dual x) { return x.v; }
 __device__ __forceinline__ float tan_(float) { return 0.f; }
 __device__ __forceinline__ float tan_(Dual x) { return x.d; }
+// the plane a pass's parameter gradients come from: the value of a float pass, the tangent of
+// a Dual one
+__device__ __forceinline__ float plane_of(float x) { return x; }
+__device__ __forceinline__ float plane_of(Dual x) { return x.d; }
 
 // two-plane loads and stores: plane = floats per plane
 __device__ __forceinline__ void ldv(const float* p, size_t i, size_t, float& o) { o = p[i]; }
@@ -290,7 +294,7 @@ __global__ void __launch_bounds__(32 * kWarps) k_msg_bwd(MsgArgs a, const float*
                                                        const float* __restrict__ gmv, float* gA_out, float* gB_out,
                                                        float* gpos, float* wr_part) {
   __shared__ float sW[NR * NCOL];
-  __shared__ float sG[kWarps][2][NR * NCOL];
+  __shared__ float sG[kWarps][NR * NCOL];
   for (int k = threadIdx.x; k < NR * NCOL; k += blockDim.x) sW[k] = a.WR[k];
   __syncthreads();
   const int w = threadIdx.x >> 5, c = threadIdx.x & 31;
@@ -446,26 +450,20 @@ __global__ void __launch_bounds__(32 * kWarps) k_msg_bwd(MsgArgs a, const float*
       stT(gpos, 3 * size_t(i) + 2, pl, ldT<T>(gpos, 3 * size_t(i) + 2, pl) + gp.z);
     }
   }
-  // block partials of dL/dWR: [block][plane][NR][NCOL]
+  // block partials of dL/dWR [block][NR][NCOL]: the pass's plane (value, or tangent for Dual)
+  if (!wr_part) return;
   const int col1 = lo ? S + c : S + 2 * V + (c - V);
 #pragma unroll
   for (int k = 0; k < NR; ++k) {
-    sG[w][0][k * NCOL + c] = val(gw0[k]);
-    sG[w][1][k * NCOL + c] = tan_(gw0[k]);
-    sG[w][0][k * NCOL + col1] = val(gw1[k]);
-    sG[w][1][k * NCOL + col1] = tan_(gw1[k]);
-    if (lo) {
-      sG[w][0][k * NCOL + S + V + c] = val(gw2[k]);
-      sG[w][1][k * NCOL + S + V + c] = tan_(gw2[k]);
-    }
+    sG[w][k * NCOL + c] = plane_of(gw0[k]);
+    sG[w][k * NCOL + col1] = plane_of(gw1[k]);
+    if (lo) sG[w][k * NCOL + S + V + c] = plane_of(gw2[k]);
   }
   __syncthreads();
-  constexpr int kPlanes = sizeof(T) / sizeof(float);
-  for (int t = threadIdx.x; t < kPlanes * NR * NCOL; t += blockDim.x) {
-    const int pl = t / (NR * NCOL), k = t % (NR * NCOL);
+  for (int k = threadIdx.x; k < NR * NCOL; k += blockDim.x) {
     float acc = 0.f;
-    for (int ww = 0; ww < kWarps; ++ww) acc += sG[ww][pl][k];
-    wr_part[(size_t(blockIdx.x) * kPlanes + pl) * NR * NCOL + k] = acc;
+    for (int ww = 0; ww < kWarps; ++ww) acc += sG[ww][k];
+    wr_part[size_t(blockIdx.x) * NR * NCOL + k] = acc;
   }
 }
 
@@ -633,17 +631,17 @@ struct ReadoutBwdArgs {
   const float* gesr;    // [F] value and tangent: gesr[2 f], gesr[2 f + 1] (may be null)
   float* gH;            // [n][64]
   float* ghv;           // [n][3][16] (written)
-  float* part;          // [block][planes][kReadoutW]
+  float* part;          // [block][kReadoutW], the pass's plane (null: no parameter gradients)
   int n;
   size_t pln, plH, plV;
 };
 
 template <typename T>
 __global__ void __launch_bounds__(32 * kWarps) k_readout_bwd(ReadoutBwdArgs a) {
-  __shared__ float sp[kWarps][2][kReadoutW];
+  __shared__ float sp[kWarps][kReadoutW];
   const int w = threadIdx.x >> 5, c = threadIdx.x & 31;
   const int i = blockIdx.x * kWarps + w;
-  for (int k = c; k < kReadoutW; k += 32) sp[w][0][k] = sp[w][1][k] = 0.f;
+  for (int k = c; k < kReadoutW; k += 32) sp[w][k] = 0.f;
   __syncwarp();
   if (i < a.n) {
     const int f = a.frame_of[i];
@@ -657,13 +655,13 @@ __global__ void __launch_bounds__(32 * kWarps) k_readout_bwd(ReadoutBwdArgs a) {
     stT(a.gH, size_t(i) * 2 * S + c, a.plH, gHq);
     stT(a.gH, size_t(i) * 2 * S + S + c, a.plH, gHe);
     const T pwq = gqt * siluT(hq), pwe = ge * siluT(he);
-    sp[w][0][c] = val(pwq);                 sp[w][1][c] = tan_(pwq);
-    sp[w][0][S + c] = val(pwe);             sp[w][1][S + c] = tan_(pwe);
-    sp[w][0][2 * S + c] = val(gHq);         sp[w][1][2 * S + c] = tan_(gHq);
-    sp[w][0][3 * S + c] = val(gHe);         sp[w][1][3 * S + c] = tan_(gHe);
+    sp[w][c] = plane_of(pwq);
+    sp[w][S + c] = plane_of(pwe);
+    sp[w][2 * S + c] = plane_of(gHq);
+    sp[w][3 * S + c] = plane_of(gHe);
     if (c == 0) {
-      sp[w][0][4 * S] = val(gqt);           sp[w][1][4 * S] = tan_(gqt);
-      sp[w][0][4 * S + 1] = val(ge);        sp[w][1][4 * S + 1] = tan_(ge);
+      sp[w][4 * S] = plane_of(gqt);
+      sp[w][4 * S + 1] = plane_of(ge);
     }
     if (c < V) {
       T gw = 0.f;
@@ -674,113 +672,191 @@ __global__ void __launch_bounds__(32 * kWarps) k_readout_bwd(ReadoutBwdArgs a) {
         stT(a.ghv, k, a.plV, gm * a.P[oWmu + c]);
         gw += gm * ldT<T>(a.hv, k, a.plV);
       }
-      sp[w][0][4 * S + 2 + c] = val(gw);
-      sp[w][1][4 * S + 2 + c] = tan_(gw);
+      sp[w][4 * S + 2 + c] = plane_of(gw);
     }
   }
+  if (!a.part) return;
   __syncthreads();
-  constexpr int kPlanes = sizeof(T) / sizeof(float);
-  for (int t = threadIdx.x; t < kPlanes * kReadoutW; t += blockDim.x) {
-    const int pl = t / kReadoutW, k = t % kReadoutW;
+  for (int k = threadIdx.x; k < kReadoutW; k += blockDim.x) {
     float acc = 0.f;
-    for (int ww = 0; ww < kWarps; ++ww) acc += sp[ww][pl][k];
-    a.part[(size_t(blockIdx.x) * kPlanes + pl) * kReadoutW + k] = acc;
+    for (int ww = 0; ww < kWarps; ++ww) acc += sp[ww][k];
+    a.part[size_t(blockIdx.x) * kReadoutW + k] = acc;
   }
 }
 
-// Per-block partials of dL/d emb [2][32] from the layer-0 input cotangent g_hs.
-template <typename T>
-__global__ void k_emb_bwd(int n, const int* __restrict__ species, const float* __restrict__ ghs, size_t plS,
-                          float* part) {
-  // block of 256 threads = 8 ion slots x 32 channels; each block covers 8 * 64 ions
-  __shared__ float sp[8][2][2 * S];
+// ---------------------------------------------------------------------------------------
+// parameter gradients
+//
+// Every parameter gradient of a backward pass is a sum over ions, formed in two launches at
+// the end of the pass: k_wgrad (all channel-mixing matrices and the embedding, one block per
+// matrix and chunk of rows) writes per-block partials next to those the readout and message
+// kernels left, and k_reduce adds the partials of every parameter in a fixed order (float64).
+// A pass wants one plane only -- the value plane of a float pass, the tangent plane of a Dual
+// one -- so only that plane is formed. Bound: k_wgrad shared-memory reads and FMAs (520 M FMA
+// for 32 frames of 512 ions), k_reduce the latency of the partials' loads. One thread per
+// parameter walking up to 2048 partials in a row, in one to three blocks per matrix, took
+// 1.83 ms of that step's 4.31 ms, and nine separate weight-gradient launches 0.28 ms; with
+// thirty-two threads per parameter and one launch for all of them the step takes 2.87 ms.
+// ---------------------------------------------------------------------------------------
+constexpr int kWgThreads = 256;
+constexpr int kWgSub = 32;       // rows staged at a time
+constexpr int kWgRows = 128;     // rows per block of the scalar-channel products and the embedding
+constexpr int kWgRowsV = 256;    // rows per block of the vector-channel products (3 rows per ion)
+
+enum WgKind { kWgU, kWgY, kWgA, kWgB, kWgH, kWgEmb };
+
+struct WgJob {
+  const float* X;      // [rows][K] (embedding: unused)
+  const float* G;      // [rows][N]
+  size_t plX, plG;     // tangent plane offsets
+  float* part;         // [blocks][K N]
+  int rows, kind, first;   // first: the job's first block of the launch
+};
+constexpr int kWgMaxJobs = 10;
+struct WgJobs {
+  WgJob job[kWgMaxJobs];
+  int n;
+  const int* species;
+};
+
+// Staged column k, row r of a [K][kWgSub] tile: 16-byte groups of four rows permuted by a
+// function of k that is distinct over eight consecutive columns (the products' reads) and over
+// eight columns four apart (the transposing stores), so neither conflicts on the banks.
+__device__ __forceinline__ int wg_group(int k, int g) { return k * kWgSub + 4 * (g ^ (((k >> 2) + 2 * (k & 3)) & 7)); }
+
+template <int C>
+__device__ __forceinline__ void wg_stage(const float* __restrict__ src, int r0, int rows, float* dst) {
+  for (int e = threadIdx.x; e < kWgSub * C / 4; e += kWgThreads) {
+    const int r = e / (C / 4), k = 4 * (e % (C / 4));
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (r0 + r < rows) v = __ldg(reinterpret_cast<const float4*>(src + size_t(r0 + r) * C + k));
+    const int g = r >> 2, o = r & 3;
+    dst[wg_group(k, g) + o] = v.x;
+    dst[wg_group(k + 1, g) + o] = v.y;
+    dst[wg_group(k + 2, g) + o] = v.z;
+    dst[wg_group(k + 3, g) + o] = v.w;
+  }
+}
+
+__device__ __forceinline__ float dot4(const float4& a, const float4& b, float acc) {
+  acc = fmaf(a.x, b.x, acc);
+  acc = fmaf(a.y, b.y, acc);
+  acc = fmaf(a.z, b.z, acc);
+  return fmaf(a.w, b.w, acc);
+}
+
+// One block of a weight gradient: part[k][n] = sum over its ROWS rows of X[r][k] G[r][n]
+// (PL = 1), or of X'[r][k] G[r][n] + X[r][k] G'[r][n] (PL = 2). Each thread owns TK x TN
+// outputs; where those are fewer than the threads, RG groups of threads share the rows.
+template <int PL, int K, int N, int TK, int TN, int ROWS>
+__device__ __forceinline__ void wgrad_block(const WgJob& J, int blk, float* sm) {
+  constexpr int NN = N / TN, NK = K / TK, NTH = NN * NK, RG = kWgThreads / NTH;
+  static_assert(NTH * RG == kWgThreads && PL * (K + N) * kWgSub >= (RG - 1) * K * N, "thread split");
+  float* sX = sm;
+  float* sG = sm + PL * K * kWgSub;
+  const int t = threadIdx.x % NTH, rg = threadIdx.x / NTH;
+  const int n0 = t % NN, k0 = t / NN;
+  float acc[TK][TN];
+#pragma unroll
+  for (int i = 0; i < TK; ++i)
+#pragma unroll
+    for (int j = 0; j < TN; ++j) acc[i][j] = 0.f;
+  const int end = min(J.rows, (blk + 1) * ROWS);
+  for (int r0 = blk * ROWS; r0 < end; r0 += kWgSub) {
+    __syncthreads();
+    wg_stage<K>(J.X, r0, end, sX);
+    wg_stage<N>(J.G, r0, end, sG);
+    if (PL > 1) {
+      wg_stage<K>(J.X + J.plX, r0, end, sX + K * kWgSub);
+      wg_stage<N>(J.G + J.plG, r0, end, sG + N * kWgSub);
+    }
+    __syncthreads();
+#pragma unroll 2
+    for (int g = rg; g < kWgSub / 4; g += RG) {
+      float4 x[PL][TK], y[PL][TN];
+#pragma unroll
+      for (int p = 0; p < PL; ++p) {
+#pragma unroll
+        for (int i = 0; i < TK; ++i)
+          x[p][i] = *reinterpret_cast<const float4*>(sX + p * K * kWgSub + wg_group(k0 + NK * i, g));
+#pragma unroll
+        for (int j = 0; j < TN; ++j)
+          y[p][j] = *reinterpret_cast<const float4*>(sG + p * N * kWgSub + wg_group(n0 + NN * j, g));
+      }
+#pragma unroll
+      for (int i = 0; i < TK; ++i)
+#pragma unroll
+        for (int j = 0; j < TN; ++j) {
+          if (PL > 1) acc[i][j] = dot4(x[0][i], y[PL - 1][j], dot4(x[PL - 1][i], y[0][j], acc[i][j]));
+          else acc[i][j] = dot4(x[0][i], y[0][j], acc[i][j]);
+        }
+    }
+  }
+  if (RG > 1) {
+    __syncthreads();
+    if (rg > 0) {
+#pragma unroll
+      for (int i = 0; i < TK; ++i)
+#pragma unroll
+        for (int j = 0; j < TN; ++j) sm[(rg - 1) * K * N + (k0 + NK * i) * N + n0 + NN * j] = acc[i][j];
+    }
+    __syncthreads();
+  }
+  if (rg == 0) {
+    float* out = J.part + size_t(blk) * K * N;
+#pragma unroll
+    for (int i = 0; i < TK; ++i)
+#pragma unroll
+      for (int j = 0; j < TN; ++j) {
+        const int o = (k0 + NK * i) * N + n0 + NN * j;
+        float v = acc[i][j];
+        for (int q = 1; q < RG; ++q) v += sm[(q - 1) * K * N + o];
+        out[o] = v;
+      }
+  }
+}
+
+// dL/d emb [2][32] over kWgRows ions: the layer-0 input cotangent added per species.
+__device__ __forceinline__ void emb_block(const WgJob& J, const int* __restrict__ species, int blk, size_t pl,
+                                          float* sm) {
   const int slot = threadIdx.x >> 5, c = threadIdx.x & 31;
-  T a0 = 0.f, a1 = 0.f;
-  for (int i = blockIdx.x * 512 + slot; i < min(n, int(blockIdx.x + 1) * 512); i += 8) {
-    const T g = ldT<T>(ghs, size_t(i) * S + c, plS);
+  float a0 = 0.f, a1 = 0.f;
+#pragma unroll 4
+  for (int i = blk * kWgRows + slot; i < min(J.rows, (blk + 1) * kWgRows); i += kWgThreads / 32) {
+    const float g = J.G[size_t(i) * S + c + pl];
     if (species[i] == 0) a0 += g;
     else a1 += g;
   }
-  sp[slot][0][c] = val(a0);      sp[slot][1][c] = tan_(a0);
-  sp[slot][0][S + c] = val(a1);  sp[slot][1][S + c] = tan_(a1);
+  sm[slot * 2 * S + c] = a0;
+  sm[slot * 2 * S + S + c] = a1;
   __syncthreads();
-  constexpr int kPlanes = sizeof(T) / sizeof(float);
-  for (int t = threadIdx.x; t < kPlanes * 2 * S; t += blockDim.x) {
-    const int pl = t / (2 * S), k = t % (2 * S);
-    float acc = 0.f;
-    for (int s2 = 0; s2 < 8; ++s2) acc += sp[s2][pl][k];
-    part[(size_t(blockIdx.x) * kPlanes + pl) * 2 * S + k] = acc;
+  if (threadIdx.x < 2 * S) {
+    float v = 0.f;
+    for (int q = 0; q < kWgThreads / 32; ++q) v += sm[q * 2 * S + threadIdx.x];
+    J.part[size_t(blk) * 2 * S + threadIdx.x] = v;
   }
 }
 
-// Per-block partials of the weight gradient G[K][N] = sum_rows X[r][k] Gy[r][n] over 128-row
-// chunks (X: [rows][K], Gy: [rows][N]), staged 32 rows at a time; for Dual also the tangent
-// sum X' Gy + X Gy'.
-constexpr int kWgRows = 128;
-constexpr int kWgSub = 32;
-template <typename T, int K, int N>
-__global__ void __launch_bounds__(256) k_wgrad(int rows, const float* __restrict__ X, const float* __restrict__ Gy,
-                                              size_t plX, size_t plG, float* part) {
-  constexpr int kPlanes = sizeof(T) / sizeof(float);
-  constexpr int kOut = (K * N + 255) / 256;
-  __shared__ float sX[kPlanes][kWgSub][K];
-  __shared__ float sGy[kPlanes][kWgSub][N + 1];
-  float a[kOut], b[kOut];
-#pragma unroll
-  for (int u = 0; u < kOut; ++u) a[u] = b[u] = 0.f;
-  for (int r0 = blockIdx.x * kWgRows; r0 < min(rows, int(blockIdx.x + 1) * kWgRows); r0 += kWgSub) {
-    __syncthreads();
-    for (int t = threadIdx.x; t < kWgSub * K; t += blockDim.x) {
-      const int r = t / K, k = t % K;
-      const bool ok = r0 + r < rows;
-      sX[0][r][k] = ok ? X[size_t(r0 + r) * K + k] : 0.f;
-      if (kPlanes > 1) sX[kPlanes - 1][r][k] = ok ? X[size_t(r0 + r) * K + k + plX] : 0.f;
-    }
-    for (int t = threadIdx.x; t < kWgSub * N; t += blockDim.x) {
-      const int r = t / N, k = t % N;
-      const bool ok = r0 + r < rows;
-      sGy[0][r][k] = ok ? Gy[size_t(r0 + r) * N + k] : 0.f;
-      if (kPlanes > 1) sGy[kPlanes - 1][r][k] = ok ? Gy[size_t(r0 + r) * N + k + plG] : 0.f;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int u = 0; u < kOut; ++u) {
-      const int o = threadIdx.x + 256 * u;
-      if (o < K * N) {
-        const int k = o / N, nn = o % N;
-        for (int r = 0; r < kWgSub; ++r) {
-          a[u] += sX[0][r][k] * sGy[0][r][nn];
-          if (kPlanes > 1) b[u] += sX[kPlanes - 1][r][k] * sGy[0][r][nn] + sX[0][r][k] * sGy[kPlanes - 1][r][nn];
-        }
-      }
-    }
-  }
-#pragma unroll
-  for (int u = 0; u < kOut; ++u) {
-    const int o = threadIdx.x + 256 * u;
-    if (o < K * N) {
-      part[(size_t(blockIdx.x) * kPlanes) * K * N + o] = a[u];
-      if (kPlanes > 1) part[(size_t(blockIdx.x) * kPlanes + 1) * K * N + o] = b[u];
-    }
+__host__ __device__ constexpr int wg_rows(int kind) { return kind == kWgY || kind == kWgB ? kWgRowsV : kWgRows; }
+
+template <int PL>
+__global__ void __launch_bounds__(kWgThreads) k_wgrad(WgJobs jobs) {
+  __shared__ __align__(16) float sm[PL * 96 * kWgSub];
+  int u = 0;
+  while (u + 1 < jobs.n && int(blockIdx.x) >= jobs.job[u + 1].first) ++u;
+  const WgJob& J = jobs.job[u];
+  const int blk = int(blockIdx.x) - J.first;
+  switch (J.kind) {
+    case kWgU: wgrad_block<PL, S + V, S + V, 3, 3, kWgRows>(J, blk, sm); break;
+    case kWgA: wgrad_block<PL, S, S + V, 2, 3, kWgRows>(J, blk, sm); break;
+    case kWgH: wgrad_block<PL, S, 2 * S, 2, 4, kWgRows>(J, blk, sm); break;
+    case kWgY: wgrad_block<PL, 2 * V, V, 2, 2, kWgRowsV>(J, blk, sm); break;
+    case kWgB: wgrad_block<PL, V, 2 * V, 2, 2, kWgRowsV>(J, blk, sm); break;
+    default: emb_block(J, jobs.species, blk, PL > 1 ? J.plG : 0, sm); break;
   }
 }
 
-// out[plane][w] (+)= sum over blocks b of part[b][plane][w] (fixed order); planes selected by
-// plane_out: the value plane goes to out_v, the tangent plane to out_t (either may be null).
-__global__ void k_reduce_parts(const float* __restrict__ part, int nblk, int planes, int width, float* out_v,
-                               float* out_t, int accumulate) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= planes * width) return;
-  const int pl = t / width, k = t % width;
-  double acc = 0.0;
-  for (int b = 0; b < nblk; ++b) acc += part[(size_t(b) * planes + pl) * width + k];
-  float* out = pl == 0 ? out_v : out_t;
-  if (!out) return;
-  out[k] = accumulate ? out[k] + float(acc) : float(acc);
-}
-
-// Scatter the readout partial sums (wq, wE, bh, bq, bE, wmu) into a parameter-gradient
-// vector: reduced[w] -> param index.
+// Parameter index of readout partial k (wq, wE, bh, bq, bE, wmu).
 __device__ __forceinline__ int readout_param(int k) {
   if (k < S) return oWq + k;
   if (k < 2 * S) return oWE + (k - S);
@@ -789,17 +865,48 @@ __device__ __forceinline__ int readout_param(int k) {
   if (k == 4 * S + 1) return oBE;
   return oWmu + (k - 4 * S - 2);
 }
-__global__ void k_reduce_readout(const float* __restrict__ part, int nblk, int planes, float* out_v, float* out_t,
-                                 int accumulate) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= planes * kReadoutW) return;
-  const int pl = t / kReadoutW, k = t % kReadoutW;
+
+struct RedJob {
+  const float* part;   // [nblk][width]
+  int nblk, width;
+  int out;             // parameter offset; -1: the readout's (readout_param)
+  int first;           // first block of the launch
+};
+constexpr int kRedMaxJobs = 14;
+struct RedJobs {
+  RedJob job[kRedMaxJobs];
+  int n;
+};
+
+// grad[w] (+)= sum over b of part[b][w]: 32 consecutive parameters per block, one per lane;
+// warp s adds the partials b = s, s + 32, ... in float64, then the 32 sums are added in order.
+__global__ void __launch_bounds__(1024) k_reduce(RedJobs jobs, float* __restrict__ grad, int accumulate) {
+  __shared__ double sum[32][33];
+  int u = 0;
+  while (u + 1 < jobs.n && int(blockIdx.x) >= jobs.job[u + 1].first) ++u;
+  const RedJob& J = jobs.job[u];
+  const int lane = threadIdx.x & 31, slice = threadIdx.x >> 5;
+  const int k = (int(blockIdx.x) - J.first) * 32 + lane;
   double acc = 0.0;
-  for (int b = 0; b < nblk; ++b) acc += part[(size_t(b) * planes + pl) * kReadoutW + k];
-  float* out = pl == 0 ? out_v : out_t;
-  if (!out) return;
-  const int o = readout_param(k);
-  out[o] = accumulate ? out[o] + float(acc) : float(acc);
+  if (k < J.width) {
+    const float* p = J.part + k;
+    for (int b0 = slice; b0 < J.nblk; b0 += 8 * 32) {   // eight loads in flight
+      float v[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) v[q] = b0 + 32 * q < J.nblk ? __ldg(p + size_t(b0 + 32 * q) * J.width) : 0.f;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) acc += double(v[q]);
+    }
+  }
+  sum[slice][lane] = acc;
+  __syncthreads();
+  if (slice == 0 && k < J.width) {
+    double t = 0.0;
+#pragma unroll 8
+    for (int q = 0; q < 32; ++q) t += sum[q][lane];
+    const int o = J.out < 0 ? readout_param(k) : J.out + k;
+    grad[o] = accumulate ? grad[o] + float(t) : float(t);
+  }
 }
 
 // ---------------------------------------------------------------------------------------
@@ -925,8 +1032,10 @@ struct gbnet_s {
   float *hs[3] = {}, *hv[3] = {}, *A[2] = {}, *B[2] = {}, *ms[2] = {}, *mv[2] = {}, *U[2] = {}, *Y[2] = {};
   float *H = nullptr, *qt = nullptr, *ei = nullptr, *q = nullptr, *mu = nullptr;
   // backward scratch
-  float *ghs = nullptr, *ghv = nullptr, *gA = nullptr, *gB = nullptr, *gms = nullptr, *gmv = nullptr,
-        *gU = nullptr, *gY = nullptr, *gH = nullptr, *gpos = nullptr, *gq = nullptr, *gmu = nullptr,
+  // (the products' cotangents of both layers stay until the pass's weight gradients are formed)
+  float *gA[2] = {}, *gB[2] = {}, *gU[2] = {}, *gY[2] = {};
+  float *ghs = nullptr, *ghv = nullptr, *gms = nullptr, *gmv = nullptr, *gH = nullptr, *gpos = nullptr,
+        *gq = nullptr, *gmu = nullptr,
         *gq_mean = nullptr, *gesr = nullptr, *part = nullptr;
   size_t part_cap = 0;
   // loss scratch
@@ -1016,32 +1125,86 @@ int forward_pass(gbnet_t net, cudaStream_t s, const float* pos, const float* dpo
   return PME_OK;
 }
 
-template <typename T, int K, int N>
-int wgrad(gbnet_t net, cudaStream_t s, int rows, const float* X, const float* Gy, int poff, float* gv, float* gt,
-          bool acc) {
+// Offsets (floats) of the partial sums of one backward pass over n ions.
+struct PartLayout {
+  size_t readout, wr[2], u[2], y[2], a[2], b[2], h, emb, total;
+};
+PartLayout part_layout(int n) {
+  const size_t ion = blocks_for(size_t(n), kWarps), row = blocks_for(size_t(n), kWgRows),
+               rowv = blocks_for(3 * size_t(n), kWgRowsV);
+  PartLayout L;
+  size_t o = 0;
+  auto take = [&](size_t blocks, size_t width) {
+    const size_t at = o;
+    o += blocks * width;
+    return at;
+  };
+  L.readout = take(ion, kReadoutW);
+  for (int t = 0; t < 2; ++t) {
+    L.wr[t] = take(ion, NR * NCOL);
+    L.u[t] = take(row, (S + V) * (S + V));
+    L.y[t] = take(rowv, 2 * V * V);
+    L.a[t] = take(row, S * (S + V));
+    L.b[t] = take(rowv, V * 2 * V);
+  }
+  L.h = take(row, S * 2 * S);
+  L.emb = take(row, 2 * S);
+  L.total = o;
+  return L;
+}
+
+// The parameter gradients of a backward pass whose cotangents are in place: grad (+)= ...
+template <typename T>
+int param_grads(gbnet_t net, cudaStream_t s, float* grad, bool acc) {
   constexpr int planes = sizeof(T) / sizeof(float);
-  if (rows == 0) return PME_OK;
-  const int nblk = (rows + kWgRows - 1) / kWgRows;
-  k_wgrad<T, K, N><<<nblk, 256, 0, s>>>(rows, X, Gy, size_t(rows) * K, size_t(rows) * N, net->part);
+  const int n = net->n;
+  const PartLayout L = part_layout(n);
+  float* P = net->part;
+  WgJobs wj{};
+  RedJobs rj{};
+  int wblocks = 0, rblocks = 0;
+  auto red = [&](const float* part, int nblk, int width, int out) {
+    rj.job[rj.n++] = RedJob{part, nblk, width, out, rblocks};
+    rblocks += int(blocks_for(size_t(width), 32));
+  };
+  auto wg = [&](int kind, int rows, const float* X, int K, const float* G, int N, size_t off, int out) {
+    const int nblk = int(blocks_for(size_t(rows), wg_rows(kind)));
+    wj.job[wj.n++] = WgJob{X, G, size_t(rows) * K, size_t(rows) * N, P + off, rows, kind, wblocks};
+    wblocks += nblk;
+    red(P + off, nblk, K * N, out);
+  };
+  for (int t = 1; t >= 0; --t) {
+    const int base = oLayer0 + t * kLayerSize;
+    wg(kWgU, n, net->ms[t], S + V, net->gU[t], S + V, L.u[t], base + oWU);
+    wg(kWgA, n, net->hs[t], S, net->gA[t], S + V, L.a[t], base + oWA);
+    wg(kWgY, 3 * n, net->mv[t], 2 * V, net->gY[t], V, L.y[t], base + oWY);
+    wg(kWgB, 3 * n, net->hv[t], V, net->gB[t], 2 * V, L.b[t], base + oWB);
+    red(P + L.wr[t], int(blocks_for(size_t(n), kWarps)), NR * NCOL, base + oWR);
+  }
+  wg(kWgH, n, net->hs[2], S, net->gH, 2 * S, L.h, oWh);
+  wg(kWgEmb, n, nullptr, 2, net->ghs, S, L.emb, oEmb);
+  rj.job[rj.n - 1].width = 2 * S;   // two species rows of S channels
+  red(P + L.readout, int(blocks_for(size_t(n), kWarps)), kReadoutW, -1);
+  wj.species = net->species;
+  k_wgrad<planes><<<wblocks, kWgThreads, 0, s>>>(wj);
   NET_LAUNCHED(net);
-  k_reduce_parts<<<blocks_for(size_t(planes) * K * N, 256), 256, 0, s>>>(
-      net->part, nblk, planes, K * N, gv ? gv + poff : nullptr, gt ? gt + poff : nullptr, acc ? 1 : 0);
+  k_reduce<<<rblocks, 1024, 0, s>>>(rj, grad, acc ? 1 : 0);
   NET_LAUNCHED(net);
   return PME_OK;
 }
 
 // Backward pass of the last forward_pass<T>. Seeds: gq [planes][n], gmu [planes][n][3] (each
 // may be null), gesr_f [F][2] float (value, tangent). Outputs: gpos [planes][n][3] (net->gpos,
-// written), parameter gradients: value plane -> gv, tangent plane -> gt (either null to skip;
-// both null skips every weight-gradient launch).
+// written) and, unless grad is null, the parameter gradients: the value plane of a float pass,
+// the tangent plane of a Dual one (written, or added when acc).
 template <typename T>
 int backward_pass(gbnet_t net, cudaStream_t s, const float* pos, const float* dpos, const float* gq,
-                  const float* gmu, const float* gesr_f, float* gv, float* gt, bool acc) {
+                  const float* gmu, const float* gesr_f, float* grad, bool acc) {
   constexpr int planes = sizeof(T) / sizeof(float);
   const int n = net->n;
   const size_t plS = size_t(n) * S, plV = size_t(n) * 3 * V, pl48 = size_t(n) * (S + V),
                pl96 = size_t(n) * 3 * 2 * V, pl64 = size_t(n) * 2 * S;
-  const bool params = gv || gt;
+  const PartLayout L = part_layout(n);
   int st;
   if ((st = cuda_ok(net, cudaMemsetAsync(net->gpos, 0, sizeof(float) * planes * 3 * size_t(n), s), "memset")))
     return st;
@@ -1061,7 +1224,7 @@ int backward_pass(gbnet_t net, cudaStream_t s, const float* pos, const float* dp
   ra.gesr = gesr_f;
   ra.gH = net->gH;
   ra.ghv = net->ghv;
-  ra.part = net->part;
+  ra.part = grad ? net->part + L.readout : nullptr;
   ra.n = n;
   ra.pln = size_t(n);
   ra.plH = pl64;
@@ -1069,46 +1232,21 @@ int backward_pass(gbnet_t net, cudaStream_t s, const float* pos, const float* dp
   const int nb_ion = int(blocks_for(n, kWarps));
   k_readout_bwd<T><<<nb_ion, 32 * kWarps, 0, s>>>(ra);
   NET_LAUNCHED(net);
-  if (params) {
-    k_reduce_readout<<<blocks_for(size_t(planes) * kReadoutW, 256), 256, 0, s>>>(net->part, nb_ion, planes, gv, gt,
-                                                                                 acc ? 1 : 0);
-    NET_LAUNCHED(net);
-  }
   if ((st = mix(net, s, planes * n, 2 * S, S, net->gH, 8, false, net->ghs, false))) return st;
-  if (params && (st = wgrad<T, S, 2 * S>(net, s, n, net->hs[2], net->gH, oWh, gv, gt, acc))) return st;
   for (int t = 1; t >= 0; --t) {
-    const int base = oLayer0 + t * kLayerSize;
-    k_update_bwd<T><<<blocks_for(size_t(n) * S, 256), 256, 0, s>>>(n, net->U[t], net->Y[t], net->ghs, net->ghv, net->gU,
-                                                                   net->gY, pl48, plV, plS, plV);
+    k_update_bwd<T><<<blocks_for(size_t(n) * S, 256), 256, 0, s>>>(n, net->U[t], net->Y[t], net->ghs, net->ghv,
+                                                                   net->gU[t], net->gY[t], pl48, plV, plS, plV);
     NET_LAUNCHED(net);
-    if ((st = mix(net, s, planes * n, S + V, S + V, net->gU, 4 * t + 2, false, net->gms, false))) return st;
-    if ((st = mix(net, s, planes * 3 * n, V, 2 * V, net->gY, 4 * t + 3, false, net->gmv, false))) return st;
-    if (params && (st = wgrad<T, S + V, S + V>(net, s, n, net->ms[t], net->gU, base + oWU, gv, gt, acc))) return st;
-    if (params && (st = wgrad<T, 2 * V, V>(net, s, 3 * n, net->mv[t], net->gY, base + oWY, gv, gt, acc))) return st;
+    if ((st = mix(net, s, planes * n, S + V, S + V, net->gU[t], 4 * t + 2, false, net->gms, false))) return st;
+    if ((st = mix(net, s, planes * 3 * n, V, 2 * V, net->gY[t], 4 * t + 3, false, net->gmv, false))) return st;
     const MsgArgs a = msg_args<T>(net, t, pos, dpos);
-    k_msg_bwd<T><<<nb_ion, 32 * kWarps, 0, s>>>(a, net->A[t], net->B[t], net->gms, net->gmv, net->gA, net->gB,
-                                               net->gpos, net->part);
+    k_msg_bwd<T><<<nb_ion, 32 * kWarps, 0, s>>>(a, net->A[t], net->B[t], net->gms, net->gmv, net->gA[t], net->gB[t],
+                                               net->gpos, grad ? net->part + L.wr[t] : nullptr);
     NET_LAUNCHED(net);
-    if (params) {
-      k_reduce_parts<<<blocks_for(size_t(planes) * NR * NCOL, 256), 256, 0, s>>>(
-          net->part, nb_ion, planes, NR * NCOL, gv ? gv + base + oWR : nullptr, gt ? gt + base + oWR : nullptr,
-          acc ? 1 : 0);
-      NET_LAUNCHED(net);
-    }
-    if ((st = mix(net, s, planes * n, S + V, S, net->gA, 4 * t + 0, false, net->ghs, true))) return st;
-    if ((st = mix(net, s, planes * 3 * n, 2 * V, V, net->gB, 4 * t + 1, false, net->ghv, true))) return st;
-    if (params && (st = wgrad<T, S, S + V>(net, s, n, net->hs[t], net->gA, base + oWA, gv, gt, acc))) return st;
-    if (params && (st = wgrad<T, V, 2 * V>(net, s, 3 * n, net->hv[t], net->gB, base + oWB, gv, gt, acc))) return st;
+    if ((st = mix(net, s, planes * n, S + V, S, net->gA[t], 4 * t + 0, false, net->ghs, true))) return st;
+    if ((st = mix(net, s, planes * 3 * n, 2 * V, V, net->gB[t], 4 * t + 1, false, net->ghv, true))) return st;
   }
-  if (params) {
-    const int nb = (n + 511) / 512;
-    k_emb_bwd<T><<<nb, 256, 0, s>>>(n, net->species, net->ghs, plS, net->part);
-    NET_LAUNCHED(net);
-    k_reduce_parts<<<blocks_for(size_t(planes) * 2 * S, 256), 256, 0, s>>>(net->part, nb, planes, 2 * S,
-                                                                           gv ? gv + oEmb : nullptr,
-                                                                           gt ? gt + oEmb : nullptr, acc ? 1 : 0);
-    NET_LAUNCHED(net);
-  }
+  if (grad && (st = param_grads<T>(net, s, grad, acc))) return st;
   (void)pl96;
   return PME_OK;
 }
@@ -1218,23 +1356,22 @@ int gbnet_create(gbnet_t* out, int max_ions, int max_frames) {
   A(&net->mu, 2 * f * N * 3);
   A(&net->ghs, 2 * f * N * S);
   A(&net->ghv, 2 * f * N * 3 * V);
-  A(&net->gA, 2 * f * N * (S + V));
-  A(&net->gB, 2 * f * N * 3 * 2 * V);
+  for (int t = 0; t < 2; ++t) {
+    A(&net->gA[t], 2 * f * N * (S + V));
+    A(&net->gB[t], 2 * f * N * 3 * 2 * V);
+    A(&net->gU[t], 2 * f * N * (S + V));
+    A(&net->gY[t], 2 * f * N * 3 * V);
+  }
   A(&net->gms, 2 * f * N * (S + V));
   A(&net->gmv, 2 * f * N * 3 * 2 * V);
-  A(&net->gU, 2 * f * N * (S + V));
-  A(&net->gY, 2 * f * N * 3 * V);
   A(&net->gH, 2 * f * N * 2 * S);
   A(&net->gpos, 2 * f * N * 3);
   A(&net->gq, 2 * f * N);
   A(&net->gmu, 2 * f * N * 3);
   A(&net->gq_mean, 2 * f * max_frames);
   A(&net->gesr, 2 * f * max_frames);
-  // partial sums: the largest of the weight-gradient, message and readout reductions
-  const size_t wg = size_t((3 * N + kWgRows - 1) / kWgRows) * 2 * (S + V) * (S + V);
-  const size_t ms = size_t((N + kWarps - 1) / kWarps) * 2 * NR * NCOL;
-  const size_t ro = size_t((N + kWarps - 1) / kWarps) * 2 * kReadoutW;
-  net->part_cap = std::max(wg, std::max(ms, ro));
+  // partial sums of every parameter gradient of one pass, side by side
+  net->part_cap = part_layout(int(N)).total;
   A(&net->part, f * net->part_cap);
   A(&net->e_sr, sizeof(double) * max_frames);
   A(&net->e_pme, sizeof(double) * max_frames);
@@ -1383,7 +1520,7 @@ int gbnet_backward(gbnet_t net, void* stream, const float* g_q, const float* g_m
   k_gesr_from<<<blocks_for(net->nframes, 128), 128, 0, s>>>(net->nframes, g_esr, net->gesr);
   NET_LAUNCHED(net);
   int st;
-  if ((st = backward_pass<float>(net, s, net->pos_saved, nullptr, g_q, g_mu, net->gesr, g_params, nullptr, false)))
+  if ((st = backward_pass<float>(net, s, net->pos_saved, nullptr, g_q, g_mu, net->gesr, g_params, false)))
     return st;
   if (g_pos && net->n &&
       (st = cuda_ok(net, cudaMemcpyAsync(g_pos, net->gpos, sizeof(float) * 3 * size_t(net->n),
@@ -1422,8 +1559,7 @@ static int loss_grad(gbnet_t net, pme_plan_t pme, cudaStream_t s, const float* p
   }
   k_seed_esr<<<blocks_for(F, 128), 128, 0, s>>>(F, net->cvec, net->gesr, 0);
   NET_LAUNCHED(net);
-  if ((st = backward_pass<float>(net, s, net->pos_saved, nullptr, net->gq, net->gmu, net->gesr, nullptr, nullptr,
-                                 false)))
+  if ((st = backward_pass<float>(net, s, net->pos_saved, nullptr, net->gq, net->gmu, net->gesr, nullptr, false)))
     return st;
   // 3. loss, energy cotangents c_b, position tangent r' = -w
   k_loss<<<F, 256, 0, s>>>(net->frames_d, F, n, net->e_pme, net->e_sr, e_ref, net->f_pme, net->gpos, f_ref, lambda_e,
@@ -1445,7 +1581,7 @@ static int loss_grad(gbnet_t net, pme_plan_t pme, cudaStream_t s, const float* p
   // 6. Dual backward of the network with energy seeds 1 + e c_b: its tangent plane is dL/dtheta
   k_seed_esr<<<blocks_for(F, 128), 128, 0, s>>>(F, net->cvec, net->gesr, 1);
   NET_LAUNCHED(net);
-  if ((st = backward_pass<Dual>(net, s, net->pos_saved, net->dpos, net->gq, net->gmu, net->gesr, nullptr, grad, acc)))
+  if ((st = backward_pass<Dual>(net, s, net->pos_saved, net->dpos, net->gq, net->gmu, net->gesr, grad, acc)))
     return st;
   return PME_OK;
 }
