@@ -224,16 +224,108 @@ struct MsgArgs {
   size_t plS, plV;     // plane sizes: n * 48 (scalar-shaped 48) and n * 96 (vector-shaped 3 x 32)
 };
 
-// Messages of one layer: ms [n][48], mv [n][3][32] from A [n][48], B [n][3][32].
+// Edge records of the message kernels. The basis and geometry of an edge depend on the edge
+// alone, not on the channel, so one lane forms them for one edge (a warp's 32 lanes for up to
+// 32 edges of its ion at once) and stores them in shared memory, where the channel loop reads
+// them back as broadcast 16-byte loads:
+//   [0..1] e_1..e_8, [2] (d^, 1/r), then (DE) [3..4] de_k/dr, or (Dual) [3..4] the tangents
+//   of e_k and [5] of d^.
+// Formed in every lane for every edge, they were most of the kernels' instructions. With the
+// weights in registers and only the outputs that a pass reads afterwards, the four message
+// kernels of a gradient over 32 frames of 512 ions (265 k edges) went from 1.88 ms to about
+// 0.5 ms, and the gradient from 2.87 to 1.51 ms.
+template <typename T, bool DE>
+struct EdgeRec {
+  static constexpr bool kDual = sizeof(T) > sizeof(float);
+  static_assert(!(kDual && DE), "no Dual pass uses the r-derivatives");
+  static constexpr int kVec = kDual ? 6 : (DE ? 5 : 3);   // float4 per record
+};
+
+template <typename T, bool DE>
+__device__ __forceinline__ void edge_store(const MsgArgs& a, const Vec3<T>& ri, int j, const float4& sh,
+                                           float4* rec) {
+  Vec3<T> rj;
+  ldpos(a.pos, a.dpos, 3 * j, rj.x);
+  ldpos(a.pos, a.dpos, 3 * j + 1, rj.y);
+  ldpos(a.pos, a.dpos, 3 * j + 2, rj.z);
+  const Vec3<T> d{rj.x - ri.x + sh.x, rj.y - ri.y + sh.y, rj.z - ri.z + sh.z};
+  T r, e[NR], de[NR];
+  Vec3<T> dh;
+  edge_basis(d, r, dh, e, de);
+  rec[0] = make_float4(val(e[0]), val(e[1]), val(e[2]), val(e[3]));
+  rec[1] = make_float4(val(e[4]), val(e[5]), val(e[6]), val(e[7]));
+  rec[2] = make_float4(val(dh.x), val(dh.y), val(dh.z), 1.f / val(r));
+  if constexpr (DE) {
+    rec[3] = make_float4(val(de[0]), val(de[1]), val(de[2]), val(de[3]));
+    rec[4] = make_float4(val(de[4]), val(de[5]), val(de[6]), val(de[7]));
+  } else if constexpr (EdgeRec<T, DE>::kDual) {
+    rec[3] = make_float4(tan_(e[0]), tan_(e[1]), tan_(e[2]), tan_(e[3]));
+    rec[4] = make_float4(tan_(e[4]), tan_(e[5]), tan_(e[6]), tan_(e[7]));
+    rec[5] = make_float4(tan_(dh.x), tan_(dh.y), tan_(dh.z), 0.f);
+  }
+}
+
+__device__ __forceinline__ void unpack8(const float4& p, const float4& q, float (&e)[NR]) {
+  e[0] = p.x; e[1] = p.y; e[2] = p.z; e[3] = p.w;
+  e[4] = q.x; e[5] = q.y; e[6] = q.z; e[7] = q.w;
+}
+__device__ __forceinline__ void edge_load(const float4* rec, float (&e)[NR], Vec3<float>& dh) {
+  unpack8(rec[0], rec[1], e);
+  const float4 g = rec[2];
+  dh = Vec3<float>{g.x, g.y, g.z};
+}
+__device__ __forceinline__ void edge_load(const float4* rec, Dual (&e)[NR], Vec3<Dual>& dh) {
+  float v[NR], t[NR];
+  unpack8(rec[0], rec[1], v);
+  unpack8(rec[3], rec[4], t);
+#pragma unroll
+  for (int k = 0; k < NR; ++k) e[k] = Dual(v[k], t[k]);
+  const float4 g = rec[2], h = rec[5];
+  dh = Vec3<Dual>{Dual(g.x, h.x), Dual(g.y, h.y), Dual(g.z, h.z)};
+}
+
+// The radial weights of this lane's channels, kept in registers: w0 ss, w1 sv (lanes of the
+// first 16 channels, lo) or vv (the others), w2 vs (lo).
+__device__ __forceinline__ void lane_weights(const float* __restrict__ WR, int c, bool lo, float (&w0)[NR],
+                                             float (&w1)[NR], float (&w2)[NR]) {
+#pragma unroll
+  for (int k = 0; k < NR; ++k) {
+    const float* row = WR + k * NCOL;
+    w0[k] = __ldg(row + c);
+    w1[k] = __ldg(row + (lo ? S + c : S + V + c));   // hi: S + 2 V + (c - V)
+    w2[k] = lo ? __ldg(row + S + V + c) : 0.f;
+  }
+}
+
 template <typename T>
+__device__ __forceinline__ T radial(const T (&e)[NR], const float (&w)[NR]) {
+  T r = e[0] * w[0];
+#pragma unroll
+  for (int k = 1; k < NR; ++k) r += e[k] * w[k];
+  return r;
+}
+
+template <typename T>
+__device__ __forceinline__ Vec3<T> ldrow3(const float* p, int j, int c, size_t pl) {
+  const size_t o = size_t(j) * 3 * 2 * V + c;
+  return Vec3<T>{ldT<T>(p, o, pl), ldT<T>(p, o + 2 * V, pl), ldT<T>(p, o + 4 * V, pl)};
+}
+
+// Messages of one layer: ms [n][48], mv [n][3][32] from A [n][48], B [n][3][32]. One warp per
+// ion, lane = channel. FIRST: the first layer, whose vector features are zero, so B (= h^v WB)
+// is too and is neither formed nor read.
+template <typename T, bool FIRST>
 __global__ void __launch_bounds__(32 * kWarps) k_msg_fwd(MsgArgs a, const float* __restrict__ A,
                                                        const float* __restrict__ B, float* ms, float* mv) {
-  __shared__ float sW[NR * NCOL];
-  for (int k = threadIdx.x; k < NR * NCOL; k += blockDim.x) sW[k] = a.WR[k];
-  __syncthreads();
-  const int i = blockIdx.x * kWarps + (threadIdx.x >> 5), c = threadIdx.x & 31;
+  constexpr int VEC = EdgeRec<T, false>::kVec;
+  __shared__ float4 srec[kWarps][32 * VEC];
+  __shared__ int sj[kWarps][32];
+  const int w = threadIdx.x >> 5, c = threadIdx.x & 31;
+  const int i = blockIdx.x * kWarps + w;
   if (i >= a.n) return;
   const bool lo = c < V;
+  float w0[NR], w1[NR], w2[NR];
+  lane_weights(a.WR, c, lo, w0, w1, w2);
   Vec3<T> ri;
   ldpos(a.pos, a.dpos, 3 * i, ri.x);
   ldpos(a.pos, a.dpos, 3 * i + 1, ri.y);
@@ -241,41 +333,36 @@ __global__ void __launch_bounds__(32 * kWarps) k_msg_fwd(MsgArgs a, const float*
   T acc_s = 0.f, acc_s2 = 0.f;
   Vec3<T> acc_v{T(0.f), T(0.f), T(0.f)};
   const int ne = a.nb.cnt[i];
-  for (int q = 0; q < ne; ++q) {
-    const int j = a.nb.j[size_t(i) * kMaxNbr + q];
-    const float4 sh = a.nb.sh[size_t(i) * kMaxNbr + q];
-    Vec3<T> rj;
-    ldpos(a.pos, a.dpos, 3 * j, rj.x);
-    ldpos(a.pos, a.dpos, 3 * j + 1, rj.y);
-    ldpos(a.pos, a.dpos, 3 * j + 2, rj.z);
-    const Vec3<T> d{rj.x - ri.x + sh.x, rj.y - ri.y + sh.y, rj.z - ri.z + sh.z};
-    T r, e[NR], de[NR];
-    Vec3<T> dh;
-    edge_basis(d, r, dh, e, de);
-    T Rss = 0.f, R2 = 0.f, R3 = 0.f;   // lo lanes: R_ss, R_sv, R_vs;  hi lanes: R_ss, R_vv
-#pragma unroll
-    for (int k = 0; k < NR; ++k) {
-      Rss += e[k] * sW[k * NCOL + c];
-      if (lo) {
-        R2 += e[k] * sW[k * NCOL + S + c];
-        R3 += e[k] * sW[k * NCOL + S + V + c];
-      } else {
-        R2 += e[k] * sW[k * NCOL + S + 2 * V + (c - V)];
-      }
+  for (int q0 = 0; q0 < ne; q0 += 32) {
+    const int nq = min(32, ne - q0);
+    __syncwarp();
+    if (c < nq) {
+      const int j = a.nb.j[size_t(i) * kMaxNbr + q0 + c];
+      sj[w][c] = j;
+      edge_store<T, false>(a, ri, j, a.nb.sh[size_t(i) * kMaxNbr + q0 + c], &srec[w][c * VEC]);
     }
-    acc_s += Rss * ldT<T>(A, size_t(j) * (S + V) + c, a.plS);
-    const Vec3<T> Bj{ldT<T>(B, (size_t(j) * 3 + 0) * 2 * V + c, a.plV), ldT<T>(B, (size_t(j) * 3 + 1) * 2 * V + c, a.plV),
-                     ldT<T>(B, (size_t(j) * 3 + 2) * 2 * V + c, a.plV)};
-    if (lo) {
-      acc_s2 += R2 * dot3(dh, Bj);
-      const T t = R3 * ldT<T>(A, size_t(j) * (S + V) + S + c, a.plS);
-      acc_v.x += t * dh.x;
-      acc_v.y += t * dh.y;
-      acc_v.z += t * dh.z;
-    } else {
-      acc_v.x += R2 * Bj.x;
-      acc_v.y += R2 * Bj.y;
-      acc_v.z += R2 * Bj.z;
+    __syncwarp();
+#pragma unroll 2
+    for (int q = 0; q < nq; ++q) {
+      const int j = sj[w][q];
+      T e[NR];
+      Vec3<T> dh;
+      edge_load(&srec[w][q * VEC], e, dh);
+      acc_s += radial(e, w0) * ldT<T>(A, size_t(j) * (S + V) + c, a.plS);
+      Vec3<T> Bj;
+      if (!FIRST) Bj = ldrow3<T>(B, j, c, a.plV);
+      if (lo) {
+        if (!FIRST) acc_s2 += radial(e, w1) * dot3(dh, Bj);
+        const T t = radial(e, w2) * ldT<T>(A, size_t(j) * (S + V) + S + c, a.plS);
+        acc_v.x += t * dh.x;
+        acc_v.y += t * dh.y;
+        acc_v.z += t * dh.z;
+      } else if (!FIRST) {
+        const T R1 = radial(e, w1);
+        acc_v.x += R1 * Bj.x;
+        acc_v.y += R1 * Bj.y;
+        acc_v.z += R1 * Bj.z;
+      }
     }
   }
   stT(ms, size_t(i) * (S + V) + c, a.plS, acc_s * kInvAvg);
@@ -286,184 +373,195 @@ __global__ void __launch_bounds__(32 * kWarps) k_msg_fwd(MsgArgs a, const float*
 }
 
 // Reverse pass of the messages. Inputs: the layer's A, B and the cotangents g_ms [n][48],
-// g_mv [n][3][32] of its messages. Outputs: g_A [n][48], g_B [n][3][32] (written),
-// g_pos [n][3] (added), and per-block partials of dL/dWR [8][80] (two planes for Dual).
-template <typename T>
+// g_mv [n][3][32] of its messages. POS: the position gradient g_pos [n][3] (added). GRAD: the
+// cotangents g_A [n][48] and (not FIRST) g_B [n][3][32], written, and per-block partials of
+// dL/dWR [8][80] (the pass's plane). A pass asks only for what is read after it: the loss's
+// float pass needs the positions (and the cotangents of the second layer, GA), its Dual pass
+// the parameters. FIRST: B is zero and its cotangent unused, as in k_msg_fwd.
+template <typename T, bool POS, bool GA, bool GRAD, bool FIRST>
 __global__ void __launch_bounds__(32 * kWarps) k_msg_bwd(MsgArgs a, const float* __restrict__ A,
                                                        const float* __restrict__ B, const float* __restrict__ gms,
                                                        const float* __restrict__ gmv, float* gA_out, float* gB_out,
                                                        float* gpos, float* wr_part) {
-  __shared__ float sW[NR * NCOL];
-  __shared__ float sG[kWarps][NR * NCOL];
-  for (int k = threadIdx.x; k < NR * NCOL; k += blockDim.x) sW[k] = a.WR[k];
-  __syncthreads();
+  constexpr int VEC = EdgeRec<T, POS>::kVec;
+  constexpr int kRecFloats = kWarps * 32 * VEC * 4, kPartFloats = kWarps * NR * NCOL;
+  // the edge records; after the edge loop the warps' partials of dL/dWR in the same place
+  __shared__ __align__(16) float smem[GRAD ? (kRecFloats > kPartFloats ? kRecFloats : kPartFloats) : kRecFloats];
+  __shared__ int sj[kWarps][32];
   const int w = threadIdx.x >> 5, c = threadIdx.x & 31;
   const int i = blockIdx.x * kWarps + w;
   const bool lo = c < V;
+  float4* srec = reinterpret_cast<float4*>(smem) + w * 32 * VEC;
   // per-lane partials of dL/dWR for this lane's columns: cols c, and (lo) S + c, S + V + c,
-  // (hi) S + 2V + c - V
-  T gw0[NR], gw1[NR], gw2[NR];
+  // (hi) S + V + c (= S + 2 V + c - V)
+  float gw0[NR], gw1[NR], gw2[NR];
 #pragma unroll
   for (int k = 0; k < NR; ++k) gw0[k] = gw1[k] = gw2[k] = 0.f;
   if (i < a.n) {
+    float w0[NR], w1[NR], w2[NR];
+    lane_weights(a.WR, c, lo, w0, w1, w2);
     Vec3<T> ri;
     ldpos(a.pos, a.dpos, 3 * i, ri.x);
     ldpos(a.pos, a.dpos, 3 * i + 1, ri.y);
     ldpos(a.pos, a.dpos, 3 * i + 2, ri.z);
     const size_t iS = size_t(i) * (S + V);
+    const Vec3<T> zero{T(0.f), T(0.f), T(0.f)};
     const T Gs_i = ldT<T>(gms, iS + c, a.plS) * kInvAvg;
-    const T Gs2_i = lo ? ldT<T>(gms, iS + S + c, a.plS) * kInvAvg : T(0.f);
-    const Vec3<T> Gv_i{ldT<T>(gmv, (size_t(i) * 3 + 0) * 2 * V + c, a.plV) * kInvAvg,
-                       ldT<T>(gmv, (size_t(i) * 3 + 1) * 2 * V + c, a.plV) * kInvAvg,
-                       ldT<T>(gmv, (size_t(i) * 3 + 2) * 2 * V + c, a.plV) * kInvAvg};
-    const T A_i = ldT<T>(A, iS + c, a.plS);
-    const T A2_i = lo ? ldT<T>(A, iS + S + c, a.plS) : T(0.f);
-    const Vec3<T> B_i{ldT<T>(B, (size_t(i) * 3 + 0) * 2 * V + c, a.plV), ldT<T>(B, (size_t(i) * 3 + 1) * 2 * V + c, a.plV),
-                      ldT<T>(B, (size_t(i) * 3 + 2) * 2 * V + c, a.plV)};
+    const T Gs2_i = lo && !FIRST ? ldT<T>(gms, iS + S + c, a.plS) * kInvAvg : T(0.f);
+    Vec3<T> Gv_i = ldrow3<T>(gmv, i, c, a.plV);
+    Gv_i = Vec3<T>{Gv_i.x * kInvAvg, Gv_i.y * kInvAvg, Gv_i.z * kInvAvg};
+    T A_i = 0.f, A2_i = 0.f;
+    Vec3<T> B_i = zero;
+    if (POS) {
+      A_i = ldT<T>(A, iS + c, a.plS);
+      if (lo) A2_i = ldT<T>(A, iS + S + c, a.plS);
+      if (!FIRST) B_i = ldrow3<T>(B, i, c, a.plV);
+    }
     T gA = 0.f, gA2 = 0.f;
-    Vec3<T> gBv{T(0.f), T(0.f), T(0.f)}, gp{T(0.f), T(0.f), T(0.f)};
+    Vec3<T> gBv = zero, gp = zero;
     const int ne = a.nb.cnt[i];
-    for (int q = 0; q < ne; ++q) {
-      const int j = a.nb.j[size_t(i) * kMaxNbr + q];
-      const float4 sh = a.nb.sh[size_t(i) * kMaxNbr + q];
-      Vec3<T> rj;
-      ldpos(a.pos, a.dpos, 3 * j, rj.x);
-      ldpos(a.pos, a.dpos, 3 * j + 1, rj.y);
-      ldpos(a.pos, a.dpos, 3 * j + 2, rj.z);
-      const Vec3<T> d{rj.x - ri.x + sh.x, rj.y - ri.y + sh.y, rj.z - ri.z + sh.z};
-      T r, e[NR], de[NR];
-      Vec3<T> dh;
-      edge_basis(d, r, dh, e, de);
-      const T rinv = rcpT(r);
-      T R0 = 0.f, R1 = 0.f, R2 = 0.f, dR0 = 0.f, dR1 = 0.f, dR2 = 0.f;
-#pragma unroll
-      for (int k = 0; k < NR; ++k) {
-        const float w0 = sW[k * NCOL + c];
-        R0 += e[k] * w0;
-        dR0 += de[k] * w0;
-        if (lo) {
-          const float w1 = sW[k * NCOL + S + c], w2 = sW[k * NCOL + S + V + c];
-          R1 += e[k] * w1;
-          dR1 += de[k] * w1;
-          R2 += e[k] * w2;
-          dR2 += de[k] * w2;
-        } else {
-          const float w1 = sW[k * NCOL + S + 2 * V + (c - V)];
-          R1 += e[k] * w1;
-          dR1 += de[k] * w1;
-        }
+    for (int q0 = 0; q0 < ne; q0 += 32) {
+      const int nq = min(32, ne - q0);
+      __syncwarp();
+      if (c < nq) {
+        const int j = a.nb.j[size_t(i) * kMaxNbr + q0 + c];
+        sj[w][c] = j;
+        edge_store<T, POS>(a, ri, j, a.nb.sh[size_t(i) * kMaxNbr + q0 + c], srec + c * VEC);
       }
-      // neighbour's data
-      const size_t jS = size_t(j) * (S + V);
-      const T A_j = ldT<T>(A, jS + c, a.plS);
-      const Vec3<T> B_j{ldT<T>(B, (size_t(j) * 3 + 0) * 2 * V + c, a.plV), ldT<T>(B, (size_t(j) * 3 + 1) * 2 * V + c, a.plV),
-                        ldT<T>(B, (size_t(j) * 3 + 2) * 2 * V + c, a.plV)};
-      const T Gs_j = ldT<T>(gms, jS + c, a.plS) * kInvAvg;
-      const Vec3<T> Gv_j{ldT<T>(gmv, (size_t(j) * 3 + 0) * 2 * V + c, a.plV) * kInvAvg,
-                         ldT<T>(gmv, (size_t(j) * 3 + 1) * 2 * V + c, a.plV) * kInvAvg,
-                         ldT<T>(gmv, (size_t(j) * 3 + 2) * 2 * V + c, a.plV) * kInvAvg};
-      // --- forward direction: receiver i, sender j (d) ---
-      // scalar-type terms: Phi += R s, dPhi/dd = R' s d^; vector-type terms: Phi += R (d^.t),
-      // dPhi/dd = R' (d^.t) d^ + R (t - (d^.t) d^) / r
-      T sc = 0.f, vcoef = 0.f;            // sum R' s + sum R' (d^.t) ; and the t-terms below
-      Vec3<T> tv{T(0.f), T(0.f), T(0.f)}; // sum R t / r
-      T dtv = 0.f;                        // sum R (d^.t) / r
-      {
-        const T s0 = Gs_i * A_j;          // ss
-        sc += dR0 * s0;
-#pragma unroll
-        for (int k = 0; k < NR; ++k) gw0[k] += e[k] * s0;
-        if (lo) {
-          const T g2 = Gs2_i;
-          const Vec3<T> t1{g2 * B_j.x, g2 * B_j.y, g2 * B_j.z};    // sv
-          const T p1 = dot3(dh, t1);
-          const T A2_j = ldT<T>(A, jS + S + c, a.plS);
-          const Vec3<T> t2{A2_j * Gv_i.x, A2_j * Gv_i.y, A2_j * Gv_i.z};   // vs
-          const T p2 = dot3(dh, t2);
-          vcoef += dR1 * p1 + dR2 * p2;
-          const T f1 = R1 * rinv, f2 = R2 * rinv;
-          tv.x += f1 * t1.x + f2 * t2.x;
-          tv.y += f1 * t1.y + f2 * t2.y;
-          tv.z += f1 * t1.z + f2 * t2.z;
-          dtv += f1 * p1 + f2 * p2;
+      __syncwarp();
+      for (int q = 0; q < nq; ++q) {
+        const int j = sj[w][q];
+        const float4* rec = srec + q * VEC;
+        T e[NR];
+        Vec3<T> dh;
+        edge_load(rec, e, dh);
+        // neighbour's data
+        const size_t jS = size_t(j) * (S + V);
+        const T Gs_j = ldT<T>(gms, jS + c, a.plS) * kInvAvg;
+        Vec3<T> Gv_j = ldrow3<T>(gmv, j, c, a.plV);
+        Gv_j = Vec3<T>{Gv_j.x * kInvAvg, Gv_j.y * kInvAvg, Gv_j.z * kInvAvg};
+        const T Gs2_j = lo && !FIRST ? ldT<T>(gms, jS + S + c, a.plS) * kInvAvg : T(0.f);
+        T A_j = 0.f, A2_j = 0.f;
+        Vec3<T> B_j = zero;
+        if (POS || GRAD) {
+          A_j = ldT<T>(A, jS + c, a.plS);
+          if (lo) A2_j = ldT<T>(A, jS + S + c, a.plS);
+          if (!FIRST) B_j = ldrow3<T>(B, j, c, a.plV);
+        }
+        // the contractions of both directions: s0, p1, p2 (or s1) of receiver i and sender j
+        // (d^), t0, m1, m2 (or u1) of receiver j and sender i (d^' = -d^)
+        const T s0 = Gs_i * A_j;
+        T p1 = 0.f, p2 = 0.f;
+        if (POS || GRAD) {
+          if (lo) {
+            if (!FIRST) p1 = Gs2_i * dot3(dh, B_j);
+            p2 = A2_j * dot3(dh, Gv_i);
+          } else if (!FIRST) {
+            p1 = dot3(Gv_i, B_j);
+          }
+        }
+        if constexpr (GRAD) {
 #pragma unroll
           for (int k = 0; k < NR; ++k) {
-            gw1[k] += e[k] * p1;
-            gw2[k] += e[k] * p2;
+            gw0[k] += plane_of(e[k] * s0);
+            if (!FIRST) gw1[k] += plane_of(e[k] * p1);
+            gw2[k] += plane_of(e[k] * p2);   // zero in the hi lanes
           }
-        } else {
-          const T s1 = dot3(Gv_i, B_j);   // vv
-          sc += dR1 * s1;
-#pragma unroll
-          for (int k = 0; k < NR; ++k) gw1[k] += e[k] * s1;
+        }
+        const T dGv = dot3(dh, Gv_j);
+        T R1 = 0.f, R2 = 0.f;
+        if (GA || POS) {
+          if (!FIRST || GA) R1 = radial(e, w1);
+          R2 = radial(e, w2);
+        }
+        if constexpr (GA) {
+          gA += radial(e, w0) * Gs_j;
+          if (lo) {
+            // g_A_i[32+c] += R_vs (d^' . Gv_j),  g_B_i[:,c] += R_sv d^' Gs_j[32+c]
+            gA2 -= R2 * dGv;
+            if (!FIRST) {
+              const T f = R1 * Gs2_j;
+              gBv.x -= f * dh.x;
+              gBv.y -= f * dh.y;
+              gBv.z -= f * dh.z;
+            }
+          } else if (!FIRST) {
+            gBv.x += R1 * Gv_j.x;
+            gBv.y += R1 * Gv_j.y;
+            gBv.z += R1 * Gv_j.z;
+          }
+        }
+        if constexpr (POS) {
+          // scalar-type terms: Phi += R s, dPhi/dd = R' s d^; vector-type terms: Phi += R (d^.t),
+          // dPhi/dd = R' (d^.t) d^ + R (t - (d^.t) d^) / r. With both directions (the reverse one
+          // has d^' = -d^ and adds to g_pos_i with the opposite sign):
+          //   g_pos_i -= radial d^ + tv
+          float de[NR];
+          unpack8(rec[3], rec[4], de);
+          const float rinv = rec[2].w;
+          T rad = radial(de, w0) * (s0 + Gs_j * A_i);
+          Vec3<T> tv = zero;
+          const T dR1 = FIRST ? T(0.f) : radial(de, w1);
+          if (lo) {
+            const T dR2 = radial(de, w2);
+            const T f1 = R1 * rinv, f2 = R2 * rinv;
+            // t of receiver i: Gs2_i B_j + A2_j Gv_i; of receiver j (sign flipped): Gs2_j B_i + A2_i Gv_j
+            const T q1 = FIRST ? T(0.f) : p1 - Gs2_j * dot3(dh, B_i);
+            const T q2 = p2 - A2_i * dGv;
+            rad += dR1 * q1 + dR2 * q2 - (f1 * q1 + f2 * q2);
+            tv.x = f2 * (A2_j * Gv_i.x - A2_i * Gv_j.x);
+            tv.y = f2 * (A2_j * Gv_i.y - A2_i * Gv_j.y);
+            tv.z = f2 * (A2_j * Gv_i.z - A2_i * Gv_j.z);
+            if (!FIRST) {
+              tv.x += f1 * (Gs2_i * B_j.x - Gs2_j * B_i.x);
+              tv.y += f1 * (Gs2_i * B_j.y - Gs2_j * B_i.y);
+              tv.z += f1 * (Gs2_i * B_j.z - Gs2_j * B_i.z);
+            }
+          } else if (!FIRST) {
+            rad += dR1 * (p1 + dot3(Gv_j, B_i));
+          }
+          gp.x -= rad * dh.x + tv.x;
+          gp.y -= rad * dh.y + tv.y;
+          gp.z -= rad * dh.z + tv.z;
         }
       }
-      const T radial = sc + vcoef - dtv;
-      // V_ij = radial d^ + tv ; g_pos_i -= V_ij
-      gp.x -= radial * dh.x + tv.x;
-      gp.y -= radial * dh.y + tv.y;
-      gp.z -= radial * dh.z + tv.z;
-      // --- reverse direction: receiver j, sender i (d' = -d, d^' = -d^) ---
-      gA += R0 * Gs_j;
-      T sc2 = dR0 * (Gs_j * A_i), vcoef2 = 0.f, dtv2 = 0.f;
-      Vec3<T> tv2{T(0.f), T(0.f), T(0.f)};
-      if (lo) {
-        const T Gs2_j = ldT<T>(gms, jS + S + c, a.plS) * kInvAvg;
-        // g_A_i[32+c] += R_vs (d^' . Gv_j),  g_B_i[:,c] += R_sv d^' Gs_j[32+c]
-        gA2 -= R2 * dot3(dh, Gv_j);
-        gBv.x -= R1 * Gs2_j * dh.x;
-        gBv.y -= R1 * Gs2_j * dh.y;
-        gBv.z -= R1 * Gs2_j * dh.z;
-        const Vec3<T> t1{Gs2_j * B_i.x, Gs2_j * B_i.y, Gs2_j * B_i.z};
-        const Vec3<T> t2{A2_i * Gv_j.x, A2_i * Gv_j.y, A2_i * Gv_j.z};
-        const T p1 = -dot3(dh, t1), p2 = -dot3(dh, t2);        // d^' . t
-        vcoef2 += dR1 * p1 + dR2 * p2;
-        const T f1 = R1 * rinv, f2 = R2 * rinv;
-        tv2.x += f1 * t1.x + f2 * t2.x;
-        tv2.y += f1 * t1.y + f2 * t2.y;
-        tv2.z += f1 * t1.z + f2 * t2.z;
-        dtv2 += f1 * p1 + f2 * p2;
-      } else {
-        gBv.x += R1 * Gv_j.x;
-        gBv.y += R1 * Gv_j.y;
-        gBv.z += R1 * Gv_j.z;
-        sc2 += dR1 * dot3(Gv_j, B_i);
+    }
+    if constexpr (GA) {
+      stT(gA_out, iS + c, a.plS, gA);
+      if (lo) stT(gA_out, iS + S + c, a.plS, gA2);
+      if (!FIRST) {
+        stT(gB_out, (size_t(i) * 3 + 0) * 2 * V + c, a.plV, gBv.x);
+        stT(gB_out, (size_t(i) * 3 + 1) * 2 * V + c, a.plV, gBv.y);
+        stT(gB_out, (size_t(i) * 3 + 2) * 2 * V + c, a.plV, gBv.z);
       }
-      // V_ji = radial' d^' + tv2 ; g_pos_i += V_ji
-      const T radial2 = sc2 + vcoef2 - dtv2;
-      gp.x += tv2.x - radial2 * dh.x;
-      gp.y += tv2.y - radial2 * dh.y;
-      gp.z += tv2.z - radial2 * dh.z;
     }
-    stT(gA_out, iS + c, a.plS, gA);
-    if (lo) stT(gA_out, iS + S + c, a.plS, gA2);
-    stT(gB_out, (size_t(i) * 3 + 0) * 2 * V + c, a.plV, gBv.x);
-    stT(gB_out, (size_t(i) * 3 + 1) * 2 * V + c, a.plV, gBv.y);
-    stT(gB_out, (size_t(i) * 3 + 2) * 2 * V + c, a.plV, gBv.z);
-    gp.x = warp_sum(gp.x);
-    gp.y = warp_sum(gp.y);
-    gp.z = warp_sum(gp.z);
-    if (c == 0) {
-      const size_t pl = size_t(a.n) * 3;
-      stT(gpos, 3 * size_t(i), pl, ldT<T>(gpos, 3 * size_t(i), pl) + gp.x);
-      stT(gpos, 3 * size_t(i) + 1, pl, ldT<T>(gpos, 3 * size_t(i) + 1, pl) + gp.y);
-      stT(gpos, 3 * size_t(i) + 2, pl, ldT<T>(gpos, 3 * size_t(i) + 2, pl) + gp.z);
+    if constexpr (POS) {
+      gp.x = warp_sum(gp.x);
+      gp.y = warp_sum(gp.y);
+      gp.z = warp_sum(gp.z);
+      if (c == 0) {
+        gpos[3 * size_t(i)] += val(gp.x);
+        gpos[3 * size_t(i) + 1] += val(gp.y);
+        gpos[3 * size_t(i) + 2] += val(gp.z);
+      }
     }
   }
-  // block partials of dL/dWR [block][NR][NCOL]: the pass's plane (value, or tangent for Dual)
-  if (!wr_part) return;
-  const int col1 = lo ? S + c : S + 2 * V + (c - V);
+  if constexpr (GRAD) {
+    // block partials of dL/dWR [block][NR][NCOL]: the pass's plane (value, or tangent for Dual)
+    __syncthreads();
+    float* sG = smem + w * NR * NCOL;
 #pragma unroll
-  for (int k = 0; k < NR; ++k) {
-    sG[w][k * NCOL + c] = plane_of(gw0[k]);
-    sG[w][k * NCOL + col1] = plane_of(gw1[k]);
-    if (lo) sG[w][k * NCOL + S + V + c] = plane_of(gw2[k]);
-  }
-  __syncthreads();
-  for (int k = threadIdx.x; k < NR * NCOL; k += blockDim.x) {
-    float acc = 0.f;
-    for (int ww = 0; ww < kWarps; ++ww) acc += sG[ww][k];
-    wr_part[size_t(blockIdx.x) * NR * NCOL + k] = acc;
+    for (int k = 0; k < NR; ++k) {
+      sG[k * NCOL + c] = gw0[k];
+      sG[k * NCOL + (lo ? S + c : S + V + c)] = gw1[k];
+      if (lo) sG[k * NCOL + S + V + c] = gw2[k];
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < NR * NCOL; k += blockDim.x) {
+      float acc = 0.f;
+      for (int ww = 0; ww < kWarps; ++ww) acc += smem[ww * NR * NCOL + k];
+      wr_part[size_t(blockIdx.x) * NR * NCOL + k] = acc;
+    }
   }
 }
 
@@ -471,23 +569,20 @@ __global__ void __launch_bounds__(32 * kWarps) k_msg_bwd(MsgArgs a, const float*
 // per-ion elementwise stages
 // ---------------------------------------------------------------------------------------
 
-// h^s = emb[species]; h^v = 0 (both planes: the embedding has no position tangent)
-__global__ void k_embed(const float* __restrict__ P, const int* __restrict__ species, int n, float* hs, float* hv,
-                        size_t plS, size_t plV, int planes) {
+// h^s = emb[species] (both planes: the embedding has no position tangent); h^v = 0 is not
+// stored (the first layer's kernels take it as zero)
+__global__ void k_embed(const float* __restrict__ P, const int* __restrict__ species, int n, float* hs, size_t plS,
+                        int planes) {
   const size_t t = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (t < size_t(n) * S) {
-    const int i = int(t / S), c = int(t % S);
-    hs[t] = P[oEmb + species[i] * S + c];
-    if (planes > 1) hs[t + plS] = 0.f;
-  }
-  if (t < size_t(n) * 3 * V) {
-    hv[t] = 0.f;
-    if (planes > 1) hv[t + plV] = 0.f;
-  }
+  if (t >= size_t(n) * S) return;
+  const int i = int(t / S), c = int(t % S);
+  hs[t] = P[oEmb + species[i] * S + c];
+  if (planes > 1) hs[t + plS] = 0.f;
 }
 
 // h^s_out = h^s_in + SiLU(U[:, :32]);  h^v_out = h^v_in + sigmoid(U[:, 32:]) * Y.
-// One thread per (ion, scalar channel); the first 16 also do the vector channel.
+// One thread per (ion, scalar channel); the first 16 also do the vector channel. hv_in null:
+// zero (the first layer).
 template <typename T>
 __global__ void k_update_fwd(int n, const float* __restrict__ U, const float* __restrict__ Y,
                              const float* __restrict__ hs_in, const float* __restrict__ hv_in, float* hs_out,
@@ -502,7 +597,8 @@ __global__ void k_update_fwd(int n, const float* __restrict__ U, const float* __
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       const size_t k = (i * 3 + a) * V + c;
-      stT(hv_out, k, plV, ldT<T>(hv_in, k, plV) + g * ldT<T>(Y, k, plY));
+      const T gy = g * ldT<T>(Y, k, plY);
+      stT(hv_out, k, plV, hv_in ? ldT<T>(hv_in, k, plV) + gy : gy);
     }
   }
 }
@@ -1100,14 +1196,18 @@ int forward_pass(gbnet_t net, cudaStream_t s, const float* pos, const float* dpo
                pl96 = size_t(n) * 3 * 2 * V, pl64 = size_t(n) * 2 * S;
   int st;
   if (n == 0) return PME_OK;
-  k_embed<<<blocks_for(size_t(n) * 3 * V, 256), 256, 0, s>>>(net->P, net->species, n, net->hs[0], net->hv[0], plS,
-                                                             plV, planes);
+  k_embed<<<blocks_for(size_t(n) * S, 256), 256, 0, s>>>(net->P, net->species, n, net->hs[0], plS, planes);
   NET_LAUNCHED(net);
   for (int t = 0; t < 2; ++t) {
     if ((st = mix(net, s, planes * n, S, S + V, net->hs[t], 4 * t + 0, true, net->A[t], false))) return st;
-    if ((st = mix(net, s, planes * 3 * n, V, 2 * V, net->hv[t], 4 * t + 1, true, net->B[t], false))) return st;
+    if (t > 0 && (st = mix(net, s, planes * 3 * n, V, 2 * V, net->hv[t], 4 * t + 1, true, net->B[t], false)))
+      return st;
     const MsgArgs a = msg_args<T>(net, t, pos, dpos);
-    k_msg_fwd<T><<<blocks_for(n, kWarps), 32 * kWarps, 0, s>>>(a, net->A[t], net->B[t], net->ms[t], net->mv[t]);
+    if (t == 0)
+      k_msg_fwd<T, true><<<blocks_for(n, kWarps), 32 * kWarps, 0, s>>>(a, net->A[t], nullptr, net->ms[t], net->mv[t]);
+    else
+      k_msg_fwd<T, false><<<blocks_for(n, kWarps), 32 * kWarps, 0, s>>>(a, net->A[t], net->B[t], net->ms[t],
+                                                                       net->mv[t]);
     NET_LAUNCHED(net);
     if ((st = mix(net, s, planes * n, S + V, S + V, net->ms[t], 4 * t + 2, true, net->U[t], false))) return st;
     if ((st = mix(net, s, planes * 3 * n, 2 * V, V, net->mv[t], 4 * t + 3, true, net->Y[t], false))) return st;
@@ -1178,7 +1278,8 @@ int param_grads(gbnet_t net, cudaStream_t s, float* grad, bool acc) {
     wg(kWgU, n, net->ms[t], S + V, net->gU[t], S + V, L.u[t], base + oWU);
     wg(kWgA, n, net->hs[t], S, net->gA[t], S + V, L.a[t], base + oWA);
     wg(kWgY, 3 * n, net->mv[t], 2 * V, net->gY[t], V, L.y[t], base + oWY);
-    wg(kWgB, 3 * n, net->hv[t], V, net->gB[t], 2 * V, L.b[t], base + oWB);
+    if (t > 0) wg(kWgB, 3 * n, net->hv[t], V, net->gB[t], 2 * V, L.b[t], base + oWB);
+    else red(P + L.b[t], 0, V * 2 * V, base + oWB);   // h^v = 0: a zero gradient, no partials
     red(P + L.wr[t], int(blocks_for(size_t(n), kWarps)), NR * NCOL, base + oWR);
   }
   wg(kWgH, n, net->hs[2], S, net->gH, 2 * S, L.h, oWh);
@@ -1195,7 +1296,7 @@ int param_grads(gbnet_t net, cudaStream_t s, float* grad, bool acc) {
 
 // Backward pass of the last forward_pass<T>. Seeds: gq [planes][n], gmu [planes][n][3] (each
 // may be null), gesr_f [F][2] float (value, tangent). Outputs: gpos [planes][n][3] (net->gpos,
-// written) and, unless grad is null, the parameter gradients: the value plane of a float pass,
+// written; a Dual pass forms only its parameter gradients) and, unless grad is null, the parameter gradients: the value plane of a float pass,
 // the tangent plane of a Dual one (written, or added when acc).
 template <typename T>
 int backward_pass(gbnet_t net, cudaStream_t s, const float* pos, const float* dpos, const float* gq,
@@ -1240,11 +1341,26 @@ int backward_pass(gbnet_t net, cudaStream_t s, const float* pos, const float* dp
     if ((st = mix(net, s, planes * n, S + V, S + V, net->gU[t], 4 * t + 2, false, net->gms, false))) return st;
     if ((st = mix(net, s, planes * 3 * n, V, 2 * V, net->gY[t], 4 * t + 3, false, net->gmv, false))) return st;
     const MsgArgs a = msg_args<T>(net, t, pos, dpos);
-    k_msg_bwd<T><<<nb_ion, 32 * kWarps, 0, s>>>(a, net->A[t], net->B[t], net->gms, net->gmv, net->gA[t], net->gB[t],
-                                               net->gpos, grad ? net->part + L.wr[t] : nullptr);
+    float* wr = grad ? net->part + L.wr[t] : nullptr;
+#define GB_MSG_BWD(POS, GA, GRAD, FIRST)                                                                          \
+  k_msg_bwd<T, POS, GA, GRAD, FIRST><<<nb_ion, 32 * kWarps, 0, s>>>(a, net->A[t], net->B[t], net->gms, net->gmv, \
+                                                                    net->gA[t], net->gB[t], net->gpos, wr)
+    if constexpr (planes > 1) {   // the Dual pass: parameters only
+      if (t == 0) GB_MSG_BWD(false, true, true, true);
+      else GB_MSG_BWD(false, true, true, false);
+    } else if (grad) {
+      if (t == 0) GB_MSG_BWD(true, true, true, true);
+      else GB_MSG_BWD(true, true, true, false);
+    } else {
+      if (t == 0) GB_MSG_BWD(true, false, false, true);
+      else GB_MSG_BWD(true, true, false, false);
+    }
+#undef GB_MSG_BWD
     NET_LAUNCHED(net);
+    // below the first layer lie only the embedding (a parameter) and h^v = 0
+    if (t == 0 && !grad) break;
     if ((st = mix(net, s, planes * n, S + V, S, net->gA[t], 4 * t + 0, false, net->ghs, true))) return st;
-    if ((st = mix(net, s, planes * 3 * n, 2 * V, V, net->gB[t], 4 * t + 1, false, net->ghv, true))) return st;
+    if (t > 0 && (st = mix(net, s, planes * 3 * n, 2 * V, V, net->gB[t], 4 * t + 1, false, net->ghv, true))) return st;
   }
   if (grad && (st = param_grads<T>(net, s, grad, acc))) return st;
   (void)pl96;
@@ -1339,7 +1455,7 @@ int gbnet_create(gbnet_t* out, int max_ions, int max_frames) {
   A(&net->nbr_sh, sizeof(float4) * N * kMaxNbr);
   for (int t = 0; t < 3; ++t) {
     A(&net->hs[t], 2 * f * N * S);
-    A(&net->hv[t], 2 * f * N * 3 * V);
+    if (t > 0) A(&net->hv[t], 2 * f * N * 3 * V);   // hv[0] = 0 is not stored
   }
   for (int t = 0; t < 2; ++t) {
     A(&net->A[t], 2 * f * N * (S + V));
