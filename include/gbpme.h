@@ -100,9 +100,10 @@ typedef struct {
                               every axis of every frame is 64 or 128 points they run as
                               power-of-two kernels (compile-time four-step transforms).
                               0 (default): automatic, the library's own when every frame's
-                              mesh takes the power-of-two kernels, or for batched plans whose
-                              meshes have no axis above 64 points (one launch per pass for
-                              all frames; faster there on GB300), cuFFT otherwise.
+                              mesh takes the power-of-two kernels, for single frames whose
+                              every axis is a product of two of 1-6, 8, 9, 10, 12, 15, 16, and
+                              for batched plans whose meshes have no axis above 64 points (one
+                              launch per pass for all frames), cuFFT otherwise.
                               1: always cuFFT. 2: always the library's own
                               (PME_ERR_UNSUPPORTED where they do not apply). 3: the library's
                               own without the power-of-two kernels. With the own transforms
@@ -142,7 +143,7 @@ int pme_plan_set_box(pme_plan_t plan, const double box[9]);
 int pme_plan_destroy(pme_plan_t plan);
 
 /* Which transforms the plan's mesh convolution uses: *kind = 0 for the library's own
- * (Stockham transforms in shared memory, the x transform fused with the influence multiply),
+ * (two-step or Stockham transforms in shared memory, the x transform fused with the influence multiply),
  * 1 for cuFFT, 2 for the library's own power-of-two kernels (every axis 64 or 128). */
 int pme_plan_fft_kind(pme_plan_t plan, int* kind);
 

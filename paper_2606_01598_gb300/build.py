@@ -3,9 +3,9 @@
 Each CUDA translation unit under ``csrc/`` is compiled in parallel to an object file under
 ``_build/`` and linked into ``lib/libgbpme.so`` against cuFFT (the only library call on the
 path: the two 3D transforms) with the CUDA runtime linked statically. Up-to-date outputs are
-reused unless ``force`` is set. The pair-term unit is compiled without implicit multiply-add
-contraction (its multiply-adds are written out), so that its fused and list-driven kernels
-round identically.
+reused unless ``force`` is set. The pair-term and the two-step transform units are compiled
+without implicit multiply-add contraction (their multiply-adds are written out), so that their
+kernel variants (fused and list-driven, with and without the virial) round identically.
 """
 from __future__ import annotations
 
@@ -24,7 +24,7 @@ LIBNAME = "libgbpme.so"
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # per-unit flags: no implicit contraction where two kernels must round the same expressions
 # identically
-UNIT_FLAGS = {"pair.cu": ["-fmad=false"]}
+UNIT_FLAGS = {"pair.cu": ["-fmad=false"], "conv_two.cu": ["-fmad=false"]}
 
 
 def find_nvcc() -> str:

@@ -208,6 +208,7 @@ struct FrameDesc {
   int tw_off[3];            // hand-written transforms: twiddle tables of the x, y, z lengths
   int conv_cols;            // pass-B tile width in (n_y, n_z) columns
   int conv_pp;              // pass A / C: consecutive x-planes per block
+  int conv_p[3], conv_q[3]; // two-step transforms: length = p q of each axis
   int item_off, nitems;     // items of the per-frame float64 sums
   FastDiv div_zh, div_y;    // division by Nz/2 + 1 and by Ny (half-spectrum index -> n)
 };
@@ -260,6 +261,7 @@ struct pme_plan_s {
   // hand-written transforms (every axis 2,3,5-smooth and short enough): no cuFFT plans
   bool conv = false;
   bool conv_p2 = false;                    // every axis 64 or 128: the power-of-two kernels
+  bool conv_two = false;                   // every axis P Q with P, Q <= 16: the two-step kernels
   float2* conv_tw = nullptr;               // twiddle tables
   int2* conv_planes1 = nullptr;            // batched plans: pass A / C block -> (frame, plane)
   int2* conv_planes2 = nullptr;            //   the same with the tangent meshes

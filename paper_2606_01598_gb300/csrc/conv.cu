@@ -29,12 +29,14 @@
 // thread waits for one round trip per batch. Layout and normalisation are those of the usual
 // unnormalised R2C / C2R pair, so the spectrum, the energy partials and Phi are laid out as
 // with a library transform. Every axis must be 2,3,5-smooth and at most kConvMaxLen long and
-// a plane must fit in shared memory; other meshes go through cuFFT.
+// a plane must fit in shared memory; other meshes go through cuFFT. Meshes whose axes all split
+// into two register steps take the kernels of conv_two.cu instead; the Stockham kernels here
+// serve the lengths that do not (125, 162, 200, 216, 243, 250) and planes that only fit here.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
 
-#include "kernels.h"
+#include "conv_dft.cuh"
 
 namespace gbpme {
 
@@ -46,80 +48,6 @@ constexpr int kConvBThreads = 256;
 constexpr int kConvPlaneThreads = 1024;  // upper bound of the pass A / C block size
 constexpr int kLoadBatch = 8;            // global loads a thread keeps in flight
 constexpr size_t kConvPlaneTarget = 4096;  // small planes are grouped up to this many entries
-
-__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
-__device__ __forceinline__ float2 cmul(float2 a, float2 b) {
-  return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
-}
-// times -i (forward transform) or +i (inverse)
-template <bool INV>
-__device__ __forceinline__ float2 rot(float2 a) {
-  return INV ? make_float2(-a.y, a.x) : make_float2(a.y, -a.x);
-}
-
-// R-point DFTs in place, X_k = sum_n v_n e^(-+2 pi i n k / R) (minus: forward).
-template <bool INV>
-__device__ __forceinline__ void dft4(float2& v0, float2& v1, float2& v2, float2& v3) {
-  const float2 t0 = cadd(v0, v2), t1 = csub(v0, v2), t2 = cadd(v1, v3), t3 = rot<INV>(csub(v1, v3));
-  v0 = cadd(t0, t2);
-  v2 = csub(t0, t2);
-  v1 = cadd(t1, t3);
-  v3 = csub(t1, t3);
-}
-
-template <int R, bool INV>
-__device__ __forceinline__ void dft(float2* v) {
-  if constexpr (R == 2) {
-    const float2 a = v[0];
-    v[0] = cadd(a, v[1]);
-    v[1] = csub(a, v[1]);
-  } else if constexpr (R == 4) {
-    dft4<INV>(v[0], v[1], v[2], v[3]);
-  } else if constexpr (R == 8) {
-    // radix-2 split: even and odd 4-point DFTs, odd outputs times w8^k
-    float2 e0 = v[0], e1 = v[2], e2 = v[4], e3 = v[6];
-    float2 o0 = v[1], o1 = v[3], o2 = v[5], o3 = v[7];
-    dft4<INV>(e0, e1, e2, e3);
-    dft4<INV>(o0, o1, o2, o3);
-    const float h = 0.70710678118654752f;   // cos(pi / 4)
-    o1 = INV ? make_float2(h * (o1.x - o1.y), h * (o1.x + o1.y)) : make_float2(h * (o1.x + o1.y), h * (o1.y - o1.x));
-    o2 = rot<INV>(o2);
-    o3 = INV ? make_float2(-h * (o3.x + o3.y), h * (o3.x - o3.y)) : make_float2(h * (o3.y - o3.x), -h * (o3.x + o3.y));
-    v[0] = cadd(e0, o0);
-    v[4] = csub(e0, o0);
-    v[1] = cadd(e1, o1);
-    v[5] = csub(e1, o1);
-    v[2] = cadd(e2, o2);
-    v[6] = csub(e2, o2);
-    v[3] = cadd(e3, o3);
-    v[7] = csub(e3, o3);
-  } else if constexpr (R == 3) {
-    const float c = -0.5f, s = 0.86602540378443865f;   // cos, sin of 2 pi / 3
-    const float2 a = v[0], sm = cadd(v[1], v[2]), d = csub(v[1], v[2]);
-    const float2 m = make_float2(a.x + c * sm.x, a.y + c * sm.y);
-    const float2 isd = make_float2(-s * d.y, s * d.x);   // i s d
-    v[0] = cadd(a, sm);
-    v[1] = INV ? cadd(m, isd) : csub(m, isd);
-    v[2] = INV ? csub(m, isd) : cadd(m, isd);
-  } else {   // R == 5
-    const float c1 = 0.30901699437494742f, c2 = -0.80901699437494742f;   // cos 2pi/5, cos 4pi/5
-    const float s1 = 0.95105651629515357f, s2 = 0.58778525229247313f;    // sin 2pi/5, sin 4pi/5
-    const float2 a = v[0];
-    const float2 s14 = cadd(v[1], v[4]), d14 = csub(v[1], v[4]);
-    const float2 s23 = cadd(v[2], v[3]), d23 = csub(v[2], v[3]);
-    const float2 m1 = make_float2(a.x + c1 * s14.x + c2 * s23.x, a.y + c1 * s14.y + c2 * s23.y);
-    const float2 m2 = make_float2(a.x + c2 * s14.x + c1 * s23.x, a.y + c2 * s14.y + c1 * s23.y);
-    const float2 n1 = make_float2(s1 * d14.x + s2 * d23.x, s1 * d14.y + s2 * d23.y);
-    const float2 n2 = make_float2(s2 * d14.x - s1 * d23.x, s2 * d14.y - s1 * d23.y);
-    const float2 in1 = make_float2(-n1.y, n1.x), in2 = make_float2(-n2.y, n2.x);   // i n
-    v[0] = cadd(a, cadd(s14, s23));
-    v[1] = INV ? cadd(m1, in1) : csub(m1, in1);
-    v[4] = INV ? csub(m1, in1) : cadd(m1, in1);
-    v[2] = INV ? cadd(m2, in2) : csub(m2, in2);
-    v[3] = INV ? csub(m2, in2) : cadd(m2, in2);
-  }
-}
 
 // Radix of the next stage for a remaining length m (2,3,5-smooth): 8 while it divides m,
 // except that 16 goes as 4 x 4 (no radix-2 stage unless the power of two is 2).
@@ -193,62 +121,6 @@ __device__ float2* fft_lines(float2* a, float2* b, int L, int nl, int ls, int es
   return a;
 }
 
-__device__ __forceinline__ void comp_add(float& s, float& c, float v) {
-  const float t = s + v;
-  c += fabsf(s) >= fabsf(v) ? (s - t) + v : (v - t) + s;
-  s = t;
-}
-
-// Block sum of per-thread compensated pairs: float within a warp, float64 across warps;
-// thread 0 gets the total.
-__device__ double block_comp_sum(float v, float c, double* wsum) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float v2 = __shfl_xor_sync(0xffffffffu, v, o);
-    const float c2 = __shfl_xor_sync(0xffffffffu, c, o);
-    c += c2;
-    comp_add(v, c, v2);
-  }
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = double(v) + double(c);
-  __syncthreads();
-  double t = 0.0;
-  if (threadIdx.x == 0)
-    for (int w = 0; w < int(blockDim.x >> 5); ++w) t += wsum[w];
-  return t;
-}
-
-// element t of a tile with c columns: row t / c, column t mod c. The float quotient is off
-// by at most one for t < 2^20, which the correction absorbs.
-__device__ __forceinline__ void split_rc(int t, int c, float rc, int& row, int& col) {
-  row = int((float(t) + 0.5f) * rc);
-  col = t - row * c;
-  if (col < 0) {
-    --row;
-    col += c;
-  } else if (col >= c) {
-    ++row;
-    col -= c;
-  }
-}
-
-struct ConvArgs {
-  FrameDesc one;
-  FrameMaps maps;
-  const int2* planes;   // batched pass A / C: block -> (frame, plane index of the frame)
-  const float2* tw;     // twiddle tables
-  float* mesh;          // pass A: rho base (input); pass C: Phi base (output)
-  float2* spec;
-  int tangent;
-  int cap;              // complex entries of each plane buffer (pass A / C)
-  const float* dconv;
-  float inv4a2;
-  double* partials;
-  double* vparts;
-  const float* gtab;
-  const int* keep;      // tangent passes: *keep == 0 skips rho / Phi (the forward's stay)
-};
-
 // Plane buffers of pass A / C: twiddles of z and y, then two buffers of cap entries.
 __device__ __forceinline__ void plane_setup(const ConvArgs& a, const FrameDesc& F, float2* sm, float2*& twz,
                                             float2*& twy, float2*& b0, float2*& b1) {
@@ -259,25 +131,6 @@ __device__ __forceinline__ void plane_setup(const ConvArgs& a, const FrameDesc& 
   b1 = b0 + a.cap;
   for (int k = threadIdx.x; k < Nz; k += blockDim.x) twz[k] = a.tw[F.tw_off[2] + k];
   for (int k = threadIdx.x; k < Ny; k += blockDim.x) twy[k] = a.tw[F.tw_off[1] + k];
-}
-
-// Pass A / C block: frame, mesh copy (0: rho / Phi, 1: the tangent one), first plane x0 and
-// plane count pc (F.conv_pp consecutive x-planes per block, fewer in the last one).
-template <bool BATCH>
-__device__ __forceinline__ const FrameDesc& plane_block(const ConvArgs& a, int& copy, int& x0, int& pc) {
-  int f = 0, local = blockIdx.x;
-  if (BATCH) {
-    const int2 m = a.planes[blockIdx.x];
-    f = m.x;
-    local = m.y;
-  }
-  const FrameDesc& F = frame_at<BATCH>(a.one, a.maps, f);
-  const int Nx = F.g.N[0], P = F.conv_pp;
-  const int per_copy = (Nx + P - 1) / P;
-  copy = local >= per_copy ? 1 : 0;
-  x0 = (local - copy * per_copy) * P;
-  pc = min(P, Nx - x0);
-  return F;
 }
 
 // Shared-memory layouts of a block's pc planes (np = ceil(Ny / 2) row pairs, Zs = Nz | 1):
@@ -567,53 +420,6 @@ __global__ void __launch_bounds__(kConvBThreads) k_conv_x(ConvArgs a) {
 // ---------------------------------------------------------------------------------------
 constexpr int kP2PlaneThreads = 1024;
 
-// 16-point DFT in registers: 4 x 4 with the twiddles w16^(n1 k1) between the two radix-4
-// steps; output in natural order.
-template <bool INV>
-__device__ __forceinline__ void dft16(float2 (&v)[16]) {
-  const float c1 = 0.92387953251128674f, s1 = 0.38268343236508978f, h = 0.70710678118654752f;
-  float2 t[4][4];
-#pragma unroll
-  for (int n1 = 0; n1 < 4; ++n1) {
-    float2 a0 = v[n1], a1 = v[n1 + 4], a2 = v[n1 + 8], a3 = v[n1 + 12];
-    dft4<INV>(a0, a1, a2, a3);
-    t[n1][0] = a0;
-    t[n1][1] = a1;
-    t[n1][2] = a2;
-    t[n1][3] = a3;
-  }
-  // forward twiddles w16^j = (cos, -sin)(2 pi j / 16); the inverse takes their conjugates
-  const float sg = INV ? -1.f : 1.f;
-  auto tw = [&](float2 a, float wr, float wi) {   // a (wr + i sg wi)
-    const float wj = sg * wi;
-    return make_float2(a.x * wr - a.y * wj, a.x * wj + a.y * wr);
-  };
-  t[1][1] = tw(t[1][1], c1, -s1);   // j = 1
-  t[1][2] = tw(t[1][2], h, -h);     // j = 2
-  t[1][3] = tw(t[1][3], s1, -c1);   // j = 3
-  t[2][1] = tw(t[2][1], h, -h);     // j = 2
-  t[2][2] = rot<INV>(t[2][2]);      // j = 4
-  t[2][3] = tw(t[2][3], -h, -h);    // j = 6
-  t[3][1] = tw(t[3][1], s1, -c1);   // j = 3
-  t[3][2] = tw(t[3][2], -h, -h);    // j = 6
-  t[3][3] = tw(t[3][3], -c1, s1);   // j = 9
-#pragma unroll
-  for (int k1 = 0; k1 < 4; ++k1) {
-    float2 b0 = t[0][k1], b1 = t[1][k1], b2 = t[2][k1], b3 = t[3][k1];
-    dft4<INV>(b0, b1, b2, b3);
-    v[k1] = b0;
-    v[k1 + 4] = b1;
-    v[k1 + 8] = b2;
-    v[k1 + 12] = b3;
-  }
-}
-
-template <int B, bool INV>
-__device__ __forceinline__ void dft_b(float2 (&u)[B]) {
-  if constexpr (B == 16) dft16<INV>(u);
-  else dft<B, INV>(u);
-}
-
 // step 1 on v[m] = x[t + B m]: the 8-point DFT and the twiddles w_L^(t k1) (tw: forward table)
 template <bool INV>
 __device__ __forceinline__ void p2_step1(float2 (&v)[8], int t, const float2* __restrict__ tw) {
@@ -665,7 +471,7 @@ __device__ __forceinline__ void r2c_plane_p2(const float* __restrict__ src, floa
     float2 u[BZ];
 #pragma unroll
     for (int t = 0; t < BZ; ++t) u[t] = Z[pr * LS + t + (BZ + 1) * k1];
-    dft_b<BZ, false>(u);
+    dft<BZ, false>(u);
 #pragma unroll
     for (int k2 = 0; k2 < BZ; ++k2) Z2[pr * LS + k1 + 8 * k2] = u[k2];
   }
@@ -694,7 +500,7 @@ __device__ __forceinline__ void r2c_plane_p2(const float* __restrict__ src, floa
     float2 u[BY];
 #pragma unroll
     for (int t = 0; t < BY; ++t) u[t] = S[(t + BY * k1) * NZH + kz];
-    dft_b<BY, false>(u);
+    dft<BY, false>(u);
 #pragma unroll
     for (int k2 = 0; k2 < BY; ++k2) dst[(k1 + 8 * k2) * NZH + kz] = u[k2];
   }
@@ -726,7 +532,7 @@ __device__ __forceinline__ void c2r_plane_p2(const float2* __restrict__ src, flo
     float2 u[BY];
 #pragma unroll
     for (int t = 0; t < BY; ++t) u[t] = S[(t + BY * k1) * NZH + kz];
-    dft_b<BY, true>(u);
+    dft<BY, true>(u);
 #pragma unroll
     for (int k2 = 0; k2 < BY; ++k2) S2[(k1 + 8 * k2) * NZH + kz] = u[k2];
   }
@@ -768,7 +574,7 @@ __device__ __forceinline__ void c2r_plane_p2(const float2* __restrict__ src, flo
     float2 u[BZ];
 #pragma unroll
     for (int t = 0; t < BZ; ++t) u[t] = Z[pr * LS + t + (BZ + 1) * k1];
-    dft_b<BZ, true>(u);
+    dft<BZ, true>(u);
     float* r0 = dst + (2 * pr) * NZ + k1;
 #pragma unroll
     for (int k2 = 0; k2 < BZ; ++k2) {
@@ -850,7 +656,7 @@ __device__ __forceinline__ void x_tile_p2(const ConvArgs& a, const FrameDesc& F,
     float2 u[BX];
 #pragma unroll
     for (int t = 0; t < BX; ++t) u[t] = T[(t + BX * k1) * NC + c];
-    dft_b<BX, false>(u);
+    dft<BX, false>(u);
 #pragma unroll
     for (int k2 = 0; k2 < BX; ++k2) T2[(k1 + 8 * k2) * NC + c] = u[k2];
   }
@@ -915,7 +721,7 @@ __device__ __forceinline__ void x_tile_p2(const ConvArgs& a, const FrameDesc& F,
     float2 u[BX];
 #pragma unroll
     for (int t = 0; t < BX; ++t) u[t] = T[(t + BX * k1) * NC + c];
-    dft_b<BX, true>(u);
+    dft<BX, true>(u);
     float2* cp = col_ptr(c);
 #pragma unroll
     for (int k2 = 0; k2 < BX; ++k2) cp[size_t(k1 + 8 * k2) * ncols] = u[k2];
@@ -962,24 +768,6 @@ ConvArgs conv_args(pme_plan_t p) {
   a.inv4a2 = float(1.0 / (4.0 * p->alpha * p->alpha));
   a.gtab = p->gtab;
   return a;
-}
-
-// The first launch of a kernel on a device raises its dynamic shared-memory limit to the
-// device's opt-in maximum (one call per kernel and device; the launch's own size decides the
-// occupancy). The plan checked its sizes against that maximum when it was made.
-template <typename K>
-int set_smem(pme_plan_t p, K kernel, unsigned& done_mask) {
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (dev < 32 && (done_mask & (1u << dev))) return PME_OK;
-  int optin = 0;
-  int st = check_cuda(p, cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev),
-                      "cudaDeviceGetAttribute");
-  if (st) return st;
-  st = check_cuda(p, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - 1024),
-                  "cudaFuncSetAttribute");
-  if (!st && dev < 32) done_mask |= 1u << dev;
-  return st;
 }
 
 }  // namespace
@@ -1053,6 +841,7 @@ int launch_conv_forward(pme_plan_t p, cudaStream_t s, bool tangent, float* mesh,
                             : (tangent ? 2 : 1) * ((F0.g.N[0] + F0.conv_pp - 1) / F0.conv_pp);
   a.planes = tangent ? p->conv_planes2 : p->conv_planes1;
   int st;
+  if (p->conv_two) return launch_two_plane(p, s, a, grid, false);
   if (p->conv_p2) {
     if (p->batch) {
       static unsigned done = 0;
@@ -1090,6 +879,7 @@ int launch_conv_inverse(pme_plan_t p, cudaStream_t s, bool tangent, float* mesh,
                             : (tangent ? 2 : 1) * ((F0.g.N[0] + F0.conv_pp - 1) / F0.conv_pp);
   a.planes = tangent ? p->conv_planes2 : p->conv_planes1;
   int st;
+  if (p->conv_two) return launch_two_plane(p, s, a, grid, true);
   if (p->conv_p2) {
     if (p->batch) {
       static unsigned done = 0;
@@ -1125,6 +915,7 @@ int launch_conv_influence(pme_plan_t p, cudaStream_t s, bool tangent, double* pa
   a.partials = partials;
   a.vparts = vparts;
   const int grid = p->batch ? p->total_blocks : p->frames_h[0].infl_nblk;
+  if (p->conv_two) return launch_two_x(p, s, a, grid);
   const size_t smem = p->conv_smem_x;
   int st;
 #define GB_CONV_X(B, V)                                                  \

@@ -97,6 +97,13 @@ int conv_planes_per_block(const int N[3]);
 size_t conv_plane_cap(const int N[3]);
 size_t conv_plane_smem(const int N[3], size_t cap);
 size_t conv_x_smem(const int N[3]);
+// two register steps per transform (conv_two.cu): L = P Q; planes, threads and shared memory of
+// a pass A / C block; shared memory of a pass-B tile
+bool two_step_factors(int L, int* P, int* Q);
+int two_planes_per_block(const int N[3], bool single);
+int two_plane_threads(const int N[3], int pp);
+size_t two_plane_smem(const int N[3], int pp);
+size_t two_x_smem(const int N[3]);
 void conv_twiddles(int L, std::vector<float2>& out);
 // keep (tangent passes, nullable): *keep == 0 means the plan's rho and Phi are those of the
 // forward on the same inputs; the passes then skip them and transform the tangent mesh only.

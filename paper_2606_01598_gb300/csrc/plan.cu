@@ -479,16 +479,19 @@ struct FrameInput {
   int ion_off, n;
 };
 
-// Whether the options ask for the hand-written transforms: fft 2 always; fft 0 (automatic)
+// Whether the options ask for the hand-written transforms: fft 2 and 3 always; fft 0
+// (automatic) whenever every frame takes the power-of-two kernels (axes of 64 or 128 points),
+// for single frames whose every axis splits into two register steps (two_step_factors), and
 // for batched plans of small meshes (no axis above kConvAutoMaxAxis), whose frames then share
-// one launch per pass instead of a cuFFT plan per mesh shape. On GB300 these passes beat
-// cuFFT on batches of 16-48 point meshes and lose to it at 128^3, where the spectrum stays in
-// L2 and cuFFT's per-point cost is lower. The axis lengths and shared-memory sizes are
-// checked by the caller.
-// Meshes whose every axis is 64 or 128 points take the power-of-two kernels (compile-time
-// four-step transforms), which beat cuFFT on GB300 for single frames too (a 128^3 R2C pass in
-// a fraction of cuFFT's three kernels), so the automatic choice takes them whenever every
-// frame qualifies.
+// one launch per pass instead of a cuFFT plan per mesh shape. The axis lengths and
+// shared-memory sizes are checked by the caller (a mesh whose planes do not fit goes to cuFFT).
+// Measured on GB300, solve of one frame, three plans in turn (us), two-step kernels against
+// cuFFT's six plus the influence pass: 32^3 20.5 / 25.9, 48^3 21.2 / 26.0, 80x81x90 28.9 / 31.5,
+// 96^3 30.8 / 36.9, 100^3 36.2 / 33.6, 144^3 51.0 / 56.7, 150^3 60.7 / 90.1, 160^3 92.8 / 85.4.
+// The two sizes where cuFFT's solve is a little faster are taken too: a backward on the
+// forward's inputs transforms one mesh here and two there, and the passes are three launches
+// instead of seven. The six lengths without two such factors stay with cuFFT (125^3: 71.9 on
+// the Stockham kernels, 52.0 on cuFFT).
 constexpr int kConvAutoMaxAxis = 64;
 
 static bool conv_wanted(const pme_plan_s* p, bool single, const std::vector<FrameInput>& fin) {
@@ -497,7 +500,12 @@ static bool conv_wanted(const pme_plan_s* p, bool single, const std::vector<Fram
   bool p2 = true;
   for (const FrameInput& f : fin) p2 = p2 && conv_p2_ok(f.mesh);
   if (p2) return true;
-  if (single) return false;
+  if (single) {
+    int P, Q;
+    for (int a = 0; a < 3; ++a)
+      if (!two_step_factors(fin[0].mesh[a], &P, &Q)) return false;
+    return true;
+  }
   for (const FrameInput& f : fin)
     for (int a = 0; a < 3; ++a)
       if (f.mesh[a] > kConvAutoMaxAxis) return false;
@@ -551,8 +559,9 @@ static int build_plan(pme_plan_s* p, const std::vector<FrameInput>& fin, double 
     if (conv && !p2) {
       for (int f = 0; f < F; ++f) smem_plane = std::max(smem_plane, conv_plane_smem(fin[f].mesh, cap));
     }
+    int optin = 0;
     if (conv) {
-      int dev = 0, optin = 0;
+      int dev = 0;
       cudaGetDevice(&dev);
       if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
         cudaGetLastError();
@@ -564,10 +573,30 @@ static int build_plan(pme_plan_s* p, const std::vector<FrameInput>& fin, double 
       return set_error(p, PME_ERR_UNSUPPORTED, "fft = 2 / 3: a mesh the library's transforms do not take");
     p->conv = conv;
     p->conv_p2 = conv && p2;
+    // two register steps per transform where every axis splits and the layout fits (it is a
+    // little larger than the general kernels'); the Stockham kernels otherwise
+    bool two = conv && !p2;
+    size_t two_plane = 0, two_x = 0;
+    int two_threads = 0;
+    for (int f = 0; f < F && two; ++f) {
+      int P, Q;
+      for (int a = 0; a < 3; ++a) two = two && two_step_factors(fin[f].mesh[a], &P, &Q);
+      if (!two) break;
+      const int pp = two_planes_per_block(fin[f].mesh, single);
+      two_plane = std::max(two_plane, two_plane_smem(fin[f].mesh, pp));
+      two_x = std::max(two_x, two_x_smem(fin[f].mesh));
+      two_threads = std::max(two_threads, two_plane_threads(fin[f].mesh, pp));
+    }
+    p->conv_two = two && two_plane + 1024 <= size_t(optin) && two_x + 1024 <= size_t(optin);
     p->conv_cap = int(cap);
     p->conv_smem_plane = smem_plane;
     p->conv_smem_x = smem_x;
     p->conv_threads = biggest >= 8192 ? 1024 : (biggest >= 2048 ? 512 : 256);
+    if (p->conv_two) {
+      p->conv_smem_plane = two_plane;
+      p->conv_smem_x = two_x;
+      p->conv_threads = two_threads;
+    }
   }
   std::vector<int> ncells(F);
   for (int f = 0; f < F; ++f) {
@@ -598,6 +627,10 @@ static int build_plan(pme_plan_s* p, const std::vector<FrameInput>& fin, double 
     if (p->conv) {
       conv_tiles(g.N, &D.infl_nblk, &D.conv_cols);
       D.conv_pp = conv_planes_per_block(g.N);
+      if (p->conv_two) {
+        D.conv_pp = two_planes_per_block(g.N, single);
+        for (int a = 0; a < 3; ++a) two_step_factors(g.N[a], &D.conv_p[a], &D.conv_q[a]);
+      }
     } else {
       D.infl_nblk = influence_blocks(g);
     }
