@@ -563,21 +563,30 @@ __global__ void __launch_bounds__(kPairThreads) k_pair(PairArgs a) {
 // hits (r, j), in stream order, to its list in global memory; list_cnt = hits, or -1 (and
 // *overflow = 1) when an ion has more than list_cap.
 // (ions of a cell sharing one candidate stream in the list pass: up to eight, so that most
-// cells walk their stream once; slots past the cell's last ion are skipped, warp-uniformly)
+// cells walk their stream once; slots past the warp's last ion are skipped, warp-uniformly)
+// Where the cells alone are too few warps for the device, each cell's ions are split over
+// 1 << split warps (build_split): a warp's time is its own chain of loads and tests, and a small
+// frame, whose cutoff reaches several images of every cell, has long chains in few warps. 64
+// ions in a 12.7 Angstrom box (8 cells of 1000 candidates): 54 us for 8 warps; with 64 warps the
+// whole forward went from 78 to 52 us.
 constexpr int kBuildSlots = 8;
 
 template <bool BATCH, bool ORTHO>
-__global__ void __launch_bounds__(kPairThreads) k_pair_build(PairArgs a, int* overflow) {
+__global__ void __launch_bounds__(kPairThreads) k_pair_build(PairArgs a, int split, int* overflow) {
   constexpr int kSlots = kBuildSlots;
   __shared__ float4 s_fi[kPairWarps][kSlots];
   __shared__ unsigned s_cand[kPairWarps][kCandCap];
   __shared__ int s_code[kPairWarps][32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int cidx = blockIdx.x * kPairWarps + w;
+  const int widx = blockIdx.x * kPairWarps + w;
+  const int cidx = widx >> split, part = widx & ((1 << split) - 1);
   if (cidx >= a.ncells) return;   // uniform per warp
   const int cell = a.cell_lo + cidx;
-  const int c_lo = a.start_c[cell], c_hi = a.start_c[cell + 1];
-  if (c_lo == c_hi) return;
+  // this warp's share of the cell's ions
+  const int cell_first = a.start_c[cell], cell_end = a.start_c[cell + 1];
+  const int per = (cell_end - cell_first + (1 << split) - 1) >> split;
+  const int c_lo = cell_first + part * per, c_hi = min(cell_end, c_lo + per);
+  if (c_lo >= c_hi) return;
   const int frame = BATCH ? a.maps.sorted_frame[c_lo] : 0;
   const FrameDesc& F = frame_at<BATCH>(a.one, a.maps, frame);
   const Geometry& g = F.g;
@@ -618,6 +627,19 @@ __global__ void __launch_bounds__(kPairThreads) k_pair_build(PairArgs a, int* ov
     }
     __syncwarp();
   }
+}
+
+// log2 of the warps per cell of the list pass: one warp where the cells make kBuildWarpsPerSM
+// warps per SM (about what stays resident); otherwise the power of two that brings the device to
+// that, at most eight and at most the mean ions per cell. (Fetching a warp's candidates into
+// shared memory ahead of the tests was measured too: no faster for small frames, and 142 -> 147
+// us for the forward at 32768 ions, whose list pass is bound by issue.)
+constexpr int kBuildWarpsPerSM = 16;
+int build_split(int ncells, int n) {
+  const long long want = (long long)kBuildWarpsPerSM * device_sm_count();
+  int split = 0;
+  while (split < 3 && ((long long)ncells << split) < want && ((long long)ncells << split) < n) ++split;
+  return split;
 }
 
 // Pair term from the lists: one warp per ion (pair-cell order); lane l takes hits l, l + 32,
@@ -760,15 +782,16 @@ int launch_pair_build(pme_plan_t p, cudaStream_t s, int n, int* overflow) {
   int st = check_cuda(p, cudaMemsetAsync(overflow, 0, sizeof(int), s), "memset");
   if (st || n == 0) return st;
   PairArgs a = pair_args(p, nullptr, nullptr);
-  const int grid = (a.ncells + kPairWarps - 1) / kPairWarps;
+  const int split = build_split(a.ncells, n);
+  const int grid = int((((long long)a.ncells << split) + kPairWarps - 1) / kPairWarps);
   if (grid == 0) return PME_OK;
   const bool ortho = plan_ortho(p);
   if (p->batch) {
-    if (ortho) k_pair_build<true, true><<<grid, kPairThreads, 0, s>>>(a, overflow);
-    else k_pair_build<true, false><<<grid, kPairThreads, 0, s>>>(a, overflow);
+    if (ortho) k_pair_build<true, true><<<grid, kPairThreads, 0, s>>>(a, split, overflow);
+    else k_pair_build<true, false><<<grid, kPairThreads, 0, s>>>(a, split, overflow);
   } else {
-    if (ortho) k_pair_build<false, true><<<grid, kPairThreads, 0, s>>>(a, overflow);
-    else k_pair_build<false, false><<<grid, kPairThreads, 0, s>>>(a, overflow);
+    if (ortho) k_pair_build<false, true><<<grid, kPairThreads, 0, s>>>(a, split, overflow);
+    else k_pair_build<false, false><<<grid, kPairThreads, 0, s>>>(a, split, overflow);
   }
   count_launch();
   return check_launch(p, "k_pair_build");
