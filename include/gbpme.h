@@ -158,12 +158,14 @@ const char* pme_status_string(int status);
  * raised since the previous pme_sync_status, clearing them. */
 int pme_sync_status(pme_plan_t plan, void* stream);
 
-/* Repeated calls. pme_forward, pme_backward and their pme_batch_* forms keep one CUDA graph
- * per pass kind: the second call with the same n and the same pointers (host arguments count
- * by the plan's staging buffers, so any host pointers qualify) records the pass once on a
- * plan-owned stream, and that call and every later identical call launch the recorded graph
- * on `stream`, with the same results. A different call runs directly; pme_plan_set_box drops
- * the graphs, and calls made while the stage timers are on always run directly. */
+/* Repeated calls. Every forward and backward entry point (single-frame, batched, with the virial,
+ * with quadrupoles) keeps one CUDA graph per pass kind: the second call with the same n records
+ * the pass once on a plan-owned stream, and that call and every later one of that n launch the
+ * recorded graph on `stream`, with the same results. The call's pointers are handed to the graph
+ * with each launch, so any buffers qualify (with recip_method 1 the pointers must be the same
+ * too). A different n runs directly, as do calls made while the stage timers are on or while
+ * `stream` is being captured by the caller (the pass is then captured into the caller's graph);
+ * pme_plan_set_box drops the graphs. */
 
 /* Forward: energy and derivatives of Eq. (1).
  *   energy     [1] float64: E                     (may be NULL)

@@ -36,6 +36,7 @@ namespace {
 constexpr int kCombThreads = kRedItem;   // one block per reduction item
 
 struct CombineArgs {
+  const PassIO* io;         // recorded passes: the caller's pointers (null: those below)
   FrameDesc one;
   FrameMaps maps;
   const float* mesh_out;
@@ -86,6 +87,15 @@ __device__ __forceinline__ float bg_factor(const CombineArgs& a, const FrameDesc
 template <bool BATCH>
 __global__ void __launch_bounds__(kCombThreads) k_combine_forward(CombineArgs a) {
   pdl_begin();
+  if (a.io) {
+    a.in = a.io->in;
+    a.force = a.io->force;
+    a.phi = a.io->phi;
+    a.field = a.io->field;
+    a.field_grad = a.io->field_grad;
+    a.energy_out = a.io->energy;
+    a.virial_out = a.io->virial;
+  }
   static_assert(kRedItem == kCombThreads, "one ion per thread");
   const int item = blockIdx.x;
   const int f = BATCH ? a.maps.item_frame[item] : 0;
@@ -234,6 +244,14 @@ __global__ void __launch_bounds__(kCombThreads) k_combine_forward(CombineArgs a)
 template <bool BATCH>
 __global__ void __launch_bounds__(kCombThreads) k_combine_backward_quad(CombineArgs a, const float* qm,
                                                                       const float* qp, float* grad_theta) {
+  if (a.io) {
+    a.in = a.io->in;
+    a.g_energy = a.io->g_energy;
+    a.grad_pos = a.io->grad_pos;
+    a.grad_q = a.io->grad_q;
+    a.grad_mu = a.io->grad_mu;
+    grad_theta = a.io->grad_theta;
+  }
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= a.in.n) return;
   const int f = BATCH ? a.maps.ion_frame[i] : 0;
@@ -307,6 +325,7 @@ k_pair_energy(int n, const float* q, const float* mu, const float* pair_out, dou
 
 CombineArgs base_args(pme_plan_t p, const IonInputs& in) {
   CombineArgs a = {};
+  a.io = live_io(p);
   a.one = p->frames_h[0];
   a.maps = p->maps;
   a.in = in;
@@ -372,6 +391,7 @@ BackwardFinish backward_finish_args(pme_plan_t p, const IonInputs& in, float* gr
                                     float* grad_mu) {
   const CombineArgs a = base_args(p, in);
   BackwardFinish f = {};
+  f.io = a.io;
   f.pair_out = p->opts.include_pair ? p->pair_out : nullptr;
   f.q = in.q;
   f.mu = in.mu;

@@ -164,9 +164,11 @@ __device__ __forceinline__ int fdiv(int x, const FastDiv& f) {
 }
 
 // A pass (forward or backward) recorded as a CUDA graph: made on the second consecutive call
-// with the same arguments, replayed while they stay the same. The key holds every pointer and
-// size of the call and the host-side state the pass depends on; post_* is the host-side state
-// the pass leaves behind.
+// of the same kind and size, replayed while they stay the same. The key holds the size of the
+// call and the host-side state the pass depends on; the call's pointers are not part of it: a
+// recorded pass reads them from the plan's PassIO in device memory, which its first node writes
+// (that node's arguments are set before each launch). (The explicit k-sum's passes bake their
+// pointers in and have them in the key.) post_* is the host-side state the pass leaves behind.
 struct PassKey {
   unsigned long long v[24];
   int len;
@@ -178,11 +180,16 @@ struct PassKey {
   }
 };
 
+struct PassIO;
+enum { kGraphForward, kGraphBackward, kGraphVirial, kGraphQuadForward, kGraphQuadBackward, kNumGraphs };
 struct PassGraph {
   PassKey key;
   PassKey last;
   bool have_last;
   cudaGraphExec_t exec;
+  cudaGraph_t graph;       // the recorded graph (owns the node below)
+  cudaGraphNode_t begin;   // its first node, which writes the call's pointers (null: baked in)
+  PassIO* io;              // host copy of what that node holds
   long long launches;   // kernels per replay (for pme_launch_count)
   int post_fwd_n;
   bool post_fwd_lists;
@@ -330,8 +337,10 @@ struct pme_plan_s {
   float2* ew_S = nullptr;     // [K] structure factor
   uint4* ew_fx = nullptr;     // [max_ions] fixed-point fractional coordinates
   float4* ew_qm = nullptr;    // [max_ions] q, mu
-  // CUDA graphs of repeated passes (0 forward, 1 backward)
+  // CUDA graphs of repeated passes (kNumGraphs kinds)
   gbpme::PassGraph* graphs = nullptr;
+  gbpme::PassIO* io_d = nullptr;       // the pointers of a recorded pass's current call
+  bool io_live = false;                // a pass is being recorded: its kernels read *io_d
   cudaStream_t cap_stream = nullptr;   // capture-only stream (nothing runs on it)
   // stage timers
   bool prof = false;

@@ -26,6 +26,7 @@ constexpr int kGatherThreads = 128;
 constexpr int kGroup = 8;
 
 struct GatherArgs {
+  const PassIO* io;       // recorded passes: the caller's pointers (null: those below)
   FrameDesc one;
   FrameMaps maps;
   MeshRecords mr;
@@ -82,6 +83,17 @@ __host__ __device__ constexpr int gather_tab_floats() {
 template <int P, int MODE, bool BATCH>
 __global__ void __launch_bounds__(kGatherThreads) k_gather(GatherArgs a) {
   pdl_begin();
+  if (MODE == 1 && a.io) {
+    a.g_energy = a.io->g_energy;
+    a.fin.q = a.io->in.q;
+    a.fin.mu = a.io->in.mu;
+    a.fin.gphi = a.io->in.gphi;
+    a.fin.gfield = a.io->in.gfield;
+    a.fin.grad_pos = a.io->grad_pos;
+    a.fin.grad_q = a.io->grad_q;
+    a.fin.grad_mu = a.io->grad_mu;
+  }
+  if (MODE == 2 && a.io) a.theta = a.io->in.theta;
   constexpr bool TAN = MODE == 1;
   constexpr int DM = MODE == 0 ? 2 : 3;
   constexpr int IPW = gather_ions_per_warp<P>();
@@ -395,6 +407,7 @@ __global__ void __launch_bounds__(kGatherThreads) k_gather(GatherArgs a) {
 // out[caller index][26]: the 13 values, then their 13 tangents.
 template <int P, bool BATCH>
 __global__ void __launch_bounds__(kGatherThreads) k_gather_qdual(GatherArgs a) {
+  if (a.io) a.theta = a.io->in.theta;
   const int gid = a.t_lo + (blockIdx.x * blockDim.x + threadIdx.x) / kGroup;
   const int l = threadIdx.x & (kGroup - 1);
   const bool valid = gid < a.t_hi;
@@ -612,6 +625,7 @@ int launch_t(pme_plan_t p, cudaStream_t s, int n, const float* mesh, const doubl
              float* out, const float* theta = nullptr, float* qout = nullptr,
              const BackwardFinish* fin = nullptr) {
   GatherArgs a;
+  a.io = live_io(p);
   a.one = p->frames_h[0];
   a.maps = p->maps;
   a.mr = p->mr;
@@ -679,6 +693,7 @@ int launch_gather_quad(pme_plan_t p, cudaStream_t s, int n, const float* mesh, c
 
 int launch_gather_qdual(pme_plan_t p, cudaStream_t s, int n, const float* mesh, const float* theta, float* out) {
   GatherArgs a;
+  a.io = live_io(p);
   a.one = p->frames_h[0];
   a.maps = p->maps;
   a.mr = p->mr;

@@ -19,6 +19,19 @@ struct IonInputs {
   int n;
 };
 
+// Every pointer a pass takes from its caller (see PassGraph).
+struct PassIO {
+  IonInputs in;
+  const double* g_energy;
+  double* energy;
+  double* virial;
+  float *force, *phi, *field, *field_grad;
+  float *grad_pos, *grad_q, *grad_mu, *grad_theta;
+};
+// Kernels take the caller's pointers as arguments and, in a recorded pass, from here (null
+// otherwise).
+inline const PassIO* live_io(pme_plan_t p) { return p->io_live ? p->io_d : nullptr; }
+
 // sort.cu: brick and pair-cell counting sorts (4 kernels), records in both orders.
 // reuse (nullable): when *reuse == 0 the plan's sorted order and primal records are those of
 // these inputs (a forward on them) and are kept; only charge sums and tangent records are
@@ -116,6 +129,7 @@ int launch_conv_inverse(pme_plan_t p, cudaStream_t s, bool tangent, float* mesh,
 // background terms, coulomb_k), done in the tangent gather's epilogue so that the backward
 // needs no separate combine launch.
 struct BackwardFinish {
+  const PassIO* io;        // recorded passes: the caller's pointers (null: those below)
   const float* pair_out;   // [n][8] tangent pair sums in caller order (null: no pair term)
   const float* q;          // [n]
   const float* mu;         // [n][3] or null

@@ -57,6 +57,7 @@ constexpr int kCandCap = 512;  // candidates listed per warp at a time
 constexpr int kSegShift = 27;  // candidate entry: (segment lane << 27) | sorted index
 
 struct PairArgs {
+  const PassIO* io;         // recorded passes: the caller's pointers (null: g_energy below)
   FrameDesc one;
   FrameMaps maps;
   PairRecords pr;
@@ -462,6 +463,7 @@ __global__ void __launch_bounds__(kPairThreads) k_pair(PairArgs a) {
   __shared__ int s_code[kPairWarps][32];                // packed (ox, oy, oz) of each segment
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   if (a.cache_bad && *a.cache_bad == 0) return;
+  if (TAN && a.io) a.g_energy = a.io->g_energy;
   if (a.vir_lost && blockIdx.x == 0 && w == 0 && lane == 0) atomicOr(a.vir_lost, kFlagVirialLost);
   // grid-stride over the cells (the launch may be capped: as a fallback it mostly exits here)
   for (int cidx = blockIdx.x * kPairWarps + w; cidx < a.ncells; cidx += gridDim.x * kPairWarps) {
@@ -648,6 +650,7 @@ int build_split(int ncells, int n) {
 template <bool TAN, bool BATCH, bool VIR = false>
 __global__ void __launch_bounds__(kPairThreads) k_pair_listed(PairArgs a, int n) {
   if (*a.cache_bad != 0) return;
+  if (TAN && a.io) a.g_energy = a.io->g_energy;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int i = blockIdx.x * kPairWarps + w;
   if (i >= n) return;   // uniform per warp
@@ -710,6 +713,7 @@ void launch_k(bool ortho, int grid, cudaStream_t s, const PairArgs& a) {
 // Arguments shared by the pair launches.
 PairArgs pair_args(pme_plan_t p, const double* g_energy, float* out) {
   PairArgs a = {};
+  a.io = live_io(p);
   a.one = p->frames_h[0];
   a.maps = p->maps;
   a.alpha = float(p->alpha);
@@ -779,7 +783,8 @@ int launch_pair(pme_plan_t p, cudaStream_t s, int n, bool tangent, const IonInpu
 }
 
 int launch_pair_build(pme_plan_t p, cudaStream_t s, int n, int* overflow) {
-  int st = check_cuda(p, cudaMemsetAsync(overflow, 0, sizeof(int), s), "memset");
+  // (a recorded pass's first node clears the flag, p->cache_bad)
+  int st = p->io_live ? PME_OK : check_cuda(p, cudaMemsetAsync(overflow, 0, sizeof(int), s), "memset");
   if (st || n == 0) return st;
   PairArgs a = pair_args(p, nullptr, nullptr);
   const int split = build_split(a.ncells, n);

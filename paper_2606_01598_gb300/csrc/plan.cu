@@ -385,7 +385,7 @@ static void free_plan(pme_plan_t p) {
                   p->plist, p->plist_cnt, p->in_saved, p->in_flags, p->vpart,
                   p->pvir, p->vitem, p->gtab, p->sb.t_bidx, p->sb.t_bfq,
                   p->sb.t_bdm, p->sb.t_cidx, p->sb.t_cfq, p->sb.t_cmu, p->conv_tw,
-                  p->conv_planes1, p->quad_out};
+                  p->conv_planes1, p->quad_out, p->io_d};
   for (void* b : bufs)
     if (b) cudaFree(b);
   for (int g = 0; g < p->nfgroups; ++g) {
@@ -958,9 +958,10 @@ static int build_plan(pme_plan_s* p, const std::vector<FrameInput>& fin, double 
   }
   if (p->gtab && ((st = launch_influence_tables(p, 0)) || (st = check_cuda(p, cudaDeviceSynchronize(), "synchronize"))))
     return st;
-  p->graphs = new (std::nothrow) PassGraph[2];
+  p->graphs = new (std::nothrow) PassGraph[kNumGraphs];
   if (!p->graphs) return set_error(p, PME_ERR_NOMEM, "host tables");
-  std::memset(p->graphs, 0, sizeof(PassGraph) * 2);
+  std::memset(p->graphs, 0, sizeof(PassGraph) * kNumGraphs);
+  if ((st = dalloc(p, &p->io_d, 1))) return st;
   if ((st = check_cuda(p, cudaStreamCreateWithFlags(&p->cap_stream, cudaStreamNonBlocking), "stream"))) return st;
   if ((st = check_cuda(p, cudaStreamCreateWithFlags(&p->side, cudaStreamNonBlocking), "stream")) ||
       (st = check_cuda(p, cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming), "event")) ||
@@ -1043,28 +1044,107 @@ static PassKey make_key(std::initializer_list<unsigned long long> vals) {
 
 static unsigned long long ptr_bits(const void* ptr) { return (unsigned long long)(uintptr_t)ptr; }
 
+static PassIO forward_io(const IonInputs& in, double* energy, double* virial, float* force, float* phi, float* field,
+                         float* field_grad) {
+  PassIO io;
+  std::memset(&io, 0, sizeof(io));   // compared bytewise
+  io.in.pos = in.pos;
+  io.in.q = in.q;
+  io.in.mu = in.mu;
+  io.in.theta = in.theta;
+  io.in.n = in.n;
+  io.energy = energy;
+  io.virial = energy ? virial : nullptr;
+  io.force = force;
+  io.phi = phi;
+  io.field = field;
+  io.field_grad = field_grad;
+  return io;
+}
+
+static PassIO backward_io(const IonInputs& in, const double* g_energy, float* grad_pos, float* grad_q, float* grad_mu,
+                          float* grad_theta) {
+  PassIO io = forward_io(in, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr);
+  io.in.gforce = in.gforce;
+  io.in.gphi = in.gphi;
+  io.in.gfield = in.gfield;
+  io.g_energy = g_energy;
+  io.grad_pos = grad_pos;
+  io.grad_q = grad_q;
+  io.grad_mu = grad_mu;
+  io.grad_theta = grad_theta;
+  return io;
+}
+
+static void drop_graph(PassGraph& G) {
+  if (G.exec) cudaGraphExecDestroy(G.exec);
+  if (G.graph) cudaGraphDestroy(G.graph);
+  delete G.io;
+  G.exec = nullptr;
+  G.graph = nullptr;
+  G.begin = nullptr;
+  G.io = nullptr;
+}
+
 static void drop_graphs(pme_plan_t p) {
   if (!p->graphs) return;
-  for (int k = 0; k < 2; ++k) {
-    if (p->graphs[k].exec) cudaGraphExecDestroy(p->graphs[k].exec);
-    p->graphs[k].exec = nullptr;
+  for (int k = 0; k < kNumGraphs; ++k) {
+    drop_graph(p->graphs[k]);
     p->graphs[k].have_last = false;
   }
 }
 
-// Run a pass, through a CUDA graph when the same call (key) comes again: the second identical
-// call records the pass on the plan's capture stream and launches the graph; later identical
-// calls only launch it. The pass sees device pointers only (host arguments are copied to and
-// from the plan's staging buffers on the stream before and after it), so staged calls replay
-// too. eligible = false, or stage timers on, runs directly.
+// First node of a recorded pass: the call's pointers to where the pass's kernels read them, and
+// the pass's flags (in_diff, cache_bad) cleared.
+__global__ void k_begin_pass(PassIO io, PassIO* dst, int* flags) {
+  if (threadIdx.x == 0) *dst = io;
+  if (threadIdx.x < 2) flags[threadIdx.x] = 0;
+}
+
+// Point a recorded pass at this call's pointers.
+static int set_pass_io(pme_plan_t p, PassGraph& G, const PassIO& io) {
+  if (std::memcmp(G.io, &io, sizeof(io)) == 0) return PME_OK;
+  PassIO arg = io;
+  PassIO* dst = p->io_d;
+  int* flags = p->in_flags;
+  void* args[] = {&arg, &dst, &flags};
+  cudaKernelNodeParams kp = {};
+  kp.func = reinterpret_cast<void*>(k_begin_pass);
+  kp.gridDim = dim3(1);
+  kp.blockDim = dim3(32);
+  kp.kernelParams = args;
+  const int st = check_cuda(p, cudaGraphExecKernelNodeSetParams(G.exec, G.begin, &kp), "graph node parameters");
+  if (st) cudaGetLastError();
+  else std::memcpy(G.io, &io, sizeof(io));
+  return st;
+}
+
+static bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cs) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return cs != cudaStreamCaptureStatusNone;
+}
+
+// Run a pass, through a CUDA graph when the same call (key) comes again: the second such call
+// records the pass on the plan's capture stream and launches the graph; later ones only launch
+// it. With io the call's pointers are not in the key: the graph's first node hands them to the
+// kernels, so calls with other buffers (outputs allocated per call, say) replay too. A graph
+// launch costs the host one call where the pass itself costs 15 to 30; of the small frames'
+// time that was most (forward + backward of 1999
+// ions with outputs allocated per call: 0.218 -> 0.105 ms; forward of 512 ions 0.109 -> 0.050 ms). Staged
+// host arguments are copied outside the pass. Stage timers, or a caller that is capturing the
+// stream itself, run the pass directly.
 template <class Run>
-static int run_pass(pme_plan_t p, int which, cudaStream_t s, const PassKey& key, bool eligible, Run&& run) {
+static int run_pass(pme_plan_t p, int which, cudaStream_t s, const PassKey& key, const PassIO* io, Run&& run) {
   PassGraph& G = p->graphs[which];
-  if (!eligible || p->prof) {
+  if (p->prof || capturing(s)) {
     G.have_last = false;
     return run(s);
   }
-  if (G.exec && G.key == key) {
+  if (G.exec && G.key == key && (!io || set_pass_io(p, G, *io) == PME_OK)) {
     int st = check_cuda(p, cudaGraphLaunch(G.exec, s), "graph launch");
     if (st) return st;
     for (long long k = 0; k < G.launches; ++k) count_launch();
@@ -1077,24 +1157,32 @@ static int run_pass(pme_plan_t p, int which, cudaStream_t s, const PassKey& key,
     G.have_last = true;
     return run(s);
   }
-  // second identical call: record the pass (nothing executes while capturing)
+  // second such call: record the pass (nothing executes while capturing)
   const long long before = pme_launch_count();
   const int save_n = p->fwd_n;
   const bool save_lists = p->fwd_lists;
-  cudaGraph_t graph = nullptr;
+  PassGraph N = {};
   int st = check_cuda(p, cudaStreamBeginCapture(p->cap_stream, cudaStreamCaptureModeThreadLocal), "begin capture");
   if (!st) {
+    if (io) k_begin_pass<<<1, 32, 0, p->cap_stream>>>(*io, p->io_d, p->in_flags);
+    p->io_live = io != nullptr;
     const int rs = run(p->cap_stream);
-    const cudaError_t ce = cudaStreamEndCapture(p->cap_stream, &graph);
-    if (rs || ce != cudaSuccess || !graph) st = rs ? rs : check_cuda(p, ce, "end capture");
+    p->io_live = false;
+    const cudaError_t ce = cudaStreamEndCapture(p->cap_stream, &N.graph);
+    if (rs || ce != cudaSuccess || !N.graph) st = rs ? rs : check_cuda(p, ce, "end capture");
   }
   const long long captured = pme_launch_count() - before;
   g_launches.fetch_sub(captured, std::memory_order_relaxed);   // recorded, not launched
-  cudaGraphExec_t exec = nullptr;
-  if (!st) st = check_cuda(p, cudaGraphInstantiate(&exec, graph, 0), "graph instantiate");
-  if (graph) cudaGraphDestroy(graph);
+  if (!st && io) {
+    size_t roots = 1;
+    st = check_cuda(p, cudaGraphGetRootNodes(N.graph, &N.begin, &roots), "graph root");
+    N.io = new (std::nothrow) PassIO(*io);
+    if (!st && (roots != 1 || !N.io)) st = PME_ERR_CUDA;
+  }
+  if (!st) st = check_cuda(p, cudaGraphInstantiate(&N.exec, N.graph, 0), "graph instantiate");
   if (st) {
     // fall back to a direct run with the host state as it was
+    drop_graph(N);
     cudaGetLastError();
     p->last_error.clear();
     p->fwd_n = save_n;
@@ -1102,8 +1190,11 @@ static int run_pass(pme_plan_t p, int which, cudaStream_t s, const PassKey& key,
     G.have_last = false;
     return run(s);
   }
-  if (G.exec) cudaGraphExecDestroy(G.exec);
-  G.exec = exec;
+  drop_graph(G);
+  G.exec = N.exec;
+  G.graph = N.graph;
+  G.begin = N.begin;
+  G.io = N.io;
   G.key = key;
   G.launches = captured;
   G.post_fwd_n = p->fwd_n;
@@ -1489,10 +1580,14 @@ int pme_forward(pme_plan_t p, void* stream, int n, const float* pos, const float
   float* fl_out = sg.out(field, 3, kOField);
   float* fg_out = sg.out(field_grad, 6, kOFG);
   if ((st = sg.ready())) return st;
-  const PassKey key = make_key({0ull, (unsigned long long)n, ptr_bits(in.pos), ptr_bits(in.q), ptr_bits(in.mu),
-                                ptr_bits(e_out), ptr_bits(f_out), ptr_bits(p_out), ptr_bits(fl_out),
-                                ptr_bits(fg_out)});
-  st = run_pass(p, 0, s, key, true,
+  const PassIO io = forward_io(in, e_out, nullptr, f_out, p_out, fl_out, fg_out);
+  // (the explicit k-sum's kernels take their pointers as arguments only)
+  const bool mesh = p->opts.recip_method == 0;
+  const PassKey key = mesh ? make_key({(unsigned long long)n})
+                           : make_key({(unsigned long long)n, ptr_bits(in.pos), ptr_bits(in.q), ptr_bits(in.mu),
+                                       ptr_bits(e_out), ptr_bits(f_out), ptr_bits(p_out), ptr_bits(fl_out),
+                                       ptr_bits(fg_out)});
+  st = run_pass(p, kGraphForward, s, key, mesh ? &io : nullptr,
                 [&](cudaStream_t cs) { return run_forward(p, cs, in, e_out, f_out, p_out, fl_out, fg_out); });
   if (st) return st;
   return sg.finish();
@@ -1523,13 +1618,17 @@ int pme_forward_virial(pme_plan_t p, void* stream, int n, const float* pos, cons
   float* fl_out = sg.out(field, 3, kOField);
   float* fg_out = sg.out(field_grad, 6, kOFG);
   if ((st = sg.ready())) return st;
-  if ((st = run_forward(p, s, in, e_out, f_out, p_out, fl_out, fg_out, v_out))) return st;
+  const PassIO io = forward_io(in, e_out, v_out, f_out, p_out, fl_out, fg_out);
+  st = run_pass(p, kGraphVirial, s, make_key({(unsigned long long)n}), &io, [&](cudaStream_t cs) {
+    return run_forward(p, cs, in, e_out, f_out, p_out, fl_out, fg_out, v_out);
+  });
+  if (st) return st;
   return sg.finish();
 }
 
 // Forward with point quadrupoles (the rank-2 channel) over every frame of the plan: sort,
 // quadrupole spread, the mesh convolution, quadrupole gather, the quadrupole pair kernel,
-// combine. Runs directly (no graph) and leaves nothing for a backward to reuse.
+// combine. Leaves nothing for a backward to reuse.
 static int run_forward_quad(pme_plan_t p, cudaStream_t s, const IonInputs& in, double* e_out,
                             float* f_out, float* p_out, float* fl_out, float* fg_out) {
   const int n = in.n;
@@ -1617,7 +1716,10 @@ int pme_forward_quad(pme_plan_t p, void* stream, int n, const float* pos, const 
   float* fl_out = sg.out(field, 3, kOField);
   float* fg_out = sg.out(field_grad, 6, kOFG);
   if ((st = sg.ready())) return st;
-  if ((st = run_forward_quad(p, s, in, e_out, f_out, p_out, fl_out, fg_out))) return st;
+  const PassIO io = forward_io(in, e_out, nullptr, f_out, p_out, fl_out, fg_out);
+  st = run_pass(p, kGraphQuadForward, s, make_key({(unsigned long long)n}), &io,
+                [&](cudaStream_t cs) { return run_forward_quad(p, cs, in, e_out, f_out, p_out, fl_out, fg_out); });
+  if (st) return st;
   return sg.finish();
 }
 
@@ -1645,7 +1747,10 @@ int pme_batch_forward_quad(pme_plan_t p, void* stream, const float* pos, const f
   float* fl_out = sg.out(field, 3, kOField);
   float* fg_out = sg.out(field_grad, 6, kOFG);
   if ((st = sg.ready())) return st;
-  if ((st = run_forward_quad(p, s, in, e_out, f_out, p_out, fl_out, fg_out))) return st;
+  const PassIO io = forward_io(in, e_out, nullptr, f_out, p_out, fl_out, fg_out);
+  st = run_pass(p, kGraphQuadForward, s, make_key({(unsigned long long)n}), &io,
+                [&](cudaStream_t cs) { return run_forward_quad(p, cs, in, e_out, f_out, p_out, fl_out, fg_out); });
+  if (st) return st;
   return sg.finish();
 }
 
@@ -1724,7 +1829,10 @@ static int backward_quad_common(pme_plan_t p, void* stream, int n, const float* 
   float* o_mu = sg.out(grad_mu, 3, kOGMu);
   float* o_th = sg.out(grad_theta, 6, kOGTheta);
   if ((st = sg.ready())) return st;
-  if ((st = run_backward_quad(p, s, in, gE, o_pos, o_q, o_mu, o_th))) return st;
+  const PassIO io = backward_io(in, gE, o_pos, o_q, o_mu, o_th);
+  st = run_pass(p, kGraphQuadBackward, s, make_key({(unsigned long long)n}), &io,
+                [&](cudaStream_t cs) { return run_backward_quad(p, cs, in, gE, o_pos, o_q, o_mu, o_th); });
+  if (st) return st;
   return sg.finish();
 }
 
@@ -1773,11 +1881,10 @@ int pme_backward(pme_plan_t p, void* stream, int n, const float* pos, const floa
   float* o_q = sg.out(grad_q, 1, kOGQ);
   float* o_mu = sg.out(grad_mu, 3, kOGMu);
   if ((st = sg.ready())) return st;
-  const PassKey key = make_key({1ull, (unsigned long long)n, ptr_bits(in.pos), ptr_bits(in.q), ptr_bits(in.mu),
-                                ptr_bits(gE), ptr_bits(in.gforce), ptr_bits(in.gphi), ptr_bits(in.gfield),
-                                ptr_bits(o_pos), ptr_bits(o_q), ptr_bits(o_mu),
-                                (unsigned long long)(long long)p->fwd_n, (unsigned long long)p->fwd_lists});
-  st = run_pass(p, 1, s, key, true,
+  const PassIO io = backward_io(in, gE, o_pos, o_q, o_mu, nullptr);
+  const PassKey key = make_key({(unsigned long long)n, (unsigned long long)(long long)p->fwd_n,
+                                (unsigned long long)p->fwd_lists});
+  st = run_pass(p, kGraphBackward, s, key, &io,
                 [&](cudaStream_t cs) { return run_backward(p, cs, in, gE, o_pos, o_q, o_mu); });
   if (st) return st;
   return sg.finish();
@@ -1808,10 +1915,14 @@ int pme_batch_forward(pme_plan_t p, void* stream, const float* pos, const float*
   float* fl_out = sg.out(field, 3, kOField);
   float* fg_out = sg.out(field_grad, 6, kOFG);
   if ((st = sg.ready())) return st;
-  const PassKey key = make_key({0ull, (unsigned long long)n, ptr_bits(in.pos), ptr_bits(in.q), ptr_bits(in.mu),
-                                ptr_bits(e_out), ptr_bits(f_out), ptr_bits(p_out), ptr_bits(fl_out),
-                                ptr_bits(fg_out)});
-  st = run_pass(p, 0, s, key, true,
+  const PassIO io = forward_io(in, e_out, nullptr, f_out, p_out, fl_out, fg_out);
+  // (the explicit k-sum's kernels take their pointers as arguments only)
+  const bool mesh = p->opts.recip_method == 0;
+  const PassKey key = mesh ? make_key({(unsigned long long)n})
+                           : make_key({(unsigned long long)n, ptr_bits(in.pos), ptr_bits(in.q), ptr_bits(in.mu),
+                                       ptr_bits(e_out), ptr_bits(f_out), ptr_bits(p_out), ptr_bits(fl_out),
+                                       ptr_bits(fg_out)});
+  st = run_pass(p, kGraphForward, s, key, mesh ? &io : nullptr,
                 [&](cudaStream_t cs) { return run_forward(p, cs, in, e_out, f_out, p_out, fl_out, fg_out); });
   if (st) return st;
   return sg.finish();
@@ -1842,7 +1953,11 @@ int pme_batch_forward_virial(pme_plan_t p, void* stream, const float* pos, const
   float* fl_out = sg.out(field, 3, kOField);
   float* fg_out = sg.out(field_grad, 6, kOFG);
   if ((st = sg.ready())) return st;
-  if ((st = run_forward(p, s, in, e_out, f_out, p_out, fl_out, fg_out, v_out))) return st;
+  const PassIO io = forward_io(in, e_out, v_out, f_out, p_out, fl_out, fg_out);
+  st = run_pass(p, kGraphVirial, s, make_key({(unsigned long long)n}), &io, [&](cudaStream_t cs) {
+    return run_forward(p, cs, in, e_out, f_out, p_out, fl_out, fg_out, v_out);
+  });
+  if (st) return st;
   return sg.finish();
 }
 
@@ -1867,11 +1982,10 @@ int pme_batch_backward(pme_plan_t p, void* stream, const float* pos, const float
   float* o_q = sg.out(grad_q, 1, kOGQ);
   float* o_mu = sg.out(grad_mu, 3, kOGMu);
   if ((st = sg.ready())) return st;
-  const PassKey key = make_key({1ull, (unsigned long long)n, ptr_bits(in.pos), ptr_bits(in.q), ptr_bits(in.mu),
-                                ptr_bits(gE), ptr_bits(in.gforce), ptr_bits(in.gphi), ptr_bits(in.gfield),
-                                ptr_bits(o_pos), ptr_bits(o_q), ptr_bits(o_mu),
-                                (unsigned long long)(long long)p->fwd_n, (unsigned long long)p->fwd_lists});
-  st = run_pass(p, 1, s, key, true,
+  const PassIO io = backward_io(in, gE, o_pos, o_q, o_mu, nullptr);
+  const PassKey key = make_key({(unsigned long long)n, (unsigned long long)(long long)p->fwd_n,
+                                (unsigned long long)p->fwd_lists});
+  st = run_pass(p, kGraphBackward, s, key, &io,
                 [&](cudaStream_t cs) { return run_backward(p, cs, in, gE, o_pos, o_q, o_mu); });
   if (st) return st;
   return sg.finish();

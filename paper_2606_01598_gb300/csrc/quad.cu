@@ -49,6 +49,7 @@ struct QuadPairArgs {
   FrameMaps maps;
   PairRecords pr;
   const int* start_c;
+  const PassIO* io;     // recorded passes: the caller's pointers (null: theta below)
   const float* theta;   // [caller index][6]
   float* out;           // [caller index][10]
   float* qout;          // [caller index][8], this kernel writes 4..6
@@ -164,6 +165,7 @@ __global__ void __launch_bounds__(kQuadThreads) k_pair_quad(QuadPairArgs a) {
   __shared__ float4 s_hit[kWarps][kHitCap];   // r (x, y, z), source j (int bits)
   __shared__ unsigned s_cand[kWarps][kCandCap];
   if (a.flag && *a.flag == 0) return;   // the lists hold: the list-driven kernel does the work
+  if (a.io) a.theta = a.io->in.theta;
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int i = blockIdx.x * kWarps + wid;
   if (i >= a.n) return;   // warp-uniform
@@ -306,6 +308,7 @@ __global__ void __launch_bounds__(kQuadThreads) k_pair_quad(QuadPairArgs a) {
 template <bool BATCH>
 __global__ void __launch_bounds__(kQuadThreads) k_pair_quad_listed(QuadPairArgs a) {
   if (*a.flag != 0) return;
+  if (a.io) a.theta = a.io->in.theta;
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int i = blockIdx.x * kWarps + wid;
   if (i >= a.n) return;   // warp-uniform
@@ -343,6 +346,7 @@ __global__ void __launch_bounds__(kQuadThreads) k_pair_quad_listed(QuadPairArgs 
 template <bool BATCH>
 __global__ void __launch_bounds__(kQuadThreads) k_pair_quad_dual(QuadPairArgs a) {
   if (*a.flag != 0) return;
+  if (a.io) a.theta = a.io->in.theta;
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int i = blockIdx.x * kWarps + wid;
   if (i >= a.n) return;   // warp-uniform
@@ -384,6 +388,7 @@ __global__ void k_flag_if_set(const int* cond, int* flags, int bit) {
 
 QuadPairArgs quad_args(pme_plan_t p, int n, const float* theta, float* out, float* qout, const int* flag) {
   QuadPairArgs a;
+  a.io = live_io(p);
   a.one = p->frames_h[0];
   a.maps = p->maps;
   a.pr = p->pr;

@@ -102,9 +102,10 @@ __device__ void block_exclusive_scan(int* count, int* start, int n) {
 // order).
 template <bool BATCH>
 __global__ void __launch_bounds__(kSortThreads)
-k_bin(FrameDesc one, FrameMaps maps, IonInputs in, SortBuffers sb, int tangent, int* flags,
+k_bin(FrameDesc one, FrameMaps maps, IonInputs in, const PassIO* io, SortBuffers sb, int tangent, int* flags,
       int nbricks, int ncells, const int* reuse, float* save, int ld) {
   pdl_begin();
+  if (io) in = io->in;
   static_assert(kRedItem == kSortThreads, "one ion per thread");
   const int item = blockIdx.x;
   const int f = BATCH ? maps.item_frame[item] : 0;
@@ -248,9 +249,10 @@ __device__ __forceinline__ int stable_rank(const int* perm, int seg_lo, int seg_
 
 template <bool BATCH>
 __global__ void __launch_bounds__(kSortThreads)
-k_rank_records(FrameDesc one, FrameMaps maps, IonInputs in, SortBuffers sb, MeshRecords mr,
+k_rank_records(FrameDesc one, FrameMaps maps, IonInputs in, const PassIO* io, SortBuffers sb, MeshRecords mr,
                PairRecords pr, int tangent, int need_mesh, int need_pair, const int* reuse) {
   pdl_begin();
+  if (io) in = io->in;
   const int n = in.n;
   int t = blockIdx.x * blockDim.x + threadIdx.x;
   const bool mesh_side = t < n;
@@ -405,9 +407,10 @@ k_rank_records(FrameDesc one, FrameMaps maps, IonInputs in, SortBuffers sb, Mesh
 
 // Bitwise comparison of the backward's inputs with the saved forward inputs.
 __global__ void __launch_bounds__(256)
-k_input_check(int n, IonInputs in, const float* saved, int ld, const int* list_cnt, int* in_diff,
+k_input_check(int n, IonInputs in, const PassIO* io, const float* saved, int ld, const int* list_cnt, int* in_diff,
               int* cache_bad) {
   pdl_begin();
+  if (io) in = io->in;
   bool same = true, lists = true;
   const int stride = gridDim.x * blockDim.x;
   const int t0 = blockIdx.x * blockDim.x + threadIdx.x;
@@ -451,7 +454,7 @@ int launch_sort_t(pme_plan_t p, cudaStream_t s, const IonInputs& in, bool tangen
   }
   {
     const int items = BATCH ? p->total_items : one.nitems;
-    pdl_launch(k_bin<BATCH>, items, kSortThreads, 0, s, one, p->maps, in, p->sb, tangent ? 1 : 0, p->flags,
+    pdl_launch(k_bin<BATCH>, items, kSortThreads, 0, s, one, p->maps, in, live_io(p), p->sb, tangent ? 1 : 0, p->flags,
                                                 p->total_bricks, p->total_cells, reuse, save,
                                                 p->max_ions);
     count_launch();
@@ -471,7 +474,7 @@ int launch_sort_t(pme_plan_t p, cudaStream_t s, const IonInputs& in, bool tangen
     count_launch();
     if ((st = check_launch(p, "k_scatter"))) return st;
     const int nblk2 = (2 * n + kSortThreads - 1) / kSortThreads;
-    pdl_launch(k_rank_records<BATCH>, nblk2, kSortThreads, 0, s, one, p->maps, in, p->sb, p->mr, p->pr,
+    pdl_launch(k_rank_records<BATCH>, nblk2, kSortThreads, 0, s, one, p->maps, in, live_io(p), p->sb, p->mr, p->pr,
                                                          tangent ? 1 : 0, need_mesh ? 1 : 0,
                                                          need_pair ? 1 : 0, reuse);
     count_launch();
@@ -483,10 +486,11 @@ int launch_sort_t(pme_plan_t p, cudaStream_t s, const IonInputs& in, bool tangen
 }  // namespace
 
 int launch_input_check(pme_plan_t p, cudaStream_t s, const IonInputs& in, bool with_lists) {
-  int st = check_cuda(p, cudaMemsetAsync(p->in_flags, 0, 2 * sizeof(int), s), "memset");
+  // (a recorded pass's first node clears the flags)
+  int st = p->io_live ? PME_OK : check_cuda(p, cudaMemsetAsync(p->in_flags, 0, 2 * sizeof(int), s), "memset");
   if (st || in.n == 0) return st;
   const int grid = std::min(4 * device_sm_count(), (3 * in.n + 255) / 256);
-  pdl_launch(k_input_check, grid, 256, 0, s, in.n, in, p->in_saved, p->max_ions, with_lists ? p->plist_cnt : nullptr,
+  pdl_launch(k_input_check, grid, 256, 0, s, in.n, in, live_io(p), p->in_saved, p->max_ions, with_lists ? p->plist_cnt : nullptr,
                                       p->in_diff, p->cache_bad);
   count_launch();
   return check_launch(p, "k_input_check");

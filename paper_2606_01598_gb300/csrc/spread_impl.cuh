@@ -26,6 +26,7 @@ struct Shape {
 };
 
 struct SpreadArgs {
+  const PassIO* io;     // recorded passes: the caller's pointers (null: theta below)
   const float* theta;   // quadrupole mode: Theta [caller index][6] (xx yy zz xy xz yz)
   FrameDesc one;
   FrameMaps maps;
@@ -92,6 +93,7 @@ __device__ __forceinline__ int up_dist(int a, int b, int n) {
 template <class SH, int P, int MODE, bool BATCH>
 __global__ void __launch_bounds__(SH::NT) k_spread(SpreadArgs a) {
   pdl_begin();
+  if (MODE >= 2 && a.io) a.theta = a.io->in.theta;
   constexpr int BX = SH::BX, BY = SH::BY, BZ = SH::BZ, NSEG = SH::NSEG, NT = SH::NT, CAP = SH::CAP,
                 NW = SH::NW, SL = SH::SL;
   constexpr bool TAN = MODE != 0;   // a second accumulator (d rho, or rho of the quadrupole modes)
@@ -523,6 +525,7 @@ int launch_order(pme_plan_t p, cudaStream_t s, int grid, const SpreadArgs& a) {
 template <class SH, int MODE, bool BATCH>
 int launch_t(pme_plan_t p, cudaStream_t s, float* mesh, const int* keep_rho, const float* theta = nullptr) {
   SpreadArgs a;
+  a.io = live_io(p);
   a.theta = theta;
   a.keep_rho = MODE == 1 ? keep_rho : nullptr;
   a.one = p->frames_h[0];
