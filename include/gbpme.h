@@ -101,6 +101,8 @@ typedef struct {
                               power-of-two kernels (compile-time four-step transforms).
                               0 (default): automatic, the library's own when every frame's
                               mesh takes the power-of-two kernels, for single frames whose
+                              axes are 64, 128 or 256 points (line by line where the planes do
+                              not fit in shared memory), for single frames whose
                               every axis is a product of two of 1-6, 8, 9, 10, 12, 15, 16, and
                               for batched plans whose meshes have no axis above 64 points (one
                               launch per pass for all frames), cuFFT otherwise.
@@ -144,7 +146,7 @@ int pme_plan_destroy(pme_plan_t plan);
 
 /* Which transforms the plan's mesh convolution uses: *kind = 0 for the library's own
  * (two-step or Stockham transforms in shared memory, the x transform fused with the influence multiply),
- * 1 for cuFFT, 2 for the library's own power-of-two kernels (every axis 64 or 128). */
+ * 1 for cuFFT, 2 for the library's own power-of-two kernels (every axis 64 or 128, or, line by line, 256). */
 int pme_plan_fft_kind(pme_plan_t plan, int* kind);
 
 /* The spread brick shape the plan uses (explicit, tuned or default): brick[3] = x, y, z edges. */

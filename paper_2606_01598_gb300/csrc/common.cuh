@@ -268,6 +268,7 @@ struct pme_plan_s {
   // hand-written transforms (every axis 2,3,5-smooth and short enough): no cuFFT plans
   bool conv = false;
   bool conv_p2 = false;                    // every axis 64 or 128: the power-of-two kernels
+  bool conv_line = false;                  // axes 64, 128 or 256, planes too large: the line kernels
   bool conv_two = false;                   // every axis P Q with P, Q <= 16: the two-step kernels
   float2* conv_tw = nullptr;               // twiddle tables
   int2* conv_planes1 = nullptr;            // batched plans: pass A / C block -> (frame, plane)

@@ -841,6 +841,7 @@ int launch_conv_forward(pme_plan_t p, cudaStream_t s, bool tangent, float* mesh,
                             : (tangent ? 2 : 1) * ((F0.g.N[0] + F0.conv_pp - 1) / F0.conv_pp);
   a.planes = tangent ? p->conv_planes2 : p->conv_planes1;
   int st;
+  if (p->conv_line) return launch_line(p, s, a, false);
   if (p->conv_two) return launch_two_plane(p, s, a, grid, false);
   if (p->conv_p2) {
     if (p->batch) {
@@ -879,6 +880,7 @@ int launch_conv_inverse(pme_plan_t p, cudaStream_t s, bool tangent, float* mesh,
                             : (tangent ? 2 : 1) * ((F0.g.N[0] + F0.conv_pp - 1) / F0.conv_pp);
   a.planes = tangent ? p->conv_planes2 : p->conv_planes1;
   int st;
+  if (p->conv_line) return launch_line(p, s, a, true);
   if (p->conv_two) return launch_two_plane(p, s, a, grid, true);
   if (p->conv_p2) {
     if (p->batch) {
@@ -915,7 +917,7 @@ int launch_conv_influence(pme_plan_t p, cudaStream_t s, bool tangent, double* pa
   a.partials = partials;
   a.vparts = vparts;
   const int grid = p->batch ? p->total_blocks : p->frames_h[0].infl_nblk;
-  if (p->conv_two) return launch_two_x(p, s, a, grid);
+  if (p->conv_two || p->conv_line) return launch_two_x(p, s, a, grid);
   const size_t smem = p->conv_smem_x;
   int st;
 #define GB_CONV_X(B, V)                                                  \

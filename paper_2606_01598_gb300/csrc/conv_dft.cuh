@@ -28,6 +28,8 @@ struct ConvArgs {
 // conv_two.cu: the passes of plans whose every axis splits into two register steps
 int launch_two_plane(pme_plan_t p, cudaStream_t s, const ConvArgs& a, int grid, bool inverse);
 int launch_two_x(pme_plan_t p, cudaStream_t s, const ConvArgs& a, int grid);
+// conv_line.cu: the z and y passes of meshes whose planes do not fit in shared memory
+int launch_line(pme_plan_t p, cudaStream_t s, const ConvArgs& a, bool inverse);
 
 namespace {
 

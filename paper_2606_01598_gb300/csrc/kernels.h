@@ -117,6 +117,7 @@ int two_planes_per_block(const int N[3], bool single);
 int two_plane_threads(const int N[3], int pp);
 size_t two_plane_smem(const int N[3], int pp);
 size_t two_x_smem(const int N[3]);
+bool line_axes_ok(const int N[3]);   // conv_line.cu: every axis 64, 128 or 256
 void conv_twiddles(int L, std::vector<float2>& out);
 // keep (tangent passes, nullable): *keep == 0 means the plan's rho and Phi are those of the
 // forward on the same inputs; the passes then skip them and transform the tangent mesh only.

@@ -484,7 +484,8 @@ struct FrameInput {
 // for single frames whose every axis splits into two register steps (two_step_factors), and
 // for batched plans of small meshes (no axis above kConvAutoMaxAxis), whose frames then share
 // one launch per pass instead of a cuFFT plan per mesh shape. The axis lengths and
-// shared-memory sizes are checked by the caller (a mesh whose planes do not fit goes to cuFFT).
+// shared-memory sizes are checked by the caller (a mesh whose planes do not fit goes to the line
+// kernels where its axes are 64, 128 or 256 points, to cuFFT otherwise).
 // Measured on GB300, solve of one frame, three plans in turn (us), two-step kernels against
 // cuFFT's six plus the influence pass: 32^3 20.5 / 25.9, 48^3 21.2 / 26.0, 80x81x90 28.9 / 31.5,
 // 96^3 30.8 / 36.9, 100^3 36.2 / 33.6, 144^3 51.0 / 56.7, 150^3 60.7 / 90.1, 160^3 92.8 / 85.4.
@@ -571,7 +572,10 @@ static int build_plan(pme_plan_s* p, const std::vector<FrameInput>& fin, double 
     }
     if (!conv && (p->opts.fft == 2 || p->opts.fft == 3))
       return set_error(p, PME_ERR_UNSUPPORTED, "fft = 2 / 3: a mesh the library's transforms do not take");
-    p->conv = conv;
+    // automatic choice, planes too large for a block: the line kernels where every axis is 64,
+    // 128 or 256 points
+    p->conv_line = !conv && p->opts.fft == 0 && single && line_axes_ok(fin[0].mesh);
+    p->conv = conv || p->conv_line;
     p->conv_p2 = conv && p2;
     // two register steps per transform where every axis splits and the layout fits (it is a
     // little larger than the general kernels'); the Stockham kernels otherwise
@@ -597,6 +601,7 @@ static int build_plan(pme_plan_s* p, const std::vector<FrameInput>& fin, double 
       p->conv_smem_x = two_x;
       p->conv_threads = two_threads;
     }
+    if (p->conv_line) p->conv_smem_x = two_x_smem(fin[0].mesh);
   }
   std::vector<int> ncells(F);
   for (int f = 0; f < F; ++f) {
@@ -627,8 +632,8 @@ static int build_plan(pme_plan_s* p, const std::vector<FrameInput>& fin, double 
     if (p->conv) {
       conv_tiles(g.N, &D.infl_nblk, &D.conv_cols);
       D.conv_pp = conv_planes_per_block(g.N);
-      if (p->conv_two) {
-        D.conv_pp = two_planes_per_block(g.N, single);
+      if (p->conv_two || p->conv_line) {
+        if (p->conv_two) D.conv_pp = two_planes_per_block(g.N, single);
         for (int a = 0; a < 3; ++a) two_step_factors(g.N[a], &D.conv_p[a], &D.conv_q[a]);
       }
     } else {
@@ -1517,7 +1522,7 @@ int pme_plan_destroy(pme_plan_t p) {
 
 int pme_plan_fft_kind(pme_plan_t p, int* kind) {
   if (!p || !kind) return PME_ERR_ARG;
-  *kind = p->conv ? (p->conv_p2 ? 2 : 0) : 1;
+  *kind = p->conv ? (p->conv_p2 || p->conv_line ? 2 : 0) : 1;
   return PME_OK;
 }
 
