@@ -127,8 +127,7 @@ struct SortBuffers {
   int* start_c;   // [total cells + 1]
   int* perm_b;    // [max_ions] unsorted placement (sorted slot -> caller index)
   int* perm_c;
-  double* qpart;  // [2 * items] Q and dQ of each reduction item
-  int* qcount;    // [frames] items finished (reset by the last one); null: no charge sums wanted
+  double* qpart;  // [2 * items] Q and dQ of each reduction item; null: no charge sums wanted
   // per-ion records formed by the binning pass in caller order (null: the rank pass forms
   // them itself), copied to their sorted slots by the rank pass
   int4* t_bidx;
@@ -315,7 +314,7 @@ struct pme_plan_s {
   int* in_flags = nullptr;     // [2]: in_diff, cache_bad (see launch_input_check)
   int* in_diff = nullptr;
   int* cache_bad = nullptr;
-  bool counts_clean = false;   // the sort's count arrays are zero (each scan re-zeroes them)
+  bool counts_clean = false;   // the sort's count arrays are zero (each scatter re-zeroes them)
   int fwd_n = -1;              // ions of that forward (-1: nothing saved / no longer valid)
   // virial partial sums
   double* vpart = nullptr;     // [6 * influence blocks] k-space sums S_ab

@@ -218,8 +218,7 @@ extern "C" int pme_spread_noalloc(void* stream, const double box[9], const int m
   v.sb.start_b = reinterpret_cast<int*>(base + kOffStartB);
   v.sb.count_c = reinterpret_cast<int*>(base + kOffCountC);
   v.sb.start_c = reinterpret_cast<int*>(base + kOffStartC);
-  v.sb.qpart = reinterpret_cast<double*>(base + kOffQpart);
-  v.sb.qcount = nullptr;   // the spread needs no charge sums: the sort skips them
+  v.sb.qpart = nullptr;   // the spread needs no charge sums: the sort skips them
   v.sb.t_bidx = nullptr;   // no room for caller-order records: the rank pass forms them
   v.sb.qsum = reinterpret_cast<double*>(base + kOffQsum);
   v.mr.idx = reinterpret_cast<int4*>(base + kOffIdx);

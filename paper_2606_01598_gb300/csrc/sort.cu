@@ -24,82 +24,81 @@ namespace {
 constexpr int kSortThreads = kRedItem;   // binning: one block per reduction item
 constexpr int kRankMaxSegment = 2048;   // longer segments keep arrival order
 
-// Exclusive scan of one count array by one block of 1024 threads; start[n] = total. Each
-// thread owns a chunk of a multiple of 4 entries and moves it with 16-byte loads and stores,
-// so both arrays are allocated padded to a multiple of 4 entries past n + 1 (entries past n
-// are read but ignored, and written with scratch values before start[n] is set). The counts
-// are dead once scanned: the scan leaves them zero for the next sort.
-__device__ void block_exclusive_scan(int* count, int* start, int n) {
-  __shared__ int warp_tot[32];
-  const int T = blockDim.x;
-  const int chunk = ((n + T - 1) / T + 3) & ~3;
-  const int lo = min(n, threadIdx.x * chunk), hi = min(n, lo + chunk);
-  // chunks of up to 16 entries stay in registers between the two passes
-  constexpr int kHold = 4;
-  int4 held[kHold];
-  const bool hold = hi - lo <= 4 * kHold;
-  int local = 0;
-  if (hold) {
-#pragma unroll
-    for (int u = 0; u < kHold; ++u) {
-      const int k = lo + 4 * u;
-      held[u] = k < hi ? __ldcg(reinterpret_cast<const int4*>(count + k)) : make_int4(0, 0, 0, 0);
-    }
-#pragma unroll
-    for (int u = 0; u < kHold; ++u) {
-      const int k = lo + 4 * u;
-      if (k < hi) {
-        const int4 c = held[u];
-        local += c.x + (k + 1 < hi ? c.y : 0) + (k + 2 < hi ? c.z : 0) + (k + 3 < hi ? c.w : 0);
-      }
-    }
-  } else {
-#pragma unroll 4
-    for (int k = lo; k < hi; k += 4) {
-      const int4 c = __ldcg(reinterpret_cast<const int4*>(count + k));
-      local += c.x + (k + 1 < hi ? c.y : 0) + (k + 2 < hi ? c.z : 0) + (k + 3 < hi ? c.w : 0);
-    }
-  }
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  int v = local;
+// Segments of a count array: one block each, kScanThreads threads on a whole number of int4s
+// (both arrays are allocated padded to a multiple of 4 entries past n + 1). A block finds its
+// own first start by adding up every count before its segment, so the blocks do not wait for
+// one another; at most kScanMaxSegs segments keep that re-reading small (91125 pair cells: 22
+// blocks reading 180 KB each on average, from L2).
+constexpr int kScanThreads = 1024;
+constexpr int kScanSeg = 4 * kScanThreads;
+constexpr int kScanMaxSegs = 64;
+__host__ __device__ __forceinline__ int scan_segment(int n) {
+  const int whole = (n + kScanSeg - 1) / kScanSeg;
+  return kScanSeg * max(1, (whole + kScanMaxSegs - 1) / kScanMaxSegs);
+}
+
+__device__ __forceinline__ int warp_inclusive(int v, int lane) {
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
     const int u = __shfl_up_sync(0xffffffffu, v, o);
     if (lane >= o) v += u;
   }
-  if (lane == 31) warp_tot[wid] = v;
+  return v;
+}
+
+// start[k] for the counts of segment seg (length len, starting at entry seg len); the last
+// segment also writes start[n] = total. The counts stay in place (k_scatter clears them).
+__device__ void scan_one_segment(const int* count, int* start, int n, int seg, int len) {
+  __shared__ int part[32];
+  __shared__ int carry;
+  const int lo = seg * len, hi = min(n, lo + len);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  int before = 0;
+#pragma unroll 4
+  for (int k = 4 * threadIdx.x; k < lo; k += kScanSeg) {
+    const int4 c = __ldcg(reinterpret_cast<const int4*>(count + k));
+    before += (c.x + c.y) + (c.z + c.w);
+  }
+  before = __reduce_add_sync(0xffffffffu, before);
+  if (lane == 0) part[wid] = before;
   __syncthreads();
   if (wid == 0) {
-    int w = (lane < (T >> 5)) ? warp_tot[lane] : 0;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int u = __shfl_up_sync(0xffffffffu, w, o);
-      if (lane >= o) w += u;
+    const int t = __reduce_add_sync(0xffffffffu, part[lane]);
+    if (lane == 0) carry = t;
+  }
+  __syncthreads();
+  int run0 = carry;
+  for (int k0 = lo; k0 < hi; k0 += kScanSeg) {
+    const int k = k0 + 4 * threadIdx.x;
+    int4 c = k < hi ? __ldcg(reinterpret_cast<const int4*>(count + k)) : make_int4(0, 0, 0, 0);
+    if (k + 1 >= hi) c.y = 0;
+    if (k + 2 >= hi) c.z = 0;
+    if (k + 3 >= hi) c.w = 0;
+    const int local = (c.x + c.y) + (c.z + c.w);
+    const int v = warp_inclusive(local, lane);
+    __syncthreads();   // part is read below in the round before
+    if (lane == 31) part[wid] = v;
+    __syncthreads();
+    const int w = warp_inclusive(part[lane], lane);   // every warp: inclusive prefix over the warps
+    const int total = __shfl_sync(0xffffffffu, w, 31);
+    const int warps_before = __shfl_sync(0xffffffffu, w, max(wid - 1, 0));
+    if (k < hi) {
+      int4 o;
+      o.x = run0 + v - local + (wid > 0 ? warps_before : 0);
+      o.y = o.x + c.x;
+      o.z = o.y + c.y;
+      o.w = o.z + c.z;
+      *reinterpret_cast<int4*>(start + k) = o;
     }
-    warp_tot[lane] = w;   // inclusive prefix over warps
+    run0 += total;
   }
-  __syncthreads();
-  int run = v - local + (wid > 0 ? warp_tot[wid - 1] : 0);
-#pragma unroll 4
-  for (int k = lo; k < hi; k += 4) {
-    const int4 c = hold ? held[(k - lo) >> 2] : __ldcg(reinterpret_cast<const int4*>(count + k));
-    int4 o;
-    o.x = run;
-    o.y = o.x + c.x;
-    o.z = o.y + (k + 1 < hi ? c.y : 0);
-    o.w = o.z + (k + 2 < hi ? c.z : 0);
-    run = o.w + (k + 3 < hi ? c.w : 0);
-    *reinterpret_cast<int4*>(start + k) = o;
-    *reinterpret_cast<int4*>(count + k) = make_int4(0, 0, 0, 0);
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) start[n] = warp_tot[31];
+  __syncthreads();   // the write of start[n] follows the padding entries of the last int4
+  if (hi == n && threadIdx.x == 0) start[n] = run0;
 }
 
 // One block per reduction item (kRedItem = kSortThreads ions of one frame, one per thread):
 // the ion's brick key and pair-cell key with one counting atomic each, its records in caller
-// order, and the item's charge sums (the last item of a frame adds the item partials in
-// order).
+// order, and the item's charge sums (k_scan adds a frame's items in order).
 template <bool BATCH>
 __global__ void __launch_bounds__(kSortThreads)
 k_bin(FrameDesc one, FrameMaps maps, IonInputs in, const PassIO* io, SortBuffers sb, int tangent, int* flags,
@@ -192,42 +191,64 @@ k_bin(FrameDesc one, FrameMaps maps, IonInputs in, const PassIO* io, SortBuffers
     qa = isfinite(qi) ? qi : 0.f;
     qb = (tangent && in.gphi) ? in.gphi[i] : 0.f;
   }
-  if (sb.qcount) {
+  if (sb.qpart) {
     double A, B;
     block_sum2_f(qa, qb, A, B);
     if (threadIdx.x == 0) {
       sb.qpart[2 * item] = A;
       sb.qpart[2 * item + 1] = B;
     }
-    if (last_item_done(sb.qcount + f, F.nitems)) {
-      double a, b;
-      strided_sum2_d(sb.qpart + 2 * F.item_off, F.nitems, 2, sb.qpart + 2 * F.item_off + 1, F.nitems, 2, a, b);
-      block_sum2_d(a, b);
-      if (threadIdx.x == 0) {
-        sb.qsum[2 * f] = a;
-        sb.qsum[2 * f + 1] = b;
-        sb.qcount[f] = 0;
-      }
-    }
   }
-  (void)nbricks;
-  (void)ncells;
 }
 
-// Segment starts from the final counts: block 0 scans the brick counts, block 1 the cell
-// counts (1024 threads each). Skipped on reuse.
-__global__ void __launch_bounds__(1024) k_scan(SortBuffers sb, int nbricks, int ncells, const int* reuse) {
+// Segment starts from the final counts (skipped on reuse) and the frames' charge sums from
+// their items' partials: blocks [0, nb) scan the brick counts, [nb, nb + nc) the cell counts, the
+// rest add the items of 32 frames each, one warp per frame. One 1024-thread block per array took
+// 50 us at 262144 ions (91125 cells) and 22 us for 256 uneven frames; the charge sums were the
+// binning pass's last block, alone on its SM for 2.8 us of every sort. Forward of 32768 ions 142.6 ->
+// 137.5 us, forward + backward of 262144 ions 1.82 -> 1.78 ms, 256 uneven frames 1.25 -> 1.23 ms.
+template <bool BATCH>
+__global__ void __launch_bounds__(kScanThreads)
+k_scan(FrameDesc one, FrameMaps maps, int nframes, SortBuffers sb, int nbricks, int ncells, int nb, int nc,
+       const int* reuse) {
   pdl_begin();
-  if (reuse && *reuse == 0) return;
-  if (blockIdx.x == 0) block_exclusive_scan(sb.count_b, sb.start_b, nbricks);
-  else block_exclusive_scan(sb.count_c, sb.start_c, ncells);
+  const int b = blockIdx.x;
+  if (b < nb + nc) {
+    if (reuse && *reuse == 0) return;
+    if (b < nb) scan_one_segment(sb.count_b, sb.start_b, nbricks, b, scan_segment(nbricks));
+    else scan_one_segment(sb.count_c, sb.start_c, ncells, b - nb, scan_segment(ncells));
+    return;
+  }
+  const int f = (b - nb - nc) * (kScanThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (f >= nframes) return;
+  const FrameDesc& F = frame_at<BATCH>(one, maps, f);
+  const double2* part = reinterpret_cast<const double2*>(sb.qpart) + F.item_off;
+  double qa = 0.0, qb = 0.0;
+#pragma unroll 4
+  for (int k = lane; k < F.nitems; k += 32) {
+    const double2 v = __ldcg(part + k);
+    qa += v.x;
+    qb += v.y;
+  }
+  qa = warp_sum_d(qa);
+  qb = warp_sum_d(qb);
+  if (lane == 0) {
+    sb.qsum[2 * f] = qa;
+    sb.qsum[2 * f + 1] = qb;
+  }
 }
 
 __global__ void __launch_bounds__(kSortThreads)
-k_scatter(int n, SortBuffers sb, int need_mesh, int need_pair, const int* reuse) {
+k_scatter(int n, SortBuffers sb, int nbricks, int ncells, int need_mesh, int need_pair, const int* reuse) {
   pdl_begin();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n || (reuse && *reuse == 0)) return;
+  if (reuse && *reuse == 0) return;
+  // the counts are dead once scanned: leave them zero for the next sort
+  for (int k = 4 * i; k < nbricks; k += 4 * gridDim.x * blockDim.x)
+    *reinterpret_cast<int4*>(sb.count_b + k) = make_int4(0, 0, 0, 0);
+  for (int k = 4 * i; k < ncells; k += 4 * gridDim.x * blockDim.x)
+    *reinterpret_cast<int4*>(sb.count_c + k) = make_int4(0, 0, 0, 0);
+  if (i >= n) return;
   if (need_mesh) {
     const int d = sb.start_b[sb.key_b[i]] + sb.slot_b[i];
     if (index_ok(d, n)) sb.perm_b[d] = i;
@@ -462,7 +483,11 @@ int launch_sort_t(pme_plan_t p, cudaStream_t s, const IonInputs& in, bool tangen
       p->counts_clean = false;
       return st;
     }
-    pdl_launch(k_scan, 2, 1024, 0, s, p->sb, p->total_bricks, p->total_cells, reuse);
+    const int nb = (p->total_bricks + scan_segment(p->total_bricks) - 1) / scan_segment(p->total_bricks);
+    const int nc = (p->total_cells + scan_segment(p->total_cells) - 1) / scan_segment(p->total_cells);
+    const int nq = p->sb.qpart ? (p->nframes + kScanThreads / 32 - 1) / (kScanThreads / 32) : 0;
+    pdl_launch(k_scan<BATCH>, nb + nc + nq, kScanThreads, 0, s, one, p->maps, p->nframes, p->sb, p->total_bricks,
+               p->total_cells, nb, nc, reuse);
     count_launch();
     if ((st = check_launch(p, "k_scan"))) {
       p->counts_clean = false;
@@ -470,7 +495,9 @@ int launch_sort_t(pme_plan_t p, cudaStream_t s, const IonInputs& in, bool tangen
     }
   }
   if (nblk > 0) {
-    pdl_launch(k_scatter, nblk, kSortThreads, 0, s, n, p->sb, need_mesh ? 1 : 0, need_pair ? 1 : 0, reuse);
+    const int clear = (std::max(p->total_bricks, p->total_cells) / 4 + kSortThreads - 1) / kSortThreads;
+    pdl_launch(k_scatter, std::max(nblk, std::min(clear, 4 * device_sm_count())), kSortThreads, 0, s, n, p->sb,
+               p->total_bricks, p->total_cells, need_mesh ? 1 : 0, need_pair ? 1 : 0, reuse);
     count_launch();
     if ((st = check_launch(p, "k_scatter"))) return st;
     const int nblk2 = (2 * n + kSortThreads - 1) / kSortThreads;
