@@ -20,7 +20,7 @@ def gb():
 
 @pytest.mark.parametrize("L,rcut", [(24.0, 4.0), (60.0, 6.0), (150.0, 4.5), (150.0, 9.0)])
 def test_pair_term_over_many_cells(gb, L, rcut):
-    # (12^3, 20^3, 66^3 and 33^3 cells: 1, 2, 64 longer, and 9 segments); ions in clumps, so that
+    # (12^3, 20^3, 66^3 and 33^3 cells: 1, 2, 36 of double length, and 9 segments); ions in clumps, so that
     # there are partners within the cutoff
     n = 2304
     rng = np.random.default_rng(17)
