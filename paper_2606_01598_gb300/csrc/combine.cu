@@ -188,10 +188,33 @@ __global__ void __launch_bounds__(kCombThreads) k_combine_forward(CombineArgs a)
     }
   }
   if (a.virial_out) {
+    // the nine block sums (each as block_sum_f forms it) with their trees interleaved: in
+    // sequence, these and the last block's fifteen were 30 of the kernel's 39 us
+    __shared__ double vpart[9][kCombThreads / 32];
+    float vc[9];
 #pragma unroll
-    for (int c = 0; c < 9; ++c) {
-      const double t = block_sum_f(vi[c]);
-      if (threadIdx.x == 0) a.vitem[9 * item + c] = t;
+    for (int c = 0; c < 9; ++c) vc[c] = 0.f;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+      for (int c = 0; c < 9; ++c) {
+        const float v2 = __shfl_xor_sync(0xffffffffu, vi[c], o), c2 = __shfl_xor_sync(0xffffffffu, vc[c], o);
+        const float t = vi[c] + v2;
+        vc[c] += c2 + (fabsf(vi[c]) >= fabsf(v2) ? (vi[c] - t) + v2 : (v2 - t) + vi[c]);
+        vi[c] = t;
+      }
+    }
+    if ((threadIdx.x & 31) == 0) {
+#pragma unroll
+      for (int c = 0; c < 9; ++c) vpart[c][threadIdx.x >> 5] = double(vi[c]) + double(vc[c]);
+    }
+    __syncthreads();
+    if (threadIdx.x < 9) {
+      double t = 0.0;
+#pragma unroll
+      for (int w = 0; w < kCombThreads / 32; ++w) t += vpart[threadIdx.x][w];
+      a.vitem[9 * item + threadIdx.x] = t;
+      __threadfence();   // before the item's ticket (last_item_done)
     }
   }
   if (!a.energy_out) return;   // uniform
@@ -204,12 +227,20 @@ __global__ void __launch_bounds__(kCombThreads) k_combine_forward(CombineArgs a)
   strided_sum2_d(a.recip_parts + F.infl_blk_off, a.recip_kind ? F.infl_nblk : 0, 1, a.eitem + F.item_off,
                  F.nitems, 1, rp, ep);
   block_sum2_d(rp, ep);
-  double W[9], S[6];
+  // the fifteen sums of the virial, W (9, over items) and S (6, over influence blocks), dealt to
+  // the warps: each is one warp's strided sum
+  __shared__ double vsum[15];
   if (a.virial_out) {
-#pragma unroll
-    for (int c = 0; c < 9; ++c) W[c] = block_sum_d(strided_sum_d(a.vitem + 9 * F.item_off + c, F.nitems, 9));
-#pragma unroll
-    for (int c = 0; c < 6; ++c) S[c] = block_sum_d(strided_sum_d(a.vparts + 6 * F.infl_blk_off + c, F.infl_nblk, 6));
+    const int lane = threadIdx.x & 31;
+    for (int c = threadIdx.x >> 5; c < 15; c += kCombThreads / 32) {
+      const double* src = c < 9 ? a.vitem + 9 * F.item_off + c : a.vparts + 6 * F.infl_blk_off + (c - 9);
+      const int m = c < 9 ? F.nitems : F.infl_nblk, st = c < 9 ? 9 : 6;
+      double t = 0.0;
+      for (int k0 = lane; k0 < m; k0 += 8 * 32) t += strided_round(src, m, st, k0, 32);
+      t = warp_sum_d(t);
+      if (lane == 0) vsum[c] = t;
+    }
+    __syncthreads();
   }
   if (threadIdx.x == 0) {
     const double V = F.g.volume;
@@ -224,7 +255,7 @@ __global__ void __launch_bounds__(kCombThreads) k_combine_forward(CombineArgs a)
       const int sidx[9] = {0, 3, 4, 3, 1, 5, 4, 5, 2};   // S_ab from xx yy zz xy xz yz
       const double diag = coef * rp + e_bg;
       for (int c = 0; c < 9; ++c)
-        a.virial_out[9 * f + c] = a.kd * (W[c] - S[sidx[c]] / V + ((c % 4) == 0 ? diag : 0.0));
+        a.virial_out[9 * f + c] = a.kd * (vsum[c] - vsum[9 + sidx[c]] / V + ((c % 4) == 0 ? diag : 0.0));
     }
     a.ecount[f] = 0;
   }
