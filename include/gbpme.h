@@ -198,6 +198,13 @@ int pme_backward(pme_plan_t plan, void* stream, int n, const float* pos, const f
                  const float* g_phi, const float* g_field, float* grad_pos, float* grad_q,
                  float* grad_mu);
 
+/* out_a = -g a [n][3], out_b = g b [n], out_c = -g c [n][3] with one device factor g (float64,
+ * rounded to float32; NULL = 1), each array skipped when its input is NULL: the gradient (dE/dr,
+ * dE/dq, dE/dmu) times g from (force, phi, field), and equally the cotangents (g_force, g_phi,
+ * g_field) of pme_backward from cotangents of that gradient. Device pointers only. */
+int pme_scale_signed(void* stream, int n, const double* g, const float* a, const float* b,
+                     const float* c, float* out_a, float* out_b, float* out_c);
+
 /* Forward plus the virial (an extension of the paper's outputs, for stress / NPT training):
  *   virial [9] float64, row-major, W_ab = -dE/d(eps_ab) for the homogeneous strain
  *   r -> (I + eps) r of the positions and the lattice vectors with the dipoles held fixed:

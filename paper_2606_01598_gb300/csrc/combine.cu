@@ -354,6 +354,20 @@ k_pair_energy(int n, const float* q, const float* mu, const float* pair_out, dou
   e_ion[i] = e;
 }
 
+// out = (-g a, g b, -g c) for per-ion arrays a [n][3], b [n], c [n][3] (null: skipped) and one
+// factor g: the gradient of an energy from its forces, potentials and fields, and the cotangents
+// of those outputs from cotangents of the gradient.
+__global__ void __launch_bounds__(256)
+k_scale_signed(int n, const double* __restrict__ g, const float* __restrict__ a, const float* __restrict__ b,
+               const float* __restrict__ c, float* oa, float* ob, float* oc) {
+  const float s = g ? float(*g) : 1.f;
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < 3 * n; t += gridDim.x * blockDim.x) {
+    if (a) oa[t] = -s * a[t];
+    if (c) oc[t] = -s * c[t];
+    if (b && t < n) ob[t] = s * b[t];
+  }
+}
+
 CombineArgs base_args(pme_plan_t p, const IonInputs& in) {
   CombineArgs a = {};
   a.io = live_io(p);
@@ -466,7 +480,16 @@ int launch_pair_energy(pme_plan_t p, cudaStream_t s, int n, const IonInputs& in,
   return check_launch(p, "k_pair_energy");
 }
 
-
 GBPME_BOUNDS_READER(bounds_hit_combine)
 
 }  // namespace gbpme
+
+extern "C" int pme_scale_signed(void* stream, int n, const double* g, const float* a, const float* b, const float* c,
+                                float* out_a, float* out_b, float* out_c) {
+  if (n < 0 || (a && !out_a) || (b && !out_b) || (c && !out_c)) return PME_ERR_ARG;
+  if (n == 0) return PME_OK;
+  const int grid = std::min((3 * n + 255) / 256, 8 * gbpme::device_sm_count());
+  gbpme::k_scale_signed<<<grid, 256, 0, static_cast<cudaStream_t>(stream)>>>(n, g, a, b, c, out_a, out_b, out_c);
+  gbpme::count_launch();
+  return cudaGetLastError() == cudaSuccess ? PME_OK : PME_ERR_CUDA;
+}
