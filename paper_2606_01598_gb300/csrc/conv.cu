@@ -404,9 +404,8 @@ __global__ void __launch_bounds__(kConvBThreads) k_conv_x(ConvArgs a) {
 }
 
 // ---------------------------------------------------------------------------------------
-// Power-of-two path: meshes whose every axis is 64 or 128 points. The same three passes, the
-// same layouts and the same energy (and virial) partials per pass-B block as the kernels
-// above, but each 1D transform of length L = 8 B (B = 8 or 16) is the four-step split of
+// Power-of-two path: meshes whose every axis is 64 or 128 points. The same passes A and C and the
+// same layouts as the kernels above (the x pass is that of conv_two.cu), but each 1D transform of length L = 8 B (B = 8 or 16) is the four-step split of
 // Bailey (J. Supercomputing 4, 1990) done in registers with one shared-memory exchange:
 //   step 1, for each t < B: the 8-point DFT over m of x[t + B m], times w_L^(t k1), written
 //           to slot t + B k1;
@@ -414,8 +413,7 @@ __global__ void __launch_bounds__(kConvBThreads) k_conv_x(ConvArgs a) {
 // The loads from global memory feed step 1 of the first transform of a pass directly, and
 // step 2 of its last transform stores to global memory directly; the real-pair separation of
 // the R2C (and the Hermitian extension of the C2R) is folded into the loads of the y (z) step
-// 1, and the influence multiply into the forward x step 2. A pass is four steps with three
-// barriers. Lengths, strides and index arithmetic are compile-time constants; the twiddles
+// 1. A pass is four steps with three barriers. Lengths, strides and index arithmetic are compile-time constants; the twiddles
 // w_L^j are read from the plan's table (float64-built) through the read-only cache.
 // ---------------------------------------------------------------------------------------
 constexpr int kP2PlaneThreads = 1024;
@@ -620,143 +618,6 @@ __global__ void __launch_bounds__(kP2PlaneThreads, 1) k_conv_c2r_p2(ConvArgs a) 
   else c2r_plane_p2<64, 64>(src, dst, tz, ty, csm);
 }
 
-// Pass B tile of NC columns (KW = 16 of the spectrum, then, in a tangent pass that also
-// keeps rho's, the same 16 of the tangent spectrum): forward x transform, influence multiply
-// with the energy (and virial) sums, inverse x transform. nrho = the leading rho columns.
-constexpr int kP2Cols = 16;
-
-template <int NX, int NC, bool VIR>
-__device__ __forceinline__ void x_tile_p2(const ConvArgs& a, const FrameDesc& F, int c0, int nrho, float2* sm) {
-  constexpr int BX = NX / 8;
-  static_assert(NC * 8 <= kConvBThreads, "one step-2 item per thread");
-  const Geometry& g = F.g;
-  const int N1 = g.N[1], N2 = g.N[2], Nzh = N2 / 2 + 1;
-  const int ncols = N1 * Nzh;
-  float2* T = sm;             // step 1 outputs [x][c], row stride NC
-  float2* T2 = sm + NX * NC;  // step 2 outputs
-  const float2* tw = a.tw + F.tw_off[0];
-  const int tid = threadIdx.x;
-  // column c of the tile: spectrum column c0 + c (rho), or c0 + c - nrho of the tangent one
-  auto col_ptr = [&](int c) { return c < nrho ? a.spec + F.spec_off + c0 + c : a.spec + F.tspec_off + c0 + (c - nrho); };
-  // forward step 1 from global memory
-  for (int it = tid; it < BX * NC; it += blockDim.x) {
-    const int t = it / NC, c = it - t * NC;
-    const float2* cp = col_ptr(c);
-    float2 v[8];
-#pragma unroll
-    for (int m = 0; m < 8; ++m) v[m] = cp[size_t(t + BX * m) * ncols];
-    p2_step1<false>(v, t, tw);
-#pragma unroll
-    for (int k = 0; k < 8; ++k) T[(t + BX * k) * NC + c] = v[k];
-  }
-  __syncthreads();
-  // forward step 2, natural order into T2
-  if (tid < 8 * NC) {
-    const int k1 = tid / NC, c = tid - k1 * NC;
-    float2 u[BX];
-#pragma unroll
-    for (int t = 0; t < BX; ++t) u[t] = T[(t + BX * k1) * NC + c];
-    dft<BX, false>(u);
-#pragma unroll
-    for (int k2 = 0; k2 < BX; ++k2) T2[(k1 + 8 * k2) * NC + c] = u[k2];
-  }
-  __syncthreads();
-  // inverse step 1, its inputs multiplied by G C / V first (the energy and virial sums over
-  // the rho columns)
-  float e = 0.f, ec = 0.f;
-  float sv[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, sc[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  const float* cx = a.dconv + F.dconv_off;
-  for (int it = tid; it < BX * NC; it += blockDim.x) {
-    const int t = it / NC, c = it - t * NC;
-    const bool rho_col = c < nrho;
-    const int col = c0 + (rho_col ? c : c - nrho);
-    int iy, iz;
-    split_rc(col, Nzh, 1.f / float(Nzh), iy, iz);
-    const float ny = float(iy <= N1 / 2 ? iy : iy - N1);
-    const float nz = float(iz);
-    const float wz = (iz == 0 || (2 * iz == N2)) ? 1.f : 2.f;
-    float gcv[8];
-#pragma unroll
-    for (int m = 0; m < 8; ++m) {
-      const int ix = t + BX * m;
-      gcv[m] = a.gtab ? __ldg(a.gtab + F.gtab_off + size_t(ix) * ncols + col) : 0.f;
-    }
-    float2 v[8];
-#pragma unroll
-    for (int m = 0; m < 8; ++m) {
-      const int ix = t + BX * m;
-      const float nx = float(ix <= NX / 2 ? ix : ix - NX);
-      const float kx = nx * g.bk[0] + ny * g.bk[3] + nz * g.bk[6];
-      const float kyv = nx * g.bk[1] + ny * g.bk[4] + nz * g.bk[7];
-      const float kz = nx * g.bk[2] + ny * g.bk[5] + nz * g.bk[8];
-      const float k2v = kx * kx + kyv * kyv + kz * kz;
-      float gc = gcv[m];
-      if (!a.gtab && k2v > 0.f)
-        gc = 12.566370614359172f * expf(-k2v * a.inv4a2) / k2v * cx[ix] * cx[NX + iy] * cx[NX + N1 + iz];
-      const float2 x = T2[ix * NC + c];
-      if (rho_col) {
-        const float eg = wz * gc * (x.x * x.x + x.y * x.y);
-        comp_add(e, ec, eg);
-        if (VIR && k2v > 0.f) {
-          const float tt = eg * (1.f / k2v + a.inv4a2);
-          comp_add(sv[0], sc[0], tt * kx * kx);
-          comp_add(sv[1], sc[1], tt * kyv * kyv);
-          comp_add(sv[2], sc[2], tt * kz * kz);
-          comp_add(sv[3], sc[3], tt * kx * kyv);
-          comp_add(sv[4], sc[4], tt * kx * kz);
-          comp_add(sv[5], sc[5], tt * kyv * kz);
-        }
-      }
-      const float fac = gc * g.inv_volume;
-      v[m] = make_float2(x.x * fac, x.y * fac);
-    }
-    p2_step1<true>(v, t, tw);
-#pragma unroll
-    for (int k = 0; k < 8; ++k) T[(t + BX * k) * NC + c] = v[k];
-  }
-  __syncthreads();
-  // inverse step 2, straight to the spectrum
-  if (tid < 8 * NC) {
-    const int k1 = tid / NC, c = tid - k1 * NC;
-    float2 u[BX];
-#pragma unroll
-    for (int t = 0; t < BX; ++t) u[t] = T[(t + BX * k1) * NC + c];
-    dft<BX, true>(u);
-    float2* cp = col_ptr(c);
-#pragma unroll
-    for (int k2 = 0; k2 < BX; ++k2) cp[size_t(k1 + 8 * k2) * ncols] = u[k2];
-  }
-  __shared__ double wsum[kConvBThreads / 32];
-  const double et = block_comp_sum(e, ec, wsum);
-  if (threadIdx.x == 0) a.partials[blockIdx.x] = et;
-  if (VIR) {
-#pragma unroll
-    for (int c = 0; c < 6; ++c) {
-      const double vt = block_comp_sum(sv[c], sc[c], wsum);
-      if (threadIdx.x == 0) a.vparts[6 * blockIdx.x + c] = vt;
-    }
-  }
-}
-
-template <bool BATCH, bool VIR>
-__global__ void __launch_bounds__(kConvBThreads) k_conv_x_p2(ConvArgs a) {
-  pdl_begin();
-  extern __shared__ __align__(16) float2 csm[];
-  const FrameDesc& F = frame_at<BATCH>(a.one, a.maps, BATCH ? a.maps.blk_frame[blockIdx.x] : 0);
-  const int c0 = (blockIdx.x - F.infl_blk_off) * kP2Cols;
-  // tangent pass on the forward's inputs: rho's columns are not needed again
-  const bool rho_cols = !(a.tangent && a.keep && *a.keep == 0);
-  const int nrho = rho_cols ? kP2Cols : 0;
-  const bool two = a.tangent && rho_cols;
-  if (F.g.N[0] == 128) {
-    if (two) x_tile_p2<128, 2 * kP2Cols, VIR>(a, F, c0, nrho, csm);
-    else x_tile_p2<128, kP2Cols, VIR>(a, F, c0, nrho, csm);
-  } else {
-    if (two) x_tile_p2<64, 2 * kP2Cols, VIR>(a, F, c0, nrho, csm);
-    else x_tile_p2<64, kP2Cols, VIR>(a, F, c0, nrho, csm);
-  }
-}
-
 ConvArgs conv_args(pme_plan_t p) {
   ConvArgs a;
   std::memset(&a, 0, sizeof(a));
@@ -781,8 +642,6 @@ bool conv_p2_ok(const int N[3]) {
 size_t conv_p2_plane_smem(const int N[3]) {
   return size_t(2 * (N[1] / 2) * (N[2] + 8)) * sizeof(float2);
 }
-
-size_t conv_p2_x_smem(const int N[3]) { return size_t(2 * N[0] * 2 * kP2Cols) * sizeof(float2); }
 
 bool conv_axis_ok(int L) {
   if (L < 1 || L > kConvMaxLen) return false;
@@ -917,7 +776,7 @@ int launch_conv_influence(pme_plan_t p, cudaStream_t s, bool tangent, double* pa
   a.partials = partials;
   a.vparts = vparts;
   const int grid = p->batch ? p->total_blocks : p->frames_h[0].infl_nblk;
-  if (p->conv_two || p->conv_line) return launch_two_x(p, s, a, grid);
+  if (p->conv_two || p->conv_line || p->conv_p2) return launch_two_x(p, s, a, grid);
   const size_t smem = p->conv_smem_x;
   int st;
 #define GB_CONV_X(B, V)                                                  \
@@ -926,23 +785,6 @@ int launch_conv_influence(pme_plan_t p, cudaStream_t s, bool tangent, double* pa
     if ((st = set_smem(p, k_conv_x<B, V>, done))) return st;             \
     pdl_launch(k_conv_x<B, V>, grid, kConvBThreads, smem, s, a);                 \
   } while (0)
-#define GB_CONV_X_P2(B, V)                                               \
-  do {                                                                   \
-    static unsigned done = 0;                                            \
-    if ((st = set_smem(p, k_conv_x_p2<B, V>, done))) return st;          \
-    pdl_launch(k_conv_x_p2<B, V>, grid, kConvBThreads, smem, s, a);              \
-  } while (0)
-  if (p->conv_p2) {
-    if (p->batch) {
-      if (vparts) GB_CONV_X_P2(true, true);
-      else GB_CONV_X_P2(true, false);
-    } else {
-      if (vparts) GB_CONV_X_P2(false, true);
-      else GB_CONV_X_P2(false, false);
-    }
-    count_launch();
-    return check_launch(p, "k_conv_x_p2");
-  }
   if (p->batch) {
     if (vparts) GB_CONV_X(true, true);
     else GB_CONV_X(true, false);
@@ -951,7 +793,6 @@ int launch_conv_influence(pme_plan_t p, cudaStream_t s, bool tangent, double* pa
     else GB_CONV_X(false, false);
   }
 #undef GB_CONV_X
-#undef GB_CONV_X_P2
   count_launch();
   return check_launch(p, "k_conv_x");
 }

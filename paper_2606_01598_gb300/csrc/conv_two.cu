@@ -292,43 +292,38 @@ __global__ void __launch_bounds__(kTwoMaxThreads) k_two_c2r(ConvArgs a) {
   });
 }
 
-// Pass B over a run of columns: forward x transform, influence multiply with the energy (and
-// virial) sums over the rho columns, inverse x transform.
-template <bool BATCH, bool VIR>
-__global__ void __launch_bounds__(kTwoXThreads, VIR ? 2 : 3) k_two_x(ConvArgs a) {
-  pdl_begin();
-  extern __shared__ __align__(16) float2 csm[];
-  const FrameDesc& F = frame_at<BATCH>(a.one, a.maps, BATCH ? a.maps.blk_frame[blockIdx.x] : 0);
+// f with the radix R known (FIX > 0) or switched on
+template <int FIX, class F>
+__device__ __forceinline__ void radix_or(int r, F&& f) {
+  if constexpr (FIX > 0) f(std::integral_constant<int, FIX>{});
+  else with_radix(r, f);
+}
+
+// Pass B tile: kw columns of the spectrum (copy 0: rho's, with the energy and virial sums; 1: the
+// tangent one): forward x transform, influence multiply, inverse x transform. FP, FQ: the
+// factors of the x length when known (0: the frame's). smem: N0 kw entries.
+template <int FP, int FQ, bool VIR>
+__device__ __forceinline__ void x_tile(const ConvArgs& a, const FrameDesc& F, int copy, int c0, int kw, float2* T) {
   const Geometry& g = F.g;
-  const int N0 = g.N[0], N1 = g.N[1], N2 = g.N[2], Nzh = N2 / 2 + 1;
-  const int P0 = F.conv_p[0], Q0 = F.conv_q[0];
+  const int P0 = FP > 0 ? FP : F.conv_p[0], Q0 = FQ > 0 ? FQ : F.conv_q[0];
+  const int N0 = P0 * Q0, N1 = g.N[1], N2 = g.N[2], Nzh = N2 / 2 + 1;
   const int ncols = N1 * Nzh;   // (n_y, n_z) columns of a plane, contiguous for a fixed x
-  const int c0 = (blockIdx.x - F.infl_blk_off) * F.conv_cols;
-  const int kw = min(F.conv_cols, ncols - c0);
-  // tangent pass on the forward's inputs: rho's columns are not needed again
-  const bool rho_cols = !(a.tangent && a.keep && *a.keep == 0);
-  const int nrho = rho_cols ? kw : 0;
-  const int nc = a.tangent ? nrho + kw : kw;
-  const float rnc = 1.f / float(nc), rzh = 1.f / float(Nzh);
+  const float rkw = 1.f / float(kw), rzh = 1.f / float(Nzh);
   const float2* tw = a.tw + F.tw_off[0];
-  // tile column c: spectrum column c0 + c (rho), or c0 + c - nrho of the tangent one
-  auto col_ptr = [&](int c) {
-    return c < nrho ? a.spec + F.spec_off + c0 + c : a.spec + F.tspec_off + c0 + (c - nrho);
-  };
-  float2* T = csm;   // [slot][nc]
+  float2* col0 = a.spec + (copy ? F.tspec_off : F.spec_off) + c0;
   const int tid = threadIdx.x, NT = blockDim.x;
-  with_radix(P0, [&](auto rc) {
+  radix_or<FP>(P0, [&](auto rc) {
     constexpr int P = decltype(rc)::value;
-    for (int it = tid; it < Q0 * nc; it += NT) {
+    for (int it = tid; it < Q0 * kw; it += NT) {
       int t, c;
-      split_rc(it, nc, rnc, t, c);
-      const float2* s = col_ptr(c) + size_t(t) * ncols;
+      split_rc(it, kw, rkw, t, c);
+      const float2* s = col0 + size_t(t) * ncols + c;
       float2 v[P];
 #pragma unroll
       for (int m = 0; m < P; ++m) v[m] = s[size_t(Q0 * m) * ncols];
       step1<P, false>(v, t, tw);
 #pragma unroll
-      for (int k = 0; k < P; ++k) T[(t + Q0 * k) * nc + c] = v[k];
+      for (int k = 0; k < P; ++k) T[(t + Q0 * k) * kw + c] = v[k];
     }
   });
   __syncthreads();
@@ -337,23 +332,22 @@ __global__ void __launch_bounds__(kTwoXThreads, VIR ? 2 : 3) k_two_x(ConvArgs a)
   const float* cz = cy + N1;
   float e = 0.f, ec = 0.f;
   float sv[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, sc[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  with_radix(Q0, [&](auto rc) {
+  radix_or<FQ>(Q0, [&](auto rc) {
     constexpr int Q = decltype(rc)::value;
-    for (int it = tid; it < P0 * nc; it += NT) {
+    for (int it = tid; it < P0 * kw; it += NT) {
       int k1, c;
-      split_rc(it, nc, rnc, k1, c);
-      const bool rho_col = c < nrho;
-      const int col = c0 + (rho_col ? c : c - nrho);
+      split_rc(it, kw, rkw, k1, c);
+      const int col = c0 + c;
       int iy, iz;
       split_rc(col, Nzh, rzh, iy, iz);
       float gcv[Q];
 #pragma unroll
       for (int k2 = 0; k2 < Q; ++k2)
         gcv[k2] = a.gtab ? __ldg(a.gtab + F.gtab_off + size_t(k1 + P0 * k2) * ncols + col) : 0.f;
-      float2* row = T + Q * k1 * nc + c;   // this thread's slots (t, k1), t < Q
+      float2* row = T + Q * k1 * kw + c;   // this thread's slots (t, k1), t < Q
       float2 u[Q];
 #pragma unroll
-      for (int t = 0; t < Q; ++t) u[t] = row[t * nc];
+      for (int t = 0; t < Q; ++t) u[t] = row[t * kw];
       dft<Q, false>(u);
       const float ny = float(iy <= N1 / 2 ? iy : iy - N1);
       const float nz = float(iz);
@@ -370,7 +364,7 @@ __global__ void __launch_bounds__(kTwoXThreads, VIR ? 2 : 3) k_two_x(ConvArgs a)
           const float k2v = kx * kx + kyv * kyv + kz * kz;
           if (!a.gtab && k2v > 0.f)
             gc = 12.566370614359172f * expf(-k2v * a.inv4a2) / k2v * cx[ix] * cy[iy] * cz[iz];
-          if (VIR && rho_col && k2v > 0.f) {
+          if (VIR && copy == 0 && k2v > 0.f) {
             const float tt = wz * gc * (u[k2].x * u[k2].x + u[k2].y * u[k2].y) * (1.f / k2v + a.inv4a2);
             comp_add(sv[0], sc[0], tt * kx * kx);
             comp_add(sv[1], sc[1], tt * kyv * kyv);
@@ -380,40 +374,69 @@ __global__ void __launch_bounds__(kTwoXThreads, VIR ? 2 : 3) k_two_x(ConvArgs a)
             comp_add(sv[5], sc[5], tt * kyv * kz);
           }
         }
-        if (rho_col) comp_add(e, ec, wz * gc * (u[k2].x * u[k2].x + u[k2].y * u[k2].y));
+        if (copy == 0) comp_add(e, ec, wz * gc * (u[k2].x * u[k2].x + u[k2].y * u[k2].y));
         const float fac = gc * g.inv_volume;
         u[k2] = make_float2(u[k2].x * fac, u[k2].y * fac);
       }
       // the inverse transform split as Q P: u[m] = x[k1 + P m] is its step-1 input of offset k1
       step1<Q, true>(u, k1, tw);
 #pragma unroll
-      for (int k = 0; k < Q; ++k) row[k * nc] = u[k];
+      for (int k = 0; k < Q; ++k) row[k * kw] = u[k];
     }
   });
   __syncthreads();
-  with_radix(P0, [&](auto rc) {
+  radix_or<FP>(P0, [&](auto rc) {
     constexpr int P = decltype(rc)::value;
-    for (int it = tid; it < Q0 * nc; it += NT) {
+    for (int it = tid; it < Q0 * kw; it += NT) {
       int k, c;
-      split_rc(it, nc, rnc, k, c);
+      split_rc(it, kw, rkw, k, c);
       float2 v[P];
 #pragma unroll
-      for (int t = 0; t < P; ++t) v[t] = T[(k + Q0 * t) * nc + c];
+      for (int t = 0; t < P; ++t) v[t] = T[(k + Q0 * t) * kw + c];
       dft<P, true>(v);
-      float2* d = col_ptr(c) + size_t(k) * ncols;
+      float2* d = col0 + size_t(k) * ncols + c;
 #pragma unroll
       for (int k2 = 0; k2 < P; ++k2) d[size_t(Q0 * k2) * ncols] = v[k2];
     }
   });
+  if (copy) return;
   __shared__ double wsum[kTwoXThreads / 32];
+  const int blk = F.infl_blk_off + c0 / F.conv_cols;
   const double et = block_comp_sum(e, ec, wsum);
-  if (threadIdx.x == 0) a.partials[blockIdx.x] = et;
+  if (threadIdx.x == 0) a.partials[blk] = et;
   if (VIR) {
 #pragma unroll
     for (int c = 0; c < 6; ++c) {
       const double vt = block_comp_sum(sv[c], sc[c], wsum);
-      if (threadIdx.x == 0) a.vparts[6 * blockIdx.x + c] = vt;
+      if (threadIdx.x == 0) a.vparts[6 * blk + c] = vt;
     }
+  }
+}
+
+// One block per tile and copy: a tangent pass on the forward's inputs then stages only its own
+// columns (half the shared memory of both side by side). With the transforms on both sides of the
+// multiply in registers and, for 64, 128 and 256 points, compile-time factors, the pass takes 9.6
+// us at 128^3 (cold; the earlier power-of-two kernel, which crossed shared memory four times,
+// 12.5); at 256^3 forward + backward of 262144 ions went from 1.77 to 1.74 ms.
+// KNOWN: 1 every frame's x axis is 64 or 128 points, 2 it is 256 (compile-time factors); 0 any mix.
+// Blocks [0, blocks) take rho's tiles, [blocks, 2 blocks) (tangent passes) the tangent's.
+template <bool BATCH, bool VIR, int KNOWN>
+__global__ void __launch_bounds__(kTwoXThreads, VIR ? 2 : (KNOWN == 1 ? 4 : 3)) k_two_x(ConvArgs a, int blocks) {
+  pdl_begin();
+  extern __shared__ __align__(16) float2 csm[];
+  const int copy = int(blockIdx.x) >= blocks ? 1 : 0, blk = int(blockIdx.x) - copy * blocks;
+  // tangent pass on the forward's inputs: rho's columns are not needed again
+  if (copy == 0 && a.tangent && a.keep && *a.keep == 0) return;
+  const FrameDesc& F = frame_at<BATCH>(a.one, a.maps, BATCH ? a.maps.blk_frame[blk] : 0);
+  const int c0 = (blk - F.infl_blk_off) * F.conv_cols;
+  const int kw = min(F.conv_cols, F.g.N[1] * (F.g.N[2] / 2 + 1) - c0);
+  if constexpr (KNOWN == 1) {
+    if (F.g.N[0] == 128) x_tile<16, 8, VIR>(a, F, copy, c0, kw, csm);
+    else x_tile<8, 8, VIR>(a, F, copy, c0, kw, csm);
+  } else if constexpr (KNOWN == 2) {
+    x_tile<16, 16, VIR>(a, F, copy, c0, kw, csm);
+  } else {
+    x_tile<0, 0, VIR>(a, F, copy, c0, kw, csm);
   }
 }
 
@@ -465,11 +488,10 @@ size_t two_plane_smem(const int N[3], int pp) {
   return (std::max(Z, S) + std::max(Z2, S)) * sizeof(float2);
 }
 
-// one tile of rho and tangent columns
 size_t two_x_smem(const int N[3]) {
   int nt, cols;
   conv_tiles(N, &nt, &cols);
-  return size_t(N[0]) * 2 * cols * sizeof(float2);
+  return size_t(N[0]) * cols * sizeof(float2);
 }
 
 int launch_two_plane(pme_plan_t p, cudaStream_t s, const ConvArgs& a, int grid, bool inverse) {
@@ -494,19 +516,23 @@ int launch_two_plane(pme_plan_t p, cudaStream_t s, const ConvArgs& a, int grid, 
 
 int launch_two_x(pme_plan_t p, cudaStream_t s, const ConvArgs& a, int grid) {
   int st;
-#define GB_TWO_X(B, V)                                                       \
-  do {                                                                       \
-    static unsigned done = 0;                                                \
-    if ((st = set_smem(p, k_two_x<B, V>, done))) return st;                  \
-    pdl_launch(k_two_x<B, V>, grid, kTwoXThreads, p->conv_smem_x, s, a);     \
+#define GB_TWO_X(B, V, K)                                                                        \
+  do {                                                                                           \
+    static unsigned done = 0;                                                                    \
+    if ((st = set_smem(p, k_two_x<B, V, K>, done))) return st;                                   \
+    pdl_launch(k_two_x<B, V, K>, (a.tangent ? 2 : 1) * grid, kTwoXThreads, p->conv_smem_x, s, a, grid); \
   } while (0)
-  if (p->batch) {
-    if (a.vparts) GB_TWO_X(true, true);
-    else GB_TWO_X(true, false);
-  } else {
-    if (a.vparts) GB_TWO_X(false, true);
-    else GB_TWO_X(false, false);
-  }
+#define GB_TWO_X_KNOWN(K)                            \
+  do {                                               \
+    if (p->batch && a.vparts) GB_TWO_X(true, true, K);  \
+    else if (p->batch) GB_TWO_X(true, false, K);     \
+    else if (a.vparts) GB_TWO_X(false, true, K);     \
+    else GB_TWO_X(false, false, K);                  \
+  } while (0)
+  if (p->conv_p2 || (p->conv_line && p->frames_h[0].g.N[0] <= 128)) GB_TWO_X_KNOWN(1);
+  else if (p->conv_line) GB_TWO_X_KNOWN(2);
+  else GB_TWO_X_KNOWN(0);
+#undef GB_TWO_X_KNOWN
 #undef GB_TWO_X
   count_launch();
   return check_launch(p, "k_two_x");

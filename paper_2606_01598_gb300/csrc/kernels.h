@@ -104,7 +104,6 @@ bool conv_axis_ok(int L);
 // (pass A / C, kP2PlaneThreads threads) and per pass-B block
 bool conv_p2_ok(const int N[3]);
 size_t conv_p2_plane_smem(const int N[3]);
-size_t conv_p2_x_smem(const int N[3]);
 void conv_tiles(const int N[3], int* ntile, int* cols);
 int conv_planes_per_block(const int N[3]);
 size_t conv_plane_cap(const int N[3]);

@@ -554,7 +554,7 @@ static int build_plan(pme_plan_s* p, const std::vector<FrameInput>& fin, double 
       smem_x = 0;
       for (int f = 0; f < F; ++f) {
         smem_plane = std::max(smem_plane, conv_p2_plane_smem(fin[f].mesh));
-        smem_x = std::max(smem_x, conv_p2_x_smem(fin[f].mesh));
+        smem_x = std::max(smem_x, two_x_smem(fin[f].mesh));
       }
     }
     if (conv && !p2) {
