@@ -97,6 +97,36 @@ __device__ __forceinline__ float warp_sum(float v) {
   return v;
 }
 
+// The warp's sums of N values, each lane left with one: halving exchanges (a lane keeps one half
+// of its values and gets the other lane's part of them) where the plain trees, one per value,
+// take five shuffles each; the same additions in the same order as warp_sum. Returns the index of
+// the value that v[0] now is the sum of (past N: none), or INT_MAX in the lanes that repeat it.
+template <int N>
+__device__ __forceinline__ int warp_sums(float (&v)[N], int lane) {
+  constexpr int PAD = N <= 8 ? 8 : 16;
+  static_assert(N <= 16, "at most sixteen values");
+  int idx = 0, o = 16;
+#pragma unroll
+  for (int h = PAD / 2; h >= 1; h >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int k = 0; k < h; ++k) {
+      if (k >= N) continue;
+      if (k + h < N) {
+        const float keep = up ? v[k + h] : v[k], give = up ? v[k] : v[k + h];
+        v[k] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+      } else {
+        v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+      }
+    }
+    idx |= up ? h : 0;
+    o >>= 1;
+  }
+  const bool first = (lane & (2 * o - 1)) == 0;
+  for (; o >= 1; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+  return first ? idx : 0x7fffffff;
+}
+
 // Per-lane state of one ion's sums.
 template <bool TAN>
 struct Acc;
@@ -120,6 +150,28 @@ struct Ion {
   float q, dq, gE;
 };
 
+// erfc(x) = e^{-x^2} erfcx(x) with the exponential the pair terms need anyway (ex): the scaled
+// function as a polynomial of degree 9 in t = 1 / (1 + x / 2), fitted to it by reweighted least
+// squares in relative error over 0 <= x <= 12 (3.9e-8; 3.3e-7 at most and 8e-8 RMS evaluated in
+// float32; beyond, e^{-x^2} is zero in float32). 13 instructions, where erfcf forms an exponential
+// of its own. Over the measured cases the outputs' error against float64 is that of erfcf. With
+// warp_sums the forward pass of 32768 ions went from 130.2 to 127.4 us, forward + backward of
+// 262144 ions from 1.74 to 1.71 ms.
+__device__ __forceinline__ float erfc_scaled(float x_half, float ex) {
+  const float t = __fdividef(1.f, 1.f + x_half);
+  float p = -5.753808096e-02f;
+  p = fmaf_(p, t, 2.767561078e-01f);
+  p = fmaf_(p, t, -4.700521231e-01f);
+  p = fmaf_(p, t, 2.569437623e-01f);
+  p = fmaf_(p, t, -1.057682279e-02f);
+  p = fmaf_(p, t, 1.949166059e-01f);
+  p = fmaf_(p, t, 2.454926074e-01f);
+  p = fmaf_(p, t, 2.819270194e-01f);
+  p = fmaf_(p, t, 2.821329236e-01f);
+  p = fmaf_(p, t, -2.028930567e-06f);
+  return p * ex;
+}
+
 template <bool TAN>
 // vir (forward only, nullable): adds 1/2 F_ij (x) r_ij, with F_ij = -(q_i grad phi_ij +
 // (grad grad phi_ij) mu_i) the force on i from j, row-major [9].
@@ -131,7 +183,7 @@ __device__ __forceinline__ void interact(const PairArgs& a, const Ion& I, int j,
   const float rr = r2 * rinv;
   const float alpha = a.alpha;
   const float ex = expf(-alpha * alpha * r2);
-  const float B0 = erfcf(alpha * rr) * rinv;
+  const float B0 = erfc_scaled(0.5f * alpha * rr, ex) * rinv;
   const float B1 = fmaf_(a.c1, ex, B0) * rinv2;
   const float B2 = fmaf_(a.c2, ex, 3.f * B1) * rinv2;
   const float B3 = fmaf_(a.c3, ex, 5.f * B2) * rinv2;
@@ -716,14 +768,10 @@ __global__ void __launch_bounds__(kPairThreads) k_pair_listed(PairArgs a, int n)
     v[5] = A.gm.y;
     v[6] = A.gm.z;
   }
-#pragma unroll
-  for (int k = 0; k < NA; ++k) v[k] = warp_sum(v[k]);
-  if (lane == 0) {
-    float* o = a.out + size_t(a.pr.idx[i].w) * (TAN ? 8 : 10);
-#pragma unroll
-    for (int k = 0; k < NA; ++k) o[k] = v[k];
-    if (TAN) o[7] = 0.f;
-  }
+  // each lane ends up with one sum
+  const int idx = warp_sums(v, lane);
+  constexpr int W = TAN ? 8 : 10;
+  if (idx < W) a.out[size_t(a.pr.idx[i].w) * W + idx] = idx < NA ? v[0] : 0.f;
 }
 
 template <bool TAN, bool BATCH>
