@@ -1280,8 +1280,7 @@ static int run_backward(pme_plan_t p, cudaStream_t s, const IonInputs& in, const
   const bool cached = reuse && pair && p->fwd_lists;
   p->fwd_n = -1;   // a backward leaves nothing for a later one
   t = prof_begin(p, B + 0, s);
-  if (reuse && (st = launch_input_check(p, s, in, cached))) return st;
-  if ((st = launch_sort(p, s, in, true, true, pair, reuse ? p->in_diff : nullptr))) return st;
+  if ((st = launch_sort(p, s, in, true, true, pair, reuse ? p->in_diff : nullptr, nullptr, cached))) return st;
   prof_end(p, t, s);
   cudaStream_t ps = p->opts.overlap_pair ? p->side : s;
   if (pair) {

@@ -96,6 +96,64 @@ __device__ void scan_one_segment(const int* count, int* start, int n, int seg, i
   if (hi == n && threadIdx.x == 0) start[n] = run0;
 }
 
+// Mesh and cell coordinates of an ion in compensated float32 (GB300's float64 rate is a small
+// fraction of its float32 rate); positions beyond the float path's range, or not finite, take
+// the float64 path.
+__device__ __forceinline__ void ion_origins(const Geometry& g, float rx, float ry, float rz, int (&m0)[3],
+                                            float (&fb)[3], int (&c)[3], float (&fc)[3]) {
+  bool fast = true;
+#pragma unroll
+  for (int b = 0; b < 3; ++b) {
+    fast = fast && stencil_origin_f(g, rx, ry, rz, b, m0[b], fb[b]);
+    fast = fast && cell_origin_f(g, rx, ry, rz, b, c[b], fc[b]);
+  }
+  if (fast) return;
+  double s[3];
+  frac_coords(g, rx, ry, rz, s);
+#pragma unroll
+  for (int b = 0; b < 3; ++b) {
+    stencil_origin(s[b], g.N[b], g.order, m0[b], fb[b]);
+    cell_origin(s[b], g.ncell[b], c[b], fc[b]);
+  }
+}
+
+// Charge and dipole of ion i (non-finite values as zero) and, tangent, its (dq, dr, d' = dmu + q dr).
+struct IonSources {
+  float q, mu[3], dq, dr[3], dp[3];
+};
+__device__ __forceinline__ IonSources ion_sources(const IonInputs& in, int i, int tangent) {
+  IonSources S;
+  S.q = in.q ? in.q[i] : 0.f;
+  if (!isfinite(S.q)) S.q = 0.f;
+  float dmu[3] = {0.f, 0.f, 0.f};
+  S.dq = tangent && in.gphi ? in.gphi[i] : 0.f;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    S.mu[a] = in.mu ? in.mu[3 * i + a] : 0.f;
+    if (!isfinite(S.mu[a])) S.mu[a] = 0.f;
+    S.dr[a] = tangent && in.gforce ? -in.gforce[3 * i + a] : 0.f;
+    if (tangent && in.gfield) dmu[a] = -in.gfield[3 * i + a];
+    S.dp[a] = dmu[a] + S.q * S.dr[a];
+  }
+  return S;
+}
+__device__ __forceinline__ void to_mesh(const Geometry& g, const float (&v)[3], float (&o)[3]) {
+#pragma unroll
+  for (int b = 0; b < 3; ++b) o[b] = v[0] * g.D[0 * 3 + b] + v[1] * g.D[1 * 3 + b] + v[2] * g.D[2 * 3 + b];
+}
+__device__ __forceinline__ void store_mesh_tangent(const Geometry& g, const MeshRecords& mr, int dest,
+                                                   const IonSources& S) {
+  float pd[3], pt[3];
+  to_mesh(g, S.dp, pd);
+  to_mesh(g, S.dr, pt);
+  mr.tq[dest] = make_float4(S.dq, pd[0], pd[1], pd[2]);
+  mr.tt[dest] = make_float4(pt[0], pt[1], pt[2], 0.f);
+}
+__device__ __forceinline__ void store_pair_tangent(const PairRecords& pr, int dest, const IonSources& S) {
+  pr.tq[dest] = make_float4(S.dq, S.dp[0], S.dp[1], S.dp[2]);
+  pr.dr[dest] = make_float4(S.dr[0], S.dr[1], S.dr[2], 0.f);
+}
+
 // One block per reduction item (kRedItem = kSortThreads ions of one frame, one per thread):
 // the ion's brick key and pair-cell key with one counting atomic each, its records in caller
 // order, and the item's charge sums (k_scan adds a frame's items in order).
@@ -140,26 +198,9 @@ k_bin(FrameDesc one, FrameMaps maps, IonInputs in, const PassIO* io, SortBuffers
       for (int a = 0; a < 6; ++a) ok = ok && isfinite(in.theta[6 * i + a]);
     }
     if (!ok) atomicOr(flags, kFlagNonFinite);
-    // mesh and cell coordinates in compensated float32 (GB300's float64 rate is a small
-    // fraction of its float32 rate); positions beyond the float path's range, or not finite,
-    // take the float64 path
     int m0[3], c[3];
     float fb[3], fc[3];
-    bool fast = true;
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      fast = fast && stencil_origin_f(g, rx, ry, rz, b, m0[b], fb[b]);
-      fast = fast && cell_origin_f(g, rx, ry, rz, b, c[b], fc[b]);
-    }
-    if (!fast) {
-      double s[3];
-      frac_coords(g, rx, ry, rz, s);
-#pragma unroll
-      for (int b = 0; b < 3; ++b) {
-        stencil_origin(s[b], g.N[b], g.order, m0[b], fb[b]);
-        cell_origin(s[b], g.ncell[b], c[b], fc[b]);
-      }
-    }
+    ion_origins(g, rx, ry, rz, m0, fb, c, fc);
     const int kb = F.brick_off + ((m0[0] / g.brick[0]) * g.nb[1] + m0[1] / g.brick[1]) * g.nb[2] +
                    m0[2] / g.brick[2];
     const int kc = F.cell_off + (c[0] * g.ncell[1] + c[1]) * g.ncell[2] + c[2];
@@ -302,73 +343,22 @@ k_rank_records(FrameDesc one, FrameMaps maps, IonInputs in, const PassIO* io, So
   const FrameDesc& F = frame_at<BATCH>(one, maps, f);
   const Geometry& g = F.g;
   const float rx = in.pos[3 * i], ry = in.pos[3 * i + 1], rz = in.pos[3 * i + 2];
-  float qi = in.q ? in.q[i] : 0.f;
-  float mu[3] = {0.f, 0.f, 0.f};
-  if (in.mu) {
-    mu[0] = in.mu[3 * i];
-    mu[1] = in.mu[3 * i + 1];
-    mu[2] = in.mu[3 * i + 2];
-  }
-  if (!isfinite(qi)) qi = 0.f;
-#pragma unroll
-  for (int a = 0; a < 3; ++a)
-    if (!isfinite(mu[a])) mu[a] = 0.f;
-  float dq = 0.f, dr[3] = {0.f, 0.f, 0.f}, dmu[3] = {0.f, 0.f, 0.f};
+  const IonSources S = ion_sources(in, i, tangent);
   if (tangent) {
-    if (in.gphi) dq = in.gphi[i];
-    if (in.gforce) {
-      dr[0] = -in.gforce[3 * i];
-      dr[1] = -in.gforce[3 * i + 1];
-      dr[2] = -in.gforce[3 * i + 2];
-    }
-    if (in.gfield) {
-      dmu[0] = -in.gfield[3 * i];
-      dmu[1] = -in.gfield[3 * i + 1];
-      dmu[2] = -in.gfield[3 * i + 2];
-    }
+    if (mesh_side) store_mesh_tangent(g, mr, dest, S);
+    else store_pair_tangent(pr, dest, S);
   }
-  // tangent dipole source d' = dmu + q dr
-  const float dp[3] = {dmu[0] + qi * dr[0], dmu[1] + qi * dr[1], dmu[2] + qi * dr[2]};
-  if (re) {
-    if (mesh_side) {
-      float pd[3], pt[3];
-#pragma unroll
-      for (int b = 0; b < 3; ++b) {
-        pd[b] = dp[0] * g.D[0 * 3 + b] + dp[1] * g.D[1 * 3 + b] + dp[2] * g.D[2 * 3 + b];
-        pt[b] = dr[0] * g.D[0 * 3 + b] + dr[1] * g.D[1 * 3 + b] + dr[2] * g.D[2 * 3 + b];
-      }
-      mr.tq[dest] = make_float4(dq, pd[0], pd[1], pd[2]);
-      mr.tt[dest] = make_float4(pt[0], pt[1], pt[2], 0.f);
-    } else {
-      pr.tq[dest] = make_float4(dq, dp[0], dp[1], dp[2]);
-      pr.dr[dest] = make_float4(dr[0], dr[1], dr[2], 0.f);
-    }
-    return;
-  }
+  if (re) return;
   if (sb.t_bidx) {
-    // primal records from the binning pass; tangent records formed here
+    // primal records from the binning pass
     if (mesh_side) {
       mr.idx[dest] = sb.t_bidx[i];
       mr.fq[dest] = sb.t_bfq[i];
       mr.dm[dest] = sb.t_bdm[i];
-      if (tangent) {
-        float pd[3], pt[3];
-#pragma unroll
-        for (int b = 0; b < 3; ++b) {
-          pd[b] = dp[0] * g.D[0 * 3 + b] + dp[1] * g.D[1 * 3 + b] + dp[2] * g.D[2 * 3 + b];
-          pt[b] = dr[0] * g.D[0 * 3 + b] + dr[1] * g.D[1 * 3 + b] + dr[2] * g.D[2 * 3 + b];
-        }
-        mr.tq[dest] = make_float4(dq, pd[0], pd[1], pd[2]);
-        mr.tt[dest] = make_float4(pt[0], pt[1], pt[2], 0.f);
-      }
     } else {
       pr.idx[dest] = sb.t_cidx[i];
       pr.fq[dest] = sb.t_cfq[i];
       pr.mu[dest] = sb.t_cmu[i];
-      if (tangent) {
-        pr.tq[dest] = make_float4(dq, dp[0], dp[1], dp[2]);
-        pr.dr[dest] = make_float4(dr[0], dr[1], dr[2], 0.f);
-      }
     }
     return;
   }
@@ -390,20 +380,11 @@ k_rank_records(FrameDesc one, FrameMaps maps, IonInputs in, const PassIO* io, So
       if (fast) fr[b] = fm[b];
       else stencil_origin(s[b], g.N[b], g.order, m0[b], fr[b]);
     }
-    float pm[3], pd[3], pt[3];
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      pm[b] = mu[0] * g.D[0 * 3 + b] + mu[1] * g.D[1 * 3 + b] + mu[2] * g.D[2 * 3 + b];
-      pd[b] = dp[0] * g.D[0 * 3 + b] + dp[1] * g.D[1 * 3 + b] + dp[2] * g.D[2 * 3 + b];
-      pt[b] = dr[0] * g.D[0 * 3 + b] + dr[1] * g.D[1 * 3 + b] + dr[2] * g.D[2 * 3 + b];
-    }
+    float pm[3];
+    to_mesh(g, S.mu, pm);
     mr.idx[dest] = make_int4(m0[0], m0[1], m0[2], i);
-    mr.fq[dest] = make_float4(fr[0], fr[1], fr[2], qi);
+    mr.fq[dest] = make_float4(fr[0], fr[1], fr[2], S.q);
     mr.dm[dest] = make_float4(pm[0], pm[1], pm[2], 0.f);
-    if (tangent) {
-      mr.tq[dest] = make_float4(dq, pd[0], pd[1], pd[2]);
-      mr.tt[dest] = make_float4(pt[0], pt[1], pt[2], 0.f);
-    }
   } else {
     int c[3];
     float fr[3];
@@ -418,10 +399,164 @@ k_rank_records(FrameDesc one, FrameMaps maps, IonInputs in, const PassIO* io, So
     }
     pr.idx[dest] = make_int4(c[0], c[1], c[2], i);
     pr.fq[dest] = make_float4(fr[0], fr[1], fr[2], __int_as_float(c[2]));
-    pr.mu[dest] = make_float4(mu[0], mu[1], mu[2], qi);
-    if (tangent) {
-      pr.tq[dest] = make_float4(dq, dp[0], dp[1], dp[2]);
-      pr.dr[dest] = make_float4(dr[0], dr[1], dr[2], 0.f);
+    pr.mu[dest] = make_float4(S.mu[0], S.mu[1], S.mu[2], S.q);
+  }
+}
+
+// ---- small systems: the whole sort in one block ------------------------------------------
+// A few hundred ions keep four (with the input check, five) kernels of one to sixteen blocks
+// busy for about 2 us each, most of it launch and memory latency. One block does the same
+// in one kernel, a thread per ion, with the counts, the starts and both orders in shared memory;
+// keys, records, order and outputs are those of the kernels above. Taken for single frames of up
+// to kSmallIons ions whose keys fit; beyond, one SM's own work outlasts the launches it saves.
+// Forward pass with this sort and with the kernels above, us: 64 ions 39.0 and 42.1, 200: 41.8
+// and 45.9, 300: 44.3 and 47.7, 400: 48.1 and 49.5, 512: 47.3 and 46.8, 1200: 57.5 and 49.9;
+// forward + backward of 64: 69.1 and 74.3, 300: 80.6 and 84.9, 400: 86.1 and 88.1.
+constexpr int kSmallIons = 384;
+constexpr int kSmallKeys = 8192;
+
+// saved / in_diff / cache_bad / list_cnt: as k_input_check (in_diff null: no check); save: as k_bin.
+__global__ void __launch_bounds__(kSmallIons)
+k_sort_small(FrameDesc one, IonInputs in, const PassIO* io, SortBuffers sb, MeshRecords mr, PairRecords pr,
+             int tangent, int need_mesh, int need_pair, int* flags, int nbricks, int ncells, float* save, int ld,
+             const float* saved, const int* list_cnt, int* in_diff, int* cache_bad) {
+  pdl_begin();
+  if (io) in = io->in;
+  extern __shared__ __align__(16) int keys[];   // [nbricks + ncells] counts, then starts
+  const int n = in.n, T = blockDim.x, tid = threadIdx.x, nk = nbricks + ncells;
+  unsigned short* order_b = reinterpret_cast<unsigned short*>(keys + nk);
+  unsigned short* order_c = order_b + kSmallIons;
+  const Geometry& g = one.g;
+  bool re = false;
+  if (in_diff) {
+    bool same = true, lists = true;
+    for (int k = tid; k < 3 * n; k += T) {
+      same = same && __float_as_int(in.pos[k]) == __float_as_int(saved[k]);
+      same = same && __float_as_int(in.mu ? in.mu[k] : 0.f) == __float_as_int(saved[4 * ld + k]);
+    }
+    for (int k = tid; k < n; k += T) {
+      same = same && __float_as_int(in.q ? in.q[k] : 0.f) == __float_as_int(saved[3 * ld + k]);
+      if (list_cnt) lists = lists && list_cnt[k] >= 0;
+    }
+    const bool diff = __syncthreads_or(!same), bad = __syncthreads_or(!lists);
+    if (tid == 0) {
+      *in_diff = diff;
+      *cache_bad = diff || bad;
+    }
+    re = !diff;
+  }
+  if (!re)
+    for (int k = tid; k < nk; k += T) keys[k] = 0;
+  __syncthreads();
+  // keys and arrival slots of this thread's ion (n <= T)
+  const int i = tid;
+  int kb = 0, kc = 0, slot_b = 0, slot_c = 0, m0[3], c[3];
+  float fb[3], fc[3];
+  double qa = 0.0, qb = 0.0;
+  if (i < n) {
+    const float qi = in.q ? in.q[i] : 0.f;
+    qa += isfinite(qi) ? double(qi) : 0.0;
+    if (tangent && in.gphi) qb += double(in.gphi[i]);
+    if (!re) {
+      const float rx = in.pos[3 * i], ry = in.pos[3 * i + 1], rz = in.pos[3 * i + 2];
+      bool ok = isfinite(rx) && isfinite(ry) && isfinite(rz) && isfinite(qi);
+      if (save) {
+        save[3 * i] = rx;
+        save[3 * i + 1] = ry;
+        save[3 * i + 2] = rz;
+        save[3 * ld + i] = qi;
+      }
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        const float m = in.mu ? in.mu[3 * i + a] : 0.f;
+        ok = ok && isfinite(m);
+        if (save) save[4 * ld + 3 * i + a] = m;
+      }
+      if (in.theta) {
+#pragma unroll
+        for (int a = 0; a < 6; ++a) ok = ok && isfinite(in.theta[6 * i + a]);
+      }
+      if (!ok) atomicOr(flags, kFlagNonFinite);
+      ion_origins(g, rx, ry, rz, m0, fb, c, fc);
+      kb = ((m0[0] / g.brick[0]) * g.nb[1] + m0[1] / g.brick[1]) * g.nb[2] + m0[2] / g.brick[2];
+      kc = nbricks + (c[0] * g.ncell[1] + c[1]) * g.ncell[2] + c[2];
+      slot_b = atomicAdd(&keys[kb], 1);
+      slot_c = atomicAdd(&keys[kc], 1);
+    }
+  }
+  block_sum2_d(qa, qb);   // (its barriers also end the counting)
+  if (tid == 0) {
+    sb.qsum[0] = qa;
+    sb.qsum[1] = qb;
+  }
+  if (re) {
+    if (!tangent) return;
+    for (int t = tid; t < 2 * n; t += T) {
+      const bool mesh_side = t < n;
+      const int dest = mesh_side ? t : t - n;
+      if (mesh_side ? !need_mesh : !need_pair) continue;
+      const int ion = mesh_side ? mr.idx[dest].w : pr.idx[dest].w;
+      if (!index_ok(ion, n)) continue;
+      const IonSources S = ion_sources(in, ion, tangent);
+      if (mesh_side) store_mesh_tangent(g, mr, dest, S);
+      else store_pair_tangent(pr, dest, S);
+    }
+    return;
+  }
+  // exclusive scan of the bricks' and the cells' counts laid end to end, in place: the bricks hold
+  // all n ions, so a cell's start is its prefix less n
+  __syncthreads();
+  {
+    __shared__ int part[32];
+    const int lane = tid & 31, wid = tid >> 5, nw = T >> 5;
+    const int chunk = ((nk + T - 1) / T) | 1,   // odd: a warp's chunks start in different banks
+               lo = min(nk, tid * chunk), hi = min(nk, lo + chunk);
+    int local = 0;
+    for (int k = lo; k < hi; ++k) local += keys[k];
+    const int v = warp_inclusive(local, lane);
+    if (lane == 31) part[wid] = v;
+    __syncthreads();
+    const int w = warp_inclusive(lane < nw ? part[lane] : 0, lane);
+    int run = v - local + __shfl_sync(0xffffffffu, w, max(wid - 1, 0)) * (wid > 0 ? 1 : 0);
+    for (int k = lo; k < hi; ++k) {
+      const int cnt = keys[k], start = k < nbricks ? run : run - n;
+      keys[k] = start;
+      if (k < nbricks) sb.start_b[k] = start;
+      else sb.start_c[k - nbricks] = start;
+      run += cnt;
+    }
+    if (tid == 0) {
+      sb.start_b[nbricks] = n;
+      sb.start_c[ncells] = n;
+    }
+  }
+  __syncthreads();
+  if (i < n) {
+    order_b[keys[kb] + slot_b] = (unsigned short)i;
+    order_c[keys[kc] + slot_c] = (unsigned short)i;
+  }
+  __syncthreads();
+  if (i < n) {
+    // rank by caller index within the brick and within the cell
+    const int b0 = keys[kb], b1 = kb + 1 < nbricks ? keys[kb + 1] : n;
+    const int c0 = keys[kc], c1 = kc + 1 < nk ? keys[kc + 1] : n;
+    int db = b0, dc = c0;
+    for (int k = b0; k < b1; ++k) db += order_b[k] < i ? 1 : 0;
+    for (int k = c0; k < c1; ++k) dc += order_c[k] < i ? 1 : 0;
+    const IonSources S = ion_sources(in, i, tangent);
+    if (need_mesh && index_ok(db, n)) {
+      float pm[3];
+      to_mesh(g, S.mu, pm);
+      mr.idx[db] = make_int4(m0[0], m0[1], m0[2], i);
+      mr.fq[db] = make_float4(fb[0], fb[1], fb[2], S.q);
+      mr.dm[db] = make_float4(pm[0], pm[1], pm[2], 0.f);
+      if (tangent) store_mesh_tangent(g, mr, db, S);
+    }
+    if (need_pair && index_ok(dc, n)) {
+      pr.idx[dc] = make_int4(c[0], c[1], c[2], i);
+      pr.fq[dc] = make_float4(fc[0], fc[1], fc[2], __int_as_float(c[2]));
+      pr.mu[dc] = make_float4(S.mu[0], S.mu[1], S.mu[2], S.q);
+      if (tangent) store_pair_tangent(pr, dc, S);
     }
   }
 }
@@ -453,9 +588,25 @@ k_input_check(int n, IonInputs in, const PassIO* io, const float* saved, int ld,
   }
 }
 
+bool sort_is_small(pme_plan_t p, int n) {
+  return !p->batch && p->nframes == 1 && p->sb.qsum && n > 0 && n <= kSmallIons && p->sb.qpart &&
+         p->total_bricks + p->total_cells <= kSmallKeys;
+}
+
+int launch_input_check(pme_plan_t p, cudaStream_t s, const IonInputs& in, bool with_lists) {
+  // (a recorded pass's first node clears the flags)
+  int st = p->io_live ? PME_OK : check_cuda(p, cudaMemsetAsync(p->in_flags, 0, 2 * sizeof(int), s), "memset");
+  if (st || in.n == 0) return st;
+  const int grid = std::min(4 * device_sm_count(), (3 * in.n + 255) / 256);
+  pdl_launch(k_input_check, grid, 256, 0, s, in.n, in, live_io(p), p->in_saved, p->max_ions, with_lists ? p->plist_cnt : nullptr,
+                                      p->in_diff, p->cache_bad);
+  count_launch();
+  return check_launch(p, "k_input_check");
+}
+
 template <bool BATCH>
 int launch_sort_t(pme_plan_t p, cudaStream_t s, const IonInputs& in, bool tangent, bool need_mesh,
-                  bool need_pair, const int* reuse, float* save) {
+                  bool need_pair, const int* reuse, float* save, bool check_lists) {
   const int n = in.n;
   const int nblk = (n + kSortThreads - 1) / kSortThreads;
   FrameDesc one = p->frames_h[0];
@@ -465,6 +616,19 @@ int launch_sort_t(pme_plan_t p, cudaStream_t s, const IonInputs& in, bool tangen
     one.nitems = std::max(1, (n + kRedItem - 1) / kRedItem);
   }
   int st = PME_OK;
+  if (!BATCH && sort_is_small(p, n)) {
+    const int nk = p->total_bricks + p->total_cells;
+    const int threads = std::max(128, (n + 31) / 32 * 32);
+    const bool check = reuse != nullptr;
+    pdl_launch(k_sort_small, 1, threads, sizeof(int) * nk + 2 * sizeof(unsigned short) * kSmallIons, s, one, in,
+               live_io(p), p->sb, p->mr, p->pr, tangent ? 1 : 0, need_mesh ? 1 : 0, need_pair ? 1 : 0, p->flags,
+               p->total_bricks, p->total_cells, save, p->max_ions, check ? p->in_saved : nullptr,
+               check && check_lists ? p->plist_cnt : nullptr, check ? p->in_diff : nullptr,
+               check ? p->cache_bad : nullptr);
+    count_launch();
+    return check_launch(p, "k_sort_small");
+  }
+  if (reuse && (st = launch_input_check(p, s, in, check_lists))) return st;
   if (!p->counts_clean) {
     st = check_cuda(p, cudaMemsetAsync(p->sb.count_b, 0, sizeof(int) * (p->total_bricks + 1), s),
                     "memset brick counts");
@@ -512,22 +676,11 @@ int launch_sort_t(pme_plan_t p, cudaStream_t s, const IonInputs& in, bool tangen
 
 }  // namespace
 
-int launch_input_check(pme_plan_t p, cudaStream_t s, const IonInputs& in, bool with_lists) {
-  // (a recorded pass's first node clears the flags)
-  int st = p->io_live ? PME_OK : check_cuda(p, cudaMemsetAsync(p->in_flags, 0, 2 * sizeof(int), s), "memset");
-  if (st || in.n == 0) return st;
-  const int grid = std::min(4 * device_sm_count(), (3 * in.n + 255) / 256);
-  pdl_launch(k_input_check, grid, 256, 0, s, in.n, in, live_io(p), p->in_saved, p->max_ions, with_lists ? p->plist_cnt : nullptr,
-                                      p->in_diff, p->cache_bad);
-  count_launch();
-  return check_launch(p, "k_input_check");
-}
-
 int launch_sort(pme_plan_t p, cudaStream_t s, const IonInputs& in, bool tangent, bool need_mesh,
-                bool need_pair, const int* reuse, float* save) {
+                bool need_pair, const int* reuse, float* save, bool check_lists) {
   if (!reuse) p->fwd_n = -1;   // the sorted records no longer belong to the saved inputs
-  return p->batch ? launch_sort_t<true>(p, s, in, tangent, need_mesh, need_pair, reuse, save)
-                  : launch_sort_t<false>(p, s, in, tangent, need_mesh, need_pair, reuse, save);
+  return p->batch ? launch_sort_t<true>(p, s, in, tangent, need_mesh, need_pair, reuse, save, check_lists)
+                  : launch_sort_t<false>(p, s, in, tangent, need_mesh, need_pair, reuse, save, check_lists);
 }
 
 GBPME_BOUNDS_READER(bounds_hit_sort)
