@@ -274,6 +274,7 @@ struct pme_plan_s {
   int2* conv_planes2 = nullptr;            //   the same with the tangent meshes
   int conv_nplanes1 = 0, conv_nplanes2 = 0;
   int conv_cap = 0, conv_threads = 0;
+  int conv_maxr = 0;                       // two-step kernels: the largest factor of any axis
   size_t conv_smem_plane = 0, conv_smem_x = 0;
   int nfgroups = 0;
   void* fft_work = nullptr;

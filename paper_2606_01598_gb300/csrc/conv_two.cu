@@ -29,8 +29,28 @@ namespace {
 constexpr int kTwoMaxThreads = 512;   // pass A / C
 constexpr int kTwoXThreads = 256;     // pass B
 
-template <class F>
+// MAXR: 10 where no factor of the plan's axes exceeds 10 (kSmallRadix; every axis up to 64
+// points and some up to 100), else 16. Without the 12- to 16-point DFTs the kernels hold 64
+// registers (76 to 80 with them, or spills), a third more warps per SM, and less code: forward +
+// backward of the uneven batch of 256 frames 1203 -> 1113 us (1148 with the large ones held to 64
+// registers), forward of 512 ions on 32^3 53.7 -> 51.7 us.
+constexpr int kSmallRadix = 10;
+template <int MAXR, class F>
 __device__ __forceinline__ void with_radix(int r, F&& f) {
+  if constexpr (MAXR <= kSmallRadix) {
+    switch (r) {
+      case 1: f(std::integral_constant<int, 1>{}); break;
+      case 2: f(std::integral_constant<int, 2>{}); break;
+      case 3: f(std::integral_constant<int, 3>{}); break;
+      case 4: f(std::integral_constant<int, 4>{}); break;
+      case 5: f(std::integral_constant<int, 5>{}); break;
+      case 6: f(std::integral_constant<int, 6>{}); break;
+      case 8: f(std::integral_constant<int, 8>{}); break;
+      case 9: f(std::integral_constant<int, 9>{}); break;
+      default: f(std::integral_constant<int, 10>{}); break;
+    }
+    return;
+  }
   switch (r) {
     case 1: f(std::integral_constant<int, 1>{}); break;
     case 2: f(std::integral_constant<int, 2>{}); break;
@@ -95,8 +115,8 @@ __device__ __forceinline__ TwoPlane two_plane(const FrameDesc& F, int pc, float2
   return T;
 }
 
-template <bool BATCH>
-__global__ void __launch_bounds__(kTwoMaxThreads) k_two_r2c(ConvArgs a) {
+template <bool BATCH, int MAXR>
+__global__ void __launch_bounds__(kTwoMaxThreads, MAXR <= kSmallRadix ? 2 : 0) k_two_r2c(ConvArgs a) {
   pdl_begin();
   extern __shared__ __align__(16) float2 csm[];
   int copy, x0, pc;
@@ -112,7 +132,7 @@ __global__ void __launch_bounds__(kTwoMaxThreads) k_two_r2c(ConvArgs a) {
   float2* S = T.b0;
   const int tid = threadIdx.x, NT = blockDim.x;
   // z step 1: complex row pr = real rows 2 pp (real part) and 2 pp + 1 (imaginary part)
-  with_radix(T.Pz, [&](auto rc) {
+  with_radix<MAXR>(T.Pz, [&](auto rc) {
     constexpr int P = decltype(rc)::value;
     for (int it = tid; it < T.rows * T.Qz; it += NT) {
       int pr, t, pl = 0, pp;
@@ -130,7 +150,7 @@ __global__ void __launch_bounds__(kTwoMaxThreads) k_two_r2c(ConvArgs a) {
     }
   });
   __syncthreads();
-  with_radix(T.Qz, [&](auto rc) {
+  with_radix<MAXR>(T.Qz, [&](auto rc) {
     constexpr int Q = decltype(rc)::value;
     for (int it = tid; it < T.rows * T.Pz; it += NT) {
       int pr, k1;
@@ -146,7 +166,7 @@ __global__ void __launch_bounds__(kTwoMaxThreads) k_two_r2c(ConvArgs a) {
   __syncthreads();
   // y step 1 on the real rows' half spectra: row 2 pp is (Z_k + conj Z_{N-k}) / 2, row 2 pp + 1
   // is (Z_k - conj Z_{N-k}) / 2i, with Z the spectrum of complex row pp
-  with_radix(T.Py, [&](auto rc) {
+  with_radix<MAXR>(T.Py, [&](auto rc) {
     constexpr int P = decltype(rc)::value;
     for (int it = tid; it < T.Qy * T.Sw; it += NT) {
       int t, col, pl = 0, kz;
@@ -170,7 +190,7 @@ __global__ void __launch_bounds__(kTwoMaxThreads) k_two_r2c(ConvArgs a) {
   });
   __syncthreads();
   // y step 2, straight to the planes' [ky][kz] blocks of the spectrum
-  with_radix(T.Qy, [&](auto rc) {
+  with_radix<MAXR>(T.Qy, [&](auto rc) {
     constexpr int Q = decltype(rc)::value;
     for (int it = tid; it < T.Py * T.Sw; it += NT) {
       int k1, col, pl = 0, kz;
@@ -188,8 +208,8 @@ __global__ void __launch_bounds__(kTwoMaxThreads) k_two_r2c(ConvArgs a) {
   });
 }
 
-template <bool BATCH>
-__global__ void __launch_bounds__(kTwoMaxThreads) k_two_c2r(ConvArgs a) {
+template <bool BATCH, int MAXR>
+__global__ void __launch_bounds__(kTwoMaxThreads, MAXR <= kSmallRadix ? 2 : 0) k_two_c2r(ConvArgs a) {
   pdl_begin();
   extern __shared__ __align__(16) float2 csm[];
   int copy, x0, pc;
@@ -205,7 +225,7 @@ __global__ void __launch_bounds__(kTwoMaxThreads) k_two_c2r(ConvArgs a) {
   float2* Z = T.b0;
   const int tid = threadIdx.x, NT = blockDim.x;
   // y step 1, read from the planes' [ky][kz] blocks
-  with_radix(T.Py, [&](auto rc) {
+  with_radix<MAXR>(T.Py, [&](auto rc) {
     constexpr int P = decltype(rc)::value;
     for (int it = tid; it < T.Qy * T.Sw; it += NT) {
       int t, col, pl = 0, kz;
@@ -222,7 +242,7 @@ __global__ void __launch_bounds__(kTwoMaxThreads) k_two_c2r(ConvArgs a) {
     }
   });
   __syncthreads();
-  with_radix(T.Qy, [&](auto rc) {
+  with_radix<MAXR>(T.Qy, [&](auto rc) {
     constexpr int Q = decltype(rc)::value;
     for (int it = tid; it < T.Py * T.Sw; it += NT) {
       int k1, col;
@@ -238,7 +258,7 @@ __global__ void __launch_bounds__(kTwoMaxThreads) k_two_c2r(ConvArgs a) {
   __syncthreads();
   // z step 1 on complex row pr = (half row 2 pp) + i (half row 2 pp + 1), extended by Hermitian
   // symmetry (the n_z = 0 and Nyquist entries of a real row's spectrum are real)
-  with_radix(T.Pz, [&](auto rc) {
+  with_radix<MAXR>(T.Pz, [&](auto rc) {
     constexpr int P = decltype(rc)::value;
     for (int it = tid; it < T.rows * T.Qz; it += NT) {
       int pr, t, pl = 0, pp;
@@ -270,7 +290,7 @@ __global__ void __launch_bounds__(kTwoMaxThreads) k_two_c2r(ConvArgs a) {
   });
   __syncthreads();
   // z step 2: real parts to row 2 pp, imaginary parts to row 2 pp + 1
-  with_radix(T.Qz, [&](auto rc) {
+  with_radix<MAXR>(T.Qz, [&](auto rc) {
     constexpr int Q = decltype(rc)::value;
     for (int it = tid; it < T.rows * T.Pz; it += NT) {
       int pr, k1, pl = 0, pp;
@@ -293,16 +313,16 @@ __global__ void __launch_bounds__(kTwoMaxThreads) k_two_c2r(ConvArgs a) {
 }
 
 // f with the radix R known (FIX > 0) or switched on
-template <int FIX, class F>
+template <int FIX, int MAXR, class F>
 __device__ __forceinline__ void radix_or(int r, F&& f) {
   if constexpr (FIX > 0) f(std::integral_constant<int, FIX>{});
-  else with_radix(r, f);
+  else with_radix<MAXR>(r, f);
 }
 
 // Pass B tile: kw columns of the spectrum (copy 0: rho's, with the energy and virial sums; 1: the
 // tangent one): forward x transform, influence multiply, inverse x transform. FP, FQ: the
 // factors of the x length when known (0: the frame's). smem: N0 kw entries.
-template <int FP, int FQ, bool VIR>
+template <int FP, int FQ, bool VIR, int MAXR = 16>
 __device__ __forceinline__ void x_tile(const ConvArgs& a, const FrameDesc& F, int copy, int c0, int kw, float2* T) {
   const Geometry& g = F.g;
   const int P0 = FP > 0 ? FP : F.conv_p[0], Q0 = FQ > 0 ? FQ : F.conv_q[0];
@@ -312,7 +332,7 @@ __device__ __forceinline__ void x_tile(const ConvArgs& a, const FrameDesc& F, in
   const float2* tw = a.tw + F.tw_off[0];
   float2* col0 = a.spec + (copy ? F.tspec_off : F.spec_off) + c0;
   const int tid = threadIdx.x, NT = blockDim.x;
-  radix_or<FP>(P0, [&](auto rc) {
+  radix_or<FP, MAXR>(P0, [&](auto rc) {
     constexpr int P = decltype(rc)::value;
     for (int it = tid; it < Q0 * kw; it += NT) {
       int t, c;
@@ -332,7 +352,7 @@ __device__ __forceinline__ void x_tile(const ConvArgs& a, const FrameDesc& F, in
   const float* cz = cy + N1;
   float e = 0.f, ec = 0.f;
   float sv[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, sc[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  radix_or<FQ>(Q0, [&](auto rc) {
+  radix_or<FQ, MAXR>(Q0, [&](auto rc) {
     constexpr int Q = decltype(rc)::value;
     for (int it = tid; it < P0 * kw; it += NT) {
       int k1, c;
@@ -385,7 +405,7 @@ __device__ __forceinline__ void x_tile(const ConvArgs& a, const FrameDesc& F, in
     }
   });
   __syncthreads();
-  radix_or<FP>(P0, [&](auto rc) {
+  radix_or<FP, MAXR>(P0, [&](auto rc) {
     constexpr int P = decltype(rc)::value;
     for (int it = tid; it < Q0 * kw; it += NT) {
       int k, c;
@@ -418,10 +438,11 @@ __device__ __forceinline__ void x_tile(const ConvArgs& a, const FrameDesc& F, in
 // multiply in registers and, for 64, 128 and 256 points, compile-time factors, the pass takes 9.6
 // us at 128^3 (cold; the earlier power-of-two kernel, which crossed shared memory four times,
 // 12.5); at 256^3 forward + backward of 262144 ions went from 1.77 to 1.74 ms.
-// KNOWN: 1 every frame's x axis is 64 or 128 points, 2 it is 256 (compile-time factors); 0 any mix.
+// KNOWN: 1 every frame's x axis is 64 or 128 points, 2 it is 256 (compile-time factors); 3 any mix
+// with factors up to kSmallRadix, 0 any mix.
 // Blocks [0, blocks) take rho's tiles, [blocks, 2 blocks) (tangent passes) the tangent's.
 template <bool BATCH, bool VIR, int KNOWN>
-__global__ void __launch_bounds__(kTwoXThreads, VIR ? 2 : (KNOWN == 1 ? 4 : 3)) k_two_x(ConvArgs a, int blocks) {
+__global__ void __launch_bounds__(kTwoXThreads, VIR ? 2 : (KNOWN == 1 || KNOWN == 3 ? 4 : 3)) k_two_x(ConvArgs a, int blocks) {
   pdl_begin();
   extern __shared__ __align__(16) float2 csm[];
   const int copy = int(blockIdx.x) >= blocks ? 1 : 0, blk = int(blockIdx.x) - copy * blocks;
@@ -436,7 +457,7 @@ __global__ void __launch_bounds__(kTwoXThreads, VIR ? 2 : (KNOWN == 1 ? 4 : 3)) 
   } else if constexpr (KNOWN == 2) {
     x_tile<16, 16, VIR>(a, F, copy, c0, kw, csm);
   } else {
-    x_tile<0, 0, VIR>(a, F, copy, c0, kw, csm);
+    x_tile<0, 0, VIR, KNOWN == 3 ? kSmallRadix : 16>(a, F, copy, c0, kw, csm);
   }
 }
 
@@ -502,13 +523,16 @@ int launch_two_plane(pme_plan_t p, cudaStream_t s, const ConvArgs& a, int grid, 
     if ((st = set_smem(p, K, done))) return st;                              \
     pdl_launch(K, grid, p->conv_threads, p->conv_smem_plane, s, a);          \
   } while (0)
-  if (inverse) {
-    if (p->batch) GB_TWO_PLANE(k_two_c2r<true>);
-    else GB_TWO_PLANE(k_two_c2r<false>);
-  } else {
-    if (p->batch) GB_TWO_PLANE(k_two_r2c<true>);
-    else GB_TWO_PLANE(k_two_r2c<false>);
-  }
+#define GB_TWO_PLANE_R(R)                                \
+  do {                                                    \
+    if (p->batch && inverse) GB_TWO_PLANE((k_two_c2r<true, R>));  \
+    else if (p->batch) GB_TWO_PLANE((k_two_r2c<true, R>)); \
+    else if (inverse) GB_TWO_PLANE((k_two_c2r<false, R>)); \
+    else GB_TWO_PLANE((k_two_r2c<false, R>));              \
+  } while (0)
+  if (p->conv_maxr <= kSmallRadix) GB_TWO_PLANE_R(kSmallRadix);
+  else GB_TWO_PLANE_R(16);
+#undef GB_TWO_PLANE_R
 #undef GB_TWO_PLANE
   count_launch();
   return check_launch(p, inverse ? "k_two_c2r" : "k_two_r2c");
@@ -531,6 +555,7 @@ int launch_two_x(pme_plan_t p, cudaStream_t s, const ConvArgs& a, int grid) {
   } while (0)
   if (p->conv_p2 || (p->conv_line && p->frames_h[0].g.N[0] <= 128)) GB_TWO_X_KNOWN(1);
   else if (p->conv_line) GB_TWO_X_KNOWN(2);
+  else if (p->conv_maxr <= kSmallRadix) GB_TWO_X_KNOWN(3);
   else GB_TWO_X_KNOWN(0);
 #undef GB_TWO_X_KNOWN
 #undef GB_TWO_X

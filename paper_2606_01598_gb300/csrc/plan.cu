@@ -581,10 +581,13 @@ static int build_plan(pme_plan_s* p, const std::vector<FrameInput>& fin, double 
     // little larger than the general kernels'); the Stockham kernels otherwise
     bool two = conv && !p2;
     size_t two_plane = 0, two_x = 0;
-    int two_threads = 0;
+    int two_threads = 0, maxr = 1;
     for (int f = 0; f < F && two; ++f) {
       int P, Q;
-      for (int a = 0; a < 3; ++a) two = two && two_step_factors(fin[f].mesh[a], &P, &Q);
+      for (int a = 0; a < 3 && two; ++a) {
+        two = two_step_factors(fin[f].mesh[a], &P, &Q);
+        if (two) maxr = std::max(maxr, P);
+      }
       if (!two) break;
       const int pp = two_planes_per_block(fin[f].mesh, single);
       two_plane = std::max(two_plane, two_plane_smem(fin[f].mesh, pp));
@@ -600,6 +603,7 @@ static int build_plan(pme_plan_s* p, const std::vector<FrameInput>& fin, double 
       p->conv_smem_plane = two_plane;
       p->conv_smem_x = two_x;
       p->conv_threads = two_threads;
+      p->conv_maxr = maxr;
     }
     if (p->conv_line) p->conv_smem_x = two_x_smem(fin[0].mesh);
   }
