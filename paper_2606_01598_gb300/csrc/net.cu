@@ -233,7 +233,10 @@ struct MsgArgs {
 // Formed in every lane for every edge, they were most of the kernels' instructions. With the
 // weights in registers and only the outputs that a pass reads afterwards, the four message
 // kernels of a gradient over 32 frames of 512 ions (265 k edges) went from 1.88 ms to about
-// 0.5 ms, and the gradient from 2.87 to 1.51 ms.
+// 0.5 ms, and the gradient from 2.87 to 1.51 ms. They wait on their neighbours' rows, so warps in
+// flight count for more than the 20 to 70 bytes that a few spill: held to 64 to 128 registers, two
+// to four blocks of eight warps per SM instead of one to three, the gradient went from 1489 to
+// 1401 us.
 template <typename T, bool DE>
 struct EdgeRec {
   static constexpr bool kDual = sizeof(T) > sizeof(float);
@@ -315,7 +318,7 @@ __device__ __forceinline__ Vec3<T> ldrow3(const float* p, int j, int c, size_t p
 // ion, lane = channel. FIRST: the first layer, whose vector features are zero, so B (= h^v WB)
 // is too and is neither formed nor read.
 template <typename T, bool FIRST>
-__global__ void __launch_bounds__(32 * kWarps) k_msg_fwd(MsgArgs a, const float* __restrict__ A,
+__global__ void __launch_bounds__(32 * kWarps, sizeof(T) > 4 ? 3 : 4) k_msg_fwd(MsgArgs a, const float* __restrict__ A,
                                                        const float* __restrict__ B, float* ms, float* mv) {
   constexpr int VEC = EdgeRec<T, false>::kVec;
   __shared__ float4 srec[kWarps][32 * VEC];
@@ -379,7 +382,7 @@ __global__ void __launch_bounds__(32 * kWarps) k_msg_fwd(MsgArgs a, const float*
 // float pass needs the positions (and the cotangents of the second layer, GA), its Dual pass
 // the parameters. FIRST: B is zero and its cotangent unused, as in k_msg_fwd.
 template <typename T, bool POS, bool GA, bool GRAD, bool FIRST>
-__global__ void __launch_bounds__(32 * kWarps) k_msg_bwd(MsgArgs a, const float* __restrict__ A,
+__global__ void __launch_bounds__(32 * kWarps, sizeof(T) > 4 ? 2 : GRAD ? 2 : 3) k_msg_bwd(MsgArgs a, const float* __restrict__ A,
                                                        const float* __restrict__ B, const float* __restrict__ gms,
                                                        const float* __restrict__ gmv, float* gA_out, float* gB_out,
                                                        float* gpos, float* wr_part) {
