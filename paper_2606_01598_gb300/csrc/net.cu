@@ -980,8 +980,8 @@ struct RedJobs {
 // grad[w] (+)= sum over b of part[b][w]: 32 consecutive parameters per block, one per lane;
 // warp s adds the partials b = s, s + 32, ... as a float32 sum and its rounding errors (Knuth's
 // two-sum; GB300 adds float64 at a small fraction of that rate), then the 32 sums, each exact to
-// about 48 bits, are added in float64 in order (1401 -> 1367 us for the
-// gradient over 32 frames of 512 ions).
+// about 48 bits, are added in float64 in order (1401 -> 1367 us for the gradient over 32 frames
+// of 512 ions).
 __global__ void __launch_bounds__(1024) k_reduce(RedJobs jobs, float* __restrict__ grad, int accumulate) {
   __shared__ double sum[32][33];
   int u = 0;
@@ -1174,10 +1174,22 @@ int cuda_ok(gbnet_t net, cudaError_t e, const char* what) {
 
 inline unsigned blocks_for(size_t m, int t) { return unsigned((m + t - 1) / t); }
 
-int mix(gbnet_t net, cudaStream_t s, int M, int K, int N, const float* X, int w, bool transposed_weights,
-        float* Y, bool acc) {
-  const uint16_t* W = net->wbf + net->wbf_offs[2 * w + (transposed_weights ? 1 : 0)];
-  const int st = launch_mix(s, M, K, N, X, W, Y, acc, net->flags);
+// One channel mixing: Y [M][N] (+)= X [M][K] with matrix w (or its transpose, the input gradient).
+struct Mix {
+  int M, K, N;
+  const float* X;
+  int w;
+  bool transposed_weights;
+  float* Y;
+  bool acc;
+};
+
+int mix(gbnet_t net, cudaStream_t s, const Mix& m, const Mix* second = nullptr) {
+  auto job = [&](const Mix& x) {
+    return MixJob{x.X, net->wbf + net->wbf_offs[2 * x.w + (x.transposed_weights ? 1 : 0)], x.Y, x.M, x.acc ? 1 : 0};
+  };
+  const int st = second ? launch_mix_pair(s, m.K, m.N, job(m), second->K, second->N, job(*second), net->flags)
+                        : launch_mix(s, m.K, m.N, job(m), net->flags);
   ++net->launches;
   return st ? fail(net, st, "channel mixing") : PME_OK;
 }
@@ -1209,9 +1221,9 @@ int forward_pass(gbnet_t net, cudaStream_t s, const float* pos, const float* dpo
   k_embed<<<blocks_for(size_t(n) * S, 256), 256, 0, s>>>(net->P, net->species, n, net->hs[0], plS, planes);
   NET_LAUNCHED(net);
   for (int t = 0; t < 2; ++t) {
-    if ((st = mix(net, s, planes * n, S, S + V, net->hs[t], 4 * t + 0, true, net->A[t], false))) return st;
-    if (t > 0 && (st = mix(net, s, planes * 3 * n, V, 2 * V, net->hv[t], 4 * t + 1, true, net->B[t], false)))
-      return st;
+    const Mix mA{planes * n, S, S + V, net->hs[t], 4 * t + 0, true, net->A[t], false};
+    const Mix mB{planes * 3 * n, V, 2 * V, net->hv[t], 4 * t + 1, true, net->B[t], false};
+    if ((st = mix(net, s, mA, t > 0 ? &mB : nullptr))) return st;   // (h^v = 0 below the first layer)
     const MsgArgs a = msg_args<T>(net, t, pos, dpos);
     if (t == 0)
       k_msg_fwd<T, true><<<blocks_for(n, kWarps), 32 * kWarps, 0, s>>>(a, net->A[t], nullptr, net->ms[t], net->mv[t]);
@@ -1219,13 +1231,14 @@ int forward_pass(gbnet_t net, cudaStream_t s, const float* pos, const float* dpo
       k_msg_fwd<T, false><<<blocks_for(n, kWarps), 32 * kWarps, 0, s>>>(a, net->A[t], net->B[t], net->ms[t],
                                                                        net->mv[t]);
     NET_LAUNCHED(net);
-    if ((st = mix(net, s, planes * n, S + V, S + V, net->ms[t], 4 * t + 2, true, net->U[t], false))) return st;
-    if ((st = mix(net, s, planes * 3 * n, 2 * V, V, net->mv[t], 4 * t + 3, true, net->Y[t], false))) return st;
+    const Mix mU{planes * n, S + V, S + V, net->ms[t], 4 * t + 2, true, net->U[t], false};
+    const Mix mY{planes * 3 * n, 2 * V, V, net->mv[t], 4 * t + 3, true, net->Y[t], false};
+    if ((st = mix(net, s, mU, &mY))) return st;
     k_update_fwd<T><<<blocks_for(size_t(n) * S, 256), 256, 0, s>>>(n, net->U[t], net->Y[t], net->hs[t], net->hv[t],
                                                                   net->hs[t + 1], net->hv[t + 1], pl48, plV, plS, plV);
     NET_LAUNCHED(net);
   }
-  if ((st = mix(net, s, planes * n, S, 2 * S, net->hs[2], 8, true, net->H, false))) return st;
+  if ((st = mix(net, s, Mix{planes * n, S, 2 * S, net->hs[2], 8, true, net->H, false}))) return st;
   k_readout_fwd<T><<<blocks_for(n, kWarps), 32 * kWarps, 0, s>>>(n, net->P, net->H, net->hv[2], net->qt, net->ei,
                                                                 net->mu, pl64, plV, size_t(n));
   NET_LAUNCHED(net);
@@ -1343,13 +1356,14 @@ int backward_pass(gbnet_t net, cudaStream_t s, const float* pos, const float* dp
   const int nb_ion = int(blocks_for(n, kWarps));
   k_readout_bwd<T><<<nb_ion, 32 * kWarps, 0, s>>>(ra);
   NET_LAUNCHED(net);
-  if ((st = mix(net, s, planes * n, 2 * S, S, net->gH, 8, false, net->ghs, false))) return st;
+  if ((st = mix(net, s, Mix{planes * n, 2 * S, S, net->gH, 8, false, net->ghs, false}))) return st;
   for (int t = 1; t >= 0; --t) {
     k_update_bwd<T><<<blocks_for(size_t(n) * S, 256), 256, 0, s>>>(n, net->U[t], net->Y[t], net->ghs, net->ghv,
                                                                    net->gU[t], net->gY[t], pl48, plV, plS, plV);
     NET_LAUNCHED(net);
-    if ((st = mix(net, s, planes * n, S + V, S + V, net->gU[t], 4 * t + 2, false, net->gms, false))) return st;
-    if ((st = mix(net, s, planes * 3 * n, V, 2 * V, net->gY[t], 4 * t + 3, false, net->gmv, false))) return st;
+    const Mix mU{planes * n, S + V, S + V, net->gU[t], 4 * t + 2, false, net->gms, false};
+    const Mix mY{planes * 3 * n, V, 2 * V, net->gY[t], 4 * t + 3, false, net->gmv, false};
+    if ((st = mix(net, s, mU, &mY))) return st;
     const MsgArgs a = msg_args<T>(net, t, pos, dpos);
     float* wr = grad ? net->part + L.wr[t] : nullptr;
 #define GB_MSG_BWD(POS, GA, GRAD, FIRST)                                                                          \
@@ -1369,8 +1383,9 @@ int backward_pass(gbnet_t net, cudaStream_t s, const float* pos, const float* dp
     NET_LAUNCHED(net);
     // below the first layer lie only the embedding (a parameter) and h^v = 0
     if (t == 0 && !grad) break;
-    if ((st = mix(net, s, planes * n, S + V, S, net->gA[t], 4 * t + 0, false, net->ghs, true))) return st;
-    if (t > 0 && (st = mix(net, s, planes * 3 * n, 2 * V, V, net->gB[t], 4 * t + 1, false, net->ghv, true))) return st;
+    const Mix mA{planes * n, S + V, S, net->gA[t], 4 * t + 0, false, net->ghs, true};
+    const Mix mB{planes * 3 * n, 2 * V, V, net->gB[t], 4 * t + 1, false, net->ghv, true};
+    if ((st = mix(net, s, mA, t > 0 ? &mB : nullptr))) return st;
   }
   if (grad && (st = param_grads<T>(net, s, grad, acc))) return st;
   (void)pl96;
@@ -1757,7 +1772,7 @@ int gbnet_mix(void* stream, int M, int k, int nout, const float* X, const unsign
     if (!dummy && cudaMalloc(&dummy, sizeof(int)) != cudaSuccess) return PME_ERR_NOMEM;
     err = dummy;
   }
-  return launch_mix(static_cast<cudaStream_t>(stream), M, k, nout, X, wt, Y, accumulate != 0, err);
+  return launch_mix(static_cast<cudaStream_t>(stream), k, nout, MixJob{X, wt, Y, M, accumulate != 0}, err);
 }
 
 int gbnet_sync_status(gbnet_t net, void* stream) {
