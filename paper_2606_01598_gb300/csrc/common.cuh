@@ -40,6 +40,17 @@ __device__ __forceinline__ void pdl_begin() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// The same, returning blockIdx.x, for kernels with const __restrict__ parameters, whose loads the
+// compiler may move over the wait: an address formed from the returned index is not known before
+// it. (The grid before the preceding one has completed by the time a block starts, so what only
+// older grids wrote may be read by any address.)
+__device__ __forceinline__ int pdl_begin_block() {
+  int b;
+  asm volatile("griddepcontrol.wait;\n\tmov.u32 %0, %%ctaid.x;" : "=r"(b) :: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  return b;
+}
+
 template <typename... KArgs, typename... Args>
 inline cudaError_t pdl_launch(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                               Args... args) {

@@ -36,6 +36,7 @@
 namespace gbnet {
 
 using gbpme::Dual;
+using gbpme::pdl_launch;
 using gbpme::rcpT;
 using gbpme::sqrtT;
 using gbpme::sincosT;
@@ -135,7 +136,8 @@ struct Nbr {
 // increasing j order.
 __global__ void k_nbr(const NetFrame* __restrict__ frames, const int* __restrict__ frame_of,
                       const float* __restrict__ pos, int n, int* cnt, int* nj, float4* nsh, int* flags) {
-  const int i = blockIdx.x * kWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const int bx = gbpme::pdl_begin_block();
+  const int i = bx * kWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (i >= n) return;
   const NetFrame F = frames[frame_of[i]];
   const float xi = pos[3 * i], yi = pos[3 * i + 1], zi = pos[3 * i + 2];
@@ -318,13 +320,14 @@ __device__ __forceinline__ Vec3<T> ldrow3(const float* p, int j, int c, size_t p
 // ion, lane = channel. FIRST: the first layer, whose vector features are zero, so B (= h^v WB)
 // is too and is neither formed nor read.
 template <typename T, bool FIRST>
-__global__ void __launch_bounds__(32 * kWarps, sizeof(T) > 4 ? 3 : 4) k_msg_fwd(MsgArgs a, const float* __restrict__ A,
-                                                       const float* __restrict__ B, float* ms, float* mv) {
+__global__ void __launch_bounds__(32 * kWarps, sizeof(T) > 4 ? 3 : 4)
+k_msg_fwd(MsgArgs a, const float* __restrict__ A, const float* __restrict__ B, float* ms, float* mv) {
+  const int bx = gbpme::pdl_begin_block();
   constexpr int VEC = EdgeRec<T, false>::kVec;
   __shared__ float4 srec[kWarps][32 * VEC];
   __shared__ int sj[kWarps][32];
   const int w = threadIdx.x >> 5, c = threadIdx.x & 31;
-  const int i = blockIdx.x * kWarps + w;
+  const int i = bx * kWarps + w;
   if (i >= a.n) return;
   const bool lo = c < V;
   float w0[NR], w1[NR], w2[NR];
@@ -382,17 +385,17 @@ __global__ void __launch_bounds__(32 * kWarps, sizeof(T) > 4 ? 3 : 4) k_msg_fwd(
 // float pass needs the positions (and the cotangents of the second layer, GA), its Dual pass
 // the parameters. FIRST: B is zero and its cotangent unused, as in k_msg_fwd.
 template <typename T, bool POS, bool GA, bool GRAD, bool FIRST>
-__global__ void __launch_bounds__(32 * kWarps, sizeof(T) > 4 ? 2 : GRAD ? 2 : 3) k_msg_bwd(MsgArgs a, const float* __restrict__ A,
-                                                       const float* __restrict__ B, const float* __restrict__ gms,
-                                                       const float* __restrict__ gmv, float* gA_out, float* gB_out,
-                                                       float* gpos, float* wr_part) {
+__global__ void __launch_bounds__(32 * kWarps, sizeof(T) > 4 || GRAD ? 2 : 3)
+k_msg_bwd(MsgArgs a, const float* __restrict__ A, const float* __restrict__ B, const float* __restrict__ gms,
+          const float* __restrict__ gmv, float* gA_out, float* gB_out, float* gpos, float* wr_part) {
+  const int bx = gbpme::pdl_begin_block();
   constexpr int VEC = EdgeRec<T, POS>::kVec;
   constexpr int kRecFloats = kWarps * 32 * VEC * 4, kPartFloats = kWarps * NR * NCOL;
   // the edge records; after the edge loop the warps' partials of dL/dWR in the same place
   __shared__ __align__(16) float smem[GRAD ? (kRecFloats > kPartFloats ? kRecFloats : kPartFloats) : kRecFloats];
   __shared__ int sj[kWarps][32];
   const int w = threadIdx.x >> 5, c = threadIdx.x & 31;
-  const int i = blockIdx.x * kWarps + w;
+  const int i = bx * kWarps + w;
   const bool lo = c < V;
   float4* srec = reinterpret_cast<float4*>(smem) + w * 32 * VEC;
   // per-lane partials of dL/dWR for this lane's columns: cols c, and (lo) S + c, S + V + c,
@@ -563,7 +566,7 @@ __global__ void __launch_bounds__(32 * kWarps, sizeof(T) > 4 ? 2 : GRAD ? 2 : 3)
     for (int k = threadIdx.x; k < NR * NCOL; k += blockDim.x) {
       float acc = 0.f;
       for (int ww = 0; ww < kWarps; ++ww) acc += smem[ww * NR * NCOL + k];
-      wr_part[size_t(blockIdx.x) * NR * NCOL + k] = acc;
+      wr_part[size_t(bx) * NR * NCOL + k] = acc;
     }
   }
 }
@@ -576,7 +579,8 @@ __global__ void __launch_bounds__(32 * kWarps, sizeof(T) > 4 ? 2 : GRAD ? 2 : 3)
 // stored (the first layer's kernels take it as zero)
 __global__ void k_embed(const float* __restrict__ P, const int* __restrict__ species, int n, float* hs, size_t plS,
                         int planes) {
-  const size_t t = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  const int bx = gbpme::pdl_begin_block();
+  const size_t t = size_t(bx) * blockDim.x + threadIdx.x;
   if (t >= size_t(n) * S) return;
   const int i = int(t / S), c = int(t % S);
   hs[t] = P[oEmb + species[i] * S + c];
@@ -590,7 +594,8 @@ template <typename T>
 __global__ void k_update_fwd(int n, const float* __restrict__ U, const float* __restrict__ Y,
                              const float* __restrict__ hs_in, const float* __restrict__ hv_in, float* hs_out,
                              float* hv_out, size_t plU, size_t plY, size_t plS, size_t plV) {
-  const size_t t = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  const int bx = gbpme::pdl_begin_block();
+  const size_t t = size_t(bx) * blockDim.x + threadIdx.x;
   if (t >= size_t(n) * S) return;
   const size_t i = t / S;
   const int c = int(t % S);
@@ -612,7 +617,8 @@ template <typename T>
 __global__ void k_update_bwd(int n, const float* __restrict__ U, const float* __restrict__ Y,
                              const float* __restrict__ ghs, const float* __restrict__ ghv, float* gU, float* gY,
                              size_t plU, size_t plY, size_t plS, size_t plV) {
-  const size_t t = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  const int bx = gbpme::pdl_begin_block();
+  const size_t t = size_t(bx) * blockDim.x + threadIdx.x;
   if (t >= size_t(n) * S) return;
   const size_t i = t / S;
   const int c = int(t % S);
@@ -636,7 +642,8 @@ template <typename T>
 __global__ void k_readout_fwd(int n, const float* __restrict__ P, const float* __restrict__ H,
                               const float* __restrict__ hv, float* qt, float* ei, float* mu, size_t plH,
                               size_t plV, size_t pln) {
-  const int i = blockIdx.x * kWarps + (threadIdx.x >> 5), c = threadIdx.x & 31;
+  const int bx = gbpme::pdl_begin_block();
+  const int i = bx * kWarps + (threadIdx.x >> 5), c = threadIdx.x & 31;
   if (i >= n) return;
   const T hq = ldT<T>(H, size_t(i) * 2 * S + c, plH) + P[oBh + c];
   const T he = ldT<T>(H, size_t(i) * 2 * S + S + c, plH) + P[oBh + S + c];
@@ -662,7 +669,8 @@ __global__ void k_readout_fwd(int n, const float* __restrict__ P, const float* _
 template <typename T>
 __global__ void k_frame_fwd(const NetFrame* __restrict__ frames, const float* __restrict__ qt,
                             const float* __restrict__ ei, float* q, double* esr, size_t pln) {
-  const NetFrame F = frames[blockIdx.x];
+  const int bx = gbpme::pdl_begin_block();
+  const NetFrame F = frames[bx];
   double sq = 0.0, sqd = 0.0, se = 0.0;
   for (int i = F.off + threadIdx.x; i < F.off + F.n; i += blockDim.x) {
     const T x = ldT<T>(qt, i, pln);
@@ -690,7 +698,7 @@ __global__ void k_frame_fwd(const NetFrame* __restrict__ frames, const float* __
     }
     mean[0] = F.n ? float(a / F.n) : 0.f;
     mean[1] = F.n ? float(b / F.n) : 0.f;
-    if (esr) esr[blockIdx.x] = e;
+    if (esr) esr[bx] = e;
   }
   __syncthreads();
   for (int i = F.off + threadIdx.x; i < F.off + F.n; i += blockDim.x) {
@@ -703,7 +711,8 @@ __global__ void k_frame_fwd(const NetFrame* __restrict__ frames, const float* __
 template <typename T>
 __global__ void k_frame_mean(const NetFrame* __restrict__ frames, const float* __restrict__ g, float* mean,
                              size_t pln) {
-  const NetFrame F = frames[blockIdx.x];
+  const int bx = gbpme::pdl_begin_block();
+  const NetFrame F = frames[bx];
   double a = 0.0, b = 0.0;
   for (int i = F.off + threadIdx.x; i < F.off + F.n; i += blockDim.x) {
     const T x = ldT<T>(g, i, pln);
@@ -714,8 +723,8 @@ __global__ void k_frame_mean(const NetFrame* __restrict__ frames, const float* _
   __syncthreads();
   b = gbpme::block_sum_d(b);
   if (threadIdx.x == 0) {
-    mean[2 * blockIdx.x] = F.n ? float(a / F.n) : 0.f;
-    mean[2 * blockIdx.x + 1] = F.n ? float(b / F.n) : 0.f;
+    mean[2 * bx] = F.n ? float(a / F.n) : 0.f;
+    mean[2 * bx + 1] = F.n ? float(b / F.n) : 0.f;
   }
 }
 
@@ -737,9 +746,10 @@ struct ReadoutBwdArgs {
 
 template <typename T>
 __global__ void __launch_bounds__(32 * kWarps) k_readout_bwd(ReadoutBwdArgs a) {
+  const int bx = gbpme::pdl_begin_block();
   __shared__ float sp[kWarps][kReadoutW];
   const int w = threadIdx.x >> 5, c = threadIdx.x & 31;
-  const int i = blockIdx.x * kWarps + w;
+  const int i = bx * kWarps + w;
   for (int k = c; k < kReadoutW; k += 32) sp[w][k] = 0.f;
   __syncwarp();
   if (i < a.n) {
@@ -779,7 +789,7 @@ __global__ void __launch_bounds__(32 * kWarps) k_readout_bwd(ReadoutBwdArgs a) {
   for (int k = threadIdx.x; k < kReadoutW; k += blockDim.x) {
     float acc = 0.f;
     for (int ww = 0; ww < kWarps; ++ww) acc += sp[ww][k];
-    a.part[size_t(blockIdx.x) * kReadoutW + k] = acc;
+    a.part[size_t(bx) * kReadoutW + k] = acc;
   }
 }
 
@@ -940,11 +950,12 @@ __host__ __device__ constexpr int wg_rows(int kind) { return kind == kWgY || kin
 
 template <int PL>
 __global__ void __launch_bounds__(kWgThreads) k_wgrad(WgJobs jobs) {
+  const int bx = gbpme::pdl_begin_block();
   __shared__ __align__(16) float sm[PL * 96 * kWgSub];
   int u = 0;
-  while (u + 1 < jobs.n && int(blockIdx.x) >= jobs.job[u + 1].first) ++u;
+  while (u + 1 < jobs.n && bx >= jobs.job[u + 1].first) ++u;
   const WgJob& J = jobs.job[u];
-  const int blk = int(blockIdx.x) - J.first;
+  const int blk = bx - J.first;
   switch (J.kind) {
     case kWgU: wgrad_block<PL, S + V, S + V, 3, 3, kWgRows>(J, blk, sm); break;
     case kWgA: wgrad_block<PL, S, S + V, 2, 3, kWgRows>(J, blk, sm); break;
@@ -983,12 +994,13 @@ struct RedJobs {
 // about 48 bits, are added in float64 in order (1401 -> 1367 us for the gradient over 32 frames
 // of 512 ions).
 __global__ void __launch_bounds__(1024) k_reduce(RedJobs jobs, float* __restrict__ grad, int accumulate) {
+  const int bx = gbpme::pdl_begin_block();
   __shared__ double sum[32][33];
   int u = 0;
-  while (u + 1 < jobs.n && int(blockIdx.x) >= jobs.job[u + 1].first) ++u;
+  while (u + 1 < jobs.n && bx >= jobs.job[u + 1].first) ++u;
   const RedJob& J = jobs.job[u];
   const int lane = threadIdx.x & 31, slice = threadIdx.x >> 5;
-  const int k = (int(blockIdx.x) - J.first) * 32 + lane;
+  const int k = (bx - J.first) * 32 + lane;
   float acc = 0.f, err = 0.f;
   if (k < J.width) {
     const float* p = J.part + k;
@@ -1027,7 +1039,8 @@ __global__ void k_loss(const NetFrame* __restrict__ frames, int nframes, int nto
                        const float* __restrict__ f_pme, const float* __restrict__ gpos_net,
                        const float* __restrict__ f_ref, double lambda_e, double lambda_f, double* cvec,
                        float* force, float* dpos, float* wneg, double* part) {
-  const NetFrame F = frames[blockIdx.x];
+  const int bx = gbpme::pdl_begin_block();
+  const NetFrame F = frames[bx];
   const double wf = 2.0 * lambda_f / (3.0 * double(ntot));
   double lf = 0.0;
   for (int t = threadIdx.x; t < 3 * F.n; t += blockDim.x) {
@@ -1042,17 +1055,18 @@ __global__ void k_loss(const NetFrame* __restrict__ frames, int nframes, int nto
   }
   lf = gbpme::block_sum_d(lf);
   if (threadIdx.x == 0) {
-    const double E = e_pme[blockIdx.x] + e_sr[blockIdx.x];
-    const double dE = (E - e_ref[blockIdx.x]) / double(max(F.n, 1));
-    cvec[blockIdx.x] = F.n ? 2.0 * lambda_e * dE / (double(nframes) * double(F.n)) : 0.0;
-    part[2 * blockIdx.x] = lambda_e * dE * dE / double(nframes);
-    part[2 * blockIdx.x + 1] = lambda_f * lf / (3.0 * double(ntot));
+    const double E = e_pme[bx] + e_sr[bx];
+    const double dE = (E - e_ref[bx]) / double(max(F.n, 1));
+    cvec[bx] = F.n ? 2.0 * lambda_e * dE / (double(nframes) * double(F.n)) : 0.0;
+    part[2 * bx] = lambda_e * dE * dE / double(nframes);
+    part[2 * bx + 1] = lambda_f * lf / (3.0 * double(ntot));
   }
 }
 
 __global__ void k_loss_total(const double* __restrict__ part, int nframes, double* loss) {
-  double le = 0.0, lf = 0.0;
-  for (int f = threadIdx.x; f < nframes; f += blockDim.x) {
+  const int bx = gbpme::pdl_begin_block();
+  double le = 0.0, lf = 0.0;   // one block
+  for (int f = bx + int(threadIdx.x); f < nframes; f += blockDim.x) {
     le += part[2 * f];
     lf += part[2 * f + 1];
   }
@@ -1068,7 +1082,8 @@ __global__ void k_loss_total(const double* __restrict__ part, int nframes, doubl
 
 // energy cotangent seeds of the Dual backward: gesr[2 f] = 1, gesr[2 f + 1] = c_f
 __global__ void k_seed_esr(int nframes, const double* __restrict__ cvec, float* gesr, int with_tangent) {
-  const int f = blockIdx.x * blockDim.x + threadIdx.x;
+  const int bx = gbpme::pdl_begin_block();
+  const int f = bx * blockDim.x + threadIdx.x;
   if (f >= nframes) return;
   gesr[2 * f] = 1.f;
   gesr[2 * f + 1] = with_tangent ? float(cvec[f]) : 0.f;
@@ -1076,17 +1091,19 @@ __global__ void k_seed_esr(int nframes, const double* __restrict__ cvec, float* 
 
 // dst[k] = s * src[k] (and optionally a second array into the tangent plane of dst)
 __global__ void k_scale(size_t m, const float* __restrict__ src, float s, float* dst) {
-  const size_t t = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  const int bx = gbpme::pdl_begin_block();
+  const size_t t = size_t(bx) * blockDim.x + threadIdx.x;
   if (t < m) dst[t] = s * src[t];
 }
 
 // bfloat16 copies of the channel-mixing matrices: W [K][N] and W^T [N][K]
 __global__ void k_cast_weights(const float* __restrict__ P, uint16_t* wbf, const int* __restrict__ offs) {
+  const int bx = gbpme::pdl_begin_block();
   const int w = blockIdx.y;
   const MixW m = mix_w(w);
   uint16_t* dW = wbf + offs[2 * w];
   uint16_t* dWt = wbf + offs[2 * w + 1];
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < m.K * m.N; t += gridDim.x * blockDim.x) {
+  for (int t = bx * blockDim.x + threadIdx.x; t < m.K * m.N; t += gridDim.x * blockDim.x) {
     const int k = t / m.N, nn = t % m.N;
     const uint32_t u = __float_as_uint(P[m.off + t]);
     const uint16_t b = uint16_t((u + 0x7FFFu + ((u >> 16) & 1u)) >> 16);
@@ -1097,7 +1114,8 @@ __global__ void k_cast_weights(const float* __restrict__ P, uint16_t* wbf, const
 
 __global__ void k_adam(int np, float* __restrict__ P, float* __restrict__ m, float* __restrict__ v,
                        const float* __restrict__ g, float lr, float b1, float b2, float eps, float c1, float c2) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  const int bx = gbpme::pdl_begin_block();
+  const int t = bx * blockDim.x + threadIdx.x;
   if (t >= np) return;
   const float gt = g[t];
   const float mt = b1 * m[t] + (1.f - b1) * gt;
@@ -1164,6 +1182,9 @@ int cuda_ok(gbnet_t net, cudaError_t e, const char* what) {
   return fail(net, PME_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
 }
 
+// A loss gradient is about eighty launches of 3 to 100 us on one stream, each waiting for the one
+// before: launched with pdl_launch they are scheduled while that one drains (32 frames of 512 ions,
+// 1220 -> 1124 us).
 #define NET_LAUNCHED(net)                                                          \
   do {                                                                             \
     gbpme::count_launch();                                                         \
@@ -1218,7 +1239,8 @@ int forward_pass(gbnet_t net, cudaStream_t s, const float* pos, const float* dpo
                pl96 = size_t(n) * 3 * 2 * V, pl64 = size_t(n) * 2 * S;
   int st;
   if (n == 0) return PME_OK;
-  k_embed<<<blocks_for(size_t(n) * S, 256), 256, 0, s>>>(net->P, net->species, n, net->hs[0], plS, planes);
+  pdl_launch(k_embed, blocks_for(size_t(n) * S, 256), 256, 0, s,
+             net->P, net->species, n, net->hs[0], plS, planes);
   NET_LAUNCHED(net);
   for (int t = 0; t < 2; ++t) {
     const Mix mA{planes * n, S, S + V, net->hs[t], 4 * t + 0, true, net->A[t], false};
@@ -1226,23 +1248,25 @@ int forward_pass(gbnet_t net, cudaStream_t s, const float* pos, const float* dpo
     if ((st = mix(net, s, mA, t > 0 ? &mB : nullptr))) return st;   // (h^v = 0 below the first layer)
     const MsgArgs a = msg_args<T>(net, t, pos, dpos);
     if (t == 0)
-      k_msg_fwd<T, true><<<blocks_for(n, kWarps), 32 * kWarps, 0, s>>>(a, net->A[t], nullptr, net->ms[t], net->mv[t]);
+      pdl_launch(k_msg_fwd<T, true>, blocks_for(n, kWarps), 32 * kWarps, 0, s, a,
+                 net->A[t], nullptr, net->ms[t], net->mv[t]);
     else
-      k_msg_fwd<T, false><<<blocks_for(n, kWarps), 32 * kWarps, 0, s>>>(a, net->A[t], net->B[t], net->ms[t],
-                                                                       net->mv[t]);
+      pdl_launch(k_msg_fwd<T, false>, blocks_for(n, kWarps), 32 * kWarps, 0, s, a,
+                 net->A[t], net->B[t], net->ms[t], net->mv[t]);
     NET_LAUNCHED(net);
     const Mix mU{planes * n, S + V, S + V, net->ms[t], 4 * t + 2, true, net->U[t], false};
     const Mix mY{planes * 3 * n, 2 * V, V, net->mv[t], 4 * t + 3, true, net->Y[t], false};
     if ((st = mix(net, s, mU, &mY))) return st;
-    k_update_fwd<T><<<blocks_for(size_t(n) * S, 256), 256, 0, s>>>(n, net->U[t], net->Y[t], net->hs[t], net->hv[t],
-                                                                  net->hs[t + 1], net->hv[t + 1], pl48, plV, plS, plV);
+    pdl_launch(k_update_fwd<T>, blocks_for(size_t(n) * S, 256), 256, 0, s, n,
+               net->U[t], net->Y[t], net->hs[t], net->hv[t], net->hs[t + 1], net->hv[t + 1], pl48, plV, plS, plV);
     NET_LAUNCHED(net);
   }
   if ((st = mix(net, s, Mix{planes * n, S, 2 * S, net->hs[2], 8, true, net->H, false}))) return st;
-  k_readout_fwd<T><<<blocks_for(n, kWarps), 32 * kWarps, 0, s>>>(n, net->P, net->H, net->hv[2], net->qt, net->ei,
-                                                                net->mu, pl64, plV, size_t(n));
+  pdl_launch(k_readout_fwd<T>, blocks_for(n, kWarps), 32 * kWarps, 0, s, n,
+             net->P, net->H, net->hv[2], net->qt, net->ei, net->mu, pl64, plV, size_t(n));
   NET_LAUNCHED(net);
-  k_frame_fwd<T><<<net->nframes, 256, 0, s>>>(net->frames_d, net->qt, net->ei, net->q, net->e_sr, size_t(n));
+  pdl_launch(k_frame_fwd<T>, net->nframes, 256, 0, s, net->frames_d, net->qt, net->ei, net->q, net->e_sr,
+             size_t(n));
   NET_LAUNCHED(net);
   (void)pl96;
   return PME_OK;
@@ -1310,9 +1334,9 @@ int param_grads(gbnet_t net, cudaStream_t s, float* grad, bool acc) {
   rj.job[rj.n - 1].width = 2 * S;   // two species rows of S channels
   red(P + L.readout, int(blocks_for(size_t(n), kWarps)), kReadoutW, -1);
   wj.species = net->species;
-  k_wgrad<planes><<<wblocks, kWgThreads, 0, s>>>(wj);
+  pdl_launch(k_wgrad<planes>, wblocks, kWgThreads, 0, s, wj);
   NET_LAUNCHED(net);
-  k_reduce<<<rblocks, 1024, 0, s>>>(rj, grad, acc ? 1 : 0);
+  pdl_launch(k_reduce, rblocks, 1024, 0, s, rj, grad, acc ? 1 : 0);
   NET_LAUNCHED(net);
   return PME_OK;
 }
@@ -1334,7 +1358,7 @@ int backward_pass(gbnet_t net, cudaStream_t s, const float* pos, const float* dp
     return st;
   if (n == 0) return PME_OK;
   if (gq) {
-    k_frame_mean<T><<<net->nframes, 256, 0, s>>>(net->frames_d, gq, net->gq_mean, size_t(n));
+    pdl_launch(k_frame_mean<T>, net->nframes, 256, 0, s, net->frames_d, gq, net->gq_mean, size_t(n));
     NET_LAUNCHED(net);
   }
   ReadoutBwdArgs ra;
@@ -1354,12 +1378,12 @@ int backward_pass(gbnet_t net, cudaStream_t s, const float* pos, const float* dp
   ra.plH = pl64;
   ra.plV = plV;
   const int nb_ion = int(blocks_for(n, kWarps));
-  k_readout_bwd<T><<<nb_ion, 32 * kWarps, 0, s>>>(ra);
+  pdl_launch(k_readout_bwd<T>, nb_ion, 32 * kWarps, 0, s, ra);
   NET_LAUNCHED(net);
   if ((st = mix(net, s, Mix{planes * n, 2 * S, S, net->gH, 8, false, net->ghs, false}))) return st;
   for (int t = 1; t >= 0; --t) {
-    k_update_bwd<T><<<blocks_for(size_t(n) * S, 256), 256, 0, s>>>(n, net->U[t], net->Y[t], net->ghs, net->ghv,
-                                                                   net->gU[t], net->gY[t], pl48, plV, plS, plV);
+    pdl_launch(k_update_bwd<T>, blocks_for(size_t(n) * S, 256), 256, 0, s, n,
+               net->U[t], net->Y[t], net->ghs, net->ghv, net->gU[t], net->gY[t], pl48, plV, plS, plV);
     NET_LAUNCHED(net);
     const Mix mU{planes * n, S + V, S + V, net->gU[t], 4 * t + 2, false, net->gms, false};
     const Mix mY{planes * 3 * n, V, 2 * V, net->gY[t], 4 * t + 3, false, net->gmv, false};
@@ -1367,8 +1391,8 @@ int backward_pass(gbnet_t net, cudaStream_t s, const float* pos, const float* dp
     const MsgArgs a = msg_args<T>(net, t, pos, dpos);
     float* wr = grad ? net->part + L.wr[t] : nullptr;
 #define GB_MSG_BWD(POS, GA, GRAD, FIRST)                                                                          \
-  k_msg_bwd<T, POS, GA, GRAD, FIRST><<<nb_ion, 32 * kWarps, 0, s>>>(a, net->A[t], net->B[t], net->gms, net->gmv, \
-                                                                    net->gA[t], net->gB[t], net->gpos, wr)
+  pdl_launch(k_msg_bwd<T, POS, GA, GRAD, FIRST>, nb_ion, 32 * kWarps, 0, s, a,                                  \
+             net->A[t], net->B[t], net->gms, net->gmv, net->gA[t], net->gB[t], net->gpos, wr)
     if constexpr (planes > 1) {   // the Dual pass: parameters only
       if (t == 0) GB_MSG_BWD(false, true, true, true);
       else GB_MSG_BWD(false, true, true, false);
@@ -1394,14 +1418,15 @@ int backward_pass(gbnet_t net, cudaStream_t s, const float* pos, const float* dp
 
 int build_neighbours(gbnet_t net, cudaStream_t s, const float* pos) {
   if (net->n == 0) return PME_OK;
-  k_nbr<<<blocks_for(net->n, kWarps), 32 * kWarps, 0, s>>>(net->frames_d, net->frame_of, pos, net->n, net->nbr_cnt,
-                                                          net->nbr_j, net->nbr_sh, net->flags);
+  pdl_launch(k_nbr, blocks_for(net->n, kWarps), 32 * kWarps, 0, s, net->frames_d, net->frame_of, pos, net->n,
+             net->nbr_cnt, net->nbr_j, net->nbr_sh, net->flags);
   NET_LAUNCHED(net);
   return PME_OK;
 }
 
 __global__ void k_gesr_from(int nframes, const double* __restrict__ g, float* out) {
-  const int f = blockIdx.x * blockDim.x + threadIdx.x;
+  const int bx = gbpme::pdl_begin_block();
+  const int f = bx * blockDim.x + threadIdx.x;
   if (f >= nframes) return;
   out[2 * f] = g ? float(g[f]) : 0.f;
   out[2 * f + 1] = 0.f;
@@ -1617,7 +1642,7 @@ int gbnet_set_params(gbnet_t net, void* stream, const float* params) {
       (st = cuda_ok(net, cudaMemsetAsync(net->av, 0, sizeof(float) * kParams, s), "memset")))
     return st;
   net->adam_step = 0;
-  k_cast_weights<<<dim3(8, kNumMix), 256, 0, s>>>(net->P, net->wbf, net->wbf_offs_d);
+  pdl_launch(k_cast_weights, dim3(8, kNumMix), 256, 0, s, net->P, net->wbf, net->wbf_offs_d);
   NET_LAUNCHED(net);
   return PME_OK;
 }
@@ -1658,7 +1683,7 @@ int gbnet_backward(gbnet_t net, void* stream, const float* g_q, const float* g_m
   if (!net) return PME_ERR_ARG;
   if (net->nframes == 0) return fail(net, PME_ERR_ARG, "no frames set");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  k_gesr_from<<<blocks_for(net->nframes, 128), 128, 0, s>>>(net->nframes, g_esr, net->gesr);
+  pdl_launch(k_gesr_from, blocks_for(net->nframes, 128), 128, 0, s, net->nframes, g_esr, net->gesr);
   NET_LAUNCHED(net);
   int st;
   if ((st = backward_pass<float>(net, s, net->pos_saved, nullptr, g_q, g_mu, net->gesr, g_params, false)))
@@ -1695,32 +1720,32 @@ static int loss_grad(gbnet_t net, pme_plan_t pme, cudaStream_t s, const float* p
     return fail(net, st, std::string("pme_batch_forward: ") + pme_last_error(pme));
   // 2. plain backward of the network with seeds (phi, dE/dmu = -field, 1): the net's part of dE/dr
   if (n) {
-    k_scale<<<blocks_for(3 * nn, 256), 256, 0, s>>>(3 * nn, net->field, -1.f, net->gmu);
+    pdl_launch(k_scale, blocks_for(3 * nn, 256), 256, 0, s, 3 * nn, net->field, -1.f, net->gmu);
     NET_LAUNCHED(net);
   }
-  k_seed_esr<<<blocks_for(F, 128), 128, 0, s>>>(F, net->cvec, net->gesr, 0);
+  pdl_launch(k_seed_esr, blocks_for(F, 128), 128, 0, s, F, net->cvec, net->gesr, 0);
   NET_LAUNCHED(net);
   if ((st = backward_pass<float>(net, s, net->pos_saved, nullptr, net->gq, net->gmu, net->gesr, nullptr, false)))
     return st;
   // 3. loss, energy cotangents c_b, position tangent r' = -w
-  k_loss<<<F, 256, 0, s>>>(net->frames_d, F, n, net->e_pme, net->e_sr, e_ref, net->f_pme, net->gpos, f_ref, lambda_e,
-                           lambda_f, net->cvec, force, net->dpos, net->wneg, net->lpart);
+  pdl_launch(k_loss, F, 256, 0, s, net->frames_d, F, n, net->e_pme, net->e_sr, e_ref, net->f_pme, net->gpos, f_ref,
+             lambda_e, lambda_f, net->cvec, force, net->dpos, net->wneg, net->lpart);
   NET_LAUNCHED(net);
-  k_loss_total<<<1, 256, 0, s>>>(net->lpart, F, loss);
+  pdl_launch(k_loss_total, 1, 256, 0, s, net->lpart, F, loss);
   NET_LAUNCHED(net);
   // 4. forward of the network carrying the tangent r'
   if ((st = forward_pass<Dual>(net, s, net->pos_saved, net->dpos))) return st;
   // 5. PME Hessian-vector product along (r', q', mu') plus c_b times the gradient: the tangents
   //    of (dE/dq, dE/dmu) land in the tangent planes of the cotangents
   if (n) {
-    k_scale<<<blocks_for(3 * nn, 256), 256, 0, s>>>(3 * nn, net->mu + 3 * nn, -1.f, net->mut_neg);
+    pdl_launch(k_scale, blocks_for(3 * nn, 256), 256, 0, s, 3 * nn, net->mu + 3 * nn, -1.f, net->mut_neg);
     NET_LAUNCHED(net);
   }
   if ((st = pme_batch_backward(pme, s, net->pos_saved, net->q_plain, net->mu_plain, net->cvec, net->wneg, net->q + nn,
                                net->mut_neg, net->gp_scratch, net->gq + nn, net->gmu + 3 * nn)))
     return fail(net, st, std::string("pme_batch_backward: ") + pme_last_error(pme));
   // 6. Dual backward of the network with energy seeds 1 + e c_b: its tangent plane is dL/dtheta
-  k_seed_esr<<<blocks_for(F, 128), 128, 0, s>>>(F, net->cvec, net->gesr, 1);
+  pdl_launch(k_seed_esr, blocks_for(F, 128), 128, 0, s, F, net->cvec, net->gesr, 1);
   NET_LAUNCHED(net);
   if ((st = backward_pass<Dual>(net, s, net->pos_saved, net->dpos, net->gq, net->gmu, net->gesr, grad, acc)))
     return st;
@@ -1742,10 +1767,10 @@ int gbnet_adam(gbnet_t net, void* stream, const float* grad, double lr, double b
   ++net->adam_step;
   const double c1 = 1.0 / (1.0 - std::pow(beta1, net->adam_step));
   const double c2 = 1.0 / (1.0 - std::pow(beta2, net->adam_step));
-  k_adam<<<blocks_for(kParams, 256), 256, 0, s>>>(kParams, net->P, net->am, net->av, grad, float(lr), float(beta1),
-                                                  float(beta2), float(eps), float(c1), float(c2));
+  pdl_launch(k_adam, blocks_for(kParams, 256), 256, 0, s, kParams,
+             net->P, net->am, net->av, grad, float(lr), float(beta1), float(beta2), float(eps), float(c1), float(c2));
   NET_LAUNCHED(net);
-  k_cast_weights<<<dim3(8, kNumMix), 256, 0, s>>>(net->P, net->wbf, net->wbf_offs_d);
+  pdl_launch(k_cast_weights, dim3(8, kNumMix), 256, 0, s, net->P, net->wbf, net->wbf_offs_d);
   NET_LAUNCHED(net);
   return PME_OK;
 }

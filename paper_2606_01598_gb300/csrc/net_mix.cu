@@ -228,24 +228,25 @@ __device__ __forceinline__ void mix_tile(const MixJob& J, int tile, int* err, un
 // 512 ions (31 products, now 19 launches) went from 1367 to 1220 us.
 template <int K1, int N1, int K2, int N2>
 __global__ void __launch_bounds__(kTile) k_mix(MixJob a, MixJob b, int blocks_a, int* err) {
+  const int bx = gbpme::pdl_begin_block();
   constexpr int kBytes1 = MixSmem<K1, N1>::bytes, kBytes2 = MixSmem<K2, N2>::bytes;
   __shared__ __align__(1024) unsigned char smem[kBytes1 > kBytes2 ? kBytes1 : kBytes2];
   __shared__ __align__(8) uint64_t mbar;
   __shared__ uint32_t tmem_slot;
   if constexpr (K2 > 0) {
-    if (int(blockIdx.x) >= blocks_a) {
-      mix_tile<K2, N2>(b, int(blockIdx.x) - blocks_a, err, smem, mbar, tmem_slot);
+    if (bx >= blocks_a) {
+      mix_tile<K2, N2>(b, bx - blocks_a, err, smem, mbar, tmem_slot);
       return;
     }
   }
-  mix_tile<K1, N1>(a, int(blockIdx.x), err, smem, mbar, tmem_slot);
+  mix_tile<K1, N1>(a, bx, err, smem, mbar, tmem_slot);
 }
 
 template <int K1, int N1, int K2, int N2>
 int launch_mix_kn(cudaStream_t s, const MixJob& a, const MixJob& b, int* err) {
   const int ba = a.M > 0 ? (a.M + kTile - 1) / kTile : 0, bb = K2 > 0 && b.M > 0 ? (b.M + kTile - 1) / kTile : 0;
   if (ba + bb == 0) return 0;
-  k_mix<K1, N1, K2, N2><<<ba + bb, kTile, 0, s>>>(a, b, ba, err);
+  gbpme::pdl_launch(k_mix<K1, N1, K2, N2>, ba + bb, kTile, 0, s, a, b, ba, err);
   gbpme::count_launch();
   return cudaGetLastError() == cudaSuccess ? 0 : PME_ERR_CUDA;
 }
