@@ -642,7 +642,7 @@ class _PMEGrad(torch.autograd.Function):
     @staticmethod
     def forward(ctx, plan, pos, q, mu, force, phi, field, gE):
         ctx.plan = plan
-        gE = gE.detach().to(torch.float64).contiguous()
+        gE = gE.detach().to(torch.float64, copy=True).contiguous()   # the caller may change its own
         ctx.save_for_backward(pos, q, mu, force, phi, field, gE)
         ctx.set_materialize_grads(False)
         return tuple(_scale_signed(plan, gE, force, phi, field))
@@ -653,11 +653,14 @@ class _PMEGrad(torch.autograd.Function):
         g = (None,) * 3
         if not (v_r is None and v_q is None and v_mu is None):
             g = ctx.plan.backward(pos.detach(), q.detach(), mu.detach(), None,
-                                  *_scale_signed(ctx.plan, gE, v_r, v_q, v_mu))
+                                  *_scale_signed(ctx.plan, gE, *(v if v is None else v.detach()
+                                                                 for v in (v_r, v_q, v_mu))))
         g_gE = None
         if ctx.needs_input_grad[7]:
-            parts = [(s * v.to(x.dtype) * x).sum() for s, v, x in ((-1.0, v_r, force), (1.0, v_q, phi),
-                                                                   (-1.0, v_mu, field)) if v is not None]
+            # through the function itself, so that under create_graph this inner product depends on
+            # pos, q and mu (torch.autograd.functional.jvp is a double backward of this kind)
+            dE = _PMEGrad.apply(ctx.plan, pos, q, mu, force, phi, field, torch.ones_like(gE))
+            parts = [(v.to(x.dtype) * x).sum() for v, x in zip((v_r, v_q, v_mu), dE) if v is not None]
             g_gE = sum(parts).to(gE.dtype).reshape(gE.shape) if parts else None
         return (None, *g, None, None, None, g_gE)
 
