@@ -636,6 +636,11 @@ int launch_t(pme_plan_t p, cudaStream_t s, int n, const float* mesh, const doubl
   a.qout = qout;
   a.finish = fin ? 1 : 0;
   a.fin = fin ? *fin : BackwardFinish{};
+  // Both meshes are read in 24-byte runs at random: with the transforms' L1 the tangent gather took
+  // 30 us at 32768 ions (1.8 waves) and 215 us at 262144, with its own 21 and 105 (forward +
+  // backward 259 -> 254 us and 1690 -> 1592 us, uneven batch of 256 frames 1101 -> 1064 us). The
+  // forward gather of 32768 ions (1.35 waves) lost 2.5 of its 9 us, that of 262144 ions gained 4.
+  constexpr int kSplitWaves = MODE == 1 ? 1 : 2;
   for (int gi = 0; gi < p->nogroups; ++gi) {
     const OrderGroup& G = p->ogroups[gi];
     a.t_lo = BATCH ? G.sorted_lo : 0;
@@ -647,7 +652,8 @@ int launch_t(pme_plan_t p, cudaStream_t s, int n, const float* mesh, const doubl
   case PP: {                                                                                    \
     const size_t per_block = size_t(kGatherThreads / 32) * gather_ions_per_warp<PP>();          \
     const int grid = int((nion + per_block - 1) / per_block);                                   \
-    pdl_launch(k_gather<PP, MODE, BATCH>, grid, kGatherThreads, 0, s, a);                               \
+    const int split = own_split<&k_gather<PP, MODE, BATCH>>(grid, kGatherThreads, kSplitWaves); \
+    launch_with(true, split, k_gather<PP, MODE, BATCH>, grid, kGatherThreads, 0, s, a);         \
     break;                                                                                      \
   }
     switch (G.order) {
