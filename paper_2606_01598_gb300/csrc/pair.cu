@@ -774,6 +774,14 @@ __global__ void __launch_bounds__(kPairThreads) k_pair_listed(PairArgs a, int n)
   if (idx < W) a.out[size_t(a.pr.idx[i].w) * W + idx] = idx < NA ? v[0] : 0.f;
 }
 
+// The list kernels read their partners' records at random beside the mesh passes, whose tiles leave
+// little L1; from eight waves on they take their own split (forward + backward of 262144 ions, 21
+// and 31 waves: 1592 -> 1559 us; of 32768 ions, 2.7 and 3.8 waves: 253.9 -> 254.6 us).
+template <auto K, typename... Args>
+void launch_l1(int grid, cudaStream_t s, Args... args) {
+  launch_with(false, own_split<K>(grid, kPairThreads, 8), K, grid, kPairThreads, 0, s, args...);
+}
+
 template <bool TAN, bool BATCH>
 void launch_k(bool ortho, int grid, cudaStream_t s, const PairArgs& a) {
   if (ortho) k_pair<TAN, BATCH, true><<<grid, kPairThreads, 0, s>>>(a);
@@ -862,11 +870,11 @@ int launch_pair_build(pme_plan_t p, cudaStream_t s, int n, int* overflow) {
   if (grid == 0) return PME_OK;
   const bool ortho = plan_ortho(p);
   if (p->batch) {
-    if (ortho) k_pair_build<true, true><<<grid, kPairThreads, 0, s>>>(a, split, overflow);
-    else k_pair_build<true, false><<<grid, kPairThreads, 0, s>>>(a, split, overflow);
+    if (ortho) launch_l1<&k_pair_build<true, true>>(grid, s, a, split, overflow);
+    else launch_l1<&k_pair_build<true, false>>(grid, s, a, split, overflow);
   } else {
-    if (ortho) k_pair_build<false, true><<<grid, kPairThreads, 0, s>>>(a, split, overflow);
-    else k_pair_build<false, false><<<grid, kPairThreads, 0, s>>>(a, split, overflow);
+    if (ortho) launch_l1<&k_pair_build<false, true>>(grid, s, a, split, overflow);
+    else launch_l1<&k_pair_build<false, false>>(grid, s, a, split, overflow);
   }
   count_launch();
   return check_launch(p, "k_pair_build");
@@ -881,13 +889,13 @@ int launch_pair_listed(pme_plan_t p, cudaStream_t s, int n, bool tangent, const 
   const int grid = (n + kPairWarps - 1) / kPairWarps;
   const bool vir = virial && !tangent;
   if (p->batch) {
-    if (tangent) k_pair_listed<true, true><<<grid, kPairThreads, 0, s>>>(a, n);
-    else if (vir) k_pair_listed<false, true, true><<<grid, kPairThreads, 0, s>>>(a, n);
-    else k_pair_listed<false, true><<<grid, kPairThreads, 0, s>>>(a, n);
+    if (tangent) launch_l1<&k_pair_listed<true, true>>(grid, s, a, n);
+    else if (vir) launch_l1<&k_pair_listed<false, true, true>>(grid, s, a, n);
+    else launch_l1<&k_pair_listed<false, true>>(grid, s, a, n);
   } else {
-    if (tangent) k_pair_listed<true, false><<<grid, kPairThreads, 0, s>>>(a, n);
-    else if (vir) k_pair_listed<false, false, true><<<grid, kPairThreads, 0, s>>>(a, n);
-    else k_pair_listed<false, false><<<grid, kPairThreads, 0, s>>>(a, n);
+    if (tangent) launch_l1<&k_pair_listed<true, false>>(grid, s, a, n);
+    else if (vir) launch_l1<&k_pair_listed<false, false, true>>(grid, s, a, n);
+    else launch_l1<&k_pair_listed<false, false>>(grid, s, a, n);
   }
   count_launch();
   return check_launch(p, "k_pair_listed");
