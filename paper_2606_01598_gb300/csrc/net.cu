@@ -1230,6 +1230,14 @@ MsgArgs msg_args(gbnet_t net, int layer, const float* pos, const float* dpos) {
   return a;
 }
 
+// The message kernels, which read their neighbours' rows at random behind the products' tiles: from
+// two waves on with their own L1 split (loss gradient over 32 frames of 512 ions, 2048 blocks of
+// which 304 to 608 are resident: 1115 -> 1100 us).
+template <auto K, typename... Args>
+static void launch_l1(unsigned grid, int threads, cudaStream_t s, Args... args) {
+  gbpme::launch_with(true, gbpme::own_split<K>(grid, threads, 2), K, grid, threads, 0, s, args...);
+}
+
 // forward pass; dpos is the position tangent (Dual passes only)
 template <typename T>
 int forward_pass(gbnet_t net, cudaStream_t s, const float* pos, const float* dpos) {
@@ -1248,11 +1256,11 @@ int forward_pass(gbnet_t net, cudaStream_t s, const float* pos, const float* dpo
     if ((st = mix(net, s, mA, t > 0 ? &mB : nullptr))) return st;   // (h^v = 0 below the first layer)
     const MsgArgs a = msg_args<T>(net, t, pos, dpos);
     if (t == 0)
-      pdl_launch(k_msg_fwd<T, true>, blocks_for(n, kWarps), 32 * kWarps, 0, s, a,
-                 net->A[t], nullptr, net->ms[t], net->mv[t]);
+      launch_l1<&k_msg_fwd<T, true>>(blocks_for(n, kWarps), 32 * kWarps, s, a, net->A[t], nullptr, net->ms[t],
+                                     net->mv[t]);
     else
-      pdl_launch(k_msg_fwd<T, false>, blocks_for(n, kWarps), 32 * kWarps, 0, s, a,
-                 net->A[t], net->B[t], net->ms[t], net->mv[t]);
+      launch_l1<&k_msg_fwd<T, false>>(blocks_for(n, kWarps), 32 * kWarps, s, a, net->A[t], net->B[t], net->ms[t],
+                                      net->mv[t]);
     NET_LAUNCHED(net);
     const Mix mU{planes * n, S + V, S + V, net->ms[t], 4 * t + 2, true, net->U[t], false};
     const Mix mY{planes * 3 * n, 2 * V, V, net->mv[t], 4 * t + 3, true, net->Y[t], false};
@@ -1391,7 +1399,7 @@ int backward_pass(gbnet_t net, cudaStream_t s, const float* pos, const float* dp
     const MsgArgs a = msg_args<T>(net, t, pos, dpos);
     float* wr = grad ? net->part + L.wr[t] : nullptr;
 #define GB_MSG_BWD(POS, GA, GRAD, FIRST)                                                                          \
-  pdl_launch(k_msg_bwd<T, POS, GA, GRAD, FIRST>, nb_ion, 32 * kWarps, 0, s, a,                                  \
+  launch_l1<&k_msg_bwd<T, POS, GA, GRAD, FIRST>>(nb_ion, 32 * kWarps, s, a,                                     \
              net->A[t], net->B[t], net->gms, net->gmv, net->gA[t], net->gB[t], net->gpos, wr)
     if constexpr (planes > 1) {   // the Dual pass: parameters only
       if (t == 0) GB_MSG_BWD(false, true, true, true);
