@@ -38,6 +38,18 @@ __device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
   return make_float2(__fmaf_rn(a.x, b.x, -(a.y * b.y)), __fmaf_rn(a.x, b.y, a.y * b.x));
 }
+// The odd radices' sums in packed instructions (f32x2: both parts in one issue slot, each rounded
+// as alone), and a + i s b crosswise as scalar multiply-adds (a pair with its halves exchanged would
+// have to be moved first). The two-step kernels issue more than they wait: forward + backward of
+// the uneven batch of 256 frames 1069.5 -> 1064.2 us, forward with virial on 80x81x90 94.0 -> 93.4 us.
+// Power-of-two DFTs stay scalar: packed too, 128^3 lost what the batch gained (258 -> 260.5 us).
+__device__ __forceinline__ float2 padd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 psub(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+__device__ __forceinline__ float2 pfma(float s, float2 a, float2 b) { return __ffma2_rn(make_float2(s, s), a, b); }
+__device__ __forceinline__ float2 pmul(float s, float2 a) { return __fmul2_rn(make_float2(s, s), a); }
+__device__ __forceinline__ float2 add_is(float2 a, float s, float2 b) {
+  return make_float2(__fmaf_rn(-s, b.y, a.x), __fmaf_rn(s, b.x, a.y));
+}
 // times -i (forward transform) or +i (inverse)
 template <bool INV>
 __device__ __forceinline__ float2 rot(float2 a) {
@@ -90,30 +102,26 @@ __device__ __forceinline__ void dft(float2* v) {
     v[7] = csub(e3, o3);
   } else if constexpr (R == 3) {
     const float c = -0.5f, s = 0.86602540378443865f;   // cos, sin of 2 pi / 3
-    const float2 a = v[0], sm = cadd(v[1], v[2]), d = csub(v[1], v[2]);
-    const float2 m = make_float2(__fmaf_rn(c, sm.x, a.x), __fmaf_rn(c, sm.y, a.y));
-    const float2 isd = make_float2(-s * d.y, s * d.x);   // i s d
-    v[0] = cadd(a, sm);
-    v[1] = INV ? cadd(m, isd) : csub(m, isd);
-    v[2] = INV ? csub(m, isd) : cadd(m, isd);
+    const float2 a = v[0], sm = padd(v[1], v[2]), d = psub(v[1], v[2]);
+    const float2 m = pfma(c, sm, a);
+    v[0] = padd(a, sm);
+    v[1] = add_is(m, INV ? s : -s, d);
+    v[2] = add_is(m, INV ? -s : s, d);
   } else if constexpr (R == 5) {
     const float c1 = 0.30901699437494742f, c2 = -0.80901699437494742f;   // cos 2pi/5, cos 4pi/5
     const float s1 = 0.95105651629515357f, s2 = 0.58778525229247313f;    // sin 2pi/5, sin 4pi/5
     const float2 a = v[0];
-    const float2 s14 = cadd(v[1], v[4]), d14 = csub(v[1], v[4]);
-    const float2 s23 = cadd(v[2], v[3]), d23 = csub(v[2], v[3]);
-    const float2 m1 = make_float2(__fmaf_rn(c2, s23.x, __fmaf_rn(c1, s14.x, a.x)),
-                                  __fmaf_rn(c2, s23.y, __fmaf_rn(c1, s14.y, a.y)));
-    const float2 m2 = make_float2(__fmaf_rn(c1, s23.x, __fmaf_rn(c2, s14.x, a.x)),
-                                  __fmaf_rn(c1, s23.y, __fmaf_rn(c2, s14.y, a.y)));
-    const float2 n1 = make_float2(__fmaf_rn(s1, d14.x, s2 * d23.x), __fmaf_rn(s1, d14.y, s2 * d23.y));
-    const float2 n2 = make_float2(__fmaf_rn(s2, d14.x, -(s1 * d23.x)), __fmaf_rn(s2, d14.y, -(s1 * d23.y)));
-    const float2 in1 = make_float2(-n1.y, n1.x), in2 = make_float2(-n2.y, n2.x);   // i n
-    v[0] = cadd(a, cadd(s14, s23));
-    v[1] = INV ? cadd(m1, in1) : csub(m1, in1);
-    v[4] = INV ? csub(m1, in1) : cadd(m1, in1);
-    v[2] = INV ? cadd(m2, in2) : csub(m2, in2);
-    v[3] = INV ? csub(m2, in2) : cadd(m2, in2);
+    const float2 s14 = padd(v[1], v[4]), d14 = psub(v[1], v[4]);
+    const float2 s23 = padd(v[2], v[3]), d23 = psub(v[2], v[3]);
+    const float2 m1 = pfma(c2, s23, pfma(c1, s14, a));
+    const float2 m2 = pfma(c1, s23, pfma(c2, s14, a));
+    const float2 n1 = pfma(s1, d14, pmul(s2, d23));
+    const float2 n2 = pfma(s2, d14, pmul(-s1, d23));
+    v[0] = padd(a, padd(s14, s23));
+    v[1] = add_is(m1, INV ? 1.f : -1.f, n1);
+    v[4] = add_is(m1, INV ? -1.f : 1.f, n1);
+    v[2] = add_is(m2, INV ? 1.f : -1.f, n2);
+    v[3] = add_is(m2, INV ? -1.f : 1.f, n2);
   } else if constexpr (R == 6) {
     dft_coprime<2, 3, INV>(v);
   } else if constexpr (R == 9) {
