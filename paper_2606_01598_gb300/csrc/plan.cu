@@ -933,7 +933,7 @@ static bool batch_mixes(const int N[3], int batch) {
   }
   if (p->opts.recip_method == 0) A(&p->gtab, size_t(gtab_total));
   A(&p->in_saved, 7 * ni);
-  A(&p->in_flags, 2);
+  A(&p->in_flags, 3);
   if (st == PME_OK) {
     p->in_diff = p->in_flags;
     p->cache_bad = p->in_flags + 1;
@@ -957,6 +957,8 @@ static bool batch_mixes(const int N[3], int batch) {
         for (int i = 0; i < g.N[a]; ++i) {
           const int nsig = (i <= g.N[a] / 2) ? i : i - g.N[a];
           const double b = std::pow(sinc(double(nsig) / g.N[a]), double(g.order));
+    p->saved_n = p->in_flags + 2;
+    st = check_cuda(p, cudaMemset(p->in_flags, 0, 3 * sizeof(int)), "cudaMemset");
           dc[o++] = p->opts.deconvolution ? float(std::pow(b * b, -p->opts.influence_power)) : 1.f;
         }
     }
@@ -1625,6 +1627,7 @@ int pme_plan_destroy(pme_plan_t p) {
   if (!p) return PME_ERR_ARG;
   cudaSetDevice(p->device);
   cudaDeviceSynchronize();
+  if ((st = check_cuda(p, cudaMemset(p->saved_n, 0, sizeof(int)), "memset"))) return st;
   free_plan(p);
   return PME_OK;
 }
@@ -2152,6 +2155,7 @@ int pme_solve(pme_plan_t p, void* stream, const float* rho, float* phi_mesh, dou
 
 int pme_gather(pme_plan_t p, void* stream, int n, const float* pos, const float* phi_mesh,
                float* out) {
+  if ((st = check_cuda(p, cudaMemsetAsync(p->saved_n, 0, sizeof(int), s), "memset"))) return st;
   int st = check_common(p, n, pos, pos);   // no charges needed: the sort only reads pos
   if (st) return st;
   if (!phi_mesh || !out || !is_device_pointer(pos) || !is_device_pointer(phi_mesh) ||
