@@ -103,10 +103,8 @@ typedef struct {
                               mesh takes the power-of-two kernels, for single frames whose
                               axes are 64, 128 or 256 points (line by line where the planes do
                               not fit in shared memory), for single frames whose
-                              every axis is a product of two of 1-6, 8, 9, 10, 12, 15, 16 and
-                              whose planes, where they take more than half of an SM's shared
-                              memory, are no more than the SMs (or two axes are multiples of 45
-                              or 75), and for batched plans whose meshes have no axis above 64 points (one
+                              every axis is a product of two of 1-6, 8, 9, 10, 12, 15, 16, and
+                              for batched plans whose meshes have no axis above 64 points (one
                               launch per pass for all frames), cuFFT otherwise.
                               1: always cuFFT. 2: always the library's own
                               (PME_ERR_UNSUPPORTED where they do not apply). 3: the library's
@@ -169,10 +167,7 @@ int pme_sync_status(pme_plan_t plan, void* stream);
  * with each launch, so any buffers qualify (with recip_method 1 the pointers must be the same
  * too). A different n runs directly, as do calls made while the stage timers are on or while
  * `stream` is being captured by the caller (the pass is then captured into the caller's graph);
- * pme_plan_set_box drops the graphs, so a plan's first call, and the first after a change of the
- * box or of n, cost the host 15 to 30 launches.
- * A backward reuses what a forward on the same inputs left in the plan only while that is in place on
- * the device, so captured passes and live calls of one plan mix in any order. */
+ * pme_plan_set_box drops the graphs. */
 
 /* Forward: energy and derivatives of Eq. (1).
  *   energy     [1] float64: E                     (may be NULL)
@@ -357,8 +352,7 @@ int pme_bounds_flags(void);
 int pme_bounds_checking(void);
 
 /* Number of the library's own kernels launched since the library was loaded (cuFFT's
- * kernels are not counted, nor is the node that hands a recorded pass its pointers: a replay
- * counts what the same call launches directly). */
+ * kernels are not counted). */
 long long pme_launch_count(void);
 
 /* ---- stage timers ------------------------------------------------------------------------

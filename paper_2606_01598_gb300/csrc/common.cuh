@@ -36,9 +36,6 @@ int device_sm_count();
 // their memory is visible (griddepcontrol.wait), then lets the next grid be scheduled
 // (griddepcontrol.launch_dependents), so consecutive kernels of a pass overlap only in their
 // launch and scheduling, never in their memory accesses. Outside such a launch both are no-ops.
-// A kernel so launched is resident while the grid before it writes, so non-coherent loads (__ldg,
-// const __restrict__ parameters), defined only on memory that nothing writes while their kernel
-// runs, are for tables that no pass writes; what passes hand on is read with plain loads.
 __device__ __forceinline__ void pdl_begin() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -309,10 +306,6 @@ struct FFTGroup {
   cufftHandle r2c, c2r, r2c2, c2r2;
 };
 
-  long long mesh_stride, spec_stride;   // from one member's mesh (half spectrum) to the next
-  // transforms of the members' meshes and, r2c2 and c2r2, of their tangent meshes too; with apart
-  // set, r2c and c2r transform one mesh each and the other two do not exist (see batch_mixes)
-  bool apart;
 }  // namespace gbpme
 
 struct pme_plan_s {
@@ -374,17 +367,12 @@ struct pme_plan_s {
   int plist_cap = 0;
   // inputs of the last forward, kept with its sorted order and records for the backward
   float* in_saved = nullptr;   // [7 max_ions]: positions, then q at 3 max_ions, mu at 4 max_ions
-  int* in_flags = nullptr;     // [3]: in_diff, cache_bad (see launch_input_check), saved_n
+  int* in_flags = nullptr;     // [2]: in_diff, cache_bad (see launch_input_check)
   int* in_diff = nullptr;
   int* cache_bad = nullptr;
   bool counts_clean = false;   // the sort's count arrays are zero (each scatter re-zeroes them)
   int fwd_n = -1;              // ions of that forward (-1: nothing saved / no longer valid)
   // virial partial sums
-  // Ions of the forward whose inputs are in in_saved while its order, records, Phi and lists are in
-  // place, else 0: kept by the passes themselves as they run on the device (fwd_n says what was
-  // enqueued last, which a caller's own graph of captured passes does not follow). A saving forward
-  // sets it; every other pass that sorts or writes rho clears it.
-  int* saved_n = nullptr;
   double* vpart = nullptr;     // [6 * influence blocks] k-space sums S_ab
   float* pvir = nullptr;       // [max_ions][9] per-ion pair virial
   double* vitem = nullptr;     // [9 * items] per-item sums

@@ -191,11 +191,11 @@ __global__ void __launch_bounds__(kGatherThreads) k_gather(GatherArgs a) {
       for (int jy = 0; jy < P; ++jy) {
         const int off = xo + yo[jy];
         const bool in_mesh = index_ok((long long)off, Mtot);
-        const float v = in_mesh ? phi_mesh[off] : 0.f;
+        const float v = in_mesh ? __ldg(phi_mesh + off) : 0.f;
 #pragma unroll
         for (int b = 0; b <= DM; ++b) r[b] += v * wy[jy][b];
         if (TAN) {
-          const float dv = in_mesh ? dphi_mesh[off] : 0.f;
+          const float dv = in_mesh ? __ldg(dphi_mesh + off) : 0.f;
 #pragma unroll
           for (int b = 0; b < 3; ++b) rt[b] += dv * wy[jy][b];
         }
@@ -292,8 +292,7 @@ __global__ void __launch_bounds__(kGatherThreads) k_gather(GatherArgs a) {
     // The gradients are linear in the moments, so each lane contracts its own z-plane's with the
     // ion's vectors and only the seven results are reduced over the lanes.
     // (Reduced first, the thirty moments took three shuffles each and the contraction ran in one
-    // lane of P: forward + backward of 262144 ions 1592 -> 1575 us, of 32768 ions 253.9 -> 252.9 us,
-    // before the list kernels had their own L1 split.)
+    // lane of P: forward + backward of 262144 ions 1592 -> 1575 us, of 32768 ions 253.9 -> 252.9 us.)
     const float gE = a.g_energy ? float(a.g_energy[frame]) : 0.f;
     const float4 dm = a.mr.dm[ion];   // m = D^T mu
     const float4 tq = a.mr.tq[ion];   // dq, dd = D^T (dmu + q dr)
@@ -454,8 +453,8 @@ __global__ void __launch_bounds__(kGatherThreads) k_gather_qdual(GatherArgs a) {
         if (y >= Ny) y -= Ny;
         const size_t off = (size_t(x) * Ny + y) * Nz + z;
         const bool in_mesh = index_ok((long long)off, Mtot);
-        const float v = in_mesh ? phi_mesh[off] : 0.f;
-        const float dv = in_mesh ? dphi_mesh[off] : 0.f;
+        const float v = in_mesh ? __ldg(phi_mesh + off) : 0.f;
+        const float dv = in_mesh ? __ldg(dphi_mesh + off) : 0.f;
 #pragma unroll
         for (int b = 0; b < 5; ++b) r[b] += v * wy[b][jy];
 #pragma unroll

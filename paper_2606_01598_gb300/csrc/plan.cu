@@ -9,14 +9,11 @@
 // per spline order; FFT: one batched cuFFT call per distinct mesh shape).
 #include <nvtx3/nvToolsExt.h>
 #include <algorithm>
-#include <array>
 #include <atomic>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
 #include <initializer_list>
-#include <map>
-#include <mutex>
 #include <new>
 #include <numeric>
 #include <vector>
@@ -388,7 +385,7 @@ static void free_plan(pme_plan_t p) {
                   p->plist, p->plist_cnt, p->in_saved, p->in_flags, p->vpart,
                   p->pvir, p->vitem, p->gtab, p->sb.t_bidx, p->sb.t_bfq,
                   p->sb.t_bdm, p->sb.t_cidx, p->sb.t_cfq, p->sb.t_cmu, p->conv_tw,
-                  p->conv_planes1, p->quad_out, p->qb_mesh, p->qb_pair, p->io_d};
+                  p->conv_planes1, p->quad_out, p->io_d};
   for (void* b : bufs)
     if (b) cudaFree(b);
   for (int g = 0; g < p->nfgroups; ++g) {
@@ -432,7 +429,7 @@ static int dalloc(pme_plan_t p, T** ptr, size_t count) {
 // them 16 bytes at a time).
 static size_t scan_entries(int n) { return (size_t(n) + 1 + 3) & ~size_t(3); }
 
-// The cell counts start zero (each scatter re-zeroes them).
+// The cell counts start zero (each scan re-zeroes them).
 static int alloc_cells(pme_plan_t p) {
   int st;
   if ((st = dalloc(p, &p->sb.count_c, scan_entries(p->total_cells)))) return st;
@@ -484,40 +481,19 @@ struct FrameInput {
 
 // Whether the options ask for the hand-written transforms: fft 2 and 3 always; fft 0
 // (automatic) whenever every frame takes the power-of-two kernels (axes of 64 or 128 points),
-// for single frames whose every axis splits into two register steps (two_step_factors) unless their
-// planes go over the device in a second wave (planes_overflow), and for batched plans of small meshes (no axis above kConvAutoMaxAxis), whose frames then share
+// for single frames whose every axis splits into two register steps (two_step_factors), and
+// for batched plans of small meshes (no axis above kConvAutoMaxAxis), whose frames then share
 // one launch per pass instead of a cuFFT plan per mesh shape. The axis lengths and
 // shared-memory sizes are checked by the caller (a mesh whose planes do not fit goes to the line
 // kernels where its axes are 64, 128 or 256 points, to cuFFT otherwise).
 // Measured on GB300, solve of one frame, three plans in turn (us), two-step kernels against
 // cuFFT's six plus the influence pass: 32^3 20.5 / 25.9, 48^3 21.2 / 26.0, 80x81x90 28.9 / 31.5,
-// 96^3 30.8 / 36.9, 100^3 36.2 / 33.6, 144^3 51.0 / 56.7, 150^3 60.7 / 90.1. (100^3 is taken: the
-// forward beside its pair term costs the same, 94.5 / 95.1, and forward + backward less, 193.7 /
-// 201.8, since a backward on the forward's inputs transforms one mesh here and two there.) The six
-// lengths without two such factors stay with cuFFT (125^3: 71.9 on the Stockham kernels, 52.0 on cuFFT).
+// 96^3 30.8 / 36.9, 100^3 36.2 / 33.6, 144^3 51.0 / 56.7, 150^3 60.7 / 90.1, 160^3 92.8 / 85.4.
+// The two sizes where cuFFT's solve is a little faster are taken too: a backward on the
+// forward's inputs transforms one mesh here and two there, and the passes are three launches
+// instead of seven. The six lengths without two such factors stay with cuFFT (125^3: 71.9 on
+// the Stockham kernels, 52.0 on cuFFT).
 constexpr int kConvAutoMaxAxis = 64;
-
-static int smem_attribute(cudaDeviceAttr which) {
-  int dev = 0, bytes = 0;
-  if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&bytes, which, dev) == cudaSuccess) return bytes;
-  cudaGetLastError();
-  return 0;
-}
-
-// Planes that take more than half of an SM's shared memory run one to an SM, and where there are more
-// of them than SMs the rest go in a second wave that leaves most of the device idle. Forward with
-// the pair term, then forward + backward (us), two-step kernels / cuFFT: 160x120x120 199 / 184 and
-// 394 / 398, 160x128x128 220 / 203 and 433 / 429, 160^3 255 / 238 and 485 / 520, 192x128x128 233 /
-// 218 and 456 / 462, 256x128x128 234 / 220 and 461 / 473; so cuFFT takes these. It is slow itself
-// where two axes or more are multiples of 45 or 75: 160x135x135 234 / 242 and 459 / 538, 160x150x150
-// 244 / 241 and 471 / 532. One wave: 150x128x128 190 / 191 and 385 / 411, 160x108x108 156 / 157 and
-// 313 / 337.
-static bool planes_overflow(const int N[3]) {
-  int slow = 0;
-  for (int a = 0; a < 3; ++a) slow += N[a] % 45 == 0 || N[a] % 75 == 0;
-  return slow < 2 && N[0] > device_sm_count() &&
-         2 * two_plane_smem(N, 1) > size_t(smem_attribute(cudaDevAttrMaxSharedMemoryPerMultiprocessor));
-}
 
 static bool conv_wanted(const pme_plan_s* p, bool single, const std::vector<FrameInput>& fin) {
   if (p->opts.fft == 2 || p->opts.fft == 3) return true;
@@ -529,110 +505,12 @@ static bool conv_wanted(const pme_plan_s* p, bool single, const std::vector<Fram
     int P, Q;
     for (int a = 0; a < 3; ++a)
       if (!two_step_factors(fin[0].mesh[a], &P, &Q)) return false;
-    // planes too large for a block: the line kernels or cuFFT
-    if (two_plane_smem(fin[0].mesh, 1) + 1024 > size_t(smem_attribute(cudaDevAttrMaxSharedMemoryPerBlockOptin)))
-      return line_axes_ok(fin[0].mesh);
-    return !planes_overflow(fin[0].mesh);
+    return true;
   }
   for (const FrameInput& f : fin)
     for (int a = 0; a < 3; ++a)
       if (f.mesh[a] > kConvAutoMaxAxis) return false;
   return true;
-}
-
-// ---- cuFFT batches -------------------------------------------------------------------------
-
-// cuFFT carries two real transforms of a batch through one complex transform for some lengths of the
-// last axis (CUDA 13.0: 39, 51, 57, 65, 69, 75, 85, 87, 91, 93, 95 among those up to 100), and each
-// then takes on the other's rounding errors. Beside rho, the tangent density of a force-matching
-// step, whose cotangents are of order 1 / n, so kept two to four digits: gradients of a mean-square
-// force loss off by 3e-4 at 905 ions on 37x37x39 and by 2e-2 at 14736 on 95x93x95, 1e-6 with the
-// transforms apart. batch_mixes finds the shapes by trial: members of order one and of order 2^-20 in
-// turn, the small ones of a batch against the same transformed alone.
-__global__ void k_trial_fill(float* v, long long M, int batch) {
-  const long long n = M * batch;
-  for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
-    unsigned h = unsigned(t) * 2654435761u;
-    h ^= h >> 15;
-    h *= 2246822519u;
-    h ^= h >> 13;
-    v[t] = (float(h >> 8) * 0x1p-24f - 0.5f) * ((t / M) & 1 ? 0x1p-20f : 1.f);
-  }
-}
-
-// out[0] = max(out[0], max |x - y|), out[1] = max(out[1], max |y|)  (bit patterns of floats >= 0)
-__global__ void k_trial_compare(const float* x, const float* y, long long n, int* out) {
-  float d = 0.f, m = 0.f;
-  for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
-    d = fmaxf(d, fabsf(x[t] - y[t]));
-    m = fmaxf(m, fabsf(y[t]));
-  }
-  atomicMax(out, __float_as_int(d));
-  atomicMax(out + 1, __float_as_int(m));
-}
-
-// Whether transforms of this shape mix the members of a batch; also true when the trial could not be
-// run. One trial per shape, device and process (the answer is the library's, the same for every plan).
-static bool batch_mixes(const int N[3], int batch) {
-  static std::mutex mu;
-  static std::map<std::array<int, 5>, bool> known;
-  int dev = 0;
-  cudaGetDevice(&dev);
-  const std::array<int, 5> key = {N[0], N[1], N[2], batch, dev};
-  std::lock_guard<std::mutex> lock(mu);
-  const auto it = known.find(key);
-  if (it != known.end()) return it->second;
-  const long long M = (long long)N[0] * N[1] * N[2], Mh = (long long)N[0] * N[1] * (N[2] / 2 + 1);
-  int dims[3] = {N[0], N[1], N[2]};
-  float *v = nullptr, *one = nullptr;
-  cufftComplex *sa = nullptr, *sb = nullptr;
-  int* res = nullptr;
-  cufftHandle h[4];
-  int made = 0;
-  const cufftType ty[4] = {CUFFT_R2C, CUFFT_C2R, CUFFT_R2C, CUFFT_C2R};
-  bool ok = cudaMalloc(&v, sizeof(float) * M * batch) == cudaSuccess && cudaMalloc(&one, sizeof(float) * M) == cudaSuccess &&
-            cudaMalloc(&sa, sizeof(cufftComplex) * Mh * batch) == cudaSuccess &&
-            cudaMalloc(&sb, sizeof(cufftComplex) * Mh * batch) == cudaSuccess &&
-            cudaMalloc(&res, 4 * sizeof(int)) == cudaSuccess && cudaMemset(res, 0, 4 * sizeof(int)) == cudaSuccess;
-  for (; made < 4 && ok; made += ok)
-    ok = cufftPlanMany(&h[made], 3, dims, nullptr, 1, 0, nullptr, 1, 0, ty[made], made < 2 ? 1 : batch) == CUFFT_SUCCESS;
-  const int grid = 4 * device_sm_count();
-  int r[4] = {0, 0, 0, 0};
-  if (ok) {
-    k_trial_fill<<<grid, 256>>>(v, M, batch);
-    count_launch();
-    // every member alone (through a buffer of its own: an odd M leaves the batch's members unaligned)
-    for (int k = 0; k < batch && ok; ++k)
-      ok = cudaMemcpyAsync(one, v + k * M, sizeof(float) * M, cudaMemcpyDeviceToDevice) == cudaSuccess &&
-           cufftExecR2C(h[0], one, sb + k * Mh) == CUFFT_SUCCESS;
-    ok = ok && cufftExecR2C(h[2], v, sa) == CUFFT_SUCCESS;
-    for (int k = 1; k < batch && ok; k += 2) {
-      k_trial_compare<<<grid, 256>>>(reinterpret_cast<float*>(sa + k * Mh), reinterpret_cast<float*>(sb + k * Mh), 2 * Mh,
-                                     res);
-      count_launch();
-    }
-    ok = ok && cudaMemcpyAsync(sa, sb, sizeof(cufftComplex) * Mh * batch, cudaMemcpyDeviceToDevice) == cudaSuccess &&
-         cufftExecC2R(h[3], sa, v) == CUFFT_SUCCESS;
-    for (int k = 1; k < batch && ok; k += 2) {
-      ok = cufftExecC2R(h[1], sb + k * Mh, one) == CUFFT_SUCCESS;
-      if (!ok) break;
-      k_trial_compare<<<grid, 256>>>(v + k * M, one, M, res + 2);
-      count_launch();
-    }
-    ok = ok && cudaGetLastError() == cudaSuccess &&
-         cudaMemcpy(r, res, 4 * sizeof(int), cudaMemcpyDeviceToHost) == cudaSuccess;
-  }
-  for (int k = 0; k < made; ++k) cufftDestroy(h[k]);
-  for (void* b : {(void*)v, (void*)one, (void*)sa, (void*)sb, (void*)res})
-    if (b) cudaFree(b);
-  cudaGetLastError();
-  if (!ok) return true;
-  float f[4];
-  std::memcpy(f, r, sizeof(f));
-  // float32 rounding between two algorithms is some 1e-6 of the largest value; mixing, 0.1
-  const bool mixes = !(f[0] <= 1e-4f * f[1] && f[2] <= 1e-4f * f[3]);
-  known[key] = mixes;
-  return mixes;
 }
 
 // Build a plan over the given frames. single: one frame whose ion count is chosen per call.
@@ -660,8 +538,7 @@ static int build_plan(pme_plan_s* p, const std::vector<FrameInput>& fin, double 
   // every axis of every frame is 2,3,5-smooth and short enough, and a plane (pass A / C) and
   // a pass-B tile fit in shared memory
   {
-    const bool wanted = conv_wanted(p, single, fin);
-    bool conv = wanted;
+    bool conv = conv_wanted(p, single, fin);
     size_t cap = 0, smem_plane = 0, smem_x = 0, biggest = 0;
     for (int f = 0; f < F && conv; ++f) {
       for (int a = 0; a < 3; ++a) conv = conv && conv_axis_ok(fin[f].mesh[a]);
@@ -685,14 +562,19 @@ static int build_plan(pme_plan_s* p, const std::vector<FrameInput>& fin, double 
     }
     int optin = 0;
     if (conv) {
-      optin = smem_attribute(cudaDevAttrMaxSharedMemoryPerBlockOptin);
+      int dev = 0;
+      cudaGetDevice(&dev);
+      if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
+        cudaGetLastError();
+        optin = 0;
+      }
       conv = smem_plane + 1024 <= size_t(optin) && smem_x + 1024 <= size_t(optin);
     }
     if (!conv && (p->opts.fft == 2 || p->opts.fft == 3))
       return set_error(p, PME_ERR_UNSUPPORTED, "fft = 2 / 3: a mesh the library's transforms do not take");
     // automatic choice, planes too large for a block: the line kernels where every axis is 64,
     // 128 or 256 points
-    p->conv_line = wanted && !conv && p->opts.fft == 0 && single && line_axes_ok(fin[0].mesh);
+    p->conv_line = !conv && p->opts.fft == 0 && single && line_axes_ok(fin[0].mesh);
     p->conv = conv || p->conv_line;
     p->conv_p2 = conv && p2;
     // two register steps per transform where every axis splits and the layout fits (it is a
@@ -848,17 +730,14 @@ static int build_plan(pme_plan_s* p, const std::vector<FrameInput>& fin, double 
     G.count = int(groups[gi].size());
     G.mesh_off = mesh_off;
     G.spec_off = spec_off;
-    G.apart = !p->conv && p->opts.recip_method == 0 && batch_mixes(G.N, std::min(2 * G.count, 4));
-    G.mesh_stride = G.apart ? (M + 1) & ~1LL : M;   // (apart: every mesh aligned as the first)
-    G.spec_stride = Mh;
     for (int k = 0; k < G.count; ++k) {
       FrameDesc& D = p->frames_h[groups[gi][k]];
-      D.mesh_off = mesh_off + k * G.mesh_stride;
-      D.tmesh_off = mesh_off + (G.count + k) * G.mesh_stride;
+      D.mesh_off = mesh_off + k * M;
+      D.tmesh_off = mesh_off + (G.count + k) * M;
       D.spec_off = spec_off + k * Mh;
       D.tspec_off = spec_off + (G.count + k) * Mh;
     }
-    mesh_off += 2LL * G.count * G.mesh_stride;
+    mesh_off += 2LL * G.count * M;
     spec_off += 2LL * G.count * Mh;
   }
   p->total_mesh = mesh_off;
@@ -953,12 +832,10 @@ static int build_plan(pme_plan_s* p, const std::vector<FrameInput>& fin, double 
   }
   if (p->opts.recip_method == 0) A(&p->gtab, size_t(gtab_total));
   A(&p->in_saved, 7 * ni);
-  A(&p->in_flags, 3);
+  A(&p->in_flags, 2);
   if (st == PME_OK) {
     p->in_diff = p->in_flags;
     p->cache_bad = p->in_flags + 1;
-    p->saved_n = p->in_flags + 2;
-    st = check_cuda(p, cudaMemset(p->in_flags, 0, 3 * sizeof(int)), "cudaMemset");
   }
   if (st) return st;
   if ((st = check_cuda(p, cudaMemset(p->flags, 0, sizeof(int)), "memset"))) return st;
@@ -1061,15 +938,15 @@ static int build_plan(pme_plan_s* p, const std::vector<FrameInput>& fin, double 
     p->maps.blk_frame = p->map_buf + 2 * Ntot + p->total_bricks;
     p->maps.item_frame = p->map_buf + 2 * Ntot + p->total_bricks + p->total_blocks;
   }
-  // cuFFT: four plans per group (two where the transforms go apart) sharing one work area
+  // cuFFT: four plans per group sharing one work area
   size_t work = 0;
   for (int gi = 0; gi < p->nfgroups && !p->conv; ++gi) {
     FFTGroup& G = p->fgroups[gi];
     int dims[3] = {G.N[0], G.N[1], G.N[2]};
     cufftHandle* hs[4] = {&G.r2c, &G.c2r, &G.r2c2, &G.c2r2};
     const cufftType ty[4] = {CUFFT_R2C, CUFFT_C2R, CUFFT_R2C, CUFFT_C2R};
-    const int batch[4] = {G.apart ? 1 : G.count, G.apart ? 1 : G.count, 2 * G.count, 2 * G.count};
-    for (int k = 0; k < (G.apart ? 2 : 4); ++k) {
+    const int batch[4] = {G.count, G.count, 2 * G.count, 2 * G.count};
+    for (int k = 0; k < 4; ++k) {
       size_t ws = 0;
       if ((st = check_fft(p, cufftCreate(hs[k]), "cufftCreate"))) return st;
       if ((st = check_fft(p, cufftSetAutoAllocation(*hs[k], 0), "cufftSetAutoAllocation"))) return st;
@@ -1083,9 +960,8 @@ static int build_plan(pme_plan_s* p, const std::vector<FrameInput>& fin, double 
     return st;
   for (int gi = 0; gi < p->nfgroups && !p->conv; ++gi) {
     FFTGroup& G = p->fgroups[gi];
-    const cufftHandle hs[4] = {G.r2c, G.c2r, G.r2c2, G.c2r2};
-    for (int k = 0; k < (G.apart ? 2 : 4); ++k)
-      if ((st = check_fft(p, cufftSetWorkArea(hs[k], p->fft_work), "cufftSetWorkArea"))) return st;
+    for (cufftHandle h : {G.r2c, G.c2r, G.r2c2, G.c2r2})
+      if ((st = check_fft(p, cufftSetWorkArea(h, p->fft_work), "cufftSetWorkArea"))) return st;
   }
   if (p->gtab && ((st = launch_influence_tables(p, 0)) || (st = check_cuda(p, cudaDeviceSynchronize(), "synchronize"))))
     return st;
@@ -1110,12 +986,9 @@ static int fft_forward(pme_plan_t p, cudaStream_t s, bool tangent, const int* ke
   int st;
   for (int gi = 0; gi < p->nfgroups; ++gi) {
     FFTGroup& G = p->fgroups[gi];
-    cufftHandle h = tangent && !G.apart ? G.r2c2 : G.r2c;
+    cufftHandle h = tangent ? G.r2c2 : G.r2c;
     if ((st = check_fft(p, cufftSetStream(h, s), "set stream"))) return st;
-    for (int k = 0; k < (G.apart ? (tangent ? 2 : 1) * G.count : 1); ++k)
-      if ((st = check_fft(p, cufftExecR2C(h, p->rho + G.mesh_off + k * G.mesh_stride,
-                                          p->spec + G.spec_off + k * G.spec_stride), "exec r2c")))
-        return st;
+    if ((st = check_fft(p, cufftExecR2C(h, p->rho + G.mesh_off, p->spec + G.spec_off), "exec r2c"))) return st;
   }
   return PME_OK;
 }
@@ -1125,12 +998,9 @@ static int fft_inverse(pme_plan_t p, cudaStream_t s, bool tangent, const int* ke
   int st;
   for (int gi = 0; gi < p->nfgroups; ++gi) {
     FFTGroup& G = p->fgroups[gi];
-    cufftHandle h = tangent && !G.apart ? G.c2r2 : G.c2r;
+    cufftHandle h = tangent ? G.c2r2 : G.c2r;
     if ((st = check_fft(p, cufftSetStream(h, s), "set stream"))) return st;
-    for (int k = 0; k < (G.apart ? (tangent ? 2 : 1) * G.count : 1); ++k)
-      if ((st = check_fft(p, cufftExecC2R(h, p->spec + G.spec_off + k * G.spec_stride,
-                                          p->phi + G.mesh_off + k * G.mesh_stride), "exec c2r")))
-        return st;
+    if ((st = check_fft(p, cufftExecC2R(h, p->spec + G.spec_off, p->phi + G.mesh_off), "exec c2r"))) return st;
   }
   return PME_OK;
 }
@@ -1627,7 +1497,6 @@ int pme_plan_set_box(pme_plan_t p, const double box[9]) {
   D.ncells = nc;
   p->g = g;
   p->fwd_n = -1;   // the saved forward belongs to the old box
-  if ((st = check_cuda(p, cudaMemset(p->saved_n, 0, sizeof(int)), "memset"))) return st;
   drop_graphs(p);  // recorded passes carry the old geometry
   std::memcpy(p->box, box, sizeof(double) * 9);
   if (p->gtab && ((st = launch_influence_tables(p, 0)) || (st = check_cuda(p, cudaDeviceSynchronize(), "synchronize"))))
@@ -2155,7 +2024,6 @@ int pme_solve(pme_plan_t p, void* stream, const float* rho, float* phi_mesh, dou
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const FFTGroup& G = p->fgroups[0];
   p->fwd_n = -1;   // the plan's rho is about to be replaced: nothing saved for a backward
-  if ((st = check_cuda(p, cudaMemsetAsync(p->saved_n, 0, sizeof(int), s), "memset"))) return st;
   if ((st = check_cuda(p, cudaMemcpyAsync(p->rho, rho, sizeof(float) * p->M, cudaMemcpyDeviceToDevice, s),
                        "copy rho")))
     return st;

@@ -160,7 +160,7 @@ __device__ __forceinline__ void store_pair_tangent(const PairRecords& pr, int de
 template <bool BATCH>
 __global__ void __launch_bounds__(kSortThreads)
 k_bin(FrameDesc one, FrameMaps maps, IonInputs in, const PassIO* io, SortBuffers sb, int tangent, int* flags,
-      const int* reuse, float* save, int ld, int* saved_n) {
+      int nbricks, int ncells, const int* reuse, float* save, int ld) {
   pdl_begin();
   if (io) in = io->in;
   static_assert(kRedItem == kSortThreads, "one ion per thread");
@@ -173,7 +173,6 @@ k_bin(FrameDesc one, FrameMaps maps, IonInputs in, const PassIO* io, SortBuffers
   // reuse: the inputs are those of the forward whose sort is still in place; only the charge
   // sums are formed
   const bool re = reuse && *reuse == 0;
-  if (!re && saved_n && item == 0 && threadIdx.x == 0) *saved_n = save ? in.n : 0;
   float qa = 0.f, qb = 0.f;
   if (re && i < hi) {
     const float qi = in.q ? in.q[i] : 0.f;
@@ -416,11 +415,11 @@ k_rank_records(FrameDesc one, FrameMaps maps, IonInputs in, const PassIO* io, So
 constexpr int kSmallIons = 384;
 constexpr int kSmallKeys = 8192;
 
-// saved / in_diff / cache_bad / list_cnt: as k_input_check (in_diff null: no check); save, saved_n: as k_bin.
+// saved / in_diff / cache_bad / list_cnt: as k_input_check (in_diff null: no check); save: as k_bin.
 __global__ void __launch_bounds__(kSmallIons)
 k_sort_small(FrameDesc one, IonInputs in, const PassIO* io, SortBuffers sb, MeshRecords mr, PairRecords pr,
              int tangent, int need_mesh, int need_pair, int* flags, int nbricks, int ncells, float* save, int ld,
-             const float* saved, const int* list_cnt, int* in_diff, int* cache_bad, int* saved_n) {
+             const float* saved, const int* list_cnt, int* in_diff, int* cache_bad) {
   pdl_begin();
   if (io) in = io->in;
   extern __shared__ __align__(16) int keys[];   // [nbricks + ncells] counts, then starts
@@ -430,7 +429,7 @@ k_sort_small(FrameDesc one, IonInputs in, const PassIO* io, SortBuffers sb, Mesh
   const Geometry& g = one.g;
   bool re = false;
   if (in_diff) {
-    bool same = *saved_n == n, lists = true;
+    bool same = true, lists = true;
     for (int k = tid; k < 3 * n; k += T) {
       same = same && __float_as_int(in.pos[k]) == __float_as_int(saved[k]);
       same = same && __float_as_int(in.mu ? in.mu[k] : 0.f) == __float_as_int(saved[4 * ld + k]);
@@ -449,7 +448,6 @@ k_sort_small(FrameDesc one, IonInputs in, const PassIO* io, SortBuffers sb, Mesh
   if (!re)
     for (int k = tid; k < nk; k += T) keys[k] = 0;
   __syncthreads();
-  if (!re && saved_n && tid == 0) *saved_n = save ? n : 0;
   // keys and arrival slots of this thread's ion (n <= T)
   const int i = tid;
   int kb = 0, kc = 0, slot_b = 0, slot_c = 0, m0[3], c[3];
@@ -563,14 +561,13 @@ k_sort_small(FrameDesc one, IonInputs in, const PassIO* io, SortBuffers sb, Mesh
   }
 }
 
-// Bitwise comparison of the backward's inputs with the saved forward inputs (which count only while
-// that forward's state is in place: *saved_n == n).
+// Bitwise comparison of the backward's inputs with the saved forward inputs.
 __global__ void __launch_bounds__(256)
 k_input_check(int n, IonInputs in, const PassIO* io, const float* saved, int ld, const int* list_cnt, int* in_diff,
-              int* cache_bad, const int* saved_n) {
+              int* cache_bad) {
   pdl_begin();
   if (io) in = io->in;
-  bool same = *saved_n == n, lists = true;
+  bool same = true, lists = true;
   const int stride = gridDim.x * blockDim.x;
   const int t0 = blockIdx.x * blockDim.x + threadIdx.x;
   for (int k = t0; k < 3 * n; k += stride) {
@@ -602,7 +599,7 @@ int launch_input_check(pme_plan_t p, cudaStream_t s, const IonInputs& in, bool w
   if (st || in.n == 0) return st;
   const int grid = std::min(4 * device_sm_count(), (3 * in.n + 255) / 256);
   pdl_launch(k_input_check, grid, 256, 0, s, in.n, in, live_io(p), p->in_saved, p->max_ions, with_lists ? p->plist_cnt : nullptr,
-                                      p->in_diff, p->cache_bad, p->saved_n);
+                                      p->in_diff, p->cache_bad);
   count_launch();
   return check_launch(p, "k_input_check");
 }
@@ -627,7 +624,7 @@ int launch_sort_t(pme_plan_t p, cudaStream_t s, const IonInputs& in, bool tangen
                live_io(p), p->sb, p->mr, p->pr, tangent ? 1 : 0, need_mesh ? 1 : 0, need_pair ? 1 : 0, p->flags,
                p->total_bricks, p->total_cells, save, p->max_ions, check ? p->in_saved : nullptr,
                check && check_lists ? p->plist_cnt : nullptr, check ? p->in_diff : nullptr,
-               check ? p->cache_bad : nullptr, p->saved_n);
+               check ? p->cache_bad : nullptr);
     count_launch();
     return check_launch(p, "k_sort_small");
   }
@@ -640,20 +637,26 @@ int launch_sort_t(pme_plan_t p, cudaStream_t s, const IonInputs& in, bool tangen
                     "memset cell counts");
     if (st) return st;
   }
-  p->counts_clean = false;   // until k_scatter, which clears them, is launched
   {
     const int items = BATCH ? p->total_items : one.nitems;
     pdl_launch(k_bin<BATCH>, items, kSortThreads, 0, s, one, p->maps, in, live_io(p), p->sb, tangent ? 1 : 0, p->flags,
-                                                reuse, save, p->max_ions, p->saved_n);
+                                                p->total_bricks, p->total_cells, reuse, save,
+                                                p->max_ions);
     count_launch();
-    if ((st = check_launch(p, "k_bin"))) return st;
+    if ((st = check_launch(p, "k_bin"))) {
+      p->counts_clean = false;
+      return st;
+    }
     const int nb = (p->total_bricks + scan_segment(p->total_bricks) - 1) / scan_segment(p->total_bricks);
     const int nc = (p->total_cells + scan_segment(p->total_cells) - 1) / scan_segment(p->total_cells);
     const int nq = p->sb.qpart ? (p->nframes + kScanThreads / 32 - 1) / (kScanThreads / 32) : 0;
     pdl_launch(k_scan<BATCH>, nb + nc + nq, kScanThreads, 0, s, one, p->maps, p->nframes, p->sb, p->total_bricks,
                p->total_cells, nb, nc, reuse);
     count_launch();
-    if ((st = check_launch(p, "k_scan"))) return st;
+    if ((st = check_launch(p, "k_scan"))) {
+      p->counts_clean = false;
+      return st;
+    }
   }
   if (nblk > 0) {
     const int clear = (std::max(p->total_bricks, p->total_cells) / 4 + kSortThreads - 1) / kSortThreads;
@@ -668,7 +671,6 @@ int launch_sort_t(pme_plan_t p, cudaStream_t s, const IonInputs& in, bool tangen
     count_launch();
     if ((st = check_launch(p, "k_rank_records"))) return st;
   }
-  p->counts_clean = true;
   return PME_OK;
 }
 
