@@ -303,6 +303,10 @@ struct FFTGroup {
   int N[3];
   int count;
   long long mesh_off, spec_off;
+  long long mesh_stride, spec_stride;   // from one member's mesh (half spectrum) to the next
+  // transforms of the members' meshes and, r2c2 and c2r2, of their tangent meshes too; with apart
+  // set, r2c and c2r transform one mesh each and the other two do not exist (see batch_mixes)
+  bool apart;
   cufftHandle r2c, c2r, r2c2, c2r2;
 };
 
