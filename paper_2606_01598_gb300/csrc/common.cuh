@@ -371,9 +371,14 @@ struct pme_plan_s {
   int plist_cap = 0;
   // inputs of the last forward, kept with its sorted order and records for the backward
   float* in_saved = nullptr;   // [7 max_ions]: positions, then q at 3 max_ions, mu at 4 max_ions
-  int* in_flags = nullptr;     // [2]: in_diff, cache_bad (see launch_input_check)
+  int* in_flags = nullptr;     // [3]: in_diff, cache_bad (see launch_input_check), saved_n
   int* in_diff = nullptr;
   int* cache_bad = nullptr;
+  // Ions of the forward whose inputs are in in_saved while its order, records, Phi and lists are in
+  // place, else 0: kept by the passes themselves as they run on the device (fwd_n says what was
+  // enqueued last, which a caller's own graph of captured passes does not follow). A saving forward
+  // sets it; every other pass that sorts or writes rho clears it.
+  int* saved_n = nullptr;
   bool counts_clean = false;   // the sort's count arrays are zero (each scatter re-zeroes them)
   int fwd_n = -1;              // ions of that forward (-1: nothing saved / no longer valid)
   // virial partial sums

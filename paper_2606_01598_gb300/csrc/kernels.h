@@ -34,12 +34,14 @@ inline const PassIO* live_io(pme_plan_t p) { return p->io_live ? p->io_d : nullp
 
 // sort.cu: brick and pair-cell counting sorts (4 kernels), records in both orders.
 // reuse (nullable, the plan's in_diff): the inputs are first compared with the saved ones bit for
-// bit: *in_diff = 1 unless they are equal, *cache_bad = 1 when *in_diff or (check_lists) a
+// bit: *in_diff = 1 unless they are equal and the saved forward's state is in place (*saved_n == n),
+// *cache_bad = 1 when *in_diff or (check_lists) a
 // recorded pair list overflowed, both 0 otherwise. When *reuse is then 0 the plan's sorted order
 // and primal records are those of these inputs (a forward on them) and are kept; only charge sums
 // and tangent records are formed. A sort without reuse clears the plan's saved-forward state.
 // save (nullable): the binning pass also copies the inputs there (positions at 0, charges at
-// 3 max_ions, dipoles at 4 max_ions) for a later backward's comparison.
+// 3 max_ions, dipoles at 4 max_ions) for a later backward's comparison. A sort that forms a new order
+// sets *saved_n to n with save and to 0 without.
 // The count arrays must be zero unless p->counts_clean is false (then they are cleared here).
 int launch_sort(pme_plan_t p, cudaStream_t s, const IonInputs& in, bool tangent, bool need_mesh,
                 bool need_pair, const int* reuse, float* save = nullptr, bool check_lists = false);

@@ -933,10 +933,12 @@ static int build_plan(pme_plan_s* p, const std::vector<FrameInput>& fin, double 
   }
   if (p->opts.recip_method == 0) A(&p->gtab, size_t(gtab_total));
   A(&p->in_saved, 7 * ni);
-  A(&p->in_flags, 2);
+  A(&p->in_flags, 3);
   if (st == PME_OK) {
     p->in_diff = p->in_flags;
     p->cache_bad = p->in_flags + 1;
+    p->saved_n = p->in_flags + 2;
+    st = check_cuda(p, cudaMemset(p->in_flags, 0, 3 * sizeof(int)), "cudaMemset");
   }
   if (st) return st;
   if ((st = check_cuda(p, cudaMemset(p->flags, 0, sizeof(int)), "memset"))) return st;
@@ -1605,6 +1607,7 @@ int pme_plan_set_box(pme_plan_t p, const double box[9]) {
   D.ncells = nc;
   p->g = g;
   p->fwd_n = -1;   // the saved forward belongs to the old box
+  if ((st = check_cuda(p, cudaMemset(p->saved_n, 0, sizeof(int)), "memset"))) return st;
   drop_graphs(p);  // recorded passes carry the old geometry
   std::memcpy(p->box, box, sizeof(double) * 9);
   if (p->gtab && ((st = launch_influence_tables(p, 0)) || (st = check_cuda(p, cudaDeviceSynchronize(), "synchronize"))))
@@ -2132,6 +2135,7 @@ int pme_solve(pme_plan_t p, void* stream, const float* rho, float* phi_mesh, dou
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const FFTGroup& G = p->fgroups[0];
   p->fwd_n = -1;   // the plan's rho is about to be replaced: nothing saved for a backward
+  if ((st = check_cuda(p, cudaMemsetAsync(p->saved_n, 0, sizeof(int), s), "memset"))) return st;
   if ((st = check_cuda(p, cudaMemcpyAsync(p->rho, rho, sizeof(float) * p->M, cudaMemcpyDeviceToDevice, s),
                        "copy rho")))
     return st;

@@ -160,7 +160,7 @@ __device__ __forceinline__ void store_pair_tangent(const PairRecords& pr, int de
 template <bool BATCH>
 __global__ void __launch_bounds__(kSortThreads)
 k_bin(FrameDesc one, FrameMaps maps, IonInputs in, const PassIO* io, SortBuffers sb, int tangent, int* flags,
-      int nbricks, int ncells, const int* reuse, float* save, int ld) {
+      const int* reuse, float* save, int ld, int* saved_n) {
   pdl_begin();
   if (io) in = io->in;
   static_assert(kRedItem == kSortThreads, "one ion per thread");
@@ -173,6 +173,7 @@ k_bin(FrameDesc one, FrameMaps maps, IonInputs in, const PassIO* io, SortBuffers
   // reuse: the inputs are those of the forward whose sort is still in place; only the charge
   // sums are formed
   const bool re = reuse && *reuse == 0;
+  if (!re && saved_n && item == 0 && threadIdx.x == 0) *saved_n = save ? in.n : 0;
   float qa = 0.f, qb = 0.f;
   if (re && i < hi) {
     const float qi = in.q ? in.q[i] : 0.f;
@@ -415,11 +416,11 @@ k_rank_records(FrameDesc one, FrameMaps maps, IonInputs in, const PassIO* io, So
 constexpr int kSmallIons = 384;
 constexpr int kSmallKeys = 8192;
 
-// saved / in_diff / cache_bad / list_cnt: as k_input_check (in_diff null: no check); save: as k_bin.
+// saved / in_diff / cache_bad / list_cnt: as k_input_check (in_diff null: no check); save, saved_n: as k_bin.
 __global__ void __launch_bounds__(kSmallIons)
 k_sort_small(FrameDesc one, IonInputs in, const PassIO* io, SortBuffers sb, MeshRecords mr, PairRecords pr,
              int tangent, int need_mesh, int need_pair, int* flags, int nbricks, int ncells, float* save, int ld,
-             const float* saved, const int* list_cnt, int* in_diff, int* cache_bad) {
+             const float* saved, const int* list_cnt, int* in_diff, int* cache_bad, int* saved_n) {
   pdl_begin();
   if (io) in = io->in;
   extern __shared__ __align__(16) int keys[];   // [nbricks + ncells] counts, then starts
@@ -429,7 +430,7 @@ k_sort_small(FrameDesc one, IonInputs in, const PassIO* io, SortBuffers sb, Mesh
   const Geometry& g = one.g;
   bool re = false;
   if (in_diff) {
-    bool same = true, lists = true;
+    bool same = *saved_n == n, lists = true;
     for (int k = tid; k < 3 * n; k += T) {
       same = same && __float_as_int(in.pos[k]) == __float_as_int(saved[k]);
       same = same && __float_as_int(in.mu ? in.mu[k] : 0.f) == __float_as_int(saved[4 * ld + k]);
@@ -448,6 +449,7 @@ k_sort_small(FrameDesc one, IonInputs in, const PassIO* io, SortBuffers sb, Mesh
   if (!re)
     for (int k = tid; k < nk; k += T) keys[k] = 0;
   __syncthreads();
+  if (!re && saved_n && tid == 0) *saved_n = save ? n : 0;
   // keys and arrival slots of this thread's ion (n <= T)
   const int i = tid;
   int kb = 0, kc = 0, slot_b = 0, slot_c = 0, m0[3], c[3];
@@ -561,13 +563,14 @@ k_sort_small(FrameDesc one, IonInputs in, const PassIO* io, SortBuffers sb, Mesh
   }
 }
 
-// Bitwise comparison of the backward's inputs with the saved forward inputs.
+// Bitwise comparison of the backward's inputs with the saved forward inputs (which count only while
+// that forward's state is in place: *saved_n == n).
 __global__ void __launch_bounds__(256)
 k_input_check(int n, IonInputs in, const PassIO* io, const float* saved, int ld, const int* list_cnt, int* in_diff,
-              int* cache_bad) {
+              int* cache_bad, const int* saved_n) {
   pdl_begin();
   if (io) in = io->in;
-  bool same = true, lists = true;
+  bool same = *saved_n == n, lists = true;
   const int stride = gridDim.x * blockDim.x;
   const int t0 = blockIdx.x * blockDim.x + threadIdx.x;
   for (int k = t0; k < 3 * n; k += stride) {
@@ -599,7 +602,7 @@ int launch_input_check(pme_plan_t p, cudaStream_t s, const IonInputs& in, bool w
   if (st || in.n == 0) return st;
   const int grid = std::min(4 * device_sm_count(), (3 * in.n + 255) / 256);
   pdl_launch(k_input_check, grid, 256, 0, s, in.n, in, live_io(p), p->in_saved, p->max_ions, with_lists ? p->plist_cnt : nullptr,
-                                      p->in_diff, p->cache_bad);
+                                      p->in_diff, p->cache_bad, p->saved_n);
   count_launch();
   return check_launch(p, "k_input_check");
 }
@@ -624,7 +627,7 @@ int launch_sort_t(pme_plan_t p, cudaStream_t s, const IonInputs& in, bool tangen
                live_io(p), p->sb, p->mr, p->pr, tangent ? 1 : 0, need_mesh ? 1 : 0, need_pair ? 1 : 0, p->flags,
                p->total_bricks, p->total_cells, save, p->max_ions, check ? p->in_saved : nullptr,
                check && check_lists ? p->plist_cnt : nullptr, check ? p->in_diff : nullptr,
-               check ? p->cache_bad : nullptr);
+               check ? p->cache_bad : nullptr, p->saved_n);
     count_launch();
     return check_launch(p, "k_sort_small");
   }
@@ -640,8 +643,7 @@ int launch_sort_t(pme_plan_t p, cudaStream_t s, const IonInputs& in, bool tangen
   {
     const int items = BATCH ? p->total_items : one.nitems;
     pdl_launch(k_bin<BATCH>, items, kSortThreads, 0, s, one, p->maps, in, live_io(p), p->sb, tangent ? 1 : 0, p->flags,
-                                                p->total_bricks, p->total_cells, reuse, save,
-                                                p->max_ions);
+                                                reuse, save, p->max_ions, p->saved_n);
     count_launch();
     if ((st = check_launch(p, "k_bin"))) {
       p->counts_clean = false;
