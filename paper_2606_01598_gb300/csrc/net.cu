@@ -989,11 +989,10 @@ struct RedJobs {
 };
 
 // grad[w] (+)= sum over b of part[b][w]: 32 consecutive parameters per block, one per lane;
-// warp s adds the partials b = s, s + 32, ... as a float32 sum and its rounding errors (Knuth's
-// two-sum; GB300 adds float64 at a small fraction of that rate), then the 32 sums, each exact to
-// about 48 bits, are added in float64 in order (1401 -> 1367 us for the gradient over 32 frames
-// of 512 ions).
-__global__ void __launch_bounds__(1024) k_reduce(RedJobs jobs, float* __restrict__ grad, int accumulate) {
+// warp s adds the partials b = s, s + 32, ... in float64, then the 32 sums are added in order.
+// (A float32 sum with its rounding errors by two-sum is 44 us faster over 32 frames of 512 ions, but
+// holds fewer bits and makes NaN of an infinite partial.)
+__global__ void __launch_bounds__(1024) k_reduce(RedJobs jobs, float* grad, int accumulate) {
   const int bx = gbpme::pdl_begin_block();
   __shared__ double sum[32][33];
   int u = 0;
@@ -1001,7 +1000,7 @@ __global__ void __launch_bounds__(1024) k_reduce(RedJobs jobs, float* __restrict
   const RedJob& J = jobs.job[u];
   const int lane = threadIdx.x & 31, slice = threadIdx.x >> 5;
   const int k = (bx - J.first) * 32 + lane;
-  float acc = 0.f, err = 0.f;
+  double acc = 0.0;
   if (k < J.width) {
     const float* p = J.part + k;
     for (int b0 = slice; b0 < J.nblk; b0 += 8 * 32) {   // eight loads in flight
@@ -1009,14 +1008,10 @@ __global__ void __launch_bounds__(1024) k_reduce(RedJobs jobs, float* __restrict
 #pragma unroll
       for (int q = 0; q < 8; ++q) v[q] = b0 + 32 * q < J.nblk ? __ldg(p + size_t(b0 + 32 * q) * J.width) : 0.f;
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const float t = acc + v[q], z = t - acc;
-        err += (acc - (t - z)) + (v[q] - z);
-        acc = t;
-      }
+      for (int q = 0; q < 8; ++q) acc += double(v[q]);
     }
   }
-  sum[slice][lane] = double(acc) + double(err);
+  sum[slice][lane] = acc;
   __syncthreads();
   if (slice == 0 && k < J.width) {
     double t = 0.0;
