@@ -36,6 +36,9 @@ int device_sm_count();
 // their memory is visible (griddepcontrol.wait), then lets the next grid be scheduled
 // (griddepcontrol.launch_dependents), so consecutive kernels of a pass overlap only in their
 // launch and scheduling, never in their memory accesses. Outside such a launch both are no-ops.
+// A kernel so launched is resident while the grid before it writes, so non-coherent loads (__ldg,
+// const __restrict__ parameters), defined only on memory that nothing writes while their kernel
+// runs, are for tables that no pass writes; what passes hand on is read with plain loads.
 __device__ __forceinline__ void pdl_begin() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -440,7 +440,7 @@ constexpr int p2_plane_entries() {
 }
 
 template <int NY, int NZ>
-__device__ __forceinline__ void r2c_plane_p2(const float* __restrict__ src, float2* __restrict__ dst,
+__device__ __forceinline__ void r2c_plane_p2(const float* src, float2* dst,
                                              const float2* __restrict__ tz, const float2* __restrict__ ty,
                                              float2* sm) {
   constexpr int NP = NY / 2, LS = NZ + 8, NZH = NZ / 2 + 1, BZ = NZ / 8, BY = NY / 8;
@@ -505,7 +505,7 @@ __device__ __forceinline__ void r2c_plane_p2(const float* __restrict__ src, floa
 }
 
 template <int NY, int NZ>
-__device__ __forceinline__ void c2r_plane_p2(const float2* __restrict__ src, float* __restrict__ dst,
+__device__ __forceinline__ void c2r_plane_p2(const float2* src, float* dst,
                                              const float2* __restrict__ tz, const float2* __restrict__ ty,
                                              float2* sm) {
   constexpr int NP = NY / 2, LS = NZ + 8, NZH = NZ / 2 + 1, BZ = NZ / 8, BY = NY / 8;

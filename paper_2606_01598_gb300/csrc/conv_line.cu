@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(kLineThreads) k_line_r2c(ConvArgs a, int block
     const float* r0 = src + pr * 2 * NZ + t;
     float2 v[P];
 #pragma unroll
-    for (int m = 0; m < P; ++m) v[m] = make_float2(__ldg(r0 + Q * m), __ldg(r0 + NZ + Q * m));
+    for (int m = 0; m < P; ++m) v[m] = make_float2(r0[Q * m], r0[NZ + Q * m]);
     line_step1<P, false>(v, t, tz);
 #pragma unroll
     for (int k = 0; k < P; ++k) csm[pr * RS + k * QO + t] = v[k];

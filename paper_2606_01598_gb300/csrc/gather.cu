@@ -191,11 +191,11 @@ __global__ void __launch_bounds__(kGatherThreads) k_gather(GatherArgs a) {
       for (int jy = 0; jy < P; ++jy) {
         const int off = xo + yo[jy];
         const bool in_mesh = index_ok((long long)off, Mtot);
-        const float v = in_mesh ? __ldg(phi_mesh + off) : 0.f;
+        const float v = in_mesh ? phi_mesh[off] : 0.f;
 #pragma unroll
         for (int b = 0; b <= DM; ++b) r[b] += v * wy[jy][b];
         if (TAN) {
-          const float dv = in_mesh ? __ldg(dphi_mesh + off) : 0.f;
+          const float dv = in_mesh ? dphi_mesh[off] : 0.f;
 #pragma unroll
           for (int b = 0; b < 3; ++b) rt[b] += dv * wy[jy][b];
         }
@@ -453,8 +453,8 @@ __global__ void __launch_bounds__(kGatherThreads) k_gather_qdual(GatherArgs a) {
         if (y >= Ny) y -= Ny;
         const size_t off = (size_t(x) * Ny + y) * Nz + z;
         const bool in_mesh = index_ok((long long)off, Mtot);
-        const float v = in_mesh ? __ldg(phi_mesh + off) : 0.f;
-        const float dv = in_mesh ? __ldg(dphi_mesh + off) : 0.f;
+        const float v = in_mesh ? phi_mesh[off] : 0.f;
+        const float dv = in_mesh ? dphi_mesh[off] : 0.f;
 #pragma unroll
         for (int b = 0; b < 5; ++b) r[b] += v * wy[b][jy];
 #pragma unroll

@@ -134,8 +134,8 @@ struct Nbr {
 
 // One warp per ion: every other ion of the frame within r_c (nearest image), compacted in
 // increasing j order.
-__global__ void k_nbr(const NetFrame* __restrict__ frames, const int* __restrict__ frame_of,
-                      const float* __restrict__ pos, int n, int* cnt, int* nj, float4* nsh, int* flags) {
+__global__ void k_nbr(const NetFrame* __restrict__ frames, const int* frame_of,
+                      const float* pos, int n, int* cnt, int* nj, float4* nsh, int* flags) {
   const int bx = gbpme::pdl_begin_block();
   const int i = bx * kWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (i >= n) return;
@@ -321,7 +321,7 @@ __device__ __forceinline__ Vec3<T> ldrow3(const float* p, int j, int c, size_t p
 // is too and is neither formed nor read.
 template <typename T, bool FIRST>
 __global__ void __launch_bounds__(32 * kWarps, sizeof(T) > 4 ? 3 : 4)
-k_msg_fwd(MsgArgs a, const float* __restrict__ A, const float* __restrict__ B, float* ms, float* mv) {
+k_msg_fwd(MsgArgs a, const float* A, const float* B, float* ms, float* mv) {
   const int bx = gbpme::pdl_begin_block();
   constexpr int VEC = EdgeRec<T, false>::kVec;
   __shared__ float4 srec[kWarps][32 * VEC];
@@ -386,8 +386,8 @@ k_msg_fwd(MsgArgs a, const float* __restrict__ A, const float* __restrict__ B, f
 // the parameters. FIRST: B is zero and its cotangent unused, as in k_msg_fwd.
 template <typename T, bool POS, bool GA, bool GRAD, bool FIRST>
 __global__ void __launch_bounds__(32 * kWarps, sizeof(T) > 4 || GRAD ? 2 : 3)
-k_msg_bwd(MsgArgs a, const float* __restrict__ A, const float* __restrict__ B, const float* __restrict__ gms,
-          const float* __restrict__ gmv, float* gA_out, float* gB_out, float* gpos, float* wr_part) {
+k_msg_bwd(MsgArgs a, const float* A, const float* B, const float* gms,
+          const float* gmv, float* gA_out, float* gB_out, float* gpos, float* wr_part) {
   const int bx = gbpme::pdl_begin_block();
   constexpr int VEC = EdgeRec<T, POS>::kVec;
   constexpr int kRecFloats = kWarps * 32 * VEC * 4, kPartFloats = kWarps * NR * NCOL;
@@ -591,22 +591,32 @@ __global__ void k_embed(const float* __restrict__ P, const int* __restrict__ spe
 // One thread per (ion, scalar channel); the first 16 also do the vector channel. hv_in null:
 // zero (the first layer).
 template <typename T>
-__global__ void k_update_fwd(int n, const float* __restrict__ U, const float* __restrict__ Y,
-                             const float* __restrict__ hs_in, const float* __restrict__ hv_in, float* hs_out,
+__global__ void k_update_fwd(int n, const float* U, const float* Y,
+                             const float* hs_in, const float* hv_in, float* hs_out,
                              float* hv_out, size_t plU, size_t plY, size_t plS, size_t plV) {
   const int bx = gbpme::pdl_begin_block();
   const size_t t = size_t(bx) * blockDim.x + threadIdx.x;
   if (t >= size_t(n) * S) return;
   const size_t i = t / S;
   const int c = int(t % S);
-  stT(hs_out, t, plS, ldT<T>(hs_in, t, plS) + siluT(ldT<T>(U, i * (S + V) + c, plU)));
+  // (every load before the first store: the compiler cannot move them past one)
+  const T h = ldT<T>(hs_in, t, plS), u = ldT<T>(U, i * (S + V) + c, plU);
+  T ug = 0.f, y[3], v[3];
   if (c < V) {
-    const T g = sigmoidT(ldT<T>(U, i * (S + V) + S + c, plU));
+    ug = ldT<T>(U, i * (S + V) + S + c, plU);
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      const size_t k = (i * 3 + a) * V + c;
-      const T gy = g * ldT<T>(Y, k, plY);
-      stT(hv_out, k, plV, hv_in ? ldT<T>(hv_in, k, plV) + gy : gy);
+      y[a] = ldT<T>(Y, (i * 3 + a) * V + c, plY);
+      if (hv_in) v[a] = ldT<T>(hv_in, (i * 3 + a) * V + c, plV);
+    }
+  }
+  stT(hs_out, t, plS, h + siluT(u));
+  if (c < V) {
+    const T g = sigmoidT(ug);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      const T gy = g * y[a];
+      stT(hv_out, (i * 3 + a) * V + c, plV, hv_in ? v[a] + gy : gy);
     }
   }
 }
@@ -614,24 +624,32 @@ __global__ void k_update_fwd(int n, const float* __restrict__ U, const float* __
 // Reverse of k_update_fwd: g_U [n][48], g_Y [n][3][16] from the output cotangents g_hs, g_hv
 // (which also pass unchanged to the layer input through the residual).
 template <typename T>
-__global__ void k_update_bwd(int n, const float* __restrict__ U, const float* __restrict__ Y,
-                             const float* __restrict__ ghs, const float* __restrict__ ghv, float* gU, float* gY,
+__global__ void k_update_bwd(int n, const float* U, const float* Y,
+                             const float* ghs, const float* ghv, float* gU, float* gY,
                              size_t plU, size_t plY, size_t plS, size_t plV) {
   const int bx = gbpme::pdl_begin_block();
   const size_t t = size_t(bx) * blockDim.x + threadIdx.x;
   if (t >= size_t(n) * S) return;
   const size_t i = t / S;
   const int c = int(t % S);
-  stT(gU, i * (S + V) + c, plU, ldT<T>(ghs, t, plS) * dsiluT(ldT<T>(U, i * (S + V) + c, plU)));
+  const T gs = ldT<T>(ghs, t, plS), u = ldT<T>(U, i * (S + V) + c, plU);
+  T ug = 0.f, gh[3], y[3];   // every load before the first store, as in k_update_fwd
   if (c < V) {
-    const T g = sigmoidT(ldT<T>(U, i * (S + V) + S + c, plU));
+    ug = ldT<T>(U, i * (S + V) + S + c, plU);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      gh[a] = ldT<T>(ghv, (i * 3 + a) * V + c, plV);
+      y[a] = ldT<T>(Y, (i * 3 + a) * V + c, plY);
+    }
+  }
+  stT(gU, i * (S + V) + c, plU, gs * dsiluT(u));
+  if (c < V) {
+    const T g = sigmoidT(ug);
     T acc = 0.f;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      const size_t k = (i * 3 + a) * V + c;
-      const T gh = ldT<T>(ghv, k, plV);
-      acc += gh * ldT<T>(Y, k, plY);
-      stT(gY, k, plY, gh * g);
+      acc += gh[a] * y[a];
+      stT(gY, (i * 3 + a) * V + c, plY, gh[a] * g);
     }
     stT(gU, i * (S + V) + S + c, plU, acc * (g * (1.f - g)));
   }
@@ -639,8 +657,8 @@ __global__ void k_update_bwd(int n, const float* __restrict__ U, const float* __
 
 // Readouts of one warp per ion: q~ (before neutralisation), site energy, dipole.
 template <typename T>
-__global__ void k_readout_fwd(int n, const float* __restrict__ P, const float* __restrict__ H,
-                              const float* __restrict__ hv, float* qt, float* ei, float* mu, size_t plH,
+__global__ void k_readout_fwd(int n, const float* __restrict__ P, const float* H,
+                              const float* hv, float* qt, float* ei, float* mu, size_t plH,
                               size_t plV, size_t pln) {
   const int bx = gbpme::pdl_begin_block();
   const int i = bx * kWarps + (threadIdx.x >> 5), c = threadIdx.x & 31;
@@ -667,8 +685,8 @@ __global__ void k_readout_fwd(int n, const float* __restrict__ P, const float* _
 // One block per frame: q = q~ - mean(q~) (both planes for Dual) and E_sr = sum of site
 // energies (float64, value only).
 template <typename T>
-__global__ void k_frame_fwd(const NetFrame* __restrict__ frames, const float* __restrict__ qt,
-                            const float* __restrict__ ei, float* q, double* esr, size_t pln) {
+__global__ void k_frame_fwd(const NetFrame* __restrict__ frames, const float* qt,
+                            const float* ei, float* q, double* esr, size_t pln) {
   const int bx = gbpme::pdl_begin_block();
   const NetFrame F = frames[bx];
   double sq = 0.0, sqd = 0.0, se = 0.0;
@@ -709,7 +727,7 @@ __global__ void k_frame_fwd(const NetFrame* __restrict__ frames, const float* __
 
 // Per-frame mean of the charge cotangent (both planes): the reverse of the neutralisation.
 template <typename T>
-__global__ void k_frame_mean(const NetFrame* __restrict__ frames, const float* __restrict__ g, float* mean,
+__global__ void k_frame_mean(const NetFrame* __restrict__ frames, const float* g, float* mean,
                              size_t pln) {
   const int bx = gbpme::pdl_begin_block();
   const NetFrame F = frames[bx];
@@ -834,11 +852,11 @@ struct WgJobs {
 __device__ __forceinline__ int wg_group(int k, int g) { return k * kWgSub + 4 * (g ^ (((k >> 2) + 2 * (k & 3)) & 7)); }
 
 template <int C>
-__device__ __forceinline__ void wg_stage(const float* __restrict__ src, int r0, int rows, float* dst) {
+__device__ __forceinline__ void wg_stage(const float* src, int r0, int rows, float* dst) {
   for (int e = threadIdx.x; e < kWgSub * C / 4; e += kWgThreads) {
     const int r = e / (C / 4), k = 4 * (e % (C / 4));
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (r0 + r < rows) v = __ldg(reinterpret_cast<const float4*>(src + size_t(r0 + r) * C + k));
+    if (r0 + r < rows) v = *reinterpret_cast<const float4*>(src + size_t(r0 + r) * C + k);
     const int g = r >> 2, o = r & 3;
     dst[wg_group(k, g) + o] = v.x;
     dst[wg_group(k + 1, g) + o] = v.y;
@@ -1006,7 +1024,7 @@ __global__ void __launch_bounds__(1024) k_reduce(RedJobs jobs, float* grad, int 
     for (int b0 = slice; b0 < J.nblk; b0 += 8 * 32) {   // eight loads in flight
       float v[8];
 #pragma unroll
-      for (int q = 0; q < 8; ++q) v[q] = b0 + 32 * q < J.nblk ? __ldg(p + size_t(b0 + 32 * q) * J.width) : 0.f;
+      for (int q = 0; q < 8; ++q) v[q] = b0 + 32 * q < J.nblk ? p[size_t(b0 + 32 * q) * J.width] : 0.f;
 #pragma unroll
       for (int q = 0; q < 8; ++q) acc += double(v[q]);
     }
@@ -1029,10 +1047,10 @@ __global__ void __launch_bounds__(1024) k_reduce(RedJobs jobs, float* grad, int 
 // Per frame (one block each): E_b = E_pme,b + E_sr,b; energy cotangent c_b; per ion: the
 // model force F = F_pme - g_pos(net), the force residual and the position tangent r' = -w.
 // part[f] = (L_E, L_F) contributions of frame f (float64).
-__global__ void k_loss(const NetFrame* __restrict__ frames, int nframes, int ntot, const double* __restrict__ e_pme,
-                       const double* __restrict__ e_sr, const double* __restrict__ e_ref,
-                       const float* __restrict__ f_pme, const float* __restrict__ gpos_net,
-                       const float* __restrict__ f_ref, double lambda_e, double lambda_f, double* cvec,
+__global__ void k_loss(const NetFrame* __restrict__ frames, int nframes, int ntot, const double* e_pme,
+                       const double* e_sr, const double* e_ref,
+                       const float* f_pme, const float* gpos_net,
+                       const float* f_ref, double lambda_e, double lambda_f, double* cvec,
                        float* force, float* dpos, float* wneg, double* part) {
   const int bx = gbpme::pdl_begin_block();
   const NetFrame F = frames[bx];
@@ -1058,7 +1076,7 @@ __global__ void k_loss(const NetFrame* __restrict__ frames, int nframes, int nto
   }
 }
 
-__global__ void k_loss_total(const double* __restrict__ part, int nframes, double* loss) {
+__global__ void k_loss_total(const double* part, int nframes, double* loss) {
   const int bx = gbpme::pdl_begin_block();
   double le = 0.0, lf = 0.0;   // one block
   for (int f = bx + int(threadIdx.x); f < nframes; f += blockDim.x) {
@@ -1076,7 +1094,7 @@ __global__ void k_loss_total(const double* __restrict__ part, int nframes, doubl
 }
 
 // energy cotangent seeds of the Dual backward: gesr[2 f] = 1, gesr[2 f + 1] = c_f
-__global__ void k_seed_esr(int nframes, const double* __restrict__ cvec, float* gesr, int with_tangent) {
+__global__ void k_seed_esr(int nframes, const double* cvec, float* gesr, int with_tangent) {
   const int bx = gbpme::pdl_begin_block();
   const int f = bx * blockDim.x + threadIdx.x;
   if (f >= nframes) return;
@@ -1085,14 +1103,14 @@ __global__ void k_seed_esr(int nframes, const double* __restrict__ cvec, float* 
 }
 
 // dst[k] = s * src[k] (and optionally a second array into the tangent plane of dst)
-__global__ void k_scale(size_t m, const float* __restrict__ src, float s, float* dst) {
+__global__ void k_scale(size_t m, const float* src, float s, float* dst) {
   const int bx = gbpme::pdl_begin_block();
   const size_t t = size_t(bx) * blockDim.x + threadIdx.x;
   if (t < m) dst[t] = s * src[t];
 }
 
 // bfloat16 copies of the channel-mixing matrices: W [K][N] and W^T [N][K]
-__global__ void k_cast_weights(const float* __restrict__ P, uint16_t* wbf, const int* __restrict__ offs) {
+__global__ void k_cast_weights(const float* P, uint16_t* wbf, const int* __restrict__ offs) {
   const int bx = gbpme::pdl_begin_block();
   const int w = blockIdx.y;
   const MixW m = mix_w(w);
@@ -1107,8 +1125,8 @@ __global__ void k_cast_weights(const float* __restrict__ P, uint16_t* wbf, const
   }
 }
 
-__global__ void k_adam(int np, float* __restrict__ P, float* __restrict__ m, float* __restrict__ v,
-                       const float* __restrict__ g, float lr, float b1, float b2, float eps, float c1, float c2) {
+__global__ void k_adam(int np, float* P, float* m, float* v,
+                       const float* g, float lr, float b1, float b2, float eps, float c1, float c2) {
   const int bx = gbpme::pdl_begin_block();
   const int t = bx * blockDim.x + threadIdx.x;
   if (t >= np) return;
@@ -1427,7 +1445,7 @@ int build_neighbours(gbnet_t net, cudaStream_t s, const float* pos) {
   return PME_OK;
 }
 
-__global__ void k_gesr_from(int nframes, const double* __restrict__ g, float* out) {
+__global__ void k_gesr_from(int nframes, const double* g, float* out) {
   const int bx = gbpme::pdl_begin_block();
   const int f = bx * blockDim.x + threadIdx.x;
   if (f >= nframes) return;

@@ -100,7 +100,7 @@ __device__ __forceinline__ void mix_tile(const MixJob& J, int tile, int* err, un
   unsigned char* sA_hi = smem;
   unsigned char* sA_lo = smem + kBytesA;
   unsigned char* sB = smem + 2 * kBytesA;
-  const float* __restrict__ X = J.X;
+  const float* X = J.X;
   const int M = J.M;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -123,7 +123,7 @@ __device__ __forceinline__ void mix_tile(const MixJob& J, int tile, int* err, un
 #pragma unroll
   for (int u = 0; u < K / 4; ++u) {
     const int e = tid + u * kTile;
-    xv[u] = (e * 4) / K < rows_left ? __ldg(X4 + e) : make_float4(0.f, 0.f, 0.f, 0.f);
+    xv[u] = (e * 4) / K < rows_left ? X4[e] : make_float4(0.f, 0.f, 0.f, 0.f);
   }
 #pragma unroll
   for (int u = 0; u < K / 4; ++u) {
@@ -140,7 +140,7 @@ __device__ __forceinline__ void mix_tile(const MixJob& J, int tile, int* err, un
   const uint2* W2 = reinterpret_cast<const uint2*>(J.Wt);
   for (int e = tid; e < NOUT * K / 4; e += kTile) {
     const int n = (e * 4) / K, k = (e * 4) % K;
-    *reinterpret_cast<uint2*>(sB + kmajor_off(n, k, K)) = __ldg(W2 + e);
+    *reinterpret_cast<uint2*>(sB + kmajor_off(n, k, K)) = W2[e];
   }
   // make the generic-proxy shared-memory writes visible to the tensor cores (async proxy)
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
