@@ -432,7 +432,7 @@ static int dalloc(pme_plan_t p, T** ptr, size_t count) {
 // them 16 bytes at a time).
 static size_t scan_entries(int n) { return (size_t(n) + 1 + 3) & ~size_t(3); }
 
-// The cell counts start zero (each scan re-zeroes them).
+// The cell counts start zero (each scatter re-zeroes them).
 static int alloc_cells(pme_plan_t p) {
   int st;
   if ((st = dalloc(p, &p->sb.count_c, scan_entries(p->total_cells)))) return st;

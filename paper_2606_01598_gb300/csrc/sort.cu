@@ -640,25 +640,20 @@ int launch_sort_t(pme_plan_t p, cudaStream_t s, const IonInputs& in, bool tangen
                     "memset cell counts");
     if (st) return st;
   }
+  p->counts_clean = false;   // until k_scatter, which clears them, is launched
   {
     const int items = BATCH ? p->total_items : one.nitems;
     pdl_launch(k_bin<BATCH>, items, kSortThreads, 0, s, one, p->maps, in, live_io(p), p->sb, tangent ? 1 : 0, p->flags,
                                                 reuse, save, p->max_ions, p->saved_n);
     count_launch();
-    if ((st = check_launch(p, "k_bin"))) {
-      p->counts_clean = false;
-      return st;
-    }
+    if ((st = check_launch(p, "k_bin"))) return st;
     const int nb = (p->total_bricks + scan_segment(p->total_bricks) - 1) / scan_segment(p->total_bricks);
     const int nc = (p->total_cells + scan_segment(p->total_cells) - 1) / scan_segment(p->total_cells);
     const int nq = p->sb.qpart ? (p->nframes + kScanThreads / 32 - 1) / (kScanThreads / 32) : 0;
     pdl_launch(k_scan<BATCH>, nb + nc + nq, kScanThreads, 0, s, one, p->maps, p->nframes, p->sb, p->total_bricks,
                p->total_cells, nb, nc, reuse);
     count_launch();
-    if ((st = check_launch(p, "k_scan"))) {
-      p->counts_clean = false;
-      return st;
-    }
+    if ((st = check_launch(p, "k_scan"))) return st;
   }
   if (nblk > 0) {
     const int clear = (std::max(p->total_bricks, p->total_cells) / 4 + kSortThreads - 1) / kSortThreads;
@@ -673,6 +668,7 @@ int launch_sort_t(pme_plan_t p, cudaStream_t s, const IonInputs& in, bool tangen
     count_launch();
     if ((st = check_launch(p, "k_rank_records"))) return st;
   }
+  p->counts_clean = true;
   return PME_OK;
 }
 
