@@ -388,7 +388,7 @@ static void free_plan(pme_plan_t p) {
                   p->plist, p->plist_cnt, p->in_saved, p->in_flags, p->vpart,
                   p->pvir, p->vitem, p->gtab, p->sb.t_bidx, p->sb.t_bfq,
                   p->sb.t_bdm, p->sb.t_cidx, p->sb.t_cfq, p->sb.t_cmu, p->conv_tw,
-                  p->conv_planes1, p->quad_out, p->io_d};
+                  p->conv_planes1, p->quad_out, p->qb_mesh, p->qb_pair, p->io_d};
   for (void* b : bufs)
     if (b) cudaFree(b);
   for (int g = 0; g < p->nfgroups; ++g) {
