@@ -631,6 +631,16 @@ def _scale_signed(plan, g, a, b, c):
     return out
 
 
+def _has_memory(t):
+    """Whether t holds its values itself: a tensor batched by vmap (is_grads_batched, jacobian with
+    vectorize=True) does not, and no kernel can be pointed at it."""
+    try:
+        t.data_ptr()
+    except RuntimeError:
+        return False
+    return True
+
+
 class _PMEGrad(torch.autograd.Function):
     """(pos, q, mu) -> gE (dE/dr, dE/dq, dE/dmu) from the forward's force, phi and field; its VJP
     is gE times the Hessian-vector product (and the inner product with the gradient for gE).
@@ -679,6 +689,10 @@ class PMEEnergy(torch.autograd.Function):
     @staticmethod
     def backward(ctx, gE):
         pos, q, mu, F, phi, field = ctx.saved_tensors
+        if not _has_memory(gE):   # the product as a torch operation, which has a batching rule
+            one = torch.ones((), dtype=torch.float64, device=F.device)
+            g = gE.to(torch.float32)
+            return (None, *(g * t for t in _PMEGrad.apply(ctx.plan, pos, q, mu, F, phi, field, one)))
         return (None, *_PMEGrad.apply(ctx.plan, pos, q, mu, F, phi, field, gE))
 
 
