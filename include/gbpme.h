@@ -103,8 +103,10 @@ typedef struct {
                               mesh takes the power-of-two kernels, for single frames whose
                               axes are 64, 128 or 256 points (line by line where the planes do
                               not fit in shared memory), for single frames whose
-                              every axis is a product of two of 1-6, 8, 9, 10, 12, 15, 16, and
-                              for batched plans whose meshes have no axis above 64 points (one
+                              every axis is a product of two of 1-6, 8, 9, 10, 12, 15, 16 and
+                              whose planes, where they take more than half of an SM's shared
+                              memory, are no more than the SMs (or two axes are multiples of 45
+                              or 75), and for batched plans whose meshes have no axis above 64 points (one
                               launch per pass for all frames), cuFFT otherwise.
                               1: always cuFFT. 2: always the library's own
                               (PME_ERR_UNSUPPORTED where they do not apply). 3: the library's

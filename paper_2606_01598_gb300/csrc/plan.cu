@@ -484,19 +484,40 @@ struct FrameInput {
 
 // Whether the options ask for the hand-written transforms: fft 2 and 3 always; fft 0
 // (automatic) whenever every frame takes the power-of-two kernels (axes of 64 or 128 points),
-// for single frames whose every axis splits into two register steps (two_step_factors), and
-// for batched plans of small meshes (no axis above kConvAutoMaxAxis), whose frames then share
+// for single frames whose every axis splits into two register steps (two_step_factors) unless their
+// planes go over the device in a second wave (planes_overflow), and for batched plans of small meshes (no axis above kConvAutoMaxAxis), whose frames then share
 // one launch per pass instead of a cuFFT plan per mesh shape. The axis lengths and
 // shared-memory sizes are checked by the caller (a mesh whose planes do not fit goes to the line
 // kernels where its axes are 64, 128 or 256 points, to cuFFT otherwise).
 // Measured on GB300, solve of one frame, three plans in turn (us), two-step kernels against
 // cuFFT's six plus the influence pass: 32^3 20.5 / 25.9, 48^3 21.2 / 26.0, 80x81x90 28.9 / 31.5,
-// 96^3 30.8 / 36.9, 100^3 36.2 / 33.6, 144^3 51.0 / 56.7, 150^3 60.7 / 90.1, 160^3 92.8 / 85.4.
-// The two sizes where cuFFT's solve is a little faster are taken too: a backward on the
-// forward's inputs transforms one mesh here and two there, and the passes are three launches
-// instead of seven. The six lengths without two such factors stay with cuFFT (125^3: 71.9 on
-// the Stockham kernels, 52.0 on cuFFT).
+// 96^3 30.8 / 36.9, 100^3 36.2 / 33.6, 144^3 51.0 / 56.7, 150^3 60.7 / 90.1. (100^3 is taken: the
+// forward beside its pair term costs the same, 94.5 / 95.1, and forward + backward less, 193.7 /
+// 201.8, since a backward on the forward's inputs transforms one mesh here and two there.) The six
+// lengths without two such factors stay with cuFFT (125^3: 71.9 on the Stockham kernels, 52.0 on cuFFT).
 constexpr int kConvAutoMaxAxis = 64;
+
+static int smem_attribute(cudaDeviceAttr which) {
+  int dev = 0, bytes = 0;
+  if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&bytes, which, dev) == cudaSuccess) return bytes;
+  cudaGetLastError();
+  return 0;
+}
+
+// Planes that take more than half of an SM's shared memory run one to an SM, and where there are more
+// of them than SMs the rest go in a second wave that leaves most of the device idle. Forward with
+// the pair term, then forward + backward (us), two-step kernels / cuFFT: 160x120x120 199 / 184 and
+// 394 / 398, 160x128x128 220 / 203 and 433 / 429, 160^3 255 / 238 and 485 / 520, 192x128x128 233 /
+// 218 and 456 / 462, 256x128x128 234 / 220 and 461 / 473; so cuFFT takes these. It is slow itself
+// where two axes or more are multiples of 45 or 75: 160x135x135 234 / 242 and 459 / 538, 160x150x150
+// 244 / 241 and 471 / 532. One wave: 150x128x128 190 / 191 and 385 / 411, 160x108x108 156 / 157 and
+// 313 / 337.
+static bool planes_overflow(const int N[3]) {
+  int slow = 0;
+  for (int a = 0; a < 3; ++a) slow += N[a] % 45 == 0 || N[a] % 75 == 0;
+  return slow < 2 && N[0] > device_sm_count() &&
+         2 * two_plane_smem(N, 1) > size_t(smem_attribute(cudaDevAttrMaxSharedMemoryPerMultiprocessor));
+}
 
 static bool conv_wanted(const pme_plan_s* p, bool single, const std::vector<FrameInput>& fin) {
   if (p->opts.fft == 2 || p->opts.fft == 3) return true;
@@ -508,7 +529,10 @@ static bool conv_wanted(const pme_plan_s* p, bool single, const std::vector<Fram
     int P, Q;
     for (int a = 0; a < 3; ++a)
       if (!two_step_factors(fin[0].mesh[a], &P, &Q)) return false;
-    return true;
+    // planes too large for a block: the line kernels or cuFFT
+    if (two_plane_smem(fin[0].mesh, 1) + 1024 > size_t(smem_attribute(cudaDevAttrMaxSharedMemoryPerBlockOptin)))
+      return line_axes_ok(fin[0].mesh);
+    return !planes_overflow(fin[0].mesh);
   }
   for (const FrameInput& f : fin)
     for (int a = 0; a < 3; ++a)
@@ -636,7 +660,8 @@ static int build_plan(pme_plan_s* p, const std::vector<FrameInput>& fin, double 
   // every axis of every frame is 2,3,5-smooth and short enough, and a plane (pass A / C) and
   // a pass-B tile fit in shared memory
   {
-    bool conv = conv_wanted(p, single, fin);
+    const bool wanted = conv_wanted(p, single, fin);
+    bool conv = wanted;
     size_t cap = 0, smem_plane = 0, smem_x = 0, biggest = 0;
     for (int f = 0; f < F && conv; ++f) {
       for (int a = 0; a < 3; ++a) conv = conv && conv_axis_ok(fin[f].mesh[a]);
@@ -660,19 +685,14 @@ static int build_plan(pme_plan_s* p, const std::vector<FrameInput>& fin, double 
     }
     int optin = 0;
     if (conv) {
-      int dev = 0;
-      cudaGetDevice(&dev);
-      if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
-        cudaGetLastError();
-        optin = 0;
-      }
+      optin = smem_attribute(cudaDevAttrMaxSharedMemoryPerBlockOptin);
       conv = smem_plane + 1024 <= size_t(optin) && smem_x + 1024 <= size_t(optin);
     }
     if (!conv && (p->opts.fft == 2 || p->opts.fft == 3))
       return set_error(p, PME_ERR_UNSUPPORTED, "fft = 2 / 3: a mesh the library's transforms do not take");
     // automatic choice, planes too large for a block: the line kernels where every axis is 64,
     // 128 or 256 points
-    p->conv_line = !conv && p->opts.fft == 0 && single && line_axes_ok(fin[0].mesh);
+    p->conv_line = wanted && !conv && p->opts.fft == 0 && single && line_axes_ok(fin[0].mesh);
     p->conv = conv || p->conv_line;
     p->conv_p2 = conv && p2;
     // two register steps per transform where every axis splits and the layout fits (it is a
@@ -1041,7 +1061,7 @@ static int build_plan(pme_plan_s* p, const std::vector<FrameInput>& fin, double 
     p->maps.blk_frame = p->map_buf + 2 * Ntot + p->total_bricks;
     p->maps.item_frame = p->map_buf + 2 * Ntot + p->total_bricks + p->total_blocks;
   }
-  // cuFFT: four plans per group sharing one work area
+  // cuFFT: four plans per group (two where the transforms go apart) sharing one work area
   size_t work = 0;
   for (int gi = 0; gi < p->nfgroups && !p->conv; ++gi) {
     FFTGroup& G = p->fgroups[gi];
