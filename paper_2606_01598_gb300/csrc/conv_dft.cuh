@@ -41,7 +41,7 @@ __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
 // The odd radices' sums in packed instructions (f32x2: both parts in one issue slot, each rounded
 // as alone), and a + i s b crosswise as scalar multiply-adds (a pair with its halves exchanged would
 // have to be moved first). The two-step kernels issue more than they wait: forward + backward of
-// the uneven batch of 256 frames 1069.5 -> 1064.2 us, forward with virial on 80x81x90 94.0 -> 93.4 us.
+// the uneven batch of 256 frames 1069.5 -> 1064.2 us.
 // Power-of-two DFTs stay scalar: packed too, 128^3 lost what the batch gained (258 -> 260.5 us).
 __device__ __forceinline__ float2 padd(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 psub(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }

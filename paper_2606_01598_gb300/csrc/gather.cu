@@ -292,7 +292,8 @@ __global__ void __launch_bounds__(kGatherThreads) k_gather(GatherArgs a) {
     // The gradients are linear in the moments, so each lane contracts its own z-plane's with the
     // ion's vectors and only the seven results are reduced over the lanes.
     // (Reduced first, the thirty moments took three shuffles each and the contraction ran in one
-    // lane of P: forward + backward of 262144 ions 1592 -> 1575 us, of 32768 ions 253.9 -> 252.9 us.)
+    // lane of P: forward + backward of 262144 ions 1592 -> 1575 us, of 32768 ions 253.9 -> 252.9 us,
+    // before the list kernels had their own L1 split.)
     const float gE = a.g_energy ? float(a.g_energy[frame]) : 0.f;
     const float4 dm = a.mr.dm[ion];   // m = D^T mu
     const float4 tq = a.mr.tq[ion];   // dq, dd = D^T (dmu + q dr)

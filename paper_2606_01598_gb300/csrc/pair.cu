@@ -754,7 +754,8 @@ __global__ void __launch_bounds__(kPairThreads) k_pair_listed(PairArgs a, int n)
 
 // The list kernels read their partners' records at random beside the mesh passes, whose tiles leave
 // little L1; from eight waves on they take their own split (forward + backward of 262144 ions, 21
-// and 31 waves: 1592 -> 1559 us; of 32768 ions, 2.7 and 3.8 waves: 253.9 -> 254.6 us).
+// and 31 waves: 1592 -> 1559 us; of 32768 ions, 2.7 and 3.8 waves: 253.9 -> 254.6 us; both before the
+// tangent gather contracted its moments).
 template <auto K, typename... Args>
 void launch_l1(int grid, cudaStream_t s, Args... args) {
   launch_with(false, own_split<K>(grid, kPairThreads, 8), K, grid, kPairThreads, 0, s, args...);
